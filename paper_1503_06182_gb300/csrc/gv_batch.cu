@@ -450,7 +450,8 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
     std::vector<double> e((size_t)x.d * (nbins + 1));
     for (int a = 0; a < x.d; ++a)
       for (int i = 0; i <= nbins; ++i) e[(size_t)a * (nbins + 1) + i] = (double)i / nbins;
-    if (cudaMemcpy(x.grid, e.data(), e.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
+    if (cudaMemcpy(x.grid + GvGridLayout{x.d, nbins}.off_e64(), e.data(), e.size() * 8,
+                   cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(x.par, x.params, sizeof x.params, cudaMemcpyHostToDevice) != cudaSuccess ||
         gv::launch_grid_pack(x.d, nbins, x.grid, B->stream) != cudaSuccess ||
         gv::launch_consts(x.ig, x.par, x.kconst, B->stream) != cudaSuccess ||
@@ -486,7 +487,9 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
           acc += B->m[b].n_tiles;
           start.push_back(acc);
           c.smem = std::max(c.smem,
-                            GvFillSmem(B->m[b].d, nbins, B->fp32 ? 4 : 8, true, maxd > 4).total);
+                            GvFillSmem(B->m[b].d, nbins, B->fp32 ? 4 : 8, true, maxd > 4, 0, false,
+                                       false, true)
+                                .total);
         }
         c.total = acc;
         B->cls.push_back(c);
@@ -690,7 +693,8 @@ int vegas_batch_grid_get(const vegas_batch* B, int index, double* edges) {
   if (!B || !edges || index < 0 || index >= B->n) return VEGAS_EINVAL;
   const Member& x = B->m[index];
   GB_TRY(cudaStreamSynchronize(B->stream));
-  GB_TRY(cudaMemcpy(edges, x.grid, sizeof(double) * x.d * (B->N + 1), cudaMemcpyDeviceToHost));
+  GB_TRY(cudaMemcpy(edges, x.grid + GvGridLayout{x.d, B->N}.off_e64(),
+                    sizeof(double) * x.d * (B->N + 1), cudaMemcpyDeviceToHost));
   return VEGAS_OK;
 }
 

@@ -1024,7 +1024,7 @@ int valid_grid(const double* e, int d, int N) {
 
 int upload_grid(vegas_ctx* c, const double* edges) {
   const size_t n = (size_t)c->ndim * (c->nbins + 1);
-  GV_TRY(cudaMemcpyAsync(c->grid, edges, n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+  GV_TRY(cudaMemcpyAsync(c->grid + GvGridLayout{c->ndim, c->nbins}.off_e64(), edges, n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   GV_TRY(gv::launch_grid_pack(c->ndim, c->nbins, c->grid, c->stream));
   GV_TRY(cudaStreamSynchronize(c->stream));
   return VEGAS_OK;
@@ -1392,7 +1392,8 @@ int vegas_grid_get(const vegas_ctx* c, double* edges) {
   if (!c || !edges) return VEGAS_EINVAL;
   const size_t n = (size_t)c->ndim * (c->nbins + 1);
   GV_TRY(cudaStreamSynchronize(c->stream));
-  GV_TRY(cudaMemcpy(edges, c->grid, n * sizeof(double), cudaMemcpyDeviceToHost));
+  GV_TRY(cudaMemcpy(edges, c->grid + GvGridLayout{c->ndim, c->nbins}.off_e64(), n * sizeof(double),
+                    cudaMemcpyDeviceToHost));
   return VEGAS_OK;
 }
 

@@ -22,13 +22,12 @@
 // Bin sums carry their own scale.  The grid refinement compresses every
 // bin's share rho through ((1-rho)/(-ln rho))^alpha, which stays far from 0
 // even for rho = 1e-100, so a bin's sum needs relative, not absolute,
-// precision.  Each bin therefore has its own exponent: F_b with w^2 < 2^(2 F_b)
-// for every event of the bin (an order-free max, per tile and then over the
-// iteration).  A tile rounds each w^2 once to a multiple of 2^(2 F_tb - 56);
-// the iteration's sum aligns the tile sums to 2^(2 F_b - 88).  Alignment
-// truncates only bits ~2^-86 below the bin's largest w^2, in a fixed way, so
-// the bin sums stay launch-shape independent; one w^2 is rounded to 2^-56 of
-// its bin's scale, so a bin sum is relatively exact to 2^-45 at worst.
+// precision.  A tile adds each w^2 (exact in the FP32 form, to 2^-62 of itself
+// in the FP64 form) to a row of 22-bit limbs at absolute positions
+// (gv_limbs.cuh) and publishes a bin's sum as at least 66 bits with its own
+// exponent code; the iteration's sum aligns the tiles' to the bin's largest
+// code with 32 more bits.  Both truncations depend on the data alone, so the
+// bin sums stay launch-shape independent.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -42,7 +41,7 @@
 #define GV_NCONST 48          // derived integrand constants per integration (doubles)
 #define GV_NCONST_F32 32      // constants 0..31 in FP64, then their FP32 copies
 #define GV_MAXPARAMS 16
-#define GV_BINE_OFF 1100      // stored bin exponent F + GV_BINE_OFF (0: no nonzero weight)
+#define GV_BINE_OFF 1200      // stored bin exponent F + GV_BINE_OFF (0: no nonzero weight)
 #define GV_BIN_QBITS 56       // bits of one w^2 below its bin's scale in a tile
 #define GV_BIN_XBITS 32       // extra low bits of the iteration's bin sums
 #define GV_BIN_FB (GV_BIN_QBITS + GV_BIN_XBITS)  // bin sums in units of 2^(2F - GV_BIN_FB)
@@ -70,27 +69,27 @@ struct GvState {
   unsigned long long it0;
 };
 
+// One bin of one axis in the FP32 form, as the fill reads it.
+struct __align__(16) GvBin32 {
+  float e, w;  // edge and width in FP32
+  float jm;    // N * (e_{i+1} - e_i) = jm 2^je, jm in [1,2]
+  int je;
+};
+
 // Grid pack of one integration (device memory, rewritten by every refine):
-//   e64[d][N+1] | wd64[d][N] | jac[d][N] | e32[d][N+1] | wd32[d][N] | jm32[d][N] | je[d][N]
-// wd = e[i+1]-e[i]; jac = N*wd (the axis' Jacobian factor) = jm32 2^je with
-// jm32 in [1,2] (FP32, for the FP32 form: mantissas multiplied in FP32,
+//   bin32[d][N] (GvBin32) | e64[d][N+1] | wd64[d][N] | jac[d][N]
+// wd = e[i+1]-e[i]; jac = N*wd (the axis' Jacobian factor) = jm 2^je with
+// jm in [1,2] (FP32, for the FP32 form: mantissas multiplied in FP32,
 // exponents summed as integers, so the product has no FP32 range limit).
+// The FP32 bins are records, so that a fill stages each by one 16-byte load.
 struct GvGridLayout {
   int d, N;
-  __host__ __device__ size_t off_e64() const { return 0; }
-  __host__ __device__ size_t off_wd64() const { return (size_t)d * (N + 1); }
+  // offsets in doubles from the (256-byte aligned) start of the pack
+  __host__ __device__ size_t off_bin32() const { return 0; }
+  __host__ __device__ size_t off_e64() const { return (size_t)2 * d * N; }
+  __host__ __device__ size_t off_wd64() const { return off_e64() + (size_t)d * (N + 1); }
   __host__ __device__ size_t off_jac() const { return off_wd64() + (size_t)d * N; }
-  // 32-bit parts, counted in doubles from the start of the pack
-  __host__ __device__ size_t off_f32_base() const { return off_jac() + (size_t)d * N; }
-  // offsets of the 32-bit tables in 32-bit words from off_f32_base()
-  __host__ __device__ size_t w_e32() const { return 0; }
-  __host__ __device__ size_t w_wd32() const { return (size_t)d * (N + 1); }
-  __host__ __device__ size_t w_jm32() const { return w_wd32() + (size_t)d * N; }
-  __host__ __device__ size_t w_je() const { return w_jm32() + (size_t)d * N; }
-  __host__ __device__ size_t doubles() const {
-    const size_t nw = w_je() + (size_t)d * N;  // 32-bit words
-    return off_f32_base() + (nw + 1) / 2;
-  }
+  __host__ __device__ size_t doubles() const { return off_jac() + (size_t)d * N; }
 };
 
 // VEGAS+ data of the stratified fill: s strata per axis, nh = s^d
@@ -305,8 +304,10 @@ struct u128 {
 
 __device__ __forceinline__ u128 add128(u128 a, u128 b) {
   u128 r;
-  r.lo = a.lo + b.lo;
-  r.hi = a.hi + b.hi + (r.lo < a.lo ? 1ull : 0ull);
+  asm("add.cc.u64 %0, %2, %4;\n\t"
+      "addc.u64 %1, %3, %5;"
+      : "=l"(r.lo), "=l"(r.hi)
+      : "l"(a.lo), "l"(a.hi), "l"(b.lo), "l"(b.hi));
   return r;
 }
 
@@ -398,16 +399,9 @@ __device__ __forceinline__ u128 gv_square_fixed_dec(const GvDecoded& d, int E) {
   return gv_shift_round(v, 2 * d.e2 - 2 * E + GV_FB);
 }
 
-// x^2 2^(GV_BIN_QBITS - 2F) for |x| = m 2^e2 < 2^F, from the high word
-// P = floor(m^2 2^-42) of the square of m 2^11 (the 64 bits below the leading
-// ones of m^2, so the truncation is below 2^-62 relative): rounded half up,
-// with rs = 2F - 2 e2 - 98 >= 8, below 2^GV_BIN_QBITS.  Each value is formed
-// on its own, so the tile's sum does not depend on the event order.
+// P = floor(m^2 2^-42), the high word of the square of m 2^11.
 __device__ __forceinline__ unsigned long long gv_square_hi(unsigned long long m) {
   return __umul64hi(m << 11, m << 11);
-}
-__device__ __forceinline__ unsigned long long gv_square_bin(unsigned long long P, int rs) {
-  return rs <= 64 ? ((P >> (rs - 1)) + 1ull) >> 1 : 0ull;
 }
 
 // The same roundings as gv_fixed_dec / gv_square_fixed_dec (half up, bit for

@@ -7,18 +7,14 @@
 //           -> g(x) -> w = J g (J in FP64 in the FP64 form; FP32 mantissas
 //           with an integer exponent in the FP32 form); the bins stay in registers
 //           (d <= 4) or go to shared memory;
-//   tile scale: block max of |w| (order-free) -> E_t (in the FP32 form a
-//           32-bit max of exponents: each weight is kept as its FP32 product
-//           and Jacobian exponent, a 24-bit significand times a power of two);
-//   pass 2: w and the exact square w^2 rounded once to fixed point at the tile
-//           scale (FP32 form: from the 24-bit significand, gv_direct*);
-//           sums in 128-bit integer registers (warp shuffle + block
-//           reduction); per-bin sums of w^2, each bin with its own exponent F
-//           (an order-free shared atomicMax in pass 1), w^2 rounded once to
-//           2^(2F - 56) and added as three 22-bit limbs with 32-bit shared
-//           atomics (32-bit shared atomics run several times faster than
-//           64-bit ones here, and 10 bits of headroom cover the 1024 events of
-//           a tile).
+//   tile scale: block max of the weights' exponents (order-free): it places
+//           the window of limbs of gv_limbs.cuh;
+//   pass 2: w^2 cut once per event into 22-bit digits at absolute positions;
+//           per axis three (FP32) or four 32-bit shared atomics add them to
+//           the event's bin, and the same digits with those of w go to
+//           per-lane columns for the tile's sums of w and w^2 (32-bit shared
+//           atomics run several times faster than 64-bit ones here).  Weights
+//           below the window take a further pass.
 // With VEGAS+ (PLUS), each thread takes GV_PLUS_SEG consecutive events (one
 // range): a binary search finds its first event's hypercube, the next events
 // step across hypercube boundaries (every hypercube holds at least 2 events),
@@ -28,16 +24,15 @@
 // its range, in event order (the range's segments), which the hypercube
 // statistics add up after the iteration.
 // With a histogram of the observable (HIST), every event with w != 0 also
-// adds w and w^2 to its observable's bin, in the same limb scheme: a per-bin
-// exponent from pass 1, then w^2 as three unsigned 22-bit limbs and w as two
-// unsigned limbs and a signed top limb (two's complement, so negative weights
-// add like positive ones).
+// adds w^2 (the same digits) and w (21-bit signed digits, so negative weights
+// add like positive ones) to its observable's bin.
 // Integer sums are order-free, so the tile's result is the same for every
 // block size / events-per-thread choice.  Apart from the Jacobian product and
 // w = J g, the bookkeeping runs on the integer pipes: the FP64 pipe of this
 // chip is a small fraction of its FP32 throughput.
 #pragma once
 #include "gv_integrands.cuh"
+#include "gv_limbs.cuh"
 #include "gv_plus_stat.cuh"
 
 template <int IG>
@@ -103,26 +98,8 @@ __device__ __forceinline__ int gv_hist_bin(Real v, Real lo, Real invw, int nh) {
   return 1 + (int)t;
 }
 
-// |w| rounded to a multiple of 2^(Fs - GV_BIN_QBITS), Fs the bin's scale
-// (|w| < 2^Fs), with w's sign: |result| < 2^56.
-__device__ __forceinline__ long long gv_hist_fixed(const GvDecoded& dw, int Fs) {
-  const int r = Fs - GV_BIN_QBITS - dw.e2;  // right shift of the mantissa (>= -55)
-  unsigned long long q;
-  if (r <= 0)
-    q = dw.m << (-r);
-  else if (r < 64)
-    q = ((dw.m >> (r - 1)) + 1ull) >> 1;
-  else
-    q = 0ull;
-  return dw.neg ? -(long long)q : (long long)q;
-}
-
-// One bin of one axis as staged in shared memory.
-struct __align__(16) GvBin32 {
-  float e, w;     // edge and width in FP32
-  float jm;       // N * (e_{i+1} - e_i) = jm 2^je, jm in [1,2]
-  int je;
-};
+// One bin of one axis as staged in shared memory (FP32 form: GvBin32 of the
+// grid pack).
 struct __align__(16) GvBin64 {
   double e, w;
 };
@@ -265,19 +242,25 @@ struct GvPair<double> {
 };
 
 // Shared-memory layout of the fill kernel (bytes), 16-byte aligned pieces:
-//   hist [4][d*N] u32     per-bin sums of w^2 in three 22-bit limbs, then the
-//                         tile's bin exponents F_tb + GV_BINE_OFF (forward only)
-//   jac  [d*N]    f64     Jacobian factor N*(e_{i+1}-e_i) (FP64 form only)
+//   evs  [R][T]   u32     the events between the two passes (GvEvent), slot
+//                         k B + tid the thread's k-th event
+//   wd   [W][T]   u32     the tile's Philox words, generated before the kernel
+//                         waits for its predecessor (see below), W = 4
+//                         ceil(d/4); over evs: a thread replaces its event's
+//                         words by the event
 //   ew   [d*N]    GvBin32 (e, w, jm, je) in the FP32 form, GvBin64 (e, w) in FP64
-//   bins [d][GV_TILE] u16 (forward kernels of the d > 4 classes only)
-//   hh   [7][nhist] u32   histogram: w^2 limbs [3], w limbs [3] (the third
-//                         signed), the tile's bin exponents (with a histogram)
+//   jac  [d*N]    f64     Jacobian factor N*(e_{i+1}-e_i) (FP64 form only)
+// After the first pass the forward fill's limbs lie over what follows evs (a
+// persistent kernel keeps the grid, so there they follow it):
+//   hist [d*N][L] u32     the bins' limbs
+//   hh   [nhist][L] u32, hw [nhist][LW] i32  the histogram's limbs of w^2 and w
+//   lq   [L][32] u32, lw [rows][32] i32   the lanes' columns of w^2 and of w
+// and beside both:
+//   bins [d][T]   u16     the events' bins (d > 4 classes only)
 //   po   [GV_PLUS_WIN] i32 hypercube offsets relative to the tile (VEGAS+)
 //   ps   [GV_PLUS_WIN + GV_TILE/GV_PLUS_SEG] double2  the tile's segments
 //                         (VEGAS+): each window hypercube's first, then each
 //                         range's continuation of an earlier hypercube
-//   wd   [ceil(d/4)][GV_TILE] uint4  the tile's Philox words, generated before
-//                         the kernel waits for its predecessor (see below)
 __host__ __device__ inline size_t gv_align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
 // The forward fill generates its tile's Philox words before it waits for the
@@ -299,20 +282,41 @@ __host__ __device__ inline bool gv_fill_hoistable(bool forward, bool plus, int d
 
 #define GV_PLUS_SEGS (GV_PLUS_WIN + GV_TILE / GV_PLUS_SEG)
 
+// Words of one event between the passes (GvEvent's layout).
+__host__ __device__ constexpr int gv_event_words32(bool f64, bool reg_bins, bool plus) {
+  return f64 ? (plus ? 4 : 2) + 2 : (plus ? 4 : 3);
+}
+
 struct GvFillSmem {
-  size_t hist, jac, ew, bins, hh, po, ps, wd, total;
+  size_t wd, ew, jac, limbs, hist, hh, hw, lq, lw, bins, po, ps, total;
+  int L;
   __host__ __device__ GvFillSmem(int d, int N, int real_bytes, bool forward, bool bins_smem,
-                                 int nhist = 0, bool plus = false, bool words = false) {
+                                 int nhist = 0, bool plus = false, bool words = false,
+                                 bool keep_grid = false, int T = GV_TILE) {
     const size_t dN = (size_t)d * N;
-    hist = 0;
-    jac = gv_align16(hist + (forward ? dN * 16 : 0));
-    ew = gv_align16(jac + (real_bytes == 8 ? dN * 8 : 0));
-    bins = gv_align16(ew + dN * 16);
-    hh = gv_align16(bins + ((forward && bins_smem) ? (size_t)d * GV_TILE * 2 : 0));
-    po = gv_align16(hh + (forward ? (size_t)nhist * 7 * 4 : 0));
+    const bool f64 = real_bytes == 8;
+    L = gv_limbs(d * N);
+    const size_t evs = forward ? (size_t)gv_event_words32(f64, !bins_smem, plus) * T * 4 : 0;
+    const size_t wds = words ? (size_t)((d + 3) / 4) * 4 * T * 4 : 0;
+    wd = 0;
+    ew = wds > evs ? wds : evs;
+    jac = ew + dN * 16;
+    const size_t first = gv_align16(jac + (f64 ? dN * 8 : 0));
+    limbs = keep_grid ? first : evs;
+    hist = limbs;
+    hh = hist + (forward ? dN * L * 4 : 0);
+    hw = hh + (forward ? (size_t)nhist * L * 4 : 0);
+    lq = hw + (forward ? (size_t)nhist * gv_hist_w_limbs(f64) * 4 : 0);
+    lw = lq + (forward ? (size_t)L * 32 * 4 : 0);
+    const size_t second = gv_align16(lw + (forward ? (size_t)gv_lane_rows(f64) * 32 * 4 : 0));
+    bins = first > second ? first : second;
+    po = gv_align16(bins + ((forward && bins_smem) ? (size_t)d * T * 2 : 0));
     ps = gv_align16(po + (plus ? (size_t)GV_PLUS_WIN * 4 : 0));
-    wd = gv_align16(ps + (plus ? (size_t)GV_PLUS_SEGS * 16 : 0));
-    total = gv_align16(wd + (words ? (size_t)((d + 3) / 4) * GV_TILE * 16 : 0));
+    total = gv_align16(ps + (plus ? (size_t)GV_PLUS_SEGS * 16 : 0));
+  }
+  // bytes of the limbs, from `limbs`
+  __host__ __device__ size_t limb_bytes(int real_bytes) const {
+    return lw + (size_t)gv_lane_rows(real_bytes == 8) * 32 * 4 - limbs;
   }
 };
 
@@ -440,17 +444,12 @@ __device__ __forceinline__ void gv_stage_grid(const double* grid, int d, int N, 
                                               int nthr) {
   const GvGridLayout L{d, N};
   const int dN = d * N;
-  const float* g32 = reinterpret_cast<const float*>(grid + L.off_f32_base());
-  for (int k = tid; k < dN; k += nthr) {
-    const int a = k / N, i = k - a * N;
-    if constexpr (sizeof(Real) == 4) {
-      GvBin32 b;
-      b.e = g32[L.w_e32() + a * (N + 1) + i];
-      b.w = g32[L.w_wd32() + k];
-      b.jm = g32[L.w_jm32() + k];
-      b.je = reinterpret_cast<const int*>(g32)[L.w_je() + k];
-      s_ew[k] = b;
-    } else {
+  if constexpr (sizeof(Real) == 4) {
+    const uint4* g = reinterpret_cast<const uint4*>(grid + L.off_bin32());
+    for (int k = tid; k < dN; k += nthr) reinterpret_cast<uint4*>(s_ew)[k] = __ldcg(g + k);
+  } else {
+    for (int k = tid; k < dN; k += nthr) {
+      const int a = k / N, i = k - a * N;
       s_jac[k] = grid[L.off_jac() + k];
       GvBin64 b;
       b.e = grid[L.off_e64() + a * (N + 1) + i];
@@ -495,74 +494,6 @@ __device__ __forceinline__ GvJac<Real> gv_map_event(const uint32_t (&r)[MAXD], i
   return J;
 }
 
-// Block-wide reductions over the NW warps of a CTA (results to every thread).
-template <int NW>
-__device__ __forceinline__ unsigned long long gv_block_max(unsigned long long v,
-                                                           unsigned long long* scratch) {
-  v = warp_max_u64(v);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) scratch[wid] = v;
-  __syncthreads();
-  unsigned long long m = scratch[0];
-#pragma unroll
-  for (int w = 1; w < NW; ++w) m = scratch[w] > m ? scratch[w] : m;
-  __syncthreads();
-  return m;
-}
-
-template <int NW>
-__device__ __forceinline__ int gv_block_max_int(int v, int* scratch) {
-  v = __reduce_max_sync(0xffffffffu, v);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) scratch[wid] = v;
-  __syncthreads();
-  int m = scratch[0];
-#pragma unroll
-  for (int w = 1; w < NW; ++w) m = max(m, scratch[w]);
-  __syncthreads();
-  return m;
-}
-
-template <int NW>
-__device__ __forceinline__ u128 gv_block_sum128(u128 v, u128* scratch) {
-  v = warp_sum128(v);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) scratch[wid] = v;
-  __syncthreads();
-  u128 s = scratch[0];
-#pragma unroll
-  for (int w = 1; w < NW; ++w) s = add128(s, scratch[w]);
-  __syncthreads();
-  return s;
-}
-
-// Bins of one event between the two passes: packed u16 pairs in registers for
-// d <= 4, shared memory otherwise.
-template <int MAXD>
-struct GvBinStore {
-  static constexpr bool REG = MAXD <= 4;
-  uint32_t q[REG ? 2 : 1];
-  __device__ __forceinline__ void put(const int (&bin)[MAXD], int d, unsigned short* s_bin,
-                                      int local) {
-    if constexpr (REG) {
-      q[0] = (uint32_t)bin[0] | ((MAXD > 1 && d > 1 ? (uint32_t)bin[1] : 0u) << 16);
-      q[1] = (MAXD > 2 && d > 2 ? (uint32_t)bin[2] : 0u) |
-             ((MAXD > 3 && d > 3 ? (uint32_t)bin[3] : 0u) << 16);
-    } else {
-#pragma unroll
-      for (int a = 0; a < MAXD; ++a)
-        if (a < d) s_bin[a * GV_TILE + local] = (unsigned short)bin[a];
-    }
-  }
-  __device__ __forceinline__ int get(int a, const unsigned short* s_bin, int local) const {
-    if constexpr (REG)
-      return (int)((q[a >> 1] >> ((a & 1) * 16)) & 0xFFFFu);
-    else
-      return s_bin[a * GV_TILE + local];
-  }
-};
-
-
 // |x| bits of a double, and its finiteness, on the integer pipes.
 __device__ __forceinline__ unsigned long long gv_abs_bits(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
@@ -571,112 +502,188 @@ __device__ __forceinline__ bool gv_finite_bits(unsigned long long absbits) {
   return absbits < 0x7FF0000000000000ull;
 }
 
-// The scale exponent of the weight u 2^e (gv_scale_exp of the double) and
-// whether that double is finite.
-__device__ __forceinline__ int gv_direct_scale(unsigned u, int e, bool& fin) {
-  const GvDirect dd = gv_direct(u, e);
-  if (dd.direct) {
-    fin = true;
-    return dd.e2 + 24;
+// The significand of the FP32 form's weight u 2^e (u the bits of the FP32
+// product J.m g): 1 with w set (m in [2^23, 2^24)), 0 if the weight is zero or
+// below the FP64 normal range, -1 if it is not finite or beyond FP64 -- as the
+// double that gv_weight assembles.
+__device__ __forceinline__ int gv_sig(unsigned u, int e, GvSig<float>& w) {
+  int ef = (int)((u >> 23) & 0xFFu);
+  unsigned m = (u & 0x7FFFFFu) | 0x800000u;
+  if (ef == 0) {  // subnormal product
+    m &= 0x7FFFFFu;
+    if (m == 0u) return 0;
+    const int lz = __clz((int)m) - 8;
+    m <<= lz;
+    ef = 1 - lz;
   }
-  const unsigned long long ab = gv_abs_bits(gv_weight_bits(u, e));
-  fin = gv_finite_bits(ab);
-  return gv_scale_exp(ab);
+  const int nf = ef + 896 + e;  // the double's exponent field
+  if (ef == 0xFF || nf >= 0x7FF) return -1;
+  if (nf <= 0) return 0;
+  w.m = m;
+  w.e2 = nf - 1046;
+  w.neg = (u >> 31) != 0u;
+  return 1;
+}
+// The FP64 form's: m in [2^52, 2^53), or 0 for a zero weight.
+__device__ __forceinline__ GvSig<double> gv_sig(double x) {
+  const GvDecoded d = gv_decode(x);
+  GvSig<double> w;
+  w.m = d.m;
+  w.e2 = d.e2;
+  w.neg = d.neg;
+  if (d.e2 == -1074 && d.m != 0ull && (d.m >> 52) == 0ull) {  // subnormal
+    const int lz = __clzll((long long)d.m) - 11;
+    w.m <<= lz;
+    w.e2 -= lz;
+  }
+  return w;
+}
+
+// One event between the two passes, in shared memory (evs, array j of slot s
+// at evs[j T + s]): FP32 form, 0: sign and significand of w (0: no weight),
+// 1: e2 + GV_SQ_OFF (12 bits) | bin 0 | bin 1 (10 bits each), 2: bin 2 | bin 3
+// | the histogram's bin; with VEGAS+, 2: bin 2 | bin 3 | e2 of q, 3: q's sign
+// and significand.  FP64 form: the double w (two words), then bins 0, 1, 2
+// and bin 3 | the histogram's bin; with VEGAS+ the double q at the end.  More
+// than 4 axes: the bins in s_bin.
+template <typename Real, int MAXD, bool PLUS, int T>
+struct GvEvent {
+  static constexpr bool REG = MAXD <= 4;
+  unsigned* e;  // evs + slot
+  __device__ __forceinline__ static unsigned pack(const int (&bin)[MAXD], int d, int i, int j) {
+    unsigned r = 0u;
+    if (REG && i < MAXD && i < d) r = (unsigned)bin[i < MAXD ? i : 0];
+    if (REG && j < MAXD && j < d) r |= (unsigned)bin[j < MAXD ? j : 0] << 10;
+    return r;
+  }
+  __device__ __forceinline__ void put(const GvSig<float>& w, const GvSig<float>& q,
+                                      const int (&bin)[MAXD], int d, int hbin) const {
+    e[0] = w.m | (w.neg ? 0x80000000u : 0u);
+    e[T] = ((unsigned)(w.e2 + GV_SQ_OFF) << 20) | pack(bin, d, 0, 1);
+    if constexpr (PLUS) {
+      e[2 * T] = ((unsigned)(q.e2 + GV_SQ_OFF) << 20) | pack(bin, d, 2, 3);
+      e[3 * T] = q.m | (q.neg ? 0x80000000u : 0u);
+    } else {
+      e[2 * T] = ((unsigned)hbin << 20) | pack(bin, d, 2, 3);
+    }
+  }
+  __device__ __forceinline__ void put(double w, double q, const int (&bin)[MAXD], int d,
+                                      int hbin) const {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(w);
+    e[0] = (unsigned)b;
+    e[T] = (unsigned)(b >> 32);
+    e[2 * T] = pack(bin, d, 0, 1);
+    e[3 * T] = ((unsigned)hbin << 20) | pack(bin, d, 2, 3);
+    if constexpr (PLUS) {
+      const unsigned long long c = (unsigned long long)__double_as_longlong(q);
+      e[4 * T] = (unsigned)c;
+      e[5 * T] = (unsigned)(c >> 32);
+    }
+  }
+  __device__ __forceinline__ void none() const {
+    e[0] = 0u;
+    if constexpr (sizeof(Real) == 8) e[T] = 0u;
+    if constexpr (PLUS) e[3 * T] = 0u;
+    if constexpr (PLUS && sizeof(Real) == 8) e[4 * T] = e[5 * T] = 0u;
+  }
+  // the weight (VEGAS+: which = 1, the bins' quantity); m = 0: none
+  template <int WHICH>
+  __device__ __forceinline__ GvSig<Real> get() const {
+    if constexpr (sizeof(Real) == 4) {
+      const unsigned sm = e[WHICH ? 3 * T : 0];
+      const unsigned x = e[WHICH ? 2 * T : T];
+      return GvSig<float>{sm & 0xFFFFFFu, (int)(x >> 20) - GV_SQ_OFF, (sm >> 31) != 0u};
+    } else {
+      const unsigned long long b =
+          ((unsigned long long)e[WHICH ? 5 * T : T] << 32) | e[WHICH ? 4 * T : 0];
+      return gv_sig(__longlong_as_double((long long)b));
+    }
+  }
+  // bins 0, 1 (lo) and 2, 3 (hi), 10 bits each, for at most 4 axes
+  __device__ __forceinline__ uint2 bins() const {
+    return sizeof(Real) == 4 ? make_uint2(e[T], e[2 * T]) : make_uint2(e[2 * T], e[3 * T]);
+  }
+  __device__ __forceinline__ int hbin() const {
+    return (int)(e[sizeof(Real) == 4 ? 2 * T : 3 * T] >> 20);
+  }
+};
+
+__device__ __forceinline__ void gv_store_partial(ulonglong2* p, const GvPartial& v) {
+  *p = make_ulonglong2(v.lo, (unsigned long long)v.hi | ((unsigned long long)(unsigned)v.code << 32));
+}
+__device__ __forceinline__ GvPartial gv_load_partial(const ulonglong2* p) {
+  const ulonglong2 v = *p;
+  return GvPartial{v.x, (unsigned)v.y, (int)(v.y >> 32)};
 }
 
 // ---------------------------------------------------------------------------
 // Forward fill of one tile: channel 0 = w, with per-bin sums of w^2.  The grid
-// of the integration must be staged and the histogram zeroed (both followed
-// by a barrier) before the call.  Used by the per-integration kernel and by
-// the persistent batched kernel, so that a tile's partial is the same
-// whichever kernel computes it.
+// of the integration must be staged (followed by a barrier) before the call;
+// `words`: the tile's Philox words lie in shared memory.  Used by the
+// per-integration kernel and by the persistent batched kernel, so that a
+// tile's partial is the same whichever kernel computes it.
+//
+// Both passes are rolled loops over the thread's events, which wait between
+// them in shared memory (in the place of their words): unrolled over events in
+// registers, the loop's constants no longer fit and were loaded again for
+// every event.
 // ---------------------------------------------------------------------------
 template <int IG, typename Real, int EPT, int MAXD, bool HIST = false, bool PLUS = false>
 __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile,
-                                             unsigned char* smem, unsigned long long* red_u64,
-                                             u128* red_128, uint32_t it,
-                                             const uint4* s_words = nullptr) {
-  constexpr int B = GV_TILE / EPT;
+                                             unsigned char* smem, const GvFillSmem& lay,
+                                             uint32_t it, bool words = false) {
+  constexpr int B = GV_TILE / EPT, T = GV_TILE;
   constexpr int NW = B / 32;
+  constexpr bool F64 = sizeof(Real) == 8;
   using Pair = typename GvPair<Real>::T;
-  const int d = a.ndim, N = a.nbins, dN = d * N;
+  using Event = GvEvent<Real, MAXD, PLUS, T>;
+  __shared__ int s_max[2][NW];
+  const int d = a.ndim, N = a.nbins, dN = d * N, L = lay.L;
   const int hb = HIST ? a.nhist : 0;
-  const GvFillSmem lay(d, N, (int)sizeof(Real), true, MAXD > 4, hb, PLUS);
-  unsigned* hh = reinterpret_cast<unsigned*>(smem + lay.hh);  // [6][hb] limbs
   const int* s_off = reinterpret_cast<const int*>(smem + lay.po);
   double2* s_seg = reinterpret_cast<double2*>(smem + lay.ps);
   const GvPlusFill* pf = a.plus;
   const long long ncall = PLUS ? *pf->ncall : a.ncall;
   const long long h0 = PLUS ? pf->tile_h0[tile] : 0;
-  double qv[EPT];  // VEGAS+: the bins' quantity F b_h (w itself otherwise)
-  int* hebin = reinterpret_cast<int*>(hh + 6 * hb);             // [hb] exponents
-  Real h_lo, h_invw;
-  if constexpr (sizeof(Real) == 4) {
-    h_lo = a.h_lo_f;
-    h_invw = a.h_invw_f;
-  } else {
-    h_lo = a.h_lo;
-    h_invw = a.h_invw;
-  }
-  int hbin[EPT];
-  unsigned* hist = reinterpret_cast<unsigned*>(smem + lay.hist);  // [3][dN] limbs
-  int* ebin = reinterpret_cast<int*>(hist + 3 * dN);               // [dN] exponents
   const double* s_jac = reinterpret_cast<const double*>(smem + lay.jac);
   const Pair* s_ew = reinterpret_cast<const Pair*>(smem + lay.ew);
   unsigned short* s_bin = reinterpret_cast<unsigned short*>(smem + lay.bins);
+  unsigned* evs = reinterpret_cast<unsigned*>(smem + lay.wd);
   const int tid = threadIdx.x;
-  GvConst<Real, GvTraits<IG>::NK> K;
-  K.load(a.kconst);
+  const long long tile0 = tile * T;
+  const int n_ev = (int)min((long long)T, ncall - tile0);  // events of this tile
 
-  // FP32 form: each weight is kept as its FP32 product and Jacobian exponent
-  // and summed through gv_direct (VEGAS+: the estimate's weight in wp, the
-  // bins' quantity in wq)
-  constexpr bool DIRECT = sizeof(Real) == 4;
-  const long long tile0 = tile * GV_TILE;
-  [[maybe_unused]] double w[EPT];
-  [[maybe_unused]] unsigned wp[EPT], wq[EPT];
-  [[maybe_unused]] int wj[EPT];
-  GvBinStore<MAXD> bs[EPT];
-  unsigned long long mx = 0ull;
-  int mE = GV_EMPTY;  // the direct form's largest weight scale
-  unsigned long long nbad = 0ull;
-  // VEGAS+: this thread's range (events tile0 + tid EPT ..), the window index
-  // of its current hypercube, that hypercube's digits and factors, and the
-  // running segment sums
-  static_assert(!PLUS || EPT == GV_PLUS_SEG, "a stratified fill thread holds one range");
-  [[maybe_unused]] int jc = PLUS ? gv_plus_cube(s_off, tid * EPT) : 0;
-  [[maybe_unused]] int jcur = -1;  // the open segment's window index
-  [[maybe_unused]] double sg1 = 0.0, sg2 = 0.0;
-  constexpr bool KEEP_DIGITS = MAXD <= 4;  // registers to spare only for few axes
-  [[maybe_unused]] unsigned cdig[MAXD];
-#pragma unroll
-  for (int k = 0; k < EPT; ++k) {
-    const int local = PLUS ? tid * EPT + k : k * B + tid;
-    const long long ev = tile0 + local;
-    if constexpr (DIRECT) {
-      wp[k] = 0u;
-      wq[k] = 0u;
-      wj[k] = 0;
-    } else {
-      w[k] = 0.0;
-    }
-    if constexpr (PLUS) qv[k] = 0.0;
-    hbin[k] = 0;
-    if (ev < ncall) {
+  int mw = GV_EMPTY;                   // the largest exponent of the thread's weights
+  [[maybe_unused]] int mq = GV_EMPTY;  // and (VEGAS+) of the bins' quantities F b_h
+  {
+    GvConst<Real, GvTraits<IG>::NK> K;
+    K.load(a.kconst);
+    unsigned nbad = 0u;
+    // VEGAS+: this thread's range (events tile0 + tid EPT ..), the window index
+    // of its current hypercube, that hypercube's digits and factors, and the
+    // running segment sums
+    static_assert(!PLUS || EPT == GV_PLUS_SEG, "a stratified fill thread holds one range");
+    [[maybe_unused]] int jc = PLUS ? gv_plus_cube(s_off, tid * EPT) : 0;
+    [[maybe_unused]] int jcur = -1;  // the open segment's window index
+    [[maybe_unused]] double sg1 = 0.0, sg2 = 0.0;
+    constexpr bool KEEP_DIGITS = MAXD <= 4;  // registers to spare only for few axes
+    [[maybe_unused]] unsigned cdig[MAXD];
+#pragma unroll 1
+    for (int k = 0; k < EPT; ++k) {
+      const int local = PLUS ? tid * EPT + k : k * B + tid;
+      const int slot = k * B + tid;
+      const Event event{evs + slot};
+      if (local >= n_ev) {
+        event.none();
+        continue;
+      }
       uint32_t r[MAXD];
-      if (s_words) {  // generated before the wait (the kernel's barrier precedes this)
+      if (words) {  // generated before the wait, by this thread
 #pragma unroll
-        for (int j = 0; j < (MAXD + 3) / 4; ++j) {
-          if (4 * j < d) {
-            const uint4 o = s_words[j * GV_TILE + local];
-            if (4 * j + 0 < MAXD) r[4 * j + 0] = o.x;
-            if (4 * j + 1 < MAXD) r[4 * j + 1] = o.y;
-            if (4 * j + 2 < MAXD) r[4 * j + 2] = o.z;
-            if (4 * j + 3 < MAXD) r[4 * j + 3] = o.w;
-          }
-        }
+        for (int j = 0; j < MAXD; ++j)
+          if (j < d) r[j] = evs[j * T + slot];
       } else {
-        gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)ev, d, r);
+        gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)(tile0 + local), d, r);
       }
       if constexpr (PLUS) {
         while (jc + 1 < GV_PLUS_WIN && s_off[jc + 1] <= local) ++jc;
@@ -696,259 +703,252 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
       Real x[MAXD];
       int bin[MAXD];
       const GvJac<Real> J = gv_map_event<Real, MAXD>(r, d, N, s_jac, s_ew, x, bin);
-      bs[k].put(bin, d, s_bin, local);
+      if constexpr (!Event::REG) {
+#pragma unroll
+        for (int ax = 0; ax < MAXD; ++ax)
+          if (ax < d) s_bin[ax * T + slot] = (unsigned short)bin[ax];
+      }
       const Real g = gv_eval<IG, Real, MAXD>(x, d, K);
-      if constexpr (HIST) hbin[k] = gv_hist_bin<Real>(gv_observable<IG, Real, MAXD>(x, K), h_lo,
-                                                      h_invw, hb - 2);
-      if constexpr (DIRECT) {
+      int hbin = 0;
+      if constexpr (HIST) {
+        if constexpr (F64)
+          hbin = gv_hist_bin<Real>(gv_observable<IG, Real, MAXD>(x, K), a.h_lo, a.h_invw, hb - 2);
+        else
+          hbin = gv_hist_bin<Real>(gv_observable<IG, Real, MAXD>(x, K), a.h_lo_f, a.h_invw_f,
+                                   hb - 2);
+      }
+      if constexpr (!F64) {
         const unsigned u = __float_as_uint(__fmul_rn(J.m, g));
-        if ((u & 0x7FFFFFFFu) != 0u) {
-          // VEGAS+: the estimate's weight u a_h and the bins' quantity u b_h,
-          // FP32 products with the hypercube's factors rounded to FP32
-          unsigned uw = u, uq = u;
-          if constexpr (PLUS) {
-            const float2 f = pf->ab32[h0 + jc];
-            uw = __float_as_uint(__fmul_rn(__uint_as_float(u), f.x));
-            uq = __float_as_uint(__fmul_rn(__uint_as_float(u), f.y));
-          }
-          bool fin, finq = true;
-          const int Ev = gv_direct_scale(uw, J.e, fin);
-          int Eq = Ev;
-          if constexpr (PLUS) Eq = gv_direct_scale(uq, J.e, finq);
-          if (fin && finq) {
-            if constexpr (PLUS) {
-              // F = u 2^e, widened exactly, into the segment (a rounded
-              // product, then the sum, as the statistics define them: the
-              // variance cancels where a hypercube's values are nearly equal)
-              double Fv = gv_weight_bits(u, J.e);
-              Fv = gv_finite_bits(gv_abs_bits(Fv)) ? Fv : 0.0;
-              sg1 += Fv;
-              sg2 += Fv * Fv;
-              wq[k] = uq;
-            }
-            wp[k] = uw;
-            wj[k] = J.e;
-            if (Ev != GV_EMPTY) mE = max(mE, Ev);
-            if (Eq != GV_EMPTY) {
-              const int F = Eq + GV_BINE_OFF;
-#pragma unroll
-              for (int ax = 0; ax < MAXD; ++ax)
-                if (ax < d) atomicMax(ebin + ax * N + bin[ax], F);
-              if constexpr (HIST) atomicMax(hebin + hbin[k], F);
-            }
-          } else {
-            ++nbad;  // counted, contributes nothing
-          }
+        // VEGAS+: the estimate's weight u a_h and the bins' quantity u b_h,
+        // FP32 products with the hypercube's factors rounded to FP32
+        unsigned uw = u;
+        [[maybe_unused]] unsigned uq = u;
+        if constexpr (PLUS) {
+          const float2 f = pf->ab32[h0 + jc];
+          uw = __float_as_uint(__fmul_rn(__uint_as_float(u), f.x));
+          uq = __float_as_uint(__fmul_rn(__uint_as_float(u), f.y));
         }
-        continue;
-      }
-      double wv = gv_weight(J, g);
-      [[maybe_unused]] double qk = 0.0;
-      if constexpr (PLUS) {
-        // F = J g into the segment (0 if not finite); the estimate's weight
-        // F C/(nh n_h), the bins' F sqrt(1/(nh n_h))
-        // (a rounded product, then the sum, as the statistics define them: the
-        // variance cancels where a hypercube's values are nearly equal)
-        const double Fv = gv_finite_bits(gv_abs_bits(wv)) ? wv : 0.0;
-        sg1 += Fv;
-        sg2 += Fv * Fv;
-        const double2 f = pf->ab[h0 + jc];
-        qk = wv * f.y;
-        wv = wv * f.x;
-      }
-      const unsigned long long ab = gv_abs_bits(wv);
-      unsigned long long bb = ab;  // |the bins' quantity|
-      bool fin = gv_finite_bits(ab);
-      if constexpr (PLUS) {
-        bb = gv_abs_bits(qk);
-        fin = fin && gv_finite_bits(bb);
-      }
-      if (fin) {
-        w[k] = wv;
-        if constexpr (PLUS) qv[k] = qk;
-        mx = ab > mx ? ab : mx;
-        if (bb != 0ull) {
-          const int F = gv_scale_exp(bb) + GV_BINE_OFF;
-#pragma unroll
-          for (int ax = 0; ax < MAXD; ++ax)
-            if (ax < d) atomicMax(ebin + ax * N + bin[ax], F);
-          if constexpr (HIST) atomicMax(hebin + hbin[k], F);
+        GvSig<float> sw = {0u, 0, false}, sq = {0u, 0, false};
+        const int kw = gv_sig(uw, J.e, sw);
+        const int kq = PLUS ? gv_sig(uq, J.e, sq) : kw;
+        const bool fin = kw >= 0 && kq >= 0;
+        if constexpr (PLUS) {
+          if (fin && (u & 0x7FFFFFFFu) != 0u) {
+            // F = u 2^e, widened exactly, into the segment (a rounded
+            // product, then the sum, as the statistics define them: the
+            // variance cancels where a hypercube's values are nearly equal)
+            double Fv = gv_weight_bits(u, J.e);
+            Fv = gv_finite_bits(gv_abs_bits(Fv)) ? Fv : 0.0;
+            sg1 += Fv;
+            sg2 += Fv * Fv;
+          }
+          if (fin && kq > 0) mq = max(mq, sq.e2);
         }
-      } else {
-        ++nbad;  // counted, contributes nothing
-      }
-    }
-  }
-  if constexpr (PLUS) {
-    // the range's last segment and its first hypercube
-    if (jcur >= 0) gv_plus_put_segment(pf, s_off, s_seg, h0, jcur, tile0, tid * EPT, sg1, sg2);
-  }
-  // the tile's scale (the barrier also orders ebin)
-  int E;
-  if constexpr (DIRECT)
-    E = gv_block_max_int<NW>(mE, reinterpret_cast<int*>(red_u64));
-  else
-    E = gv_scale_exp(gv_block_max<NW>(mx, red_u64));
-
-  u128 s1 = {0ull, 0ull}, s2 = {0ull, 0ull};
-  if (E != GV_EMPTY) {
-#pragma unroll
-    for (int k = 0; k < EPT; ++k) {
-      bool any;
-      if constexpr (DIRECT)
-        any = (wp[k] & 0x7FFFFFFFu) != 0u || (PLUS && (wq[k] & 0x7FFFFFFFu) != 0u);
-      else
-        any = gv_abs_bits(w[k]) != 0ull || (PLUS && gv_abs_bits(qv[k]) != 0ull);
-      if (any) {
-        const int local = PLUS ? tid * EPT + k : k * B + tid;
-        // bins: w^2 (VEGAS+: q^2) at its bin's scale, a 56-bit value, as three
-        // 22-bit limbs, from P = floor(m^2 2^-42) of its 53-bit significand m
-        // and c = 2 e2 + 98 + 2 GV_BINE_OFF
-        unsigned long long P;
-        int c;
-        [[maybe_unused]] GvDecoded dw;
-        if constexpr (DIRECT) {
-          const GvDirect dd = gv_direct(wp[k], wj[k]);
-          if (dd.direct) {
-            const unsigned long long M = (unsigned long long)dd.m * dd.m;
-            s1 = add128(s1, gv_direct_fixed(dd.m, dd.e2 - E + GV_FB, dd.neg));
-            s2 = add128(s2, gv_direct_square(M, 2 * (dd.e2 - E) + GV_FB));
-            P = M << 16;  // m = dd.m 2^29
-            c = 2 * (dd.e2 - 29) + 98 + 2 * GV_BINE_OFF;
-            if constexpr (HIST) dw = GvDecoded{(unsigned long long)dd.m << 29, dd.e2 - 29, dd.neg};
-          } else {
-            dw = gv_decode(gv_weight_bits(wp[k], wj[k]));
-            P = gv_square_hi(dw.m);
-            c = 2 * dw.e2 + 98 + 2 * GV_BINE_OFF;
-            if (dw.m != 0ull) {
-              s1 = add128(s1, gv_fixed_tile(dw, E));
-              s2 = add128(s2, gv_square_tile(dw, P, E));
-            } else if (!PLUS) {
-              continue;  // below the FP64 range: zero
-            }
-          }
-          if constexpr (PLUS) {
-            // the bins' terms from the bins' quantity
-            const GvDirect dq = gv_direct(wq[k], wj[k]);
-            if (dq.direct) {
-              P = ((unsigned long long)dq.m * dq.m) << 16;
-              c = 2 * (dq.e2 - 29) + 98 + 2 * GV_BINE_OFF;
-            } else {
-              const GvDecoded q = gv_decode(gv_weight_bits(wq[k], wj[k]));
-              if (q.m == 0ull) continue;  // below the FP64 range: zero
-              P = gv_square_hi(q.m);
-              c = 2 * q.e2 + 98 + 2 * GV_BINE_OFF;
-            }
-          }
+        if (fin && kw > 0) mw = max(mw, sw.e2);
+        if (fin && (kw > 0 || kq > 0)) {
+          if (kw <= 0) sw = GvSig<float>{0u, 0, false};
+          if (PLUS && kq <= 0) sq = GvSig<float>{0u, 0, false};
+          event.put(sw, sq, bin, d, hbin);
         } else {
-          dw = gv_decode(w[k]);
-          const unsigned long long Pw = gv_square_hi(dw.m);
-          s1 = add128(s1, gv_fixed_tile(dw, E));
-          s2 = add128(s2, gv_square_tile(dw, Pw, E));
-          const GvDecoded dq = PLUS ? gv_decode(qv[k]) : dw;
-          P = PLUS ? gv_square_hi(dq.m) : Pw;
-          c = 2 * dq.e2 + 98 + 2 * GV_BINE_OFF;
+          event.none();
         }
-#pragma unroll
-        for (int ax = 0; ax < MAXD; ++ax) {
-          if (ax < d) {
-            const int bi = ax * N + bs[k].get(ax, s_bin, local);
-            const unsigned long long q = gv_square_bin(P, 2 * ebin[bi] - c);
-            const unsigned l0 = (unsigned)(q & 0x3FFFFFull);
-            const unsigned l1 = (unsigned)((q >> 22) & 0x3FFFFFull);
-            const unsigned l2 = (unsigned)(q >> 44);
-            if (l0) atomicAdd(hist + bi, l0);
-            if (l1) atomicAdd(hist + dN + bi, l1);
-            if (l2) atomicAdd(hist + 2 * dN + bi, l2);
-          }
+        if (!fin) ++nbad;  // counted, contributes nothing
+      } else {
+        double wv = gv_weight(J, g);
+        [[maybe_unused]] double qk = 0.0;
+        bool fin = gv_finite_bits(gv_abs_bits(wv));
+        if constexpr (PLUS) {
+          // F = J g into the segment (0 if not finite); the estimate's weight
+          // F C/(nh n_h), the bins' F sqrt(1/(nh n_h))
+          // (a rounded product, then the sum, as the statistics define them: the
+          // variance cancels where a hypercube's values are nearly equal)
+          const double Fv = fin ? wv : 0.0;
+          sg1 += Fv;
+          sg2 += Fv * Fv;
+          const double2 f = pf->ab[h0 + jc];
+          qk = wv * f.y;
+          wv = wv * f.x;
+          fin = gv_finite_bits(gv_abs_bits(wv)) && gv_finite_bits(gv_abs_bits(qk));
         }
-        if constexpr (HIST) {
-          // the observable's bin: w^2 as the axis bins, then w (signed)
-          const int hk = hbin[k];
-          const int Fh = hebin[hk];
-          const unsigned long long q = gv_square_bin(P, 2 * Fh - c);
-          const unsigned l0 = (unsigned)(q & 0x3FFFFFull);
-          const unsigned l1 = (unsigned)((q >> 22) & 0x3FFFFFull);
-          const unsigned l2 = (unsigned)(q >> 44);
-          if (l0) atomicAdd(hh + hk, l0);
-          if (l1) atomicAdd(hh + hb + hk, l1);
-          if (l2) atomicAdd(hh + 2 * hb + hk, l2);
-          const long long v = gv_hist_fixed(dw, Fh - GV_BINE_OFF);
-          const unsigned m0 = (unsigned)((unsigned long long)v & 0x3FFFFFull);
-          const unsigned m1 = (unsigned)(((unsigned long long)v >> 22) & 0x3FFFFFull);
-          const unsigned m2 = (unsigned)(int)(v >> 44);  // signed, |v >> 44| <= 2^12
-          if (m0) atomicAdd(hh + 3 * hb + hk, m0);
-          if (m1) atomicAdd(hh + 4 * hb + hk, m1);
-          if (m2) atomicAdd(hh + 5 * hb + hk, m2);
+        if (fin) {
+          event.put(wv, qk, bin, d, hbin);
+          if (gv_abs_bits(wv) != 0ull) mw = max(mw, gv_scale_exp(gv_abs_bits(wv)) - 53);
+          if constexpr (PLUS)
+            if (gv_abs_bits(qk) != 0ull) mq = max(mq, gv_scale_exp(gv_abs_bits(qk)) - 53);
+        } else {
+          event.none();
+          ++nbad;  // counted, contributes nothing
         }
       }
     }
+    if constexpr (PLUS) {
+      // the range's last segment and its first hypercube
+      if (jcur >= 0) gv_plus_put_segment(pf, s_off, s_seg, h0, jcur, tile0, tid * EPT, sg1, sg2);
+    }
+    if (nbad) atomicAdd(&a.st->nonfinite_iter, (unsigned long long)nbad);
   }
-  if constexpr (PLUS) {
-    // the hypercubes this tile holds whole (the barrier of the tile's scale
-    // ordered the staged segments)
-    __shared__ double2 s_pr[PLUS ? B : 1];
-    gv_plus_tile_stats<B>(pf, s_off, s_seg, h0, tile, s_pr);
-  }
-  const u128 t1 = gv_block_sum128<NW>(s1, red_128);
-  const u128 t2 = gv_block_sum128<NW>(s2, red_128);
-  gv_allow_next_grid();
+
+  // pass 2, once for each window of limbs (one, unless weights lie below it)
+  unsigned* hist = reinterpret_cast<unsigned*>(smem + lay.hist);  // [dN][L]
+  [[maybe_unused]] unsigned* hh = reinterpret_cast<unsigned*>(smem + lay.hh);  // [hb][L]
+  [[maybe_unused]] int* hw = reinterpret_cast<int*>(smem + lay.hw);            // [hb][HW]
+  unsigned* lq = reinterpret_cast<unsigned*>(smem + lay.lq);
+  int* lw = reinterpret_cast<int*>(smem + lay.lw);
+  constexpr int HW = gv_hist_w_limbs(F64);
+  const int lane = tid & 31, wid = tid >> 5;
+  const unsigned a_hist = gv_shared_address(hist), a_lq = gv_shared_address(lq + lane),
+                 a_lw = gv_shared_address(lw + lane);
+  [[maybe_unused]] const unsigned a_hh = gv_shared_address(hh), a_hw = gv_shared_address(hw);
+  const unsigned L4 = 4u * (unsigned)L, axis4 = L4 * (unsigned)N;  // bytes of a bin, of an axis
   // the tile's slots: slot k at out[k ks] (tile-major or slot-major partials)
   const size_t ks = a.slot_major ? (size_t)a.n_tiles : (size_t)1;
   ulonglong2* out = a.part + (a.slot_major ? (size_t)tile : (size_t)tile * a.nacc);
-  if (tid == 0) {
-    out[0] = make_ulonglong2(t1.lo, t1.hi);
-    out[ks] = make_ulonglong2(t2.lo, t2.hi);
-    a.tileE[tile] = E;
-  }
-  if (nbad) atomicAdd(&a.st->nonfinite_iter, nbad);
-  for (int k = tid; k < dN; k += B) {
-    // Q = l0 + l1 2^22 + l2 2^44 (< 2^67) in units of 2^(2 F_tb - GV_BIN_QBITS),
-    // with F_tb + GV_BINE_OFF in bits 96.. of the partial
-    const unsigned long long l0 = hist[k], l1 = hist[dN + k], l2 = hist[2 * dN + k];
-    u128 v = {l0, 0ull};
-    v = add128(v, u128{l1 << 22, l1 >> 42});
-    v = add128(v, u128{l2 << 44, l2 >> 20});
-    out[(2 + k) * ks] = make_ulonglong2(v.lo, v.hi | ((unsigned long long)(unsigned)ebin[k] << 32));
-  }
-  if constexpr (HIST) {
-    for (int k = tid; k < hb; k += B) {
-      const unsigned long long eh = (unsigned long long)(unsigned)hebin[k] << 32;
-      // w^2: as the axis bins
-      const unsigned long long l0 = hh[k], l1 = hh[hb + k], l2 = hh[2 * hb + k];
-      u128 v = {l0, 0ull};
-      v = add128(v, u128{l1 << 22, l1 >> 42});
-      v = add128(v, u128{l2 << 44, l2 >> 20});
-      out[(2 + dN + k) * ks] = make_ulonglong2(v.lo, v.hi | eh);
-      // w: M = m0 + m1 2^22 + m2 2^44 with m2 signed (|M| < 2^67) as a 96-bit
-      // two's complement value in units of 2^(F_tb - GV_BIN_QBITS)
-      const unsigned long long m0 = hh[3 * hb + k], m1 = hh[4 * hb + k];
-      const long long m2 = (long long)(int)hh[5 * hb + k];
-      u128 t = {m0, 0ull};
-      t = add128(t, u128{m1 << 22, m1 >> 42});
-      t = add128(t, u128{(unsigned long long)m2 << 44, (unsigned long long)(m2 >> 20)});
-      out[(2 + dN + hb + k) * ks] = make_ulonglong2(t.lo, (t.hi & 0xFFFFFFFFull) | eh);
+  int E = GV_EMPTY;         // the tile's scale: |w| < 2^E
+  u128 sum = {0ull, 0ull};  // warp 0: of w^2, warp 1: of w, at the tile's scale
+  // weights at limb indices of at least up_w have been added (VEGAS+: q, up_q)
+  int up_w = 0x40000000;
+  [[maybe_unused]] int up_q = 0x40000000;
+  bool first = true;
+  for (;;) {
+    mw = __reduce_max_sync(0xffffffffu, mw);
+    if constexpr (PLUS) mq = __reduce_max_sync(0xffffffffu, mq);
+    if (lane == 0) {
+      s_max[0][wid] = mw;
+      if constexpr (PLUS) s_max[1][wid] = mq;
     }
+    __syncthreads();
+    mw = __reduce_max_sync(0xffffffffu, s_max[0][lane % NW]);
+    if constexpr (PLUS) mq = __reduce_max_sync(0xffffffffu, s_max[1][lane % NW]);
+    const bool have_w = mw != GV_EMPTY, have_q = PLUS ? mq != GV_EMPTY : have_w;
+    GvWindow vw = gv_window<Real>(have_w ? mw : 0, L);
+    GvWindow vq = PLUS ? gv_window<Real>(have_q ? mq : 0, L) : vw;
+    if (!have_w) vw.base = up_w;  // nothing (left)
+    if (PLUS && !have_q) vq.base = up_q;
+    if (first && have_w) E = mw + GvSig<Real>::BITS;
+    {
+      uint4* z = reinterpret_cast<uint4*>(smem + lay.limbs);
+      const int nz = (int)((lay.limb_bytes((int)sizeof(Real)) + 15) / 16);
+      for (int k = tid; k < nz; k += B) z[k] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    __syncthreads();
+    mw = GV_EMPTY;
+    mq = GV_EMPTY;
+#pragma unroll 1
+    for (int k = 0; k < EPT; ++k) {
+      const int slot = k * B + tid;
+      const Event event{evs + slot};
+      const auto add_bins = [&](const unsigned (&l)[4], int pos) {
+        unsigned row = a_hist + 4u * (unsigned)pos;
+        const uint2 b = Event::REG ? event.bins() : make_uint2(0u, 0u);
+#pragma unroll
+        for (int ax = 0; ax < MAXD; ++ax) {
+          if (ax < d) {
+            unsigned bin;
+            if constexpr (Event::REG)
+              bin = ((ax < 2 ? b.x : b.y) >> (10 * (ax & 1))) & 0x3FFu;
+            else
+              bin = s_bin[ax * T + slot];
+            gv_bin_add_square<Real>(l, row + bin * L4);
+            row += axis4;
+          }
+        }
+      };
+      {
+        const GvSig<Real> s = event.template get<0>();
+        const int h = s.e2 + GvSig<Real>::H;
+        const int limb = gv_limb_index(h), pos = limb - vw.base;
+        if (s.m != 0 && limb < up_w) {
+          if (pos >= 0) {
+            unsigned l[4];
+            gv_square_digits(s, h + GV_SQ_OFF - 11 * limb, l);
+            gv_lane_add_square<Real>(l, a_lq + pos * 128);
+            gv_lane_add_w(s, a_lw, vw.wbase);
+            if constexpr (!PLUS) add_bins(l, pos);
+            if constexpr (HIST) {
+              const int hbin = event.hbin();
+              gv_bin_add_square<Real>(l, a_hh + 4 * (pos + hbin * L));
+              gv_hist_add_w<Real>(s, a_hw + 4 * (hbin * HW), vw.hbase);
+            }
+          } else {
+            mw = max(mw, s.e2);
+          }
+        }
+      }
+      if constexpr (PLUS) {
+        const GvSig<Real> s = event.template get<1>();
+        const int h = s.e2 + GvSig<Real>::H;
+        const int limb = gv_limb_index(h), pos = limb - vq.base;
+        if (s.m != 0 && limb < up_q) {
+          if (pos >= 0) {
+            unsigned l[4];
+            gv_square_digits(s, h + GV_SQ_OFF - 11 * limb, l);
+            add_bins(l, pos);
+          } else {
+            mq = max(mq, s.e2);
+          }
+        }
+      }
+    }
+    const bool more = __syncthreads_or((int)(mw != GV_EMPTY || (PLUS && mq != GV_EMPTY))) != 0;
+    if (first) gv_allow_next_grid();
+    if (have_w && wid == 0) {
+      const int r0 = gv_square_row0(F64, L);
+      const u192 t = gv_lane_total<false>(lq, L, r0);
+      sum = add128(sum, gv_tile_fixed(t, 22 * (vw.base + r0) - 2 * GV_SQ_OFF - 2 * E + GV_FB));
+    } else if (have_w && wid == 1) {
+      const u192 t = gv_lane_total<true>(reinterpret_cast<const unsigned*>(lw), gv_lane_rows(F64), 0);
+      sum = add128(sum, gv_tile_fixed(t, 22 * vw.wbase - GV_SQ_OFF - E + GV_FB));
+    }
+    for (int k = tid; k < dN; k += B) {
+      ulonglong2* o = out + (2 + k) * ks;
+      GvPartial v = gv_bin_partial(hist + k * L, L, vq.base);
+      if (!first) v = gv_partial_add(v, gv_load_partial(o));
+      gv_store_partial(o, v);
+    }
+    if constexpr (HIST) {
+      for (int k = tid; k < hb; k += B) {
+        ulonglong2* o = out + (2 + dN + k) * ks;
+        GvPartial v = gv_bin_partial(hh + k * L, L, vw.base);
+        if (!first) v = gv_partial_add(v, gv_load_partial(o));
+        gv_store_partial(o, v);
+        o = out + (2 + dN + hb + k) * ks;
+        v = gv_hist_partial(hw + k * HW, HW, vw.hbase);
+        if (!first) v = gv_hist_partial_add(v, gv_load_partial(o));
+        gv_store_partial(o, v);
+      }
+    }
+    if (!more) break;
+    first = false;
+    up_w = vw.base;
+    if constexpr (PLUS) up_q = vq.base;
+  }
+  if (lane == 0 && wid < 2) out[wid == 0 ? ks : (size_t)0] = make_ulonglong2(sum.lo, sum.hi);
+  if (tid == 0) a.tileE[tile] = E;
+  if constexpr (PLUS) {
+    // the hypercubes this tile holds whole (the barriers above ordered the
+    // staged segments)
+    __shared__ double2 s_pr[PLUS ? B : 1];
+    gv_plus_tile_stats<B>(pf, s_off, s_seg, h0, tile, s_pr);
   }
 }
 
 // The Philox words of a tile's events at counter `it` into shared memory
-// (layout [ceil(d/4)][GV_TILE]); each thread makes the words of the events it
-// will evaluate (local index tid + k B), so no barrier is needed before use.
-template <int MAXD>
+// (word a of slot s at s_words[a T + s]); each thread makes the words of the
+// events it will evaluate, so no barrier is needed before use.
+template <int MAXD, int T, int B, bool PLUS>
 __device__ __forceinline__ void gv_tile_words(const GvFillArgs& a, uint32_t it, long long tile,
-                                              uint4* s_words, int B) {
+                                              unsigned* s_words) {
   const int d = a.ndim;
-  const long long t0 = tile * GV_TILE;
-  for (int local = threadIdx.x; local < GV_TILE; local += B) {
+  const long long t0 = tile * T;
+#pragma unroll 1
+  for (int k = 0; k < T / B; ++k) {
+    const int local = PLUS ? (int)threadIdx.x * (T / B) + k : k * B + (int)threadIdx.x;
+    const int slot = k * B + (int)threadIdx.x;
     uint32_t r[MAXD];
     gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)(t0 + local), d, r);
 #pragma unroll
-    for (int j = 0; j < (MAXD + 3) / 4; ++j)
-      if (4 * j < d)
-        s_words[j * GV_TILE + local] =
-            make_uint4(r[4 * j], 4 * j + 1 < MAXD ? r[4 * j + 1] : 0u,
-                       4 * j + 2 < MAXD ? r[4 * j + 2] : 0u, 4 * j + 3 < MAXD ? r[4 * j + 3] : 0u);
+    for (int j = 0; j < MAXD; ++j)
+      if (j < d) s_words[j * T + slot] = r[j];
   }
 }
 
@@ -973,28 +973,19 @@ struct GvFillBlocks {
 template <int IG, typename Real, int EPT, int MAXD, bool HIST = false, bool PLUS = false>
 __global__ void __launch_bounds__(GV_TILE / EPT, (GvFillBlocks<Real, EPT, MAXD, PLUS>::value))
     gv_fill_kernel(const GvFillArgs a) {
-  constexpr int B = GV_TILE / EPT;
-  constexpr int NW = B / 32;
+  constexpr int B = GV_TILE / EPT, T = GV_TILE;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned long long red_u64[NW];
-  __shared__ u128 red_128[NW];
   const int d = a.ndim, N = a.nbins;
   const bool hoist = MAXD <= 8 && a.hoist;  // set by the host (gv_fill_hoistable)
   const GvFillSmem lay(d, N, (int)sizeof(Real), true, MAXD > 4, HIST ? a.nhist : 0, PLUS, hoist);
-  unsigned* hist = reinterpret_cast<unsigned*>(smem + lay.hist);
-  for (int k = threadIdx.x; k < 4 * d * N; k += B) hist[k] = 0u;
-  if constexpr (HIST) {
-    unsigned* hh = reinterpret_cast<unsigned*>(smem + lay.hh);
-    for (int k = threadIdx.x; k < 7 * a.nhist; k += B) hh[k] = 0u;
-  }
   // the tile's words at the counter this iteration should have (the stage's
   // first counter, which no running kernel writes, plus the iteration index),
   // made while the previous iteration's reduce and refinement finish
-  uint4* s_words = reinterpret_cast<uint4*>(smem + lay.wd);
+  unsigned* s_words = reinterpret_cast<unsigned*>(smem + lay.wd);
   uint32_t itg = 0u;
   if (hoist) {
     itg = (uint32_t)(a.st->it0 + (unsigned long long)a.kst);
-    gv_tile_words<MAXD>(a, itg, blockIdx.x, s_words, B);
+    gv_tile_words<MAXD, T, B, PLUS>(a, itg, blockIdx.x, s_words);
   }
   gv_wait_prior_grid();  // grid, constants and iteration counter come from earlier kernels
   if constexpr (PLUS) {
@@ -1025,10 +1016,10 @@ __global__ void __launch_bounds__(GV_TILE / EPT, (GvFillBlocks<Real, EPT, MAXD, 
     }
   }
   const uint32_t it = (uint32_t)a.st->it;
-  if (hoist && it != itg) gv_tile_words<MAXD>(a, it, blockIdx.x, s_words, B);  // (not expected)
+  if (hoist && it != itg) gv_tile_words<MAXD, T, B, PLUS>(a, it, blockIdx.x, s_words);  // (not expected)
   __syncthreads();
-  gv_fill_tile<IG, Real, EPT, MAXD, HIST, PLUS>(a, blockIdx.x, smem, red_u64, red_128, it,
-                                                hoist ? s_words : nullptr);
+  gv_fill_tile<IG, Real, EPT, MAXD, HIST, PLUS>(a, blockIdx.x, smem, lay, it,
+                                                hoist);
 }
 
 // Single-event diagnostics (no shared memory): weight and bins of the given
@@ -1044,11 +1035,7 @@ __global__ void gv_eval_events_kernel(const GvFillArgs a, uint32_t it, const lon
   const double* e64 = a.grid + L.off_e64();
   const double* wd64 = a.grid + L.off_wd64();
   const double* jac = a.grid + L.off_jac();
-  const float* g32 = reinterpret_cast<const float*>(a.grid + L.off_f32_base());
-  const float* e32 = g32 + L.w_e32();
-  const float* wd32 = g32 + L.w_wd32();
-  const float* jm32 = g32 + L.w_jm32();
-  const int* je = reinterpret_cast<const int*>(g32 + L.w_je());
+  const GvBin32* b32 = reinterpret_cast<const GvBin32*>(a.grid + L.off_bin32());
   GvConst<Real, GvTraits<IG>::NK> K;
   K.load(a.kconst);
   uint32_t r[MAXD];
@@ -1064,9 +1051,9 @@ __global__ void gv_eval_events_kernel(const GvFillArgs a, uint32_t it, const lon
       const int k = ax * N + i;
       if constexpr (sizeof(Real) == 4) {
         const float f = fmaf(__uint2float_rn(lo), 0x1p-32f, 0x1p-33f);
-        x[ax] = fmaf(f, wd32[k], e32[ax * (N + 1) + i]);
-        J.m = (ax == 0) ? jm32[k] : __fmul_rn(J.m, jm32[k]);
-        J.e = (ax == 0) ? je[k] : J.e + je[k];
+        x[ax] = fmaf(f, b32[k].w, b32[k].e);
+        J.m = (ax == 0) ? b32[k].jm : __fmul_rn(J.m, b32[k].jm);
+        J.e = (ax == 0) ? b32[k].je : J.e + b32[k].je;
       } else {
         const double f = ((double)lo + 0.5) * 0x1p-32;
         x[ax] = __dadd_rn(e64[ax * (N + 1) + i], __dmul_rn(f, wd64[k]));

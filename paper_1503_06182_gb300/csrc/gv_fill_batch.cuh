@@ -20,10 +20,7 @@ __global__ void __launch_bounds__(GV_TILE / EPT,
                          const long long* __restrict__ item_start, int n, long long total,
                          unsigned long long* counter) {
   constexpr int B = GV_TILE / EPT;
-  constexpr int NW = B / 32;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned long long red_u64[NW];
-  __shared__ u128 red_128[NW];
   __shared__ long long s_item;
   __shared__ int s_pos;
   int cur = -1;
@@ -52,9 +49,7 @@ __global__ void __launch_bounds__(GV_TILE / EPT,
     const int b = order[pos];
     const long long tile = item - item_start[pos];
     const GvFillArgs a = args[b];
-    const GvFillSmem lay(a.ndim, a.nbins, (int)sizeof(Real), true, MAXD > 4);
-    unsigned* hist = reinterpret_cast<unsigned*>(smem + lay.hist);
-    for (int k = threadIdx.x; k < 4 * a.ndim * a.nbins; k += B) hist[k] = 0u;
+    const GvFillSmem lay(a.ndim, a.nbins, (int)sizeof(Real), true, MAXD > 4, 0, false, false, true);
     if (b != cur) {
       gv_stage_grid<Real>(a.grid, a.ndim, a.nbins, reinterpret_cast<double*>(smem + lay.jac),
                           reinterpret_cast<typename GvPair<Real>::T*>(smem + lay.ew),
@@ -63,7 +58,7 @@ __global__ void __launch_bounds__(GV_TILE / EPT,
     }
     const uint32_t it = (uint32_t)a.st->it;
     __syncthreads();
-    gv_fill_tile<IG, Real, EPT, MAXD>(a, tile, smem, red_u64, red_128, it);
+    gv_fill_tile<IG, Real, EPT, MAXD>(a, tile, smem, lay, it);
     __syncthreads();
   }
 }

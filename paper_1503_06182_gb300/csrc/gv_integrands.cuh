@@ -99,9 +99,15 @@ struct GvConst {
   // the constants kernel stores after them (no conversions per CTA)
   __device__ __forceinline__ void load(const double* k) {
     if constexpr (sizeof(Real) == 4) {
-      const float* kf = reinterpret_cast<const float*>(k + GV_NCONST_F32);
+      const float4* kf = reinterpret_cast<const float4*>(k + GV_NCONST_F32);
 #pragma unroll
-      for (int i = 0; i < NC; ++i) v[i] = kf[i];
+      for (int i = 0; i < NC; i += 4) {
+        const float4 q = __ldg(kf + i / 4);
+        v[i] = q.x;
+        if (i + 1 < NC) v[i + 1] = q.y;
+        if (i + 2 < NC) v[i + 2] = q.z;
+        if (i + 3 < NC) v[i + 3] = q.w;
+      }
     } else {
 #pragma unroll
       for (int i = 0; i < NC; ++i) v[i] = k[i];

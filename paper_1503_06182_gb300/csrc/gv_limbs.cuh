@@ -1,0 +1,349 @@
+// gv_limbs.cuh -- exact sums of a tile's weights and of their squares in
+// 32-bit shared-memory limbs.
+//
+// A weight is w = m 2^h with an integer significand m (24 bits in the FP32
+// form, 53 in the FP64 form).  Its square is cut into 22-bit digits at
+// absolute positions: the digit of limb index i counts units of
+// 2^(22 i - 2 GV_SQ_OFF).  The digits of one event are therefore the same for
+// every bin it falls into, and adding the event to a bin is three (FP32) or
+// four 32-bit shared atomics with no further arithmetic; 1024 events of a
+// tile leave 10 bits of headroom.  A row of L limbs per bin covers the events
+// whose limb index lies within L - 4 of the tile's largest (at L = 9: weights
+// down to 2^-55 of the tile's largest); a tile with smaller weights takes
+// them in further passes over a lower window, so no weight is lost, and the
+// passes a tile takes depend on its events alone.
+//
+// Before this, every bin of a tile had its own exponent (an atomicMax per
+// axis and event) and every event shifted and split its square once per axis:
+// about 45 instructions per axis and event against 8 now, and the tile's own
+// sums took 128-bit shifts, adds and shuffles in every thread; they now go to
+// per-lane columns of limbs with the same digits.  Bound by instruction issue
+// before and after.  One FP32 fill of 1e6 events alone, before and now (with
+// the rolled passes of gv_fill.cuh): Drell-Yan (4 axes) 28.7 and 23.3 us,
+// 685 and 490 instructions per event; NLO-shaped (13 axes) 97 and 65 us; with
+// a 60-bin histogram 34.5 and 30.1 us; 3-jet (5 axes, 3e6 events) 101 and
+// 73 us.
+#pragma once
+#include "gv_common.cuh"
+
+#define GV_LIMB_BITS 22
+#define GV_LIMB_MASK 0x3FFFFFu
+#define GV_SQ_OFF 1144  // 11 x 104: keeps every limb index positive (h >= -1126)
+#define GV_W21_OFF 1155 // 21 x 55: the histogram's 21-bit digits of w
+
+// Limbs per bin: 9 up to 1024 bins in all; above, fewer, so that the largest
+// shapes still fit shared memory.  Odd, so that consecutive bins start in
+// different banks.
+__host__ __device__ inline int gv_limbs(int dN) { return dN <= 1024 ? 9 : (dN <= 2048 ? 7 : 5); }
+// Rows of the per-lane columns of w (22-bit digits) and limbs per histogram
+// bin of w (21-bit digits), for the window of 9 limbs.
+__host__ __device__ constexpr int gv_lane_rows(bool f64) { return f64 ? 7 : 5; }
+__host__ __device__ constexpr int gv_hist_w_limbs(bool f64) { return f64 ? 9 : 7; }
+
+struct u192 {
+  unsigned long long l0, l1, l2;
+};
+
+__device__ __forceinline__ void add192(u192& r, const u192& x) {
+  asm("add.cc.u64 %0, %0, %3;\n\t"
+      "addc.cc.u64 %1, %1, %4;\n\t"
+      "addc.u64 %2, %2, %5;"
+      : "+l"(r.l0), "+l"(r.l1), "+l"(r.l2)
+      : "l"(x.l0), "l"(x.l1), "l"(x.l2));
+}
+
+// Arithmetic shift right of a 192-bit two's complement value.
+__device__ __forceinline__ u192 sar192(u192 v, int s) {
+  const unsigned long long ext = (unsigned long long)((long long)v.l2 >> 63);
+  if (s <= 0) return v;
+  if (s >= 192) return {ext, ext, ext};
+  while (s >= 64) {
+    v.l0 = v.l1;
+    v.l1 = v.l2;
+    v.l2 = ext;
+    s -= 64;
+  }
+  if (s > 0) {
+    v.l0 = (v.l0 >> s) | (v.l1 << (64 - s));
+    v.l1 = (v.l1 >> s) | (v.l2 << (64 - s));
+    v.l2 = (unsigned long long)((long long)v.l2 >> s);
+  }
+  return v;
+}
+
+// Left shift by 0 <= s < 64 (callers keep the result below 2^190).
+__device__ __forceinline__ u192 shl192(u192 v, int s) {
+  if (s <= 0) return v;
+  v.l2 = (v.l2 << s) | (v.l1 >> (64 - s));
+  v.l1 = (v.l1 << s) | (v.l0 >> (64 - s));
+  v.l0 <<= s;
+  return v;
+}
+
+// Adds v to the 32-bit word at shared-memory address p + OFF (p as
+// gv_shared_address gives it): one instruction, address offset included.
+template <int OFF>
+__device__ __forceinline__ void gv_red(unsigned p, unsigned v) {
+  asm volatile("red.shared.add.u32 [%0+%2], %1;" ::"r"(p), "r"(v), "n"(OFF) : "memory");
+}
+// The same where v != 0, without a branch.
+template <int OFF>
+__device__ __forceinline__ void gv_red_nonzero(unsigned p, unsigned v) {
+  asm volatile(
+      "{\n\t"
+      ".reg .pred nz;\n\t"
+      "setp.ne.u32 nz, %1, 0;\n\t"
+      "@nz red.shared.add.u32 [%0+%2], %1;\n\t"
+      "}" ::"r"(p),
+      "r"(v), "n"(OFF)
+      : "memory");
+}
+__device__ __forceinline__ unsigned gv_shared_address(const void* p) {
+  return (unsigned)__cvta_generic_to_shared(p);
+}
+
+// Limb index and residue of h: h + GV_SQ_OFF = 11 limb + rem, for
+// 0 <= h + GV_SQ_OFF < 4096 (5958 = ceil(2^16 / 11)).
+__device__ __forceinline__ int gv_limb_index(int h) {
+  return (int)(((unsigned)(h + GV_SQ_OFF) * 5958u) >> 16);
+}
+
+// A significand and the exponent of its last bit.
+template <typename Real>
+struct GvSig;
+template <>
+struct GvSig<float> {
+  static constexpr int H = 0;  // the square's digits are those of m^2 2^(2 (e2 + H))
+  static constexpr int BITS = 24;
+  unsigned m;
+  int e2;
+  bool neg;
+};
+template <>
+struct GvSig<double> {
+  static constexpr int H = 21;  // of floor(m^2 2^-42), 64 bits
+  static constexpr int BITS = 53;
+  unsigned long long m;
+  int e2;
+  bool neg;
+};
+
+// The digits of (M << 2 rem), M the square: l[i] at limb index limb + i.
+// FP32: M < 2^48 is exact, and the fourth digit is zero except for rem = 10.
+__device__ __forceinline__ void gv_square_digits(const GvSig<float>& w, int rem, unsigned (&l)[4]) {
+  const unsigned long long M = (unsigned long long)w.m * w.m;
+  const unsigned lo = (unsigned)M, hi = (unsigned)(M >> 32), s = 2u * (unsigned)rem;
+  l[0] = (lo << s) & GV_LIMB_MASK;
+  l[1] = __funnelshift_r(lo, hi, 22u - s) & GV_LIMB_MASK;
+  l[2] = (__funnelshift_r(lo, hi, 24u) >> (20u - s)) & GV_LIMB_MASK;
+  l[3] = rem == 10 ? hi >> 14 : 0u;
+}
+// FP64: the high 64 bits of the 106-bit square (truncated below 2^-62 of it).
+__device__ __forceinline__ void gv_square_digits(const GvSig<double>& w, int rem,
+                                                 unsigned (&l)[4]) {
+  const unsigned long long P = __umul64hi(w.m << 11, w.m << 11);
+  const unsigned s = 2u * (unsigned)rem;
+  l[0] = ((unsigned)P << s) & GV_LIMB_MASK;
+  l[1] = __funnelshift_r((unsigned)P, (unsigned)(P >> 32), 22u - s) & GV_LIMB_MASK;
+  l[2] = (unsigned)(P >> (44u - s)) & GV_LIMB_MASK;
+  l[3] = (unsigned)(P >> 46) >> (20u - s);
+}
+
+// The window of one pass: the squares' limb indices [base, base + L - 4] (their
+// digits reach base + L - 1), and the lowest digit of w in units of 22 and 21
+// bits.
+struct GvWindow {
+  int base, wbase, hbase;
+};
+template <typename Real>
+__device__ __forceinline__ GvWindow gv_window(int e2max, int L) {
+  GvWindow v;
+  v.base = gv_limb_index(e2max + GvSig<Real>::H) - (L - 4);
+  const int t = 11 * v.base - GvSig<Real>::H;  // e2 + GV_SQ_OFF of the smallest weight taken
+  v.wbase = (t + 2200) / 22 - 100;             // (t > -2200)
+  v.hbase = (t + GV_W21_OFF - GV_SQ_OFF + 2100) / 21 - 100;
+  return v;
+}
+
+// Adds one weight to the columns of its lane: the square's digits and those
+// of w (shared-memory addresses of the digits' first rows, 128 bytes a row).
+// A lane's column takes at most 32 events of a tile, so the top digit of w
+// needs no mask.
+__device__ __forceinline__ unsigned gv_signed_digit(unsigned d, int s) { return (d ^ s) - s; }
+__device__ __forceinline__ void gv_lane_add_w(const GvSig<float>& w, unsigned lw, int wbase) {
+  const unsigned t = (unsigned)(w.e2 + GV_SQ_OFF);
+  const unsigned idx = (t * 2979u) >> 16;  // t / 22
+  const unsigned sh = t - 22u * idx;
+  const int s = w.neg ? -1 : 0;
+  const unsigned p = lw + (idx - (unsigned)wbase) * 128u;
+  gv_red<0>(p, gv_signed_digit((w.m << sh) & GV_LIMB_MASK, s));
+  gv_red<128>(p, gv_signed_digit(w.m >> (22u - sh), s));
+}
+__device__ __forceinline__ void gv_lane_add_w(const GvSig<double>& w, unsigned lw, int wbase) {
+  const unsigned t = (unsigned)(w.e2 + GV_SQ_OFF);
+  const unsigned idx = (t * 2979u) >> 16;
+  const unsigned sh = t - 22u * idx;
+  const int s = w.neg ? -1 : 0;
+  const unsigned p = lw + (idx - (unsigned)wbase) * 128u;
+  gv_red<0>(p, gv_signed_digit(((unsigned)w.m << sh) & GV_LIMB_MASK, s));
+  gv_red<128>(p, gv_signed_digit((unsigned)(w.m >> (22u - sh)) & GV_LIMB_MASK, s));
+  gv_red<256>(p, gv_signed_digit((unsigned)(w.m >> (44u - sh)) & GV_LIMB_MASK, s));
+  gv_red<384>(p, gv_signed_digit((unsigned)(w.m >> 45) >> (21u - sh), s));
+}
+template <typename Real>
+__device__ __forceinline__ void gv_lane_add_square(const unsigned (&l)[4], unsigned p) {
+  gv_red<0>(p, l[0]);
+  gv_red<128>(p, l[1]);
+  gv_red<256>(p, l[2]);
+  if constexpr (sizeof(Real) == 8)
+    gv_red<384>(p, l[3]);
+  else
+    gv_red_nonzero<384>(p, l[3]);
+}
+// The square's digits into a bin's row at address p.
+template <typename Real>
+__device__ __forceinline__ void gv_bin_add_square(const unsigned (&l)[4], unsigned p) {
+  gv_red<0>(p, l[0]);
+  gv_red<4>(p, l[1]);
+  gv_red<8>(p, l[2]);
+  if constexpr (sizeof(Real) == 8)
+    gv_red<12>(p, l[3]);
+  else
+    gv_red_nonzero<12>(p, l[3]);
+}
+// w in 21-bit signed digits into a histogram bin's limbs (address of the
+// bin's row): |digit| < 2^21, so 1024 of them stay in 32 bits with either
+// sign.
+template <typename Real>
+__device__ __forceinline__ void gv_hist_add_w(const GvSig<Real>& w, unsigned row, int hbase) {
+  const unsigned t = (unsigned)(w.e2 + GV_W21_OFF);
+  const unsigned idx = t / 21u;
+  const unsigned sh = t - 21u * idx;
+  const int s = w.neg ? -1 : 0;
+  const unsigned long long m = w.m;
+  const unsigned p = row + (idx - (unsigned)hbase) * 4u;
+  gv_red<0>(p, gv_signed_digit((unsigned)(m << sh) & 0x1FFFFFu, s));
+  gv_red<4>(p, gv_signed_digit((unsigned)(m >> (21u - sh)) & 0x1FFFFFu, s));
+  gv_red<8>(p, gv_signed_digit((unsigned)(m >> (42u - sh)) & 0x1FFFFFu, s));
+  if constexpr (sizeof(Real) == 8) gv_red<12>(p, gv_signed_digit((unsigned)(m >> (63u - sh)), s));
+}
+
+// Rows of the squares' columns left out of their total: the FP64 form's 204
+// bits from row 0 of nine would pass 192; rows 0 and 1 lie 2^54 below the unit
+// of the tile's fixed point there.
+__host__ __device__ constexpr int gv_square_row0(bool f64, int L) { return f64 && L > 7 ? 2 : 0; }
+
+// Warp-collective total of a lane column's digits [row0, rows), in units of
+// row row0 (every lane returns it).
+template <bool SIGNED>
+__device__ __forceinline__ u192 gv_lane_total(const unsigned* col, int rows, int row0) {
+  const int lane = threadIdx.x & 31;
+  u192 acc = {0ull, 0ull, 0ull};
+  for (int j = rows - 1; j >= row0; --j) {
+    const unsigned v = col[j * 32 + lane];
+    u192 s;
+    if constexpr (SIGNED) {
+      const long long x = (long long)__reduce_add_sync(0xffffffffu, v & 0xFFFFu) +
+                          ((long long)__reduce_add_sync(0xffffffffu, (int)v >> 16) << 16);
+      const unsigned long long ext = (unsigned long long)(x >> 63);
+      s = {(unsigned long long)x, ext, ext};
+    } else {
+      s = {__reduce_add_sync(0xffffffffu, v), 0ull, 0ull};
+    }
+    acc = shl192(acc, GV_LIMB_BITS);
+    add192(acc, s);
+  }
+  return acc;
+}
+// The total in a tile's fixed point: v 2^p as a 128-bit integer (bits below
+// its unit truncated).
+__device__ __forceinline__ u128 gv_tile_fixed(const u192& v, int p) {
+  const u192 r = p >= 0 ? shl192(v, p) : sar192(v, -p);
+  return u128{r.l0, r.l1};
+}
+
+// A bin's partial: 96 bits and an exponent code F + GV_BINE_OFF with the value
+// in units of 2^(2 F - GV_BIN_QBITS).  From the row's top nonzero limb and the
+// three below it (zeros below the row), so the value is at least 2^66.
+struct GvPartial {
+  unsigned long long lo;
+  unsigned hi;
+  int code;  // 0: empty
+};
+__device__ __forceinline__ GvPartial gv_partial_norm(unsigned long long lo, unsigned long long hi,
+                                                     int code) {
+  if (hi >> 32) {  // 97 or 98 bits: drop one digit
+    lo = (lo >> GV_LIMB_BITS) | (hi << (64 - GV_LIMB_BITS));
+    hi >>= GV_LIMB_BITS;
+    code += GV_LIMB_BITS / 2;
+  }
+  return GvPartial{lo, (unsigned)hi, code};
+}
+__device__ __forceinline__ GvPartial gv_bin_partial(const unsigned* row, int L, int base) {
+  int t = L - 1;
+  unsigned a = row[t];
+  while (a == 0u && t > 0) a = row[--t];
+  if (a == 0u) return GvPartial{0ull, 0u, 0};
+  const unsigned b = t > 0 ? row[t - 1] : 0u, c = t > 1 ? row[t - 2] : 0u,
+                 d = t > 2 ? row[t - 3] : 0u;
+  const u128 x = add128(add128(u128{(unsigned long long)d + ((unsigned long long)c << 22), 0ull},
+                               u128{(unsigned long long)b << 44, b >> 20}),
+                        u128{0ull, (unsigned long long)a << 2});
+  // unit 2^(22 i - 2 GV_SQ_OFF) = 2^(2 F - 56) for the lowest digit i = base + t - 3
+  return gv_partial_norm(x.lo, x.hi, 11 * (base + t - 3) - GV_SQ_OFF + GV_BIN_QBITS / 2 +
+                                         GV_BINE_OFF);
+}
+// The sum of two partials of a bin (a later pass over lower weights): the
+// smaller unit aligned to the larger one, bits below it dropped.
+__device__ __forceinline__ GvPartial gv_partial_add(GvPartial x, GvPartial y) {
+  if (x.code == 0) return y;
+  if (y.code == 0) return x;
+  if (x.code < y.code) {
+    const GvPartial t = x;
+    x = y;
+    y = t;
+  }
+  const u192 s = sar192(u192{y.lo, y.hi, 0ull}, 2 * (x.code - y.code));
+  const u128 r = add128(u128{x.lo, x.hi}, u128{s.l0, s.l1});
+  return gv_partial_norm(r.lo, r.hi, x.code);
+}
+// A histogram bin's partial of w: 96-bit two's complement in units of
+// 2^(F - GV_BIN_QBITS), from its row of signed 21-bit digits.
+__device__ __forceinline__ GvPartial gv_hist_partial(const int* row, int rows, int hbase) {
+  int t = rows - 1;
+  int a = row[t];
+  while (a == 0 && t > 0) a = row[--t];
+  if (a == 0) return GvPartial{0ull, 0u, 0};
+  u192 v = {(unsigned long long)(long long)a, (unsigned long long)((long long)a >> 63), 0ull};
+#pragma unroll
+  for (int i = 1; i <= 3; ++i) {
+    const long long q = t >= i ? (long long)row[t - i] : 0ll;
+    v = shl192(v, 21);
+    const unsigned long long ext = (unsigned long long)(q >> 63);
+    add192(v, u192{(unsigned long long)q, ext, ext});
+  }
+  return GvPartial{v.l0, (unsigned)v.l1,
+                   21 * (hbase + t - 3) - GV_W21_OFF + GV_BIN_QBITS + GV_BINE_OFF};
+}
+__device__ __forceinline__ GvPartial gv_hist_partial_add(GvPartial x, GvPartial y) {
+  if (x.code == 0) return y;
+  if (y.code == 0) return x;
+  if (x.code < y.code) {
+    const GvPartial t = x;
+    x = y;
+    y = t;
+  }
+  const unsigned long long xh = (unsigned long long)(long long)(int)x.hi;
+  const unsigned long long yh = (unsigned long long)(long long)(int)y.hi;
+  const unsigned long long ye = (unsigned long long)((long long)yh >> 63);
+  const u192 s = sar192(u192{y.lo, yh, ye}, x.code - y.code);
+  u192 r = {x.lo, xh, (unsigned long long)((long long)xh >> 63)};
+  add192(r, s);
+  // |x|, |y| < 2^95: halve if the sum leaves 95 bits (it stays two's complement)
+  const long long top = (long long)r.l1;
+  if (top != (long long)(int)top) {
+    r = sar192(r, 1);
+    x.code += 1;
+  }
+  return GvPartial{r.l0, (unsigned)r.l1, x.code};
+}

@@ -6,7 +6,7 @@
 // of 32) x (tile ranges): each CTA owns 32 slots and a range of tiles; its 8
 // warps stride over the tiles, align every partial to the largest exponent
 // the slot has in the range (channel sums: the tiles' scales; bin sums: the
-// bins' own exponents, formed by the fill kernel with order-free atomicMax)
+// bins' own exponent codes, gv_limbs.cuh)
 // and add in 192-bit integers; the warps' sums are combined in shared memory
 // and published with that exponent.  No sum is formed with atomics.  Integer
 // addition is associative, and the alignment depends only on the data and on
@@ -33,50 +33,7 @@
 #include "gv_combine.cuh"
 #include "gv_ff.cuh"
 #include "gv_integrands.cuh"
-
-struct u192 {
-  unsigned long long l0, l1, l2;
-};
-
-__device__ __forceinline__ void add192(u192& r, const u192& x) {
-  const unsigned long long a0 = r.l0 + x.l0;
-  const unsigned long long c0 = a0 < r.l0 ? 1ull : 0ull;
-  const unsigned long long t1 = r.l1 + x.l1;
-  const unsigned long long c1 = t1 < r.l1 ? 1ull : 0ull;
-  const unsigned long long a1 = t1 + c0;
-  const unsigned long long c1b = a1 < t1 ? 1ull : 0ull;
-  r.l0 = a0;
-  r.l1 = a1;
-  r.l2 = r.l2 + x.l2 + c1 + c1b;
-}
-
-// Arithmetic shift right of a 192-bit two's complement value.
-__device__ __forceinline__ u192 sar192(u192 v, int s) {
-  const unsigned long long ext = (unsigned long long)((long long)v.l2 >> 63);
-  if (s <= 0) return v;
-  if (s >= 192) return {ext, ext, ext};
-  while (s >= 64) {
-    v.l0 = v.l1;
-    v.l1 = v.l2;
-    v.l2 = ext;
-    s -= 64;
-  }
-  if (s > 0) {
-    v.l0 = (v.l0 >> s) | (v.l1 << (64 - s));
-    v.l1 = (v.l1 >> s) | (v.l2 << (64 - s));
-    v.l2 = (unsigned long long)((long long)v.l2 >> s);
-  }
-  return v;
-}
-
-// Left shift by 0 <= s < 64 (callers keep the result below 2^149).
-__device__ __forceinline__ u192 shl192(u192 v, int s) {
-  if (s <= 0) return v;
-  v.l2 = (v.l2 << s) | (v.l1 >> (64 - s));
-  v.l1 = (v.l1 << s) | (v.l0 >> (64 - s));
-  v.l0 <<= s;
-  return v;
-}
+#include "gv_limbs.cuh"
 
 // Slots (GvSlot: 192 bits and an exponent) are written by one thread and read
 // by CTAs that took a ticket after the writer's fence: L2 loads.
@@ -248,21 +205,15 @@ __device__ __forceinline__ void pack_axis_tables(double* grid, const double* e_s
   double* e64 = grid + L.off_e64() + (size_t)ax * (N + 1);
   double* wd64 = grid + L.off_wd64() + (size_t)ax * N;
   double* jac = grid + L.off_jac() + (size_t)ax * N;
-  float* w32 = reinterpret_cast<float*>(grid + L.off_f32_base());
-  float* e32 = w32 + L.w_e32() + (size_t)ax * (N + 1);
-  float* wd32 = w32 + L.w_wd32() + (size_t)ax * N;
-  float* jm32 = w32 + L.w_jm32() + (size_t)ax * N;
-  int* je = reinterpret_cast<int*>(w32 + L.w_je()) + (size_t)ax * N;
+  GvBin32* b32 = reinterpret_cast<GvBin32*>(grid + L.off_bin32()) + (size_t)ax * N;
   for (int i = tid; i <= N; i += nthr) {
     const double e = e_src[i];
     e64[i] = e;
-    e32[i] = (float)e;
     if (i < N) {
       const double w = e_src[i + 1] - e;
       const double j = (double)N * w;
       wd64[i] = w;
       jac[i] = j;
-      wd32[i] = (float)w;
       // j = m 2^x with m in [1,2): exponent from the bits (j > 0; a subnormal
       // j is scaled into the normal range first)
       const bool sub = j < 0x1p-1000;
@@ -270,8 +221,7 @@ __device__ __forceinline__ void pack_axis_tables(double* grid, const double* e_s
       const long long b = __double_as_longlong(js);
       const int x = (int)((b >> 52) & 0x7FF) - 1023;
       const double m = __longlong_as_double((b & 0xFFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
-      jm32[i] = (float)m;
-      je[i] = sub ? x - 200 : x;
+      b32[i] = GvBin32{(float)e, (float)w, (float)m, sub ? x - 200 : x};
     }
   }
 }
@@ -770,8 +720,9 @@ __device__ __forceinline__ u192 warp_sum192(u192 v) {
   return v;
 }
 
+// Four CTAs per SM (64 registers): the 32-thread form would otherwise take 127.
 template <int GT>
-__global__ void __launch_bounds__(256) gv_reduce_slots_kernel(const GvReduceArgs a) {
+__global__ void __launch_bounds__(256, 4) gv_reduce_slots_kernel(const GvReduceArgs a) {
   constexpr int NG = 256 / GT;  // slots per CTA
   constexpr int WPG = GT / 32;  // warps per slot
   constexpr int G = GV_RED_TILES_PER_LOAD;
@@ -888,8 +839,9 @@ __global__ void __launch_bounds__(256) gv_reduce_slots_kernel(const GvReduceArgs
 }
 
 // Batched: one launch reduces many integrations; task i names the
-// integration and the block coordinates of CTA i.
-__global__ void __launch_bounds__(256) gv_reduce_batch_kernel(const GvReduceArgs* args,
+// integration and the block coordinates of CTA i.  Four CTAs per SM, as
+// above (72 registers otherwise).
+__global__ void __launch_bounds__(256, 4) gv_reduce_batch_kernel(const GvReduceArgs* args,
                                                               const int4* tasks, int k, int last,
                                                               double inv_m1) {
   extern __shared__ __align__(16) double sm[];
