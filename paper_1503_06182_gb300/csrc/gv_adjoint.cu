@@ -47,7 +47,7 @@ __device__ __forceinline__ void rs_step(const u128 (&x)[2 * N], u128 (&y)[N], in
 // FP32 products J.m g and the event's Jacobian exponent J.e.
 template <typename Real>
 constexpr size_t stage_bytes() {
-  return sizeof(Real) == 8 ? (size_t)GV_TILE * kNch * 8 : (size_t)GV_TILE * (kNch + 1) * 4;
+  return sizeof(Real) != 4 ? (size_t)GV_TILE * kNch * 8 : (size_t)GV_TILE * (kNch + 1) * 4;
 }
 
 // A weight's two fixed-point terms through the general FP64 route.
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(GV_TILE / EPT, AdjBlocks<Real, EPT>::value)
   __shared__ u128 red_sum[NW][kNsum];
   __shared__ int s_E[kNch];
   const int d = a.ndim, N = a.nbins;
-  const GvFillSmem lay(d, N, (int)sizeof(Real), false, false);
+  const GvFillSmem lay(d, N, GvForm<Real>::ID, false, false);
   double* s_jac = reinterpret_cast<double*>(smem + lay.jac);
   Pair* s_ew = reinterpret_cast<Pair*>(smem + lay.ew);
   // channel c of the thread's k-th event at [(k kNch + c) B + tid]: FP64
@@ -92,7 +92,13 @@ __global__ void __launch_bounds__(GV_TILE / EPT, AdjBlocks<Real, EPT>::value)
   gv_wait_prior_grid();
   gv_stage_grid<Real>(a.grid, d, N, s_jac, s_ew, tid, B);
   GvConst<Real, DK_NK> K;
-  K.load(a.kconst);
+  if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
+    __shared__ GvX s_k[XK_N];  // (the barrier below)
+    if (tid < XK_N) s_k[tid] = gv_x_consts(a.kconst)[tid];
+    K.k = s_k;
+  } else {
+    K.load(a.kconst);
+  }
   const uint32_t it = (uint32_t)a.st->it;
   __syncthreads();
 
@@ -121,11 +127,15 @@ __global__ void __launch_bounds__(GV_TILE / EPT, AdjBlocks<Real, EPT>::value)
     if (ev < a.ncall) {
       uint32_t r[MAXD];
       gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)ev, d, r);
-      Real x[MAXD];
+      typename GvForm<Real>::Coord x[MAXD];
       int bin[MAXD];
       const GvJac<Real> J = gv_map_event<Real, MAXD>(r, d, N, s_jac, s_ew, x, bin);
       Real gr[GV_NGRAD];
-      const Real g = gv_drell_yan<Real, true>(x, K, gr);
+      Real g;
+      if constexpr (GvForm<Real>::ID == GV_FORM_X64)
+        g = gv_drell_yan_x<true>(x, K.k, gr);
+      else
+        g = gv_drell_yan<Real, true>(x, K, gr);
       bool finite = true;
       if constexpr (F32) {
         je = J.e;
@@ -288,14 +298,16 @@ static cudaError_t gv_launch_adj_ept(int ept, const GvFillArgs& a, int n_tiles, 
 }
 
 namespace gv {
-cudaError_t launch_fill_adjoint(int fp32, int ept, const GvFillArgs& a, int n_tiles, size_t smem,
+cudaError_t launch_fill_adjoint(int form, int ept, const GvFillArgs& a, int n_tiles, size_t smem,
                                 cudaStream_t s, bool pdl) {
   if (a.ndim <= 4)
-    return fp32 ? gv_launch_adj_ept<float, 4>(ept, a, n_tiles, smem, s, pdl)
-                : gv_launch_adj_ept<double, 4>(ept, a, n_tiles, smem, s, pdl);
+    return form == GV_FORM_F32   ? gv_launch_adj_ept<float, 4>(ept, a, n_tiles, smem, s, pdl)
+           : form == GV_FORM_X64 ? gv_launch_adj_ept<GvX, 4>(ept, a, n_tiles, smem, s, pdl)
+                                 : gv_launch_adj_ept<double, 4>(ept, a, n_tiles, smem, s, pdl);
   if (a.ndim <= 16)
-    return fp32 ? gv_launch_adj_ept<float, 16>(ept, a, n_tiles, smem, s, pdl)
-                : gv_launch_adj_ept<double, 16>(ept, a, n_tiles, smem, s, pdl);
+    return form == GV_FORM_F32   ? gv_launch_adj_ept<float, 16>(ept, a, n_tiles, smem, s, pdl)
+           : form == GV_FORM_X64 ? gv_launch_adj_ept<GvX, 16>(ept, a, n_tiles, smem, s, pdl)
+                                 : gv_launch_adj_ept<double, 16>(ept, a, n_tiles, smem, s, pdl);
   return cudaErrorInvalidValue;
 }
 }  // namespace gv

@@ -66,7 +66,7 @@ double tile_cost(int ig, int d) {
 }
 
 struct Member {
-  int ig, d, np, n_tiles, nacc, gx, gy;
+  int ig, d, np, form, n_tiles, nacc, gx, gy;
   int64_t ncall;
   double params[GV_MAXPARAMS];
   double* grid;
@@ -104,7 +104,7 @@ struct vegas_batch {
   // one work list per dimension class (members of at most 4, 8, 16 axes) and
   // integrand
   struct FillClass {
-    int maxd = 0, ig = 0, n = 0, ctas = 0;
+    int maxd = 0, ig = 0, form = 0, n = 0, ctas = 0;
     long long total = 0;
     size_t smem = 0;
     int* d_order = nullptr;
@@ -133,6 +133,9 @@ struct vegas_batch {
 
 namespace {
 
+// Work lists: dimension class, integrand and, in FP64, the arithmetic.
+constexpr int kMaxLists = 18;
+
 // Dimension class of a member (the same classes as the single-context fill).
 int dim_class(int ig, int d) { return (d <= 4 && ig != VEGAS_EE3J) ? 4 : d <= 8 ? 8 : 16; }
 
@@ -141,17 +144,21 @@ cudaError_t fill_class(vegas_batch* B, const vegas_batch::FillClass& c, int ept,
                        cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(c.d_counter, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
-  auto f = c.maxd == 4 ? (B->fp32 ? gv::fill_batch_f4 : gv::fill_batch_d4)
-           : c.maxd == 8 ? (B->fp32 ? gv::fill_batch_f8 : gv::fill_batch_d8)
-                         : (B->fp32 ? gv::fill_batch_f16 : gv::fill_batch_d16);
+  static decltype(&gv::fill_batch_f4) const fs[3][3] = {
+      {gv::fill_batch_d4, gv::fill_batch_d8, gv::fill_batch_d16},
+      {gv::fill_batch_f4, gv::fill_batch_f8, gv::fill_batch_f16},
+      {gv::fill_batch_x4, gv::fill_batch_x8, gv::fill_batch_x16}};
+  auto f = fs[c.form][c.maxd == 4 ? 0 : (c.maxd == 8 ? 1 : 2)];
   return f(c.ig, ept, ctas, c.smem, s, B->d_fill, c.d_order, c.d_start, c.n, c.total,
            c.d_counter);
 }
 
 int class_occupancy(vegas_batch* B, const vegas_batch::FillClass& c, int ept) {
-  auto f = c.maxd == 4 ? (B->fp32 ? gv::fill_batch_occ_f4 : gv::fill_batch_occ_d4)
-           : c.maxd == 8 ? (B->fp32 ? gv::fill_batch_occ_f8 : gv::fill_batch_occ_d8)
-                         : (B->fp32 ? gv::fill_batch_occ_f16 : gv::fill_batch_occ_d16);
+  static decltype(&gv::fill_batch_occ_f4) const fs[3][3] = {
+      {gv::fill_batch_occ_d4, gv::fill_batch_occ_d8, gv::fill_batch_occ_d16},
+      {gv::fill_batch_occ_f4, gv::fill_batch_occ_f8, gv::fill_batch_occ_f16},
+      {gv::fill_batch_occ_x4, gv::fill_batch_occ_x8, gv::fill_batch_occ_x16}};
+  auto f = fs[c.form][c.maxd == 4 ? 0 : (c.maxd == 8 ? 1 : 2)];
   return std::max(1, f(c.ig, ept, c.smem));
 }
 
@@ -393,6 +400,9 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
     for (int i = 0; i < GV_MAXPARAMS; ++i)
       x.params[i] = i < x.np ? params[(size_t)b * VEGAS_MAX_PARAMS + i] : 0.0;
     x.params[GV_MAXPARAMS - 1] = (double)x.np;
+    x.form = precision ? GV_FORM_F32
+             : gv_x64_applies(x.ig, x.params, x.np, x.d * nbins) ? GV_FORM_X64
+                                                                 : GV_FORM_F64;
     x.n_tiles = (int)((x.ncall + GV_TILE - 1) / GV_TILE);
     x.nacc = 2 + x.d * nbins;
     int tpc = 0;
@@ -405,7 +415,7 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
     q[2] = off;
     off = a256(off + GV_MAXPARAMS * 8);
     q[3] = off;
-    off = a256(off + GV_NCONST * 8);
+    off = a256(off + GV_NCONST_ALL * 8);
     q[4] = off;  // cpart
     off = a256(off + (size_t)x.gy * x.gx * 32 * sizeof(GvSlot));
     q[5] = off;
@@ -420,9 +430,9 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
   const size_t o_order = off;
   off = a256(off + (size_t)n * 4);
   const size_t o_start = off;
-  off = a256(off + (size_t)(n + 9) * 8);
-  const size_t o_ccount = off;  // up to nine list counters, one per 128-byte line
-  off = a256(off + 9 * 128);
+  off = a256(off + (size_t)(n + kMaxLists) * 8);
+  const size_t o_ccount = off;  // the list counters, one per 128-byte line
+  off = a256(off + kMaxLists * 128);
   if (cudaMalloc(&B->dmem, off) != cudaSuccess) {
     cudaGetLastError();
     vegas_batch_free(B);
@@ -458,16 +468,23 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
         gv::launch_reset(x.st, B->stream) != cudaSuccess)
       st = VEGAS_ECUDA;
   }
-  // work lists, one per dimension class and integrand: largest expected cost first
+  // work lists, one per dimension class, integrand and arithmetic: largest
+  // expected cost first
   if (!st) {
     std::vector<int> order;
     std::vector<long long> start;
     int pos = 0, slot = 0;
-    for (int maxd : {4, 8, 16}) {
-      for (int ig : {VEGAS_GAUSS, VEGAS_DY, VEGAS_EE3J}) {
+    for (int cl = 0; cl < kMaxLists; ++cl) {
+      {
+        const int maxd = cl % 3 == 0 ? 4 : (cl % 3 == 1 ? 8 : 16);
+        const int ig = cl / 3 % 3 == 0 ? VEGAS_GAUSS : (cl / 3 % 3 == 1 ? VEGAS_DY : VEGAS_EE3J);
+        const int form = precision ? GV_FORM_F32 : (cl < 9 ? GV_FORM_X64 : GV_FORM_F64);
+        if (precision && cl >= 9) continue;
         std::vector<int> mem;
         for (int b = 0; b < n; ++b)
-          if (B->m[b].ig == ig && dim_class(B->m[b].ig, B->m[b].d) == maxd) mem.push_back(b);
+          if (B->m[b].ig == ig && B->m[b].form == form &&
+              dim_class(B->m[b].ig, B->m[b].d) == maxd)
+            mem.push_back(b);
         if (mem.empty()) continue;
         std::stable_sort(mem.begin(), mem.end(), [&](int p, int q) {
           return B->m[p].n_tiles * tile_cost(B->m[p].ig, B->m[p].d) >
@@ -476,6 +493,7 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
         vegas_batch::FillClass c;
         c.maxd = maxd;
         c.ig = ig;
+        c.form = form;
         c.n = (int)mem.size();
         c.d_order = (int*)(base + o_order) + pos;
         c.d_start = (long long*)(base + o_start) + pos + slot;
@@ -487,7 +505,7 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
           acc += B->m[b].n_tiles;
           start.push_back(acc);
           c.smem = std::max(c.smem,
-                            GvFillSmem(B->m[b].d, nbins, B->fp32 ? 4 : 8, true, maxd > 4, 0, false,
+                            GvFillSmem(B->m[b].d, nbins, form, true, maxd > 4, 0, false,
                                        false, true)
                                 .total);
         }
@@ -509,7 +527,8 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
     std::vector<double> cost(B->cls.size(), 0.0);
     for (size_t i = 0; i < B->cls.size(); ++i)
       for (int b = 0; b < n; ++b)
-        if (B->m[b].ig == B->cls[i].ig && dim_class(B->m[b].ig, B->m[b].d) == B->cls[i].maxd)
+        if (B->m[b].ig == B->cls[i].ig && B->m[b].form == B->cls[i].form &&
+            dim_class(B->m[b].ig, B->m[b].d) == B->cls[i].maxd)
           cost[i] += (double)B->m[b].n_tiles * tile_cost(B->m[b].ig, B->m[b].d);
     for (size_t i = 0; i < B->cls.size(); ++i) B->launch_order.push_back((int)i);
     std::stable_sort(B->launch_order.begin(), B->launch_order.end(),

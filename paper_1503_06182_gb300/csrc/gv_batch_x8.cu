@@ -1,0 +1,3 @@
+// Batched fill kernels: GvX, at most 8 axes (4 and 8 events per thread).
+#include "gv_fill_batch.cuh"
+GV_DEFINE_FILL_BATCH(x8, GvX, 8)

@@ -28,21 +28,21 @@
 #include "gv_fill.cuh"
 
 namespace gv {
-cudaError_t launch_fill_gauss(int fp32, int ept, const GvFillArgs& a, int n_tiles, size_t smem,
+cudaError_t launch_fill_gauss(int form, int ept, const GvFillArgs& a, int n_tiles, size_t smem,
                               cudaStream_t s, bool pdl);
-cudaError_t launch_fill_dy(int fp32, int ept, const GvFillArgs& a, int n_tiles, size_t smem,
+cudaError_t launch_fill_dy(int form, int ept, const GvFillArgs& a, int n_tiles, size_t smem,
                            cudaStream_t s, bool pdl);
-cudaError_t launch_fill_ee3j(int fp32, int ept, const GvFillArgs& a, int n_tiles, size_t smem,
+cudaError_t launch_fill_ee3j(int form, int ept, const GvFillArgs& a, int n_tiles, size_t smem,
                              cudaStream_t s, bool pdl);
-cudaError_t launch_fill_dynlo(int fp32, int ept, const GvFillArgs& a, int n_tiles, size_t smem,
+cudaError_t launch_fill_dynlo(int form, int ept, const GvFillArgs& a, int n_tiles, size_t smem,
                              cudaStream_t s, bool pdl);
-cudaError_t launch_fill_gauss_eval(int fp32, const GvFillArgs& a, uint32_t it, const long long* ev,
+cudaError_t launch_fill_gauss_eval(int form, const GvFillArgs& a, uint32_t it, const long long* ev,
                                    long long n, double* w, int* bins, cudaStream_t s);
-cudaError_t launch_fill_dy_eval(int fp32, const GvFillArgs& a, uint32_t it, const long long* ev,
+cudaError_t launch_fill_dy_eval(int form, const GvFillArgs& a, uint32_t it, const long long* ev,
                                 long long n, double* w, int* bins, cudaStream_t s);
-cudaError_t launch_fill_ee3j_eval(int fp32, const GvFillArgs& a, uint32_t it, const long long* ev,
+cudaError_t launch_fill_ee3j_eval(int form, const GvFillArgs& a, uint32_t it, const long long* ev,
                                   long long n, double* w, int* bins, cudaStream_t s);
-cudaError_t launch_fill_dynlo_eval(int fp32, const GvFillArgs& a, uint32_t it, const long long* ev,
+cudaError_t launch_fill_dynlo_eval(int form, const GvFillArgs& a, uint32_t it, const long long* ev,
                                   long long n, double* w, int* bins, cudaStream_t s);
 // The last CUDA error behind a VEGAS_ECUDA status, per host thread.
 cudaError_t& last_cuda_error() {
@@ -64,13 +64,13 @@ namespace {
 
 cudaError_t& gv_last_cuda_error() { return gv::last_cuda_error(); }
 
-cudaError_t launch_fill_any(int ig, int fp32, int ept, const GvFillArgs& a, int n_tiles,
+cudaError_t launch_fill_any(int ig, int form, int ept, const GvFillArgs& a, int n_tiles,
                             size_t smem, cudaStream_t s, bool pdl) {
   switch (ig) {
-    case GV_GAUSS: return gv::launch_fill_gauss(fp32, ept, a, n_tiles, smem, s, pdl);
-    case GV_DY: return gv::launch_fill_dy(fp32, ept, a, n_tiles, smem, s, pdl);
-    case GV_EE3J: return gv::launch_fill_ee3j(fp32, ept, a, n_tiles, smem, s, pdl);
-    case GV_DYNLO: return gv::launch_fill_dynlo(fp32, ept, a, n_tiles, smem, s, pdl);
+    case GV_GAUSS: return gv::launch_fill_gauss(form, ept, a, n_tiles, smem, s, pdl);
+    case GV_DY: return gv::launch_fill_dy(form, ept, a, n_tiles, smem, s, pdl);
+    case GV_EE3J: return gv::launch_fill_ee3j(form, ept, a, n_tiles, smem, s, pdl);
+    case GV_DYNLO: return gv::launch_fill_dynlo(form, ept, a, n_tiles, smem, s, pdl);
   }
   return cudaErrorInvalidValue;
 }
@@ -115,11 +115,11 @@ static_assert(sizeof(GvState) <= kHostRecOff, "state fits before the records");
 std::mutex g_tune_mu;
 std::map<std::string, int> g_tune;
 
-std::string tune_key(int dev, int ig, int fp32, int mode, int d, int N, int n_tiles) {
+std::string tune_key(int dev, int ig, int form, int mode, int d, int N, int n_tiles) {
   char buf[160];
   int lg = 0;
   while ((1 << (lg + 1)) <= n_tiles && lg < 30) ++lg;
-  snprintf(buf, sizeof buf, "dev%d:ig%d:fp%d:m%d:d%d:N%d:t%d", dev, ig, fp32, mode, maxd_class(d),
+  snprintf(buf, sizeof buf, "dev%d:ig%d:fp%d:m%d:d%d:N%d:t%d", dev, ig, form, mode, maxd_class(d),
            N, lg);
   return buf;
 }
@@ -292,7 +292,7 @@ int ensure_pinned(vegas_ctx* c, size_t need) {
 }
 
 struct Plan {
-  int ig, fp32, mode, itmx, n_tiles, nacc, nch, ept, reduce_ctas, tiles_per_cta;
+  int ig, form, mode, itmx, n_tiles, nacc, nch, ept, reduce_ctas, tiles_per_cta;
   int nhist;  // histogram bins with underflow and overflow (0: none)
   int slot_major;  // slot-major partials and the single-level reduce (forward stages)
   int hoist;       // the fill makes its Philox words before it waits (gv_fill_hoistable)
@@ -514,10 +514,10 @@ int ensure_consts(vegas_ctx* c, int ig, const double* params, int np) {
 cudaError_t launch_fill_plan(const vegas_ctx* c, const Plan& p, int ept, bool pdl = false,
                              int k = 0) {
   const GvFillArgs a = fill_args(c, p, k);
-  if (p.mode) return gv::launch_fill_adjoint(p.fp32, ept, a, p.n_tiles, p.smem, c->stream, pdl);
-  if (p.nhist) return gv::launch_fill_hist(p.ig, p.fp32, a, p.n_tiles, p.smem, c->stream, pdl);
-  if (p.plus) return gv::launch_fill_plus(p.ig, p.fp32, a, p.n_tiles, p.smem, c->stream, pdl);
-  return launch_fill_any(p.ig, p.fp32, ept, a, p.n_tiles, p.smem, c->stream, pdl);
+  if (p.mode) return gv::launch_fill_adjoint(p.form, ept, a, p.n_tiles, p.smem, c->stream, pdl);
+  if (p.nhist) return gv::launch_fill_hist(p.ig, p.form, a, p.n_tiles, p.smem, c->stream, pdl);
+  if (p.plus) return gv::launch_fill_plus(p.ig, p.form, a, p.n_tiles, p.smem, c->stream, pdl);
+  return launch_fill_any(p.ig, p.form, ept, a, p.n_tiles, p.smem, c->stream, pdl);
 }
 
 // Pick events per thread by timing one fill launch per candidate.  Runs
@@ -598,7 +598,7 @@ int autotune_chained(vegas_ctx* c, Plan& p, const std::string& key) {
 }
 
 int autotune(vegas_ctx* c, Plan& p) {
-  const std::string key = tune_key(c->device, p.ig, p.fp32, p.mode, c->ndim, c->nbins, p.n_tiles);
+  const std::string key = tune_key(c->device, p.ig, p.form, p.mode, c->ndim, c->nbins, p.n_tiles);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(key);
@@ -656,9 +656,20 @@ int autotune(vegas_ctx* c, Plan& p) {
   return VEGAS_OK;
 }
 
-int make_plan(vegas_ctx* c, int64_t ncall, int itmx, int ig, int mode, Plan& p) {
+// The arithmetic of a stage's events: FP32, or FP64 on 64-bit significands
+// where gv_x64_applies, else on the FP64 pipe.  The stratified fill stays on
+// the FP64 pipe: its allocation floors a function of each hypercube's
+// variance, and weights that differ in their last bits would give other
+// allocations than before from the same seed.
+int form_of(const vegas_ctx* c, int ig, const double* params, int np, bool plus) {
+  if (c->fp32) return GV_FORM_F32;
+  return !plus && gv_x64_applies(ig, params, np, c->ndim * c->nbins) ? GV_FORM_X64 : GV_FORM_F64;
+}
+
+int make_plan(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* params, int np,
+              int mode, Plan& p) {
   p.ig = ig;
-  p.fp32 = c->fp32;
+  p.form = form_of(c, ig, params, np, mode == 0 && c->strat);
   p.mode = mode;
   p.itmx = itmx;
   p.ncall = ncall;
@@ -685,9 +696,9 @@ int make_plan(vegas_ctx* c, int64_t ncall, int itmx, int ig, int mode, Plan& p) 
   p.nhist = (mode == 0 && c->hist_nh > 0) ? c->hist_nh + 2 : 0;
   p.nacc = mode ? 2 * GV_MAXCH : 2 + c->ndim * c->nbins + 2 * p.nhist;
   {
-    const GvFillSmem plain(c->ndim, c->nbins, c->fp32 ? 4 : 8, mode == 0, c->ndim > 4, p.nhist,
+    const GvFillSmem plain(c->ndim, c->nbins, p.form, mode == 0, c->ndim > 4, p.nhist,
                            p.plus != 0, false);
-    const GvFillSmem words(c->ndim, c->nbins, c->fp32 ? 4 : 8, mode == 0, c->ndim > 4, p.nhist,
+    const GvFillSmem words(c->ndim, c->nbins, p.form, mode == 0, c->ndim > 4, p.nhist,
                            p.plus != 0, true);
     p.hoist = gv_fill_hoistable(mode == 0, p.plus != 0, c->ndim) &&
                       words.total <= GV_WORDS_SMEM_MAX
@@ -873,7 +884,7 @@ int enqueue_stage(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* p
   if (st) return st;
   if (mode && (ig != VEGAS_DY || c->strat)) return VEGAS_EINVAL;
   Plan p;
-  st = make_plan(c, ncall, itmx, ig, mode, p);
+  st = make_plan(c, ncall, itmx, ig, params, np, mode, p);
   if (st) return st;
   st = ensure_consts(c, ig, params, np);
   if (st) return st;
@@ -923,7 +934,7 @@ int enqueue_stage(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* p
   }
   char kb[400];
   snprintf(kb, sizeof kb, "graph:%d:%d:%d:%lld:%d:%d:%d:%a:%d%d:%llu:%u:%p:%p:h%d:%a:%a:p%d:%d:%p",
-           ig, p.fp32, mode, (long long)ncall, itmx, p.ept, c->adapt, c->alpha, c->timing, c->pdl,
+           ig, p.form, mode, (long long)ncall, itmx, p.ept, c->adapt, c->alpha, c->timing, c->pdl,
            (unsigned long long)c->seed, c->batch, c->ws, (void*)c->stream, p.nhist, c->hist_lo,
            c->hist_hi, p.plus, c->beta_j, c->plus_mem);
   const std::string key(kb);
@@ -1104,7 +1115,7 @@ int vegas_init(int ndim, int nbins, uint64_t seed, vegas_ctx** out) {
   const size_t o_par = off;
   off = align256(off + GV_MAXPARAMS * 8);
   const size_t o_k = off;
-  off = align256(off + GV_NCONST * 8);
+  off = align256(off + GV_NCONST_ALL * 8);
   const size_t o_sums = off;
   off = align256(off + (size_t)c->nacc_max * 8);
   const size_t o_tick = off;
@@ -1493,11 +1504,12 @@ int vegas_eval_events(vegas_ctx* c, int id, const double* params, int np, uint32
     a.kconst = c->kconst;
     a.grid = c->grid;
     a.st = c->st;
+    const int form = form_of(c, id, params, np, false);
     switch (id) {
-      case GV_GAUSS: e = gv::launch_fill_gauss_eval(c->fp32, a, iteration, dev, n, dw, db, c->stream); break;
-      case GV_DY: e = gv::launch_fill_dy_eval(c->fp32, a, iteration, dev, n, dw, db, c->stream); break;
-      case GV_EE3J: e = gv::launch_fill_ee3j_eval(c->fp32, a, iteration, dev, n, dw, db, c->stream); break;
-      default: e = gv::launch_fill_dynlo_eval(c->fp32, a, iteration, dev, n, dw, db, c->stream); break;
+      case GV_GAUSS: e = gv::launch_fill_gauss_eval(form, a, iteration, dev, n, dw, db, c->stream); break;
+      case GV_DY: e = gv::launch_fill_dy_eval(form, a, iteration, dev, n, dw, db, c->stream); break;
+      case GV_EE3J: e = gv::launch_fill_ee3j_eval(form, a, iteration, dev, n, dw, db, c->stream); break;
+      default: e = gv::launch_fill_dynlo_eval(form, a, iteration, dev, n, dw, db, c->stream); break;
     }
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(w, dw, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream);

@@ -40,6 +40,8 @@
 #define GV_EMPTY (-0x40000000)  // scale of a tile / iteration with no nonzero value
 #define GV_NCONST 48          // derived integrand constants per integration (doubles)
 #define GV_NCONST_F32 32      // constants 0..31 in FP64, then their FP32 copies
+#define GV_NCONST_X 24        // and the 64-bit-significand constants (GvX) after all of them
+#define GV_NCONST_ALL (GV_NCONST + 2 * GV_NCONST_X)  // doubles in all
 #define GV_MAXPARAMS 16
 #define GV_BINE_OFF 1200      // stored bin exponent F + GV_BINE_OFF (0: no nonzero weight)
 #define GV_BIN_QBITS 56       // bits of one w^2 below its bin's scale in a tile
@@ -48,6 +50,27 @@
 #define GV_HIST_MAX 1000      // histogram bins of the observable (plus underflow and overflow)
 
 enum { GV_GAUSS = 0, GV_DY = 1, GV_EE3J = 2, GV_DYNLO = 3 };
+
+// Arithmetic of an event: the FP64 pipe, FP32, or 64-bit significands on the
+// integer pipes (gv_x64.cuh).
+enum { GV_FORM_F64 = 0, GV_FORM_F32 = 1, GV_FORM_X64 = 2 };
+
+// Whether the FP64 form runs on 64-bit significands: parameters of ordinary
+// size (every derived constant finite, momentum fractions above 2^-60, y_cut
+// far above the fixed point's resolution) and at most 2048 bins in all (its
+// 32-byte grid records, with the limbs, must fit shared memory in the
+// persistent kernel too).  Others stay on the FP64 pipe: same results to
+// rounding, several times the time (1e6 Drell-Yan events: 345 us).
+inline bool gv_x64_applies(int ig, const double* p, int np, int dN) {
+  const auto in = [](double v, double lo, double hi) { return v >= lo && v <= hi; };
+  if (dN > 2048) return false;
+  if (ig == GV_GAUSS) return in(p[0], 1e-6, 1e6) && (np < 2 || in(p[1], -1e30, 1e30));
+  if (ig == GV_EE3J) return in(p[0], 1e-9, 1.0) && (np < 2 || in(p[1], 1e-100, 1e100));
+  return in(p[0], 1e-3, 1e9) && in(p[1], 1e-9, 1e9) && in(p[2], 1e-9, 1e9) &&
+         in(p[3], 1e-6, 1.0 - 1e-6) && in(p[4], 1e-12, 1e3) && p[5] >= 1e-9 * p[0] &&
+         p[6] <= 0.999 * p[0] && in(p[7], -64.0, 64.0) && in(p[8], -64.0, 64.0) &&
+         in(p[9], 1e-30, 1e30);
+}
 
 // Device-side state of one integration (one context or one batch member).
 // nonfinite_iter and the tickets return to zero at the end of every iteration.
@@ -532,9 +555,9 @@ namespace gv {
 cudaError_t launch_plus_finish(const GvPlusArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_plus_alloc(const GvPlusArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_plus_layout(const GvPlusArgs& a, cudaStream_t s, bool pdl);
-cudaError_t launch_fill_plus(int ig, int fp32, const GvFillArgs& a, int n_tiles, size_t smem,
+cudaError_t launch_fill_plus(int ig, int form, const GvFillArgs& a, int n_tiles, size_t smem,
                              cudaStream_t s, bool pdl);
-cudaError_t launch_fill_adjoint(int fp32, int ept, const GvFillArgs& a, int n_tiles,
+cudaError_t launch_fill_adjoint(int form, int ept, const GvFillArgs& a, int n_tiles,
                                 size_t smem, cudaStream_t s, bool pdl);
 void reduce_grid(int n_tiles, int nacc, int* tiles_per_cta, int* gx, int* gy);
 size_t reduce_smem_bytes(int N);  // dynamic shared memory of the reduce kernels
@@ -542,7 +565,7 @@ cudaError_t launch_reduce(const GvReduceArgs& a, size_t smem, cudaStream_t s, bo
 // the single-level reduce of slot-major partials (plain forward stages)
 cudaError_t launch_reduce_slots(const GvReduceArgs& a, size_t smem, cudaStream_t s, bool pdl);
 cudaError_t launch_hist(const GvHistArgs& a, cudaStream_t s, bool pdl);
-cudaError_t launch_fill_hist(int ig, int fp32, const GvFillArgs& a, int n_tiles, size_t smem,
+cudaError_t launch_fill_hist(int ig, int form, const GvFillArgs& a, int n_tiles, size_t smem,
                              cudaStream_t s, bool pdl);
 cudaError_t launch_reduce_batch(const GvReduceArgs* args, const int4* tasks, int ntasks, int k,
                                 int last, double inv_m1, size_t smem, cudaStream_t s);

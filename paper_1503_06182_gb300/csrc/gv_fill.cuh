@@ -34,30 +34,66 @@
 #include "gv_integrands.cuh"
 #include "gv_limbs.cuh"
 #include "gv_plus_stat.cuh"
+#include "gv_xint.cuh"
+
+// The arithmetic of an event: Real = float, double or GvX (FP64 results on the
+// integer pipes).  W: the weight's type; Coord: a sampled variable's.
+template <typename Real>
+struct GvForm {
+  using W = Real;
+  using Coord = Real;
+  static constexpr int ID = sizeof(Real) == 4 ? GV_FORM_F32 : GV_FORM_F64;
+};
+template <>
+struct GvForm<GvX> {
+  using W = double;
+  using Coord = unsigned long long;
+  static constexpr int ID = GV_FORM_X64;
+};
 
 template <int IG>
 struct GvTraits;
 template <>
 struct GvTraits<GV_GAUSS> {
-  static constexpr int NK = 2;
+  static constexpr int NK = 2, NX = 2;  // constants; as GvX
 };
 template <>
 struct GvTraits<GV_DY> {
-  static constexpr int NK = DK_NK;
+  static constexpr int NK = DK_NK, NX = XK_N;
 };
 template <>
 struct GvTraits<GV_EE3J> {
-  static constexpr int NK = 3;
+  static constexpr int NK = 3, NX = 1;
 };
 template <>
 struct GvTraits<GV_DYNLO> {
-  static constexpr int NK = NK_NK;
+  static constexpr int NK = NK_NK, NX = XK_N;
 };
+static_assert(XK_N <= GV_NCONST_X, "room for the GvX constants");
+
+// The GvX constants stay in (shared) memory: too many for registers.
+template <int NC>
+struct GvConst<GvX, NC> {
+  const GvX* k;
+  __device__ __forceinline__ const GvX& operator[](int i) const { return k[i]; }
+};
+__device__ __forceinline__ const GvX* gv_x_consts(const double* kconst) {
+  return reinterpret_cast<const GvX*>(kconst + GV_NCONST);
+}
 
 template <int IG, typename Real, int MAXD>
-__device__ __forceinline__ Real gv_eval(const Real (&x)[MAXD], int d,
+__device__ __forceinline__ Real gv_eval(const typename GvForm<Real>::Coord (&x)[MAXD], int d,
                                         const GvConst<Real, GvTraits<IG>::NK>& K) {
-  if constexpr (IG == GV_GAUSS) {
+  if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
+    if constexpr (IG == GV_GAUSS)
+      return gv_gauss_x<MAXD>(x, d, K.k);
+    else if constexpr (IG == GV_DY)
+      return gv_drell_yan_x<false>(x, K.k, nullptr);
+    else if constexpr (IG == GV_DYNLO)
+      return gv_dy_nlo_x<MAXD>(x, d, K.k);
+    else
+      return gv_ee3j_x(x, K.k);
+  } else if constexpr (IG == GV_GAUSS) {
     return gv_gauss<Real, MAXD>(x, d, K[GK_INV2S2], K[GK_SHIFT]);
   } else if constexpr (IG == GV_DY) {
     return gv_drell_yan<Real, false>(x, K, nullptr);
@@ -73,10 +109,21 @@ __device__ __forceinline__ Real gv_eval(const Real (&x)[MAXD], int d,
 // m_ll = sqrt(tau s) in GeV, with tau as the integrand forms it; 3-jet the
 // thrust max(x1, x2, x3), x3 = 2 - x1 - x2.
 template <int IG, typename Real, int MAXD>
-__device__ __forceinline__ Real gv_observable(const Real (&x)[MAXD],
-                                              const GvConst<Real, GvTraits<IG>::NK>& K) {
-  using Mt = GvMath<Real>;
-  if constexpr (IG == GV_GAUSS) {
+__device__ __forceinline__ typename GvForm<Real>::W gv_observable(
+    const typename GvForm<Real>::Coord (&x)[MAXD], const GvConst<Real, GvTraits<IG>::NK>& K) {
+  using Mt = GvMath<typename GvForm<Real>::W>;
+  if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
+    if constexpr (IG == GV_GAUSS) {
+      return x_to_double(x_from_q64(x[0]));
+    } else if constexpr (IG == GV_DY || IG == GV_DYNLO) {  // sqrt(s) 2^(log2(tau) / 2)
+      const unsigned long long lt = K[XK_B2].m - xi_mulhi(K[XK_A2].m, x[0]);
+      return x_to_double(x_mul(K[XK_SQRTS], x_exp2(lt, K[XK_B2].e - 1, true)));
+    } else {  // (x3 = 2 - x1 - x2 where it is below 1; elsewhere the weight is 0)
+      const unsigned long long x3 = 0ull - (x[0] + x[1]);
+      const unsigned long long t = x[0] > x[1] ? x[0] : x[1];
+      return x_to_double(x_from_q64(t > x3 ? t : x3));
+    }
+  } else if constexpr (IG == GV_GAUSS) {
     return x[0];
   } else if constexpr (IG == GV_DY || IG == GV_DYNLO) {
     const Real tau = Mt::exp(Mt::fma(x[0], K[DK_L], K[DK_LOGTAULO]));
@@ -140,6 +187,10 @@ struct GvJac<float> {
   float m;
   int e;
 };
+template <>
+struct GvJac<GvX> {
+  GvX v;
+};
 
 // x 2^E for a double x, on the integer pipes: zero, infinity and NaN pass
 // through, a result beyond FP64 becomes infinity (counted as non-finite by
@@ -158,6 +209,9 @@ __device__ __forceinline__ double gv_ldexp_bits(double x, int E) {
 // w = J g as a double.
 __device__ __forceinline__ double gv_weight(const GvJac<double>& J, double g) {
   return __dmul_rn(J.v, g);
+}
+__device__ __forceinline__ double gv_weight(const GvJac<GvX>& J, const GvX& g) {
+  return x_to_double(x_mul(J.v, g));
 }
 __device__ __forceinline__ double gv_weight(const GvJac<float>& J, float g) {
   const float p = __fmul_rn(J.m, g);
@@ -240,6 +294,16 @@ template <>
 struct GvPair<double> {
   using T = GvBin64;
 };
+// One bin as the 64-bit-significand form reads it: edge and width as
+// fractions, and the Jacobian factor N w = jm 2^je, jm in [2^63, 2^64).
+struct __align__(16) GvBinX {
+  unsigned long long e, w, jm;
+  long long je;
+};
+template <>
+struct GvPair<GvX> {
+  using T = GvBinX;
+};
 
 // Shared-memory layout of the fill kernel (bytes), 16-byte aligned pieces:
 //   evs  [R][T]   u32     the events between the two passes (GvEvent), slot
@@ -248,8 +312,9 @@ struct GvPair<double> {
 //                         waits for its predecessor (see below), W = 4
 //                         ceil(d/4); over evs: a thread replaces its event's
 //                         words by the event
-//   ew   [d*N]    GvBin32 (e, w, jm, je) in the FP32 form, GvBin64 (e, w) in FP64
-//   jac  [d*N]    f64     Jacobian factor N*(e_{i+1}-e_i) (FP64 form only)
+//   ew   [d*N]    GvBin32 (e, w, jm, je) in FP32, GvBin64 (e, w) on the FP64
+//                         pipe, GvBinX with 64-bit significands
+//   jac  [d*N]    f64     Jacobian factor N*(e_{i+1}-e_i) (FP64 pipe only)
 // After the first pass the forward fill's limbs lie over what follows evs (a
 // persistent kernel keeps the grid, so there they follow it):
 //   hist [d*N][L] u32     the bins' limbs
@@ -290,18 +355,18 @@ __host__ __device__ constexpr int gv_event_words32(bool f64, bool reg_bins, bool
 struct GvFillSmem {
   size_t wd, ew, jac, limbs, hist, hh, hw, lq, lw, bins, po, ps, total;
   int L;
-  __host__ __device__ GvFillSmem(int d, int N, int real_bytes, bool forward, bool bins_smem,
+  __host__ __device__ GvFillSmem(int d, int N, int form, bool forward, bool bins_smem,
                                  int nhist = 0, bool plus = false, bool words = false,
                                  bool keep_grid = false, int T = GV_TILE) {
     const size_t dN = (size_t)d * N;
-    const bool f64 = real_bytes == 8;
+    const bool f64 = form != GV_FORM_F32;
     L = gv_limbs(d * N);
     const size_t evs = forward ? (size_t)gv_event_words32(f64, !bins_smem, plus) * T * 4 : 0;
     const size_t wds = words ? (size_t)((d + 3) / 4) * 4 * T * 4 : 0;
     wd = 0;
     ew = wds > evs ? wds : evs;
-    jac = ew + dN * 16;
-    const size_t first = gv_align16(jac + (f64 ? dN * 8 : 0));
+    jac = ew + dN * (form == GV_FORM_X64 ? 32 : 16);
+    const size_t first = gv_align16(jac + (form == GV_FORM_F64 ? dN * 8 : 0));
     limbs = keep_grid ? first : evs;
     hist = limbs;
     hh = hist + (forward ? dN * L * 4 : 0);
@@ -315,8 +380,8 @@ struct GvFillSmem {
     total = gv_align16(ps + (plus ? (size_t)GV_PLUS_SEGS * 16 : 0));
   }
   // bytes of the limbs, from `limbs`
-  __host__ __device__ size_t limb_bytes(int real_bytes) const {
-    return lw + (size_t)gv_lane_rows(real_bytes == 8) * 32 * 4 - limbs;
+  __host__ __device__ size_t limb_bytes(bool f64) const {
+    return lw + (size_t)gv_lane_rows(f64) * 32 * 4 - limbs;
   }
 };
 
@@ -437,6 +502,14 @@ __device__ __forceinline__ void gv_plus_strat(const unsigned (&c)[MAXD], int d, 
   }
 }
 
+// A bin's record from its edge and width (e in [0, 1), 0 < w < 1, exact to
+// 2^-64); N w is exact: 53 + 10 bits.
+__device__ __forceinline__ GvBinX gv_bin_x(double e, double w, int N) {
+  const GvX E = x_from(e), W = x_from(w);
+  const GvX j = x_norm((W.m >> 11) * (unsigned long long)N, W.e + 11);
+  return GvBinX{E.m ? x_to_q64(E) : 0ull, x_to_q64(W), j.m, (long long)j.e};
+}
+
 // Stage the grid of one integration into shared memory.
 template <typename Real>
 __device__ __forceinline__ void gv_stage_grid(const double* grid, int d, int N, double* s_jac,
@@ -447,6 +520,11 @@ __device__ __forceinline__ void gv_stage_grid(const double* grid, int d, int N, 
   if constexpr (sizeof(Real) == 4) {
     const uint4* g = reinterpret_cast<const uint4*>(grid + L.off_bin32());
     for (int k = tid; k < dN; k += nthr) reinterpret_cast<uint4*>(s_ew)[k] = __ldcg(g + k);
+  } else if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
+    for (int k = tid; k < dN; k += nthr) {
+      const int a = k / N, i = k - a * N;
+      s_ew[k] = gv_bin_x(grid[L.off_e64() + a * (N + 1) + i], grid[L.off_wd64() + k], N);
+    }
   } else {
     for (int k = tid; k < dN; k += nthr) {
       const int a = k / N, i = k - a * N;
@@ -464,11 +542,14 @@ __device__ __forceinline__ void gv_stage_grid(const double* grid, int d, int N, 
 // written, J the FP64 product of the factors N (e_{i+1}-e_i); FP32: x with
 // FP32 edges and one fma, J as FP32 mantissa product and exponent sum.  The
 // product starts from the first factor (J = 1 * f0 * f1 ... exactly).
+// 64-bit significands: x = e + w (2 lo + 1) 2^-33 in fractions, J the product
+// of the normalised factors.
 template <typename Real, int MAXD>
 __device__ __forceinline__ GvJac<Real> gv_map_event(const uint32_t (&r)[MAXD], int d, int N,
                                                     const double* s_jac,
                                                     const typename GvPair<Real>::T* s_ew,
-                                                    Real (&x)[MAXD], int (&bin)[MAXD]) {
+                                                    typename GvForm<Real>::Coord (&x)[MAXD],
+                                                    int (&bin)[MAXD]) {
   GvJac<Real> J;
 #pragma unroll
   for (int a = 0; a < MAXD; ++a) {
@@ -477,7 +558,11 @@ __device__ __forceinline__ GvJac<Real> gv_map_event(const uint32_t (&r)[MAXD], i
       const int i = (int)(v >> 32);
       const uint32_t lo = (uint32_t)v;
       const auto ew = s_ew[a * N + i];
-      if constexpr (sizeof(Real) == 4) {
+      if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
+        x[a] = ew.e + xi_mul64x32(ew.w, lo) + (ew.w >> 33);
+        const GvX j = {ew.jm, (int)ew.je, 0u};
+        J.v = (a == 0) ? j : x_mul(J.v, j);
+      } else if constexpr (sizeof(Real) == 4) {
         const float f = fmaf(__uint2float_rn(lo), 0x1p-32f, 0x1p-33f);
         x[a] = fmaf(f, ew.w, ew.e);
         J.m = (a == 0) ? ew.jm : __fmul_rn(J.m, ew.jm);
@@ -634,9 +719,10 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
                                              uint32_t it, bool words = false) {
   constexpr int B = GV_TILE / EPT, T = GV_TILE;
   constexpr int NW = B / 32;
-  constexpr bool F64 = sizeof(Real) == 8;
+  using W = typename GvForm<Real>::W;
+  constexpr bool F64 = sizeof(W) == 8;
   using Pair = typename GvPair<Real>::T;
-  using Event = GvEvent<Real, MAXD, PLUS, T>;
+  using Event = GvEvent<W, MAXD, PLUS, T>;
   __shared__ int s_max[2][NW];
   const int d = a.ndim, N = a.nbins, dN = d * N, L = lay.L;
   const int hb = HIST ? a.nhist : 0;
@@ -657,7 +743,15 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
   [[maybe_unused]] int mq = GV_EMPTY;  // and (VEGAS+) of the bins' quantities F b_h
   {
     GvConst<Real, GvTraits<IG>::NK> K;
-    K.load(a.kconst);
+    if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
+      constexpr int NX = GvTraits<IG>::NX;
+      __shared__ GvX s_k[NX];
+      if (tid < NX) s_k[tid] = gv_x_consts(a.kconst)[tid];
+      __syncthreads();
+      K.k = s_k;
+    } else {
+      K.load(a.kconst);
+    }
     unsigned nbad = 0u;
     // VEGAS+: this thread's range (events tile0 + tid EPT ..), the window index
     // of its current hypercube, that hypercube's digits and factors, and the
@@ -700,7 +794,7 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
           gv_plus_digits<MAXD>((unsigned)(h0 + jc), d, (unsigned)pf->s, pf->inv_s, cdig);
         gv_plus_strat<MAXD>(cdig, d, (unsigned)pf->s, pf->magic, r);
       }
-      Real x[MAXD];
+      typename GvForm<Real>::Coord x[MAXD];
       int bin[MAXD];
       const GvJac<Real> J = gv_map_event<Real, MAXD>(r, d, N, s_jac, s_ew, x, bin);
       if constexpr (!Event::REG) {
@@ -712,10 +806,9 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
       int hbin = 0;
       if constexpr (HIST) {
         if constexpr (F64)
-          hbin = gv_hist_bin<Real>(gv_observable<IG, Real, MAXD>(x, K), a.h_lo, a.h_invw, hb - 2);
+          hbin = gv_hist_bin<W>(gv_observable<IG, Real, MAXD>(x, K), a.h_lo, a.h_invw, hb - 2);
         else
-          hbin = gv_hist_bin<Real>(gv_observable<IG, Real, MAXD>(x, K), a.h_lo_f, a.h_invw_f,
-                                   hb - 2);
+          hbin = gv_hist_bin<W>(gv_observable<IG, Real, MAXD>(x, K), a.h_lo_f, a.h_invw_f, hb - 2);
       }
       if constexpr (!F64) {
         const unsigned u = __float_as_uint(__fmul_rn(J.m, g));
@@ -820,14 +913,14 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
     mw = __reduce_max_sync(0xffffffffu, s_max[0][lane % NW]);
     if constexpr (PLUS) mq = __reduce_max_sync(0xffffffffu, s_max[1][lane % NW]);
     const bool have_w = mw != GV_EMPTY, have_q = PLUS ? mq != GV_EMPTY : have_w;
-    GvWindow vw = gv_window<Real>(have_w ? mw : 0, L);
-    GvWindow vq = PLUS ? gv_window<Real>(have_q ? mq : 0, L) : vw;
+    GvWindow vw = gv_window<W>(have_w ? mw : 0, L);
+    GvWindow vq = PLUS ? gv_window<W>(have_q ? mq : 0, L) : vw;
     if (!have_w) vw.base = up_w;  // nothing (left)
     if (PLUS && !have_q) vq.base = up_q;
-    if (first && have_w) E = mw + GvSig<Real>::BITS;
+    if (first && have_w) E = mw + GvSig<W>::BITS;
     {
       uint4* z = reinterpret_cast<uint4*>(smem + lay.limbs);
-      const int nz = (int)((lay.limb_bytes((int)sizeof(Real)) + 15) / 16);
+      const int nz = (int)((lay.limb_bytes(F64) + 15) / 16);
       for (int k = tid; k < nz; k += B) z[k] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncthreads();
@@ -848,26 +941,26 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
               bin = ((ax < 2 ? b.x : b.y) >> (10 * (ax & 1))) & 0x3FFu;
             else
               bin = s_bin[ax * T + slot];
-            gv_bin_add_square<Real>(l, row + bin * L4);
+            gv_bin_add_square<W>(l, row + bin * L4);
             row += axis4;
           }
         }
       };
       {
-        const GvSig<Real> s = event.template get<0>();
-        const int h = s.e2 + GvSig<Real>::H;
+        const GvSig<W> s = event.template get<0>();
+        const int h = s.e2 + GvSig<W>::H;
         const int limb = gv_limb_index(h), pos = limb - vw.base;
         if (s.m != 0 && limb < up_w) {
           if (pos >= 0) {
             unsigned l[4];
             gv_square_digits(s, h + GV_SQ_OFF - 11 * limb, l);
-            gv_lane_add_square<Real>(l, a_lq + pos * 128);
+            gv_lane_add_square<W>(l, a_lq + pos * 128);
             gv_lane_add_w(s, a_lw, vw.wbase);
             if constexpr (!PLUS) add_bins(l, pos);
             if constexpr (HIST) {
               const int hbin = event.hbin();
-              gv_bin_add_square<Real>(l, a_hh + 4 * (pos + hbin * L));
-              gv_hist_add_w<Real>(s, a_hw + 4 * (hbin * HW), vw.hbase);
+              gv_bin_add_square<W>(l, a_hh + 4 * (pos + hbin * L));
+              gv_hist_add_w<W>(s, a_hw + 4 * (hbin * HW), vw.hbase);
             }
           } else {
             mw = max(mw, s.e2);
@@ -875,8 +968,8 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
         }
       }
       if constexpr (PLUS) {
-        const GvSig<Real> s = event.template get<1>();
-        const int h = s.e2 + GvSig<Real>::H;
+        const GvSig<W> s = event.template get<1>();
+        const int h = s.e2 + GvSig<W>::H;
         const int limb = gv_limb_index(h), pos = limb - vq.base;
         if (s.m != 0 && limb < up_q) {
           if (pos >= 0) {
@@ -963,7 +1056,7 @@ __device__ __forceinline__ void gv_tile_words(const GvFillArgs& a, uint32_t it, 
 template <typename Real, int EPT, int MAXD, bool PLUS>
 struct GvFillBlocks {
   static constexpr int B = GV_TILE / EPT;
-  static constexpr int value = sizeof(Real) != 4       ? 0
+  static constexpr int value = GvForm<Real>::ID != GV_FORM_F32 ? 0
                                : (PLUS && MAXD == 8)   ? 3
                                : MAXD <= 8             ? 65536 / (64 * B)
                                : (!PLUS && EPT == 4)   ? 3
@@ -977,7 +1070,7 @@ __global__ void __launch_bounds__(GV_TILE / EPT, (GvFillBlocks<Real, EPT, MAXD, 
   extern __shared__ __align__(16) unsigned char smem[];
   const int d = a.ndim, N = a.nbins;
   const bool hoist = MAXD <= 8 && a.hoist;  // set by the host (gv_fill_hoistable)
-  const GvFillSmem lay(d, N, (int)sizeof(Real), true, MAXD > 4, HIST ? a.nhist : 0, PLUS, hoist);
+  const GvFillSmem lay(d, N, GvForm<Real>::ID, true, MAXD > 4, HIST ? a.nhist : 0, PLUS, hoist);
   // the tile's words at the counter this iteration should have (the stage's
   // first counter, which no running kernel writes, plus the iteration index),
   // made while the previous iteration's reduce and refinement finish
@@ -1037,10 +1130,13 @@ __global__ void gv_eval_events_kernel(const GvFillArgs a, uint32_t it, const lon
   const double* jac = a.grid + L.off_jac();
   const GvBin32* b32 = reinterpret_cast<const GvBin32*>(a.grid + L.off_bin32());
   GvConst<Real, GvTraits<IG>::NK> K;
-  K.load(a.kconst);
+  if constexpr (GvForm<Real>::ID == GV_FORM_X64)
+    K.k = gv_x_consts(a.kconst);
+  else
+    K.load(a.kconst);
   uint32_t r[MAXD];
   gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)events[j], d, r);
-  Real x[MAXD];
+  typename GvForm<Real>::Coord x[MAXD];
   GvJac<Real> J;
 #pragma unroll
   for (int ax = 0; ax < MAXD; ++ax) {
@@ -1049,7 +1145,12 @@ __global__ void gv_eval_events_kernel(const GvFillArgs a, uint32_t it, const lon
       const int i = (int)(v >> 32);
       const uint32_t lo = (uint32_t)v;
       const int k = ax * N + i;
-      if constexpr (sizeof(Real) == 4) {
+      if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
+        const GvBinX b = gv_bin_x(e64[ax * (N + 1) + i], wd64[k], N);
+        x[ax] = b.e + xi_mul64x32(b.w, lo) + (b.w >> 33);
+        const GvX f = {b.jm, (int)b.je, 0u};
+        J.v = (ax == 0) ? f : x_mul(J.v, f);
+      } else if constexpr (sizeof(Real) == 4) {
         const float f = fmaf(__uint2float_rn(lo), 0x1p-32f, 0x1p-33f);
         x[ax] = fmaf(f, b32[k].w, b32[k].e);
         J.m = (ax == 0) ? b32[k].jm : __fmul_rn(J.m, b32[k].jm);

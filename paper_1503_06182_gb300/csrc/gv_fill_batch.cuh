@@ -1,6 +1,6 @@
 // gv_fill_batch.cuh -- the persistent fill kernel of the batched form and its
 // launch helpers, instantiated per precision and dimension class in
-// gv_batch_{f,d}{4,8,16}.cu (so that they compile in parallel).  Each class
+// gv_batch_{f,d,x}{4,8,16}.cu (so that they compile in parallel).  Each class
 // (at most 4, 8 or 16 axes) and integrand runs its own work list with code
 // unrolled for it: one kernel holding the three integrands needed the
 // registers of two (219 instead of 96-126 at 16 axes, one CTA per SM
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(GV_TILE / EPT,
     const int b = order[pos];
     const long long tile = item - item_start[pos];
     const GvFillArgs a = args[b];
-    const GvFillSmem lay(a.ndim, a.nbins, (int)sizeof(Real), true, MAXD > 4, 0, false, false, true);
+    const GvFillSmem lay(a.ndim, a.nbins, GvForm<Real>::ID, true, MAXD > 4, 0, false, false, true);
     if (b != cur) {
       gv_stage_grid<Real>(a.grid, a.ndim, a.nbins, reinterpret_cast<double*>(smem + lay.jac),
                           reinterpret_cast<typename GvPair<Real>::T*>(smem + lay.ew),
@@ -159,3 +159,6 @@ GV_DECLARE_FILL_BATCH(f16)
 GV_DECLARE_FILL_BATCH(d4)
 GV_DECLARE_FILL_BATCH(d8)
 GV_DECLARE_FILL_BATCH(d16)
+GV_DECLARE_FILL_BATCH(x4)
+GV_DECLARE_FILL_BATCH(x8)
+GV_DECLARE_FILL_BATCH(x16)

@@ -130,14 +130,20 @@ static cudaError_t gv_launch_eval_t(const GvFillArgs& a, uint32_t it, const long
                               long long n, double* w, int* bins, cudaStream_t s);             \
   cudaError_t NAME##_eval_f64(const GvFillArgs& a, uint32_t it, const long long* ev,          \
                               long long n, double* w, int* bins, cudaStream_t s);             \
-  cudaError_t NAME(int fp32, int ept, const GvFillArgs& a, int n_tiles, size_t smem,          \
+  cudaError_t NAME##_x64(int ept, const GvFillArgs& a, int n_tiles, size_t smem,              \
+                         cudaStream_t s, bool pdl);                                           \
+  cudaError_t NAME##_eval_x64(const GvFillArgs& a, uint32_t it, const long long* ev,          \
+                              long long n, double* w, int* bins, cudaStream_t s);             \
+  cudaError_t NAME(int form, int ept, const GvFillArgs& a, int n_tiles, size_t smem,          \
                    cudaStream_t s, bool pdl) {                                                \
-    return fp32 ? NAME##_f32(ept, a, n_tiles, smem, s, pdl)                                   \
-                : NAME##_f64(ept, a, n_tiles, smem, s, pdl);                                  \
+    return form == GV_FORM_F32   ? NAME##_f32(ept, a, n_tiles, smem, s, pdl)                  \
+           : form == GV_FORM_X64 ? NAME##_x64(ept, a, n_tiles, smem, s, pdl)                  \
+                                 : NAME##_f64(ept, a, n_tiles, smem, s, pdl);                 \
   }                                                                                           \
-  cudaError_t NAME##_eval(int fp32, const GvFillArgs& a, uint32_t it, const long long* ev,    \
+  cudaError_t NAME##_eval(int form, const GvFillArgs& a, uint32_t it, const long long* ev,    \
                           long long n, double* w, int* bins, cudaStream_t s) {                \
-    return fp32 ? NAME##_eval_f32(a, it, ev, n, w, bins, s)                                   \
-                : NAME##_eval_f64(a, it, ev, n, w, bins, s);                                  \
+    return form == GV_FORM_F32   ? NAME##_eval_f32(a, it, ev, n, w, bins, s)                  \
+           : form == GV_FORM_X64 ? NAME##_eval_x64(a, it, ev, n, w, bins, s)                  \
+                                 : NAME##_eval_f64(a, it, ev, n, w, bins, s);                 \
   }                                                                                           \
   }

@@ -34,6 +34,7 @@
 #include "gv_ff.cuh"
 #include "gv_integrands.cuh"
 #include "gv_limbs.cuh"
+#include "gv_xint.cuh"
 
 // Slots (GvSlot: 192 bits and an exponent) are written by one thread and read
 // by CTAs that took a ticket after the writer's fence: L2 loads.
@@ -1001,6 +1002,31 @@ __global__ void gv_consts_kernel(int ig, const double* p, double* K) {
   }
   float* kf = reinterpret_cast<float*>(K + GV_NCONST_F32);
   for (int i = 0; i < GV_NCONST_F32; ++i) kf[i] = (float)K[i];
+  // 64-bit significands (read only where gv_x64_applies)
+  GvX* X = reinterpret_cast<GvX*>(K + GV_NCONST);
+  for (int i = 0; i < GV_NCONST_X; ++i) X[i] = x_zero();
+  if (ig == GV_GAUSS) {
+    X[XK_INV2S2] = x_mul(x_from(K[GK_INV2S2]), GV_X_LOG2E);
+    X[XK_MSHIFT] = x_from(-K[GK_SHIFT]);
+  } else if (ig == GV_EE3J) {
+    X[XK_YCUT].m = x_to_q64(x_from(K[EK_YCUT]));
+  } else {
+    const GvX B = x_mul(x_from(-K[DK_LOGTAULO]), GV_X_LOG2E);
+    const GvX A = x_mul(x_from(K[DK_L]), GV_X_LOG2E);
+    const int sh = B.e - A.e;
+    X[XK_B2] = B;
+    X[XK_A2].m = sh < 64 ? A.m >> max(sh, 0) : 0ull;
+    X[XK_CP] = x_mul(x_mul(x_from(K[DK_L]), GV_X_LN2), x_from(K[DK_PREF]));
+    X[XK_SQRTS] = x_from(K[DK_SQRTS]);
+    X[XK_MMZ2] = x_from(-K[DK_MZ2]);
+    X[XK_BETA2] = x_mul(x_from(K[NK_BETA]), GV_X_LOG2E);
+    const int from[] = {DK_GM2, DK_KAPPA, DK_CA0, DK_CA1, DK_CA2, DK_CB1, DK_CB2, DK_A,
+                        DK_B,   DK_NORM,  DK_MZ,  DK_GZ,  DK_DKAPPA, DK_DCA1, DK_DCA2, DK_DCB2};
+    const int to[] = {XK_GM2, XK_KAPPA, XK_CA0, XK_CA1, XK_CA2, XK_CB1, XK_CB2, XK_A,
+                      XK_B,   XK_NORM,  XK_MZ,  XK_GZ,  XK_DKAPPA, XK_DCA1, XK_DCA2, XK_DCB2};
+    for (int i = 0; i < 16; ++i) X[to[i]] = x_from(K[from[i]]);
+    X[XK_INVI0] = x_from(K[NK_INVI0]);
+  }
 }
 
 // Reset the per-iteration state (at creation and after the autotuner's
