@@ -64,7 +64,7 @@ extern "C" {
 #define VEGAS_MAX_BINS 1024
 #define VEGAS_MAX_DIM_BINS 4096 /* ndim * nbins */
 #define VEGAS_NGRAD 5           /* Drell-Yan gradient: M_Z, Gamma_Z, sin2_thetaW, a, b */
-#define VEGAS_TILE 1024         /* canonical events per tile */
+#define VEGAS_TILE 1024         /* most events per tile (the unit of the exact sums) */
 
 /* ---- options (vegas_set_option / vegas_batch_set_option) ---- */
 #define VEGAS_OPT_ALPHA 0     /* grid damping exponent alpha >= 0 (default 1.5) */

@@ -56,7 +56,7 @@ int batch_check_params(int ig, int ndim, const double* p, int np) {
   return VEGAS_EINVAL;
 }
 
-// Rough relative cost of one tile, for the largest-first order only.
+// Rough relative cost of one event, for the largest-first order only.
 double tile_cost(int ig, int d) {
   switch (ig) {
     case VEGAS_GAUSS: return 1.0 + 0.25 * d;
@@ -66,7 +66,7 @@ double tile_cost(int ig, int d) {
 }
 
 struct Member {
-  int ig, d, np, form, n_tiles, nacc, gx, gy;
+  int ig, d, np, form, tile_events, n_tiles, nacc, gx, gy;
   int64_t ncall;
   double params[GV_MAXPARAMS];
   double* grid;
@@ -211,6 +211,7 @@ int upload_tables(vegas_batch* B) {
     a.nbins = B->N;
     a.nch = 1;
     a.nacc = x.nacc;
+    a.tile_events = x.tile_events;
     a.ncall = x.ncall;
     a.seed = B->seed;
     a.batch = (unsigned)b;
@@ -403,7 +404,8 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
     x.form = precision ? GV_FORM_F32
              : gv_x64_applies(x.ig, x.params, x.np, x.d * nbins) ? GV_FORM_X64
                                                                  : GV_FORM_F64;
-    x.n_tiles = (int)((x.ncall + GV_TILE - 1) / GV_TILE);
+    x.tile_events = gv_tile_events(x.ncall, x.form);
+    x.n_tiles = (int)((x.ncall + x.tile_events - 1) / x.tile_events);
     x.nacc = 2 + x.d * nbins;
     int tpc = 0;
     gv::reduce_grid(x.n_tiles, x.nacc, &tpc, &x.gx, &x.gy);
@@ -487,8 +489,8 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
             mem.push_back(b);
         if (mem.empty()) continue;
         std::stable_sort(mem.begin(), mem.end(), [&](int p, int q) {
-          return B->m[p].n_tiles * tile_cost(B->m[p].ig, B->m[p].d) >
-                 B->m[q].n_tiles * tile_cost(B->m[q].ig, B->m[q].d);
+          return (double)B->m[p].n_tiles * B->m[p].tile_events * tile_cost(B->m[p].ig, B->m[p].d) >
+                 (double)B->m[q].n_tiles * B->m[q].tile_events * tile_cost(B->m[q].ig, B->m[q].d);
         });
         vegas_batch::FillClass c;
         c.maxd = maxd;
@@ -529,7 +531,7 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
       for (int b = 0; b < n; ++b)
         if (B->m[b].ig == B->cls[i].ig && B->m[b].form == B->cls[i].form &&
             dim_class(B->m[b].ig, B->m[b].d) == B->cls[i].maxd)
-          cost[i] += (double)B->m[b].n_tiles * tile_cost(B->m[b].ig, B->m[b].d);
+          cost[i] += (double)B->m[b].n_tiles * B->m[b].tile_events * tile_cost(B->m[b].ig, B->m[b].d);
     for (size_t i = 0; i < B->cls.size(); ++i) B->launch_order.push_back((int)i);
     std::stable_sort(B->launch_order.begin(), B->launch_order.end(),
                      [&](int p, int q) { return cost[p] > cost[q]; });

@@ -115,12 +115,13 @@ static_assert(sizeof(GvState) <= kHostRecOff, "state fits before the records");
 std::mutex g_tune_mu;
 std::map<std::string, int> g_tune;
 
-std::string tune_key(int dev, int ig, int form, int mode, int d, int N, int n_tiles) {
+std::string tune_key(int dev, int ig, int form, int mode, int d, int N, int T,
+                     int n_tiles) {
   char buf[160];
   int lg = 0;
   while ((1 << (lg + 1)) <= n_tiles && lg < 30) ++lg;
-  snprintf(buf, sizeof buf, "dev%d:ig%d:fp%d:m%d:d%d:N%d:t%d", dev, ig, form, mode, maxd_class(d),
-           N, lg);
+  snprintf(buf, sizeof buf, "dev%d:ig%d:fp%d:m%d:d%d:N%d:T%d:t%d", dev, ig, form, mode,
+           maxd_class(d), N, T, lg);
   return buf;
 }
 
@@ -221,9 +222,9 @@ size_t grid_doubles(int d, int N) { return GvGridLayout{d, N}.doubles(); }
 // chained iterations per autotuning trial (iteration records are sized for them)
 constexpr int kTuneIter = 8;
 
-size_t workspace_bytes(int d, int N, int64_t ncall, int itmx, int mode, int nhist,
+size_t workspace_bytes(int d, int N, int64_t ncall, int itmx, int mode, int nhist, int T,
                        bool plus_f = false) {
-  const int64_t n_tiles = (ncall + GV_TILE - 1) / GV_TILE;
+  const int64_t n_tiles = (ncall + T - 1) / T;
   const int nch = mode ? GV_MAXCH : 1;
   const int nacc = mode ? 2 * GV_MAXCH : 2 + d * N + 2 * nhist;
   int tpc = 0, gx = 0, gy = 0;
@@ -292,7 +293,7 @@ int ensure_pinned(vegas_ctx* c, size_t need) {
 }
 
 struct Plan {
-  int ig, form, mode, itmx, n_tiles, nacc, nch, ept, reduce_ctas, tiles_per_cta;
+  int ig, form, mode, itmx, tile_events, n_tiles, nacc, nch, ept, reduce_ctas, tiles_per_cta;
   int nhist;  // histogram bins with underflow and overflow (0: none)
   int slot_major;  // slot-major partials and the single-level reduce (forward stages)
   int hoist;       // the fill makes its Philox words before it waits (gv_fill_hoistable)
@@ -327,6 +328,7 @@ GvFillArgs fill_args(const vegas_ctx* c, const Plan& p, int k = 0) {
   a.slot_major = p.slot_major;
   a.hoist = p.hoist;
   a.n_tiles = p.n_tiles;
+  a.tile_events = p.tile_events;
   a.nhist = p.nhist;
   if (p.nhist) {
     const double invw = (double)c->hist_nh / (c->hist_hi - c->hist_lo);
@@ -598,7 +600,7 @@ int autotune_chained(vegas_ctx* c, Plan& p, const std::string& key) {
 }
 
 int autotune(vegas_ctx* c, Plan& p) {
-  const std::string key = tune_key(c->device, p.ig, p.form, p.mode, c->ndim, c->nbins, p.n_tiles);
+  const std::string key = tune_key(c->device, p.ig, p.form, p.mode, c->ndim, c->nbins, p.tile_events, p.n_tiles);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(key);
@@ -688,7 +690,9 @@ int make_plan(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* param
     cap = ncall + 2 * p.nh;
   }
   p.cap = cap;
-  const int64_t nt = (cap + GV_TILE - 1) / GV_TILE;
+  // the adjoint's and the stratified fill's tiles have one size
+  p.tile_events = mode || p.plus ? GV_TILE : gv_tile_events(ncall, p.form);
+  const int64_t nt = (cap + p.tile_events - 1) / p.tile_events;
   if (nt > 0x7fffffff) return VEGAS_EINVAL;
   p.n_tiles = (int)nt;
   p.nch = mode ? GV_MAXCH : 1;
@@ -709,7 +713,7 @@ int make_plan(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* param
   int gx = 0, gy = 0;
   gv::reduce_grid(p.n_tiles, p.nacc, &p.tiles_per_cta, &gx, &gy);
   p.reduce_ctas = gx * gy;
-  const size_t need = workspace_bytes(c->ndim, c->nbins, cap, itmx, mode, p.nhist, p.plus != 0);
+  const size_t need = workspace_bytes(c->ndim, c->nbins, cap, itmx, mode, p.nhist, p.tile_events, p.plus != 0);
   int st = ensure_workspace(c, need);
   if (st) return st;
   char* w = (char*)c->ws;
@@ -1244,8 +1248,10 @@ int vegas_set_stream(vegas_ctx* c, void* stream) {
 int vegas_workspace_size(const vegas_ctx* c, int64_t ncall, int itmx, size_t* bytes) {
   if (!c || !bytes || ncall < 2 || itmx < 1) return VEGAS_EINVAL;
   const int nhist = c->hist_nh > 0 ? c->hist_nh + 2 : 0;
-  *bytes = std::max(workspace_bytes(c->ndim, c->nbins, ncall, itmx, 0, nhist),
-                    workspace_bytes(c->ndim, c->nbins, ncall, itmx, 1, 0));
+  // FP64's tiles are no larger than FP32's: room for either
+  const int T = std::min(gv_tile_events(ncall, GV_FORM_F32), gv_tile_events(ncall, GV_FORM_X64));
+  *bytes = std::max(workspace_bytes(c->ndim, c->nbins, ncall, itmx, 0, nhist, T),
+                    workspace_bytes(c->ndim, c->nbins, ncall, itmx, 1, 0, GV_TILE));
   return VEGAS_OK;
 }
 

@@ -2,7 +2,7 @@
 //
 // One VEGAS iteration (Section 2.1: events evaluated independently, all events
 // combined, serial grid optimisation) runs as two kernels:
-//   fill   : one CTA per tile of GV_TILE consecutive events; uniforms from
+//   fill   : one CTA per tile of up to GV_TILE consecutive events; uniforms from
 //            Philox4x32-10, grid map, integrand, then exact integer
 //            accumulation of sum w, sum w^2 and the per-bin sums of w^2
 //            into a per-tile partial;
@@ -32,7 +32,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-#define GV_TILE 1024          // canonical events per tile
+#define GV_TILE 1024          // most events of a tile (see gv_tile_events)
 #define GV_FB 96              // fixed-point bits below a tile's scale
 #define GV_MAXD 16            // maximum number of axes
 #define GV_NGRAD 5            // Drell-Yan gradient components
@@ -54,6 +54,29 @@ enum { GV_GAUSS = 0, GV_DY = 1, GV_EE3J = 2, GV_DYNLO = 3 };
 // Arithmetic of an event: the FP64 pipe, FP32, or 64-bit significands on the
 // integer pipes (gv_x64.cuh).
 enum { GV_FORM_F64 = 0, GV_FORM_F32 = 1, GV_FORM_X64 = 2 };
+
+// Events per tile of a stage of ncall events (plain forward stages, single or
+// batched): 128 to GV_TILE, a function of the call count and the arithmetic
+// alone, so that results do not depend on the launch shape.  One tile is one
+// CTA: the size minimises the rounds of tiles over the 152 SMs times a tile's
+// time, its events plus a fixed part (staging, zeroing, epilogue) worth t0
+// events.  Ten iterations with 128 and with 1024 events a tile: 1e4 calls of
+// the FP64 NLO-shaped weight on 13 axes 297 and 619 us, of FP64 Drell-Yan 199
+// and 287, of FP32 Drell-Yan 159 and 162; with 256 and 1024: 1e5 calls of FP64
+// NLO 578 and 632, of FP32 Drell-Yan 196 and 176 (there the rule keeps 1024).
+inline int gv_tile_events(long long ncall, int form) {
+  const long long t0 = form == GV_FORM_F32 ? 256 : 96;
+  long long best = 0;
+  int T = GV_TILE;
+  for (int t = GV_TILE; t >= 128; t /= 2) {
+    const long long tiles = (ncall + t - 1) / t, cost = (tiles + 151) / 152 * (t + t0);
+    if (best == 0 || cost < best) {
+      best = cost;
+      T = t;
+    }
+  }
+  return T;
+}
 
 // Whether the FP64 form runs on 64-bit significands: parameters of ordinary
 // size (every derived constant finite, momentum fractions above 2^-60, y_cut
@@ -148,6 +171,7 @@ struct GvPlusFill {
 // Arguments of the fill kernels (forward and adjoint).
 struct GvFillArgs {
   int ndim, nbins, nch, nacc;
+  int tile_events;               // events per tile
   long long ncall;
   unsigned long long seed;
   unsigned batch;

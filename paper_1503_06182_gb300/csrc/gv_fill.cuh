@@ -1,6 +1,6 @@
 // gv_fill.cuh -- the fused per-event kernel of one VEGAS iteration.
 //
-// One CTA evaluates one tile of GV_TILE consecutive events (Section 2.1: each
+// One CTA evaluates one tile of up to GV_TILE consecutive events (Section 2.1: each
 // event generated and evaluated independently), with EPT events per thread:
 //   pass 1: Philox words -> bins and in-bin positions -> x on the adaptive grid
 //           ((edge, width) pairs and Jacobian factors staged in shared memory)
@@ -717,7 +717,7 @@ template <int IG, typename Real, int EPT, int MAXD, bool HIST = false, bool PLUS
 __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile,
                                              unsigned char* smem, const GvFillSmem& lay,
                                              uint32_t it, bool words = false) {
-  constexpr int B = GV_TILE / EPT, T = GV_TILE;
+  constexpr int B = GV_TILE / EPT, T = GV_TILE;  // T: stride of the arrays
   constexpr int NW = B / 32;
   using W = typename GvForm<Real>::W;
   constexpr bool F64 = sizeof(W) == 8;
@@ -736,8 +736,9 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
   unsigned short* s_bin = reinterpret_cast<unsigned short*>(smem + lay.bins);
   unsigned* evs = reinterpret_cast<unsigned*>(smem + lay.wd);
   const int tid = threadIdx.x;
-  const long long tile0 = tile * T;
-  const int n_ev = (int)min((long long)T, ncall - tile0);  // events of this tile
+  const long long tile0 = tile * a.tile_events;
+  const int n_ev = (int)min((long long)a.tile_events, ncall - tile0);  // events of this tile
+  const int nk = PLUS ? EPT : (a.tile_events + B - 1) / B;             // events per thread
 
   int mw = GV_EMPTY;                   // the largest exponent of the thread's weights
   [[maybe_unused]] int mq = GV_EMPTY;  // and (VEGAS+) of the bins' quantities F b_h
@@ -763,7 +764,7 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
     constexpr bool KEEP_DIGITS = MAXD <= 4;  // registers to spare only for few axes
     [[maybe_unused]] unsigned cdig[MAXD];
 #pragma unroll 1
-    for (int k = 0; k < EPT; ++k) {
+    for (int k = 0; k < nk; ++k) {
       const int local = PLUS ? tid * EPT + k : k * B + tid;
       const int slot = k * B + tid;
       const Event event{evs + slot};
@@ -927,7 +928,7 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
     mw = GV_EMPTY;
     mq = GV_EMPTY;
 #pragma unroll 1
-    for (int k = 0; k < EPT; ++k) {
+    for (int k = 0; k < nk; ++k) {
       const int slot = k * B + tid;
       const Event event{evs + slot};
       const auto add_bins = [&](const unsigned (&l)[4], int pos) {
@@ -1032,9 +1033,10 @@ template <int MAXD, int T, int B, bool PLUS>
 __device__ __forceinline__ void gv_tile_words(const GvFillArgs& a, uint32_t it, long long tile,
                                               unsigned* s_words) {
   const int d = a.ndim;
-  const long long t0 = tile * T;
+  const long long t0 = tile * a.tile_events;
+  const int nk = PLUS ? T / B : (a.tile_events + B - 1) / B;
 #pragma unroll 1
-  for (int k = 0; k < T / B; ++k) {
+  for (int k = 0; k < nk; ++k) {
     const int local = PLUS ? (int)threadIdx.x * (T / B) + k : k * B + (int)threadIdx.x;
     const int slot = k * B + (int)threadIdx.x;
     uint32_t r[MAXD];

@@ -1,6 +1,7 @@
 """GPU path: the tile's limb sums at the edges of their windows (requires a
 GB300).  Weights over hundreds of binades take several windows per tile, and
 the number of bins chooses the row length (9, 7 or 5 limbs)."""
+import math
 from fractions import Fraction
 
 import numpy as np
@@ -65,3 +66,33 @@ def test_wide_weights_identical_across_launch_shapes():
         B.close()
     for per, grid in outs[1:]:
         assert np.array_equal(per, outs[0][0]) and np.array_equal(grid, outs[0][1])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("ncall", [2, 127, 128, 129, 19456, 19457, 38913, 77824, 100_001])
+def test_sums_at_the_edges_of_the_tile_sizes(ncall, precision):
+    """Every tile size and its last, partly filled tile: the sums against sums
+    of the events' own weights, rounded once (math.fsum; the squares' own
+    roundings add 2^-53), and the same bits for every block size."""
+    p = (0.1, 0.1)  # weights of both signs
+    sums = []
+    for ept in (1, 2, 4, 8):
+        g = v.Vegas(3, 40, 11, precision=precision)
+        try:
+            g.set(v.VEGAS_OPT_EPT, ept)
+            g.iterate(ncall, 1, v.VEGAS_GAUSS, p)
+            sums.append(g.last_sums())
+            if ept == 8:
+                g.grid = np.tile(np.arange(41) / 40, (3, 1))
+                w, bins = g.eval_events(v.VEGAS_GAUSS, p, 0, np.arange(ncall))
+        finally:
+            g.close()
+    assert all(np.array_equal(s, sums[0]) for s in sums[1:])
+    w2 = w * w
+    scale = math.fsum(np.abs(w))
+    assert abs(sums[0][0] - math.fsum(w)) <= 2.0 ** -52 * scale
+    assert abs(sums[0][1] - math.fsum(w2)) <= 2.0 ** -51 * sums[0][1]
+    for a in range(3):
+        for b in range(40):
+            want = math.fsum(w2[bins[:, a] == b])
+            assert abs(sums[0][2 + 40 * a + b] - want) <= 2.0 ** -51 * want
