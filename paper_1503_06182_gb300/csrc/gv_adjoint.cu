@@ -7,63 +7,40 @@
 // fixed-point sums (values and squares) to the tile's partial, as the forward
 // fill does for its one channel.
 //
-// The six values of each event are staged in shared memory (FP32 form: the
-// FP32 products J.m g and the exponent J.e, 28 KB a tile; FP64 form: the
-// weights, 48 KB), not held in registers across the tile's maximum, so that
-// two 512-thread or three 256-thread CTAs share an SM.  In the FP32 form a
-// weight is a 24-bit significand times a power of two, and its fixed-point
-// terms are formed from that significand (gv_direct*: one 32 x 32 -> 64 bit
-// square), the same exactly rounded integers as through the double, with
-// less integer work.  All six channels share the block-wide
-// steps: one barrier after the per-warp maxima, one after the tile scales,
-// one after the per-warp sums.  Each warp's twelve 128-bit sums leave the warp
-// by a reduce-scatter (every shuffle step halves the values a lane carries),
-// so a warp shuffles 13 128-bit values instead of 12 x 5.
+// Bound by instruction issue.  As in the forward fill, both passes are rolled
+// loops and the events' six values wait between them in shared memory (FP32
+// form: the FP32 products J.m g and the exponent J.e, 28 KB a tile; FP64 form:
+// the weights, 48 KB); the second pass adds each value's and its square's
+// digits to per-lane columns of limbs (gv_limbs.cuh): about 45 instructions a
+// channel, where 128-bit shifts and adds in registers and a reduce-scatter of
+// twelve 128-bit sums per warp took twice that.  1e7 FP32 events on 4 axes: 370
+// before, 283 us now (1136 and 918 instructions per event, 83% of issue slots,
+// 1.7 warps waiting to issue); 1e5 FP64 events 75 and 38 us.
 #include "gv_fill_inst.cuh"
 
 namespace {
 
-constexpr int kNch = GV_MAXCH;     // channels
-constexpr int kNsum = 2 * kNch;    // per channel: sum v, sum v^2
-static_assert(kNsum == 12, "the reduce-scatter below is laid out for 12 sums");
+constexpr int kNch = GV_MAXCH;   // channels
+constexpr int kNsum = 2 * kNch;  // per channel: sum v, sum v^2
+constexpr int kL = 9;            // limbs of a square's column
 
-// One reduce-scatter step over lane distance `mask`: the lane with that bit
-// set keeps the upper half of x, its partner the lower half, and each adds
-// the partner's copy of the half it keeps.
-template <int N>
-__device__ __forceinline__ void rs_step(const u128 (&x)[2 * N], u128 (&y)[N], int mask,
-                                        bool up) {
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    const u128 send = up ? x[i] : x[i + N];
-    const u128 keep = up ? x[i + N] : x[i];
-    const u128 recv = {shfl_xor_u64(send.lo, mask), shfl_xor_u64(send.hi, mask)};
-    y[i] = add128(keep, recv);
-  }
-}
-
-// Bytes of the per-event values staged in shared memory after the grid, for
-// the tile's GV_TILE events: FP64 form, the six weights; FP32 form, the six
-// FP32 products J.m g and the event's Jacobian exponent J.e.
+// Shared memory of the adjoint fill (bytes, 16-byte aligned): the events'
+// values, the lanes' columns, the grid.
 template <typename Real>
-constexpr size_t stage_bytes() {
-  return sizeof(Real) != 4 ? (size_t)GV_TILE * kNch * 8 : (size_t)GV_TILE * (kNch + 1) * 4;
-}
-
-// A weight's two fixed-point terms through the general FP64 route.
-__device__ __forceinline__ void adj_add_double(double x, int E, u128& s1, u128& s2) {
-  if (gv_abs_bits(x) == 0ull) return;
-  const GvDecoded dv = gv_decode(x);
-  s1 = add128(s1, gv_fixed_tile(dv, E));
-  s2 = add128(s2, gv_square_tile(dv, gv_square_hi(dv.m), E));
-}
+struct AdjSmem {
+  static constexpr bool F64 = GvForm<Real>::ID != GV_FORM_F32;
+  static constexpr int WORDS = F64 ? 2 * kNch : kNch + 1;  // per event
+  static constexpr int ROWS = kL + gv_lane_rows(F64);      // per channel: of v^2, then of v
+  static constexpr size_t lanes = (size_t)WORDS * GV_TILE * 4;
+  static constexpr size_t grid = lanes + (size_t)kNch * ROWS * 32 * 4;
+};
 
 // Register budget of the FP32 kernels: 64 registers at 1024 or 512 threads
-// (one or two CTAs per SM), 80 at 256 (three CTAs; the staging buffer allows
-// no fourth).  The FP64 kernels would spill under it and keep their own.
+// (one or two CTAs per SM), and four CTAs at 256.  The FP64 kernels would
+// spill under it and keep their own.
 template <typename Real, int EPT>
 struct AdjBlocks {
-  static constexpr int value = sizeof(Real) == 4 ? (EPT == 4 ? 3 : (EPT == 2 ? 2 : 1)) : 1;
+  static constexpr int value = GvForm<Real>::ID == GV_FORM_F32 ? (EPT == 4 ? 4 : (EPT == 2 ? 2 : 1)) : 1;
 };
 
 }  // namespace
@@ -71,23 +48,24 @@ struct AdjBlocks {
 template <typename Real, int EPT, int MAXD>
 __global__ void __launch_bounds__(GV_TILE / EPT, AdjBlocks<Real, EPT>::value)
     gv_fill_adjoint_kernel(const GvFillArgs a) {
-  constexpr int B = GV_TILE / EPT;
+  constexpr int B = GV_TILE / EPT, T = GV_TILE;  // T: stride of the events' arrays
   constexpr int NW = B / 32;
-  constexpr bool F32 = sizeof(Real) == 4;
+  using Lay = AdjSmem<Real>;
+  using W = typename GvForm<Real>::W;
   using Pair = typename GvPair<Real>::T;
+  constexpr bool F64 = Lay::F64;
+  constexpr int kOdd = 1 << 30;  // on J.e: a product or exponent out of the ordinary
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int red_max[NW][kNch];
-  __shared__ u128 red_sum[NW][kNsum];
-  __shared__ int s_E[kNch];
+  __shared__ int s_max[kNch][NW], s_E[kNch];
+  __shared__ int4 s_win[kNch];  // the window's base and wbase, the limb index below which
+                                // values are still to be added, whether there are any
+  __shared__ u128 s_sum[kNsum];
   const int d = a.ndim, N = a.nbins;
   const GvFillSmem lay(d, N, GvForm<Real>::ID, false, false);
-  double* s_jac = reinterpret_cast<double*>(smem + lay.jac);
-  Pair* s_ew = reinterpret_cast<Pair*>(smem + lay.ew);
-  // channel c of the thread's k-th event at [(k kNch + c) B + tid]: FP64
-  // form, the weight; FP32 form, the bits of J.m g, and J.e at s_je[k B + tid]
-  double* s_v = reinterpret_cast<double*>(smem + lay.total);
-  unsigned* s_p = reinterpret_cast<unsigned*>(smem + lay.total);
-  int* s_je = reinterpret_cast<int*>(smem + lay.total + (size_t)GV_TILE * kNch * 4);
+  double* s_jac = reinterpret_cast<double*>(smem + Lay::grid + lay.jac);
+  Pair* s_ew = reinterpret_cast<Pair*>(smem + Lay::grid + lay.ew);
+  unsigned* evs = reinterpret_cast<unsigned*>(smem);            // [WORDS][T]
+  unsigned* cols = reinterpret_cast<unsigned*>(smem + Lay::lanes);  // [channel][ROWS][32]
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   gv_wait_prior_grid();
   gv_stage_grid<Real>(a.grid, d, N, s_jac, s_ew, tid, B);
@@ -99,188 +77,186 @@ __global__ void __launch_bounds__(GV_TILE / EPT, AdjBlocks<Real, EPT>::value)
   } else {
     K.load(a.kconst);
   }
+  if (tid < kNsum) s_sum[tid] = u128{0ull, 0ull};
+  if (tid < kNch) s_E[tid] = GV_EMPTY;
   const uint32_t it = (uint32_t)a.st->it;
   __syncthreads();
 
   const long long tile = blockIdx.x;
-  const long long tile0 = tile * GV_TILE;
-  // per channel the largest scale gv_scale_exp(|w|) of the thread's weights
-  // (the scale of the largest |w|: the scale is monotonic in |w|)
-  int mE[kNch];
+  const long long tile0 = tile * a.tile_events;
+  const int n_ev = (int)min((long long)a.tile_events, a.ncall - tile0);
+  const int nk = (a.tile_events + B - 1) / B;
+  int mE[kNch];  // per channel the largest exponent of the thread's values
 #pragma unroll
   for (int c = 0; c < kNch; ++c) mE[c] = GV_EMPTY;
-  unsigned long long nbad = 0ull;
-#pragma unroll
-  for (int k = 0; k < EPT; ++k) {
-    const long long ev = tile0 + k * B + tid;
-    int Ev[kNch];
-#pragma unroll
-    for (int c = 0; c < kNch; ++c) Ev[c] = GV_EMPTY;
-    [[maybe_unused]] unsigned pu[kNch];
-    [[maybe_unused]] double vals[kNch];
-    [[maybe_unused]] int je = 0;
-#pragma unroll
-    for (int c = 0; c < kNch; ++c) {
-      pu[c] = 0u;
-      vals[c] = 0.0;
-    }
-    if (ev < a.ncall) {
+  unsigned nbad = 0u;
+#pragma unroll 1
+  for (int k = 0; k < nk; ++k) {
+    const int slot = k * B + tid;
+    bool keep = false;
+    if (slot < n_ev) {
       uint32_t r[MAXD];
-      gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)ev, d, r);
+      gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)(tile0 + slot), d, r);
       typename GvForm<Real>::Coord x[MAXD];
       int bin[MAXD];
       const GvJac<Real> J = gv_map_event<Real, MAXD>(r, d, N, s_jac, s_ew, x, bin);
-      Real gr[GV_NGRAD];
-      Real g;
+      Real gr[1 + GV_NGRAD];
       if constexpr (GvForm<Real>::ID == GV_FORM_X64)
-        g = gv_drell_yan_x<true>(x, K.k, gr);
+        gr[0] = gv_drell_yan_x<true>(x, K.k, gr + 1);
       else
-        g = gv_drell_yan<Real, true>(x, K, gr);
-      bool finite = true;
-      if constexpr (F32) {
-        je = J.e;
-        pu[0] = __float_as_uint(__fmul_rn(J.m, g));
-#pragma unroll
-        for (int p = 0; p < GV_NGRAD; ++p) pu[1 + p] = __float_as_uint(__fmul_rn(J.m, gr[p]));
+        gr[0] = gv_drell_yan<Real, true>(x, K, gr + 1);
+      int ex[kNch];
+      keep = true;  // every channel finite
+      if constexpr (!F64) {
+        // ordinary: every product zero or a normal FP32 number, and every
+        // weight in FP64's normal range whatever the product's exponent;
+        // otherwise gv_sig sorts it out, here and below
+        bool odd = J.e < -890 || J.e > 890;
+        unsigned pu[kNch];
 #pragma unroll
         for (int c = 0; c < kNch; ++c) {
-          if ((pu[c] & 0x7FFFFFFFu) == 0u) continue;
-          const GvDirect w = gv_direct(pu[c], je);
-          if (w.direct) {
-            Ev[c] = w.e2 + 24;  // the double's exponent field - 1022
-          } else {
-            const unsigned long long bits = gv_abs_bits(gv_weight_bits(pu[c], je));
-            finite &= gv_finite_bits(bits);
-            Ev[c] = gv_scale_exp(bits);
+          pu[c] = __float_as_uint(__fmul_rn(J.m, gr[c]));
+          const unsigned ef = (pu[c] >> 23) & 0xFFu;
+          odd = odd || ef == 0xFFu || (ef == 0u && (pu[c] << 1) != 0u);
+          ex[c] = ef ? (int)ef + J.e - 150 : GV_EMPTY;
+          evs[c * T + slot] = pu[c];
+        }
+        if (odd) {
+#pragma unroll
+          for (int c = 0; c < kNch; ++c) {
+            GvSig<float> s;
+            const int ks = gv_sig(pu[c], J.e, s);
+            keep = keep && ks >= 0;
+            ex[c] = ks > 0 ? s.e2 : GV_EMPTY;
           }
         }
+        evs[kNch * T + slot] = (unsigned)(odd ? J.e + kOdd : J.e);
       } else {
-        vals[0] = gv_weight(J, g);
-#pragma unroll
-        for (int p = 0; p < GV_NGRAD; ++p) vals[1 + p] = gv_weight(J, gr[p]);
 #pragma unroll
         for (int c = 0; c < kNch; ++c) {
-          const unsigned long long bits = gv_abs_bits(vals[c]);
-          finite &= gv_finite_bits(bits);
-          Ev[c] = gv_scale_exp(bits);
+          const double v = gv_weight(J, gr[c]);
+          const unsigned long long b = gv_abs_bits(v);
+          keep = keep && gv_finite_bits(b);
+          ex[c] = b ? gv_scale_exp(b) - 53 : GV_EMPTY;
+          const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+          evs[2 * c * T + slot] = (unsigned)u;
+          evs[(2 * c + 1) * T + slot] = (unsigned)(u >> 32);
         }
       }
-      if (!finite) {
-        ++nbad;
+      if (keep) {
 #pragma unroll
-        for (int c = 0; c < kNch; ++c) {
-          pu[c] = 0u;
-          vals[c] = 0.0;
-          Ev[c] = GV_EMPTY;
-        }
+        for (int c = 0; c < kNch; ++c) mE[c] = max(mE[c], ex[c]);
+      } else {
+        ++nbad;  // counted, contributes nothing
       }
     }
+    if (!keep) {
 #pragma unroll
-    for (int c = 0; c < kNch; ++c) {
-      mE[c] = max(mE[c], Ev[c]);
-      if constexpr (F32)
-        s_p[(k * kNch + c) * B + tid] = pu[c];
-      else
-        s_v[(k * kNch + c) * B + tid] = vals[c];
+      for (int j = 0; j < Lay::WORDS; ++j) evs[j * T + slot] = 0u;
     }
-    if constexpr (F32) s_je[k * B + tid] = je;
   }
   gv_allow_next_grid();
 
-  // tile scales: warp maxima, then one thread per channel over the warps
+  // pass 2, once for each set of windows (see gv_fill_tile)
+  bool first = true;
+  for (;;) {
 #pragma unroll
-  for (int c = 0; c < kNch; ++c) {
-    const int m = __reduce_max_sync(0xffffffffu, mE[c]);
-    if (lane == 0) red_max[wid][c] = m;
-  }
-  __syncthreads();
-  if (tid < kNch) {
-    int E = red_max[0][tid];
+    for (int c = 0; c < kNch; ++c) {
+      const int m = __reduce_max_sync(0xffffffffu, mE[c]);
+      if (lane == 0) s_max[c][wid] = m;
+    }
+    __syncthreads();
+    if (tid < kNch) {
+      int m = s_max[tid][0];
 #pragma unroll
-    for (int w = 1; w < NW; ++w) E = max(E, red_max[w][tid]);
-    s_E[tid] = E;
-  }
-  __syncthreads();
-
-  // This thread's exact sums, two channels at a time: channels c and c + 3
-  // hold sums 2c, 2c+1 and 2c+6, 2c+7, which meet in the first step of the
-  // warp's reduce-scatter (lane distance 16), so that step runs as soon as
-  // the pair is formed.
-  [[maybe_unused]] int jek[EPT];
-  if constexpr (F32) {
+      for (int w = 1; w < NW; ++w) m = max(m, s_max[tid][w]);
+      const bool have = m != GV_EMPTY;
+      const int up = first ? 0x40000000 : s_win[tid].x;
+      const GvWindow v = gv_window<W>(have ? m : 0, kL);
+      if (first && have) s_E[tid] = m + GvSig<W>::BITS;
+      s_win[tid] = make_int4(have ? v.base : up, v.wbase, up, have);
+    }
+    {
+      uint4* z = reinterpret_cast<uint4*>(cols);
+      for (int k = tid; k < kNch * Lay::ROWS * 8; k += B) z[k] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    __syncthreads();
+    const unsigned a_cols = gv_shared_address(cols + lane);
 #pragma unroll
-    for (int k = 0; k < EPT; ++k) jek[k] = s_je[k * B + tid];
-  }
-  const bool up16 = (lane & 16) != 0;
-  u128 a6[6];
+    for (int c = 0; c < kNch; ++c) mE[c] = GV_EMPTY;
+#pragma unroll 1
+    for (int k = 0; k < nk; ++k) {
+      const int slot = k * B + tid;
+      [[maybe_unused]] const int je = F64 ? 0 : (int)evs[(F64 ? 0 : kNch) * T + slot];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    u128 s[4];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int ch = c + 3 * h;
-      const int E = s_E[ch];
-      u128 s1 = {0ull, 0ull}, s2 = {0ull, 0ull};
-      if (E != GV_EMPTY) {
-#pragma unroll
-        for (int k = 0; k < EPT; ++k) {
-          if constexpr (F32) {
-            const unsigned u = s_p[(k * kNch + ch) * B + tid];
-            if ((u & 0x7FFFFFFFu) != 0u) {
-              const GvDirect w = gv_direct(u, jek[k]);
-              if (w.direct) {
-                s1 = add128(s1, gv_direct_fixed(w.m, w.e2 - E + GV_FB, w.neg));
-                s2 = add128(s2, gv_direct_square((unsigned long long)w.m * w.m,
-                                                   2 * (w.e2 - E) + GV_FB));
-              } else {
-                adj_add_double(gv_weight_bits(u, jek[k]), E, s1, s2);
-              }
-            }
+      for (int c = 0; c < kNch; ++c) {
+        GvSig<W> s;
+        bool any;
+        if constexpr (!F64) {
+          const unsigned u = evs[c * T + slot];
+          if (je < kOdd / 2) {
+            const int ef = (int)((u >> 23) & 0xFFu);
+            any = ef != 0;
+            s.m = (u & 0x7FFFFFu) | 0x800000u;
+            s.e2 = ef + je - 150;
+            s.neg = (u >> 31) != 0u;
           } else {
-            adj_add_double(s_v[(k * kNch + ch) * B + tid], E, s1, s2);
+            any = gv_sig(u, je - kOdd, s) > 0;
+          }
+        } else {
+          s = gv_sig(__longlong_as_double((long long)(
+              ((unsigned long long)evs[(2 * c + 1) * T + slot] << 32) | evs[2 * c * T + slot])));
+          any = s.m != 0ull;
+        }
+        const int4 win = s_win[c];
+        const int h = s.e2 + GvSig<W>::H, limb = gv_limb_index(h);
+        if (any && limb < win.z) {
+          const int pos = limb - win.x;
+          if (pos >= 0) {
+            unsigned l[4];
+            gv_square_digits(s, h + GV_SQ_OFF - 11 * limb, l);
+            gv_lane_add_square<W>(l, a_cols + (c * Lay::ROWS + pos) * 128);
+            gv_lane_add_w(s, a_cols + (c * Lay::ROWS + kL) * 128, win.y);
+          } else {
+            mE[c] = max(mE[c], s.e2);
           }
         }
       }
-      s[2 * h] = s1;
-      s[2 * h + 1] = s2;
     }
-    const u128 x2[4] = {s[0], s[1], s[2], s[3]};
-    u128 y[2];
-    rs_step<2>(x2, y, 16, up16);
-    a6[2 * c] = y[0];
-    a6[2 * c + 1] = y[1];
+    bool left = false;
+#pragma unroll
+    for (int c = 0; c < kNch; ++c) left = left || mE[c] != GV_EMPTY;
+    const bool more = __syncthreads_or((int)left) != 0;
+    for (int j = wid; j < kNsum; j += NW) {
+      const int c = j >> 1, E = s_E[c];
+      const int4 win = s_win[c];
+      if (!win.w) continue;
+      const unsigned* col = cols + c * Lay::ROWS * 32;
+      const u128 t =
+          (j & 1) ? gv_lane_total<false>(col, kL, 22 * win.x - 2 * GV_SQ_OFF - 2 * E + GV_FB)
+                  : gv_lane_total<true>(col + kL * 32, gv_lane_rows(F64),
+                                        22 * win.y - GV_SQ_OFF - E + GV_FB);
+      if (lane == 0) s_sum[j] = add128(s_sum[j], t);
+    }
+    if (!more) break;
+    first = false;
+    __syncthreads();  // the windows and the columns, read above
   }
-  // the remaining steps: lane distances 8, 4, 2, then both lanes of a pair
-  u128 a3[3], a2[2], a1[1];
-  rs_step<3>(a6, a3, 8, (lane & 8) != 0);
-  const u128 a4[4] = {a3[0], a3[1], a3[2], u128{0ull, 0ull}};
-  rs_step<2>(a4, a2, 4, (lane & 4) != 0);
-  rs_step<1>(a2, a1, 2, (lane & 2) != 0);
-  const u128 o = {shfl_xor_u64(a1[0].lo, 1), shfl_xor_u64(a1[0].hi, 1)};
-  const u128 t = add128(a1[0], o);
-  // sum index of this lane: 6 b4 + 3 b3 + (2 b2 + b1), b_i bit i of the
-  // lane; 2 b2 + b1 = 3 is padding; of the two lanes holding an index, the
-  // even one publishes it
-  const int local = ((lane >> 1) & 2) | ((lane >> 1) & 1);
-  const int j = 6 * ((lane >> 4) & 1) + 3 * ((lane >> 3) & 1) + local;
-  if (local < 3 && (lane & 1) == 0) red_sum[wid][j] = t;
   __syncthreads();
   if (tid < kNsum) {
-    u128 tot = red_sum[0][tid];
-#pragma unroll
-    for (int w = 1; w < NW; ++w) tot = add128(tot, red_sum[w][tid]);
-    ulonglong2* out = a.part + (size_t)tile * a.nacc;
-    out[tid] = make_ulonglong2(tot.lo, tot.hi);
+    const u128 t = s_sum[tid];
+    ulonglong2* out = a.part + (a.slot_major ? (size_t)tid * a.n_tiles + tile : (size_t)tile * a.nacc + tid);
+    *out = make_ulonglong2(t.lo, t.hi);
     if ((tid & 1) == 0) a.tileE[tile * kNch + tid / 2] = s_E[tid / 2];
   }
-  if (nbad) atomicAdd(&a.st->nonfinite_iter, nbad);
+  if (nbad) atomicAdd(&a.st->nonfinite_iter, (unsigned long long)nbad);
 }
 
 template <typename Real, int EPT, int MAXD>
 static cudaError_t gv_launch_adj_t(const GvFillArgs& a, int n_tiles, size_t smem, cudaStream_t s,
                                    bool pdl) {
   auto k = gv_fill_adjoint_kernel<Real, EPT, MAXD>;
-  const size_t total = smem + stage_bytes<Real>();  // the grid, then the staged values
+  const size_t total = AdjSmem<Real>::grid + smem;  // the events and columns, then the grid
   cudaError_t e = gv_prepare(k, total);
   if (e != cudaSuccess) return e;
   return gv_launch(k, dim3(n_tiles), dim3(GV_TILE / EPT), total, s, pdl, a);

@@ -506,7 +506,7 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
           order.push_back(b);
           acc += B->m[b].n_tiles;
           start.push_back(acc);
-          c.smem = std::max(c.smem,
+          c.smem = std::max<size_t>(c.smem,
                             GvFillSmem(B->m[b].d, nbins, form, true, maxd > 4, 0, false,
                                        false, true)
                                 .total);

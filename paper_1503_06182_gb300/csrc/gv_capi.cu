@@ -690,13 +690,15 @@ int make_plan(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* param
     cap = ncall + 2 * p.nh;
   }
   p.cap = cap;
-  // the adjoint's and the stratified fill's tiles have one size
-  p.tile_events = mode || p.plus ? GV_TILE : gv_tile_events(ncall, p.form);
+  // the stratified fill's tiles have one size
+  p.tile_events = p.plus ? GV_TILE : gv_tile_events(ncall, p.form);
   const int64_t nt = (cap + p.tile_events - 1) / p.tile_events;
   if (nt > 0x7fffffff) return VEGAS_EINVAL;
   p.n_tiles = (int)nt;
   p.nch = mode ? GV_MAXCH : 1;
-  p.slot_major = mode == 0 ? 1 : 0;
+  // the adjoint's twelve slots: one CTA each while its threads hold every
+  // tile's partial; beyond, the two-level reduce has more CTAs reading
+  p.slot_major = mode == 0 || p.n_tiles <= 2048 ? 1 : 0;
   p.nhist = (mode == 0 && c->hist_nh > 0) ? c->hist_nh + 2 : 0;
   p.nacc = mode ? 2 * GV_MAXCH : 2 + c->ndim * c->nbins + 2 * p.nhist;
   {
@@ -1251,7 +1253,7 @@ int vegas_workspace_size(const vegas_ctx* c, int64_t ncall, int itmx, size_t* by
   // FP64's tiles are no larger than FP32's: room for either
   const int T = std::min(gv_tile_events(ncall, GV_FORM_F32), gv_tile_events(ncall, GV_FORM_X64));
   *bytes = std::max(workspace_bytes(c->ndim, c->nbins, ncall, itmx, 0, nhist, T),
-                    workspace_bytes(c->ndim, c->nbins, ncall, itmx, 1, 0, GV_TILE));
+                    workspace_bytes(c->ndim, c->nbins, ncall, itmx, 1, 0, T));
   return VEGAS_OK;
 }
 

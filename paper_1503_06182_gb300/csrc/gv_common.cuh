@@ -389,132 +389,8 @@ __device__ __forceinline__ GvDecoded gv_decode(double x) {
   return r;
 }
 
-// round(m * 2^s) for a 128-bit m = (hi, lo), s of either sign (round half up).
-__device__ __forceinline__ u128 gv_shift_round(u128 v, int s) {
-  if (s > 0) {
-    if (s >= 64) {
-      v.hi = v.lo << (s - 64);
-      v.lo = 0ull;
-    } else {
-      v.hi = (v.hi << s) | (v.lo >> (64 - s));
-      v.lo <<= s;
-    }
-    return v;
-  }
-  if (s == 0) return v;
-  const int rs = -s;
-  if (rs > 127) return {0ull, 0ull};
-  // add half a unit of the last kept bit, then shift right
-  u128 h;
-  if (rs - 1 >= 64) {
-    h.lo = 0ull;
-    h.hi = 1ull << (rs - 1 - 64);
-  } else {
-    h.lo = 1ull << (rs - 1);
-    h.hi = 0ull;
-  }
-  v = add128(v, h);
-  if (rs >= 64) {
-    v.lo = v.hi >> (rs - 64);
-    v.hi = 0ull;
-  } else {
-    v.lo = (v.lo >> rs) | (v.hi << (64 - rs));
-    v.hi >>= rs;
-  }
-  return v;
-}
-
-__device__ __forceinline__ u128 gv_negate_if(u128 v, bool neg) {
-  if (neg) {
-    v.lo = ~v.lo + 1ull;
-    v.hi = ~v.hi + (v.lo == 0 ? 1ull : 0ull);
-  }
-  return v;
-}
-
-// round(x 2^(GV_FB - E)) from a decoded x with |x| < 2^E, two's complement.
-__device__ __forceinline__ u128 gv_fixed_dec(const GvDecoded& d, int E) {
-  u128 v = {d.m, 0ull};
-  v = gv_shift_round(v, d.e2 - E + GV_FB);
-  return gv_negate_if(v, d.neg);
-}
-
-// round(x^2 2^(GV_FB - 2E)), with the square formed exactly in integers
-// (m^2 has at most 106 bits): the sum of squares is then exact too.
-__device__ __forceinline__ u128 gv_square_fixed_dec(const GvDecoded& d, int E) {
-  u128 v = {d.m * d.m, __umul64hi(d.m, d.m)};
-  return gv_shift_round(v, 2 * d.e2 - 2 * E + GV_FB);
-}
-
-// P = floor(m^2 2^-42), the high word of the square of m 2^11.
-__device__ __forceinline__ unsigned long long gv_square_hi(unsigned long long m) {
-  return __umul64hi(m << 11, m << 11);
-}
-
-// The same roundings as gv_fixed_dec / gv_square_fixed_dec (half up, bit for
-// bit), specialised to the shifts that occur in a tile for normal x (|x| <
-// 2^E, so the mantissa shift of x is at most GV_FB - 53 and that of x^2 at
-// least 106 - GV_FB; subnormal x take the general routine), on 64-bit
-// pieces.  round(v 2^-r) = ((v >> (r-1)) + 1) >> 1.
-__device__ __forceinline__ u128 gv_fixed_tile(const GvDecoded& d, int E) {
-  const int s = d.e2 - E + GV_FB;  // <= GV_FB - 53 unless x is subnormal
-  if (s > GV_FB - 53) return gv_fixed_dec(d, E);
-  u128 v;
-  if (s > 0) {
-    v.lo = d.m << s;
-    v.hi = d.m >> (64 - s);
-  } else if (s == 0) {
-    v.lo = d.m;
-    v.hi = 0ull;
-  } else {
-    const int r = -s;
-    v.lo = r <= 54 ? ((d.m >> (r - 1)) + 1ull) >> 1 : 0ull;
-    v.hi = 0ull;
-  }
-  return gv_negate_if(v, d.neg);
-}
-// x^2 from its exact 128-bit mantissa square (hi = floor(m^2 2^-64) taken
-// from P = floor(m^2 2^-42), see gv_square_hi; lo = m^2 mod 2^64).
-__device__ __forceinline__ u128 gv_square_tile(const GvDecoded& d, unsigned long long P, int E) {
-  const int k = 2 * E - 2 * d.e2 - GV_FB - 1;  // r - 1 >= 105 - GV_FB unless x is subnormal
-  if (k < 105 - GV_FB) return gv_square_fixed_dec(d, E);
-  const unsigned long long hi = P >> 22, lo = d.m * d.m;
-  u128 t;
-  if (k < 64) {
-    t.lo = (lo >> k) | (hi << (64 - k));
-    t.hi = hi >> k;
-  } else {
-    t.lo = k < 128 ? hi >> (k - 64) : 0ull;
-    t.hi = 0ull;
-  }
-  // (t + 1) >> 1
-  t.lo += 1ull;
-  t.hi += t.lo == 0ull ? 1ull : 0ull;
-  t.lo = (t.lo >> 1) | (t.hi << 63);
-  t.hi >>= 1;
-  return t;
-}
-
 __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v, int m) {
   return __shfl_xor_sync(0xffffffffu, v, m);
-}
-
-__device__ __forceinline__ u128 warp_sum128(u128 v) {
-#pragma unroll
-  for (int m = 16; m > 0; m >>= 1) {
-    u128 o = {shfl_xor_u64(v.lo, m), shfl_xor_u64(v.hi, m)};
-    v = add128(v, o);
-  }
-  return v;
-}
-
-__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
-#pragma unroll
-  for (int m = 16; m > 0; m >>= 1) {
-    unsigned long long o = shfl_xor_u64(v, m);
-    v = o > v ? o : v;
-  }
-  return v;
 }
 
 // ----------------------------------------------------------------------------

@@ -225,63 +225,9 @@ __device__ __forceinline__ double gv_weight(const GvJac<float>& J, float g) {
   return gv_ldexp_bits(gv_widen(p), J.e);
 }
 
-// FP32 form, for the exact sums: the weight p 2^e of an FP32 product
-// p = J.m g.  Where p is normal and p 2^e a normal double ("direct"), the
-// weight is m 2^e2 with m the 24-bit significand of p and e2 = nf - 1046, nf
-// its FP64 exponent field (the double gv_weight assembles holds m << 29).
-// Its tile fixed-point terms are formed from m (a 32 x 32 -> 64 bit square):
-// the same exactly rounded integers as through the double, with less integer
-// work.  Every other case takes the double, formed as gv_weight forms it.
-struct GvDirect {
-  bool direct;
-  unsigned m;
-  int e2;
-  bool neg;
-};
-__device__ __forceinline__ GvDirect gv_direct(unsigned u, int e) {
-  const int ef = (int)((u >> 23) & 0xFFu);
-  const int nf = ef + 896 + e;
-  GvDirect w;
-  w.direct = ef != 0 && ef != 0xFF && nf > 0 && nf < 0x7FF;
-  w.m = (u & 0x7FFFFFu) | 0x800000u;
-  w.e2 = nf - 1046;
-  w.neg = (u >> 31) != 0u;
-  return w;
-}
+// The double gv_weight assembles, from the product's bits.
 __device__ __forceinline__ double gv_weight_bits(unsigned u, int e) {
   return gv_ldexp_bits(gv_widen(__uint_as_float(u)), e);
-}
-
-// round(m 2^s), half up, for m < 2^24 and s <= 72, with the sign: the tile's
-// fixed-point value of a direct weight (|w| < 2^E, s = e2 - E + GV_FB), as
-// gv_fixed_tile rounds the equal double.
-__device__ __forceinline__ u128 gv_direct_fixed(unsigned long long m, int s, bool neg) {
-  u128 v;
-  if (s >= 0) {
-    v.lo = s < 64 ? m << s : 0ull;
-    v.hi = s > 40 ? (s < 64 ? m >> (64 - s) : m << (s - 64)) : 0ull;
-  } else {
-    const int r = -s;
-    v.lo = r < 64 ? ((m >> (r - 1)) + 1ull) >> 1 : 0ull;
-    v.hi = 0ull;
-  }
-  return gv_negate_if(v, neg);
-}
-
-// round(M 2^t), half up, for the square M = m^2 < 2^48 of a direct weight's
-// significand and t = 2 (e2 - E) + GV_FB <= 48: the tile's fixed-point square,
-// as gv_square_tile rounds it.
-__device__ __forceinline__ u128 gv_direct_square(unsigned long long M, int t) {
-  u128 v;
-  if (t >= 0) {
-    v.lo = M << t;
-    v.hi = t > 16 ? M >> (64 - t) : 0ull;
-  } else {
-    const int r = -t;
-    v.lo = r < 64 ? ((M >> (r - 1)) + 1ull) >> 1 : 0ull;
-    v.hi = 0ull;
-  }
-  return v;
 }
 
 template <typename Real>
@@ -326,7 +272,7 @@ struct GvPair<GvX> {
 //   ps   [GV_PLUS_WIN + GV_TILE/GV_PLUS_SEG] double2  the tile's segments
 //                         (VEGAS+): each window hypercube's first, then each
 //                         range's continuation of an earlier hypercube
-__host__ __device__ inline size_t gv_align16(size_t b) { return (b + 15) & ~(size_t)15; }
+__host__ __device__ inline unsigned gv_align16(unsigned b) { return (b + 15u) & ~15u; }
 
 // The forward fill generates its tile's Philox words before it waits for the
 // previous kernel (the words depend only on the seed, the counter and the
@@ -353,35 +299,35 @@ __host__ __device__ constexpr int gv_event_words32(bool f64, bool reg_bins, bool
 }
 
 struct GvFillSmem {
-  size_t wd, ew, jac, limbs, hist, hh, hw, lq, lw, bins, po, ps, total;
+  unsigned wd, ew, jac, limbs, hist, hh, hw, lq, lw, bins, po, ps, total;
   int L;
   __host__ __device__ GvFillSmem(int d, int N, int form, bool forward, bool bins_smem,
                                  int nhist = 0, bool plus = false, bool words = false,
                                  bool keep_grid = false, int T = GV_TILE) {
-    const size_t dN = (size_t)d * N;
+    const unsigned dN = (unsigned)(d * N);
     const bool f64 = form != GV_FORM_F32;
     L = gv_limbs(d * N);
-    const size_t evs = forward ? (size_t)gv_event_words32(f64, !bins_smem, plus) * T * 4 : 0;
-    const size_t wds = words ? (size_t)((d + 3) / 4) * 4 * T * 4 : 0;
+    const unsigned evs = forward ? gv_event_words32(f64, !bins_smem, plus) * T * 4 : 0;
+    const unsigned wds = words ? (d + 3) / 4 * 4 * T * 4 : 0;
     wd = 0;
     ew = wds > evs ? wds : evs;
     jac = ew + dN * (form == GV_FORM_X64 ? 32 : 16);
-    const size_t first = gv_align16(jac + (form == GV_FORM_F64 ? dN * 8 : 0));
+    const unsigned first = gv_align16(jac + (form == GV_FORM_F64 ? dN * 8 : 0));
     limbs = keep_grid ? first : evs;
     hist = limbs;
     hh = hist + (forward ? dN * L * 4 : 0);
-    hw = hh + (forward ? (size_t)nhist * L * 4 : 0);
-    lq = hw + (forward ? (size_t)nhist * gv_hist_w_limbs(f64) * 4 : 0);
-    lw = lq + (forward ? (size_t)L * 32 * 4 : 0);
-    const size_t second = gv_align16(lw + (forward ? (size_t)gv_lane_rows(f64) * 32 * 4 : 0));
+    hw = hh + (forward ? nhist * L * 4 : 0);
+    lq = hw + (forward ? nhist * gv_hist_w_limbs(f64) * 4 : 0);
+    lw = lq + (forward ? L * 32 * 4 : 0);
+    const unsigned second = gv_align16(lw + (forward ? gv_lane_rows(f64) * 32 * 4 : 0));
     bins = first > second ? first : second;
-    po = gv_align16(bins + ((forward && bins_smem) ? (size_t)d * T * 2 : 0));
-    ps = gv_align16(po + (plus ? (size_t)GV_PLUS_WIN * 4 : 0));
-    total = gv_align16(ps + (plus ? (size_t)GV_PLUS_SEGS * 16 : 0));
+    po = gv_align16(bins + ((forward && bins_smem) ? d * T * 2 : 0));
+    ps = gv_align16(po + (plus ? GV_PLUS_WIN * 4 : 0));
+    total = gv_align16(ps + (plus ? GV_PLUS_SEGS * 16 : 0));
   }
   // bytes of the limbs, from `limbs`
-  __host__ __device__ size_t limb_bytes(bool f64) const {
-    return lw + (size_t)gv_lane_rows(f64) * 32 * 4 - limbs;
+  __host__ __device__ unsigned limb_bytes(bool f64) const {
+    return lw + gv_lane_rows(f64) * 32 * 4 - limbs;
   }
 };
 
@@ -985,16 +931,13 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
     }
     const bool more = __syncthreads_or((int)(mw != GV_EMPTY || (PLUS && mq != GV_EMPTY))) != 0;
     if (first) gv_allow_next_grid();
-    if (have_w && wid == 0) {
-      const int r0 = gv_square_row0(F64, L);
-      const u192 t = gv_lane_total<false>(lq, L, r0);
-      sum = add128(sum, gv_tile_fixed(t, 22 * (vw.base + r0) - 2 * GV_SQ_OFF - 2 * E + GV_FB));
-    } else if (have_w && wid == 1) {
-      const u192 t = gv_lane_total<true>(reinterpret_cast<const unsigned*>(lw), gv_lane_rows(F64), 0);
-      sum = add128(sum, gv_tile_fixed(t, 22 * vw.wbase - GV_SQ_OFF - E + GV_FB));
-    }
-    for (int k = tid; k < dN; k += B) {
-      ulonglong2* o = out + (2 + k) * ks;
+    if (have_w && wid == 0)
+      sum = add128(sum, gv_lane_total<false>(lq, L, 22 * vw.base - 2 * GV_SQ_OFF - 2 * E + GV_FB));
+    else if (have_w && wid == 1)
+      sum = add128(sum, gv_lane_total<true>(reinterpret_cast<const unsigned*>(lw), gv_lane_rows(F64),
+                                            22 * vw.wbase - GV_SQ_OFF - E + GV_FB));
+    ulonglong2* o = out + (size_t)(2 + tid) * ks;
+    for (int k = tid; k < dN; k += B, o += (size_t)B * ks) {
       GvPartial v = gv_bin_partial(hist + k * L, L, vq.base);
       if (!first) v = gv_partial_add(v, gv_load_partial(o));
       gv_store_partial(o, v);

@@ -228,38 +228,41 @@ __device__ __forceinline__ void gv_hist_add_w(const GvSig<Real>& w, unsigned row
   if constexpr (sizeof(Real) == 8) gv_red<12>(p, gv_signed_digit((unsigned)(m >> (63u - sh)), s));
 }
 
-// Rows of the squares' columns left out of their total: the FP64 form's 204
-// bits from row 0 of nine would pass 192; rows 0 and 1 lie 2^54 below the unit
-// of the tile's fixed point there.
-__host__ __device__ constexpr int gv_square_row0(bool f64, int L) { return f64 && L > 7 ? 2 : 0; }
-
-// Warp-collective total of a lane column's digits [row0, rows), in units of
-// row row0 (every lane returns it).
+// Warp-collective total of a lane column's `rows` digits (at most 16) as a
+// 128-bit integer, row 0 counting units of 2^p (bits below 1 truncated row by
+// row): lane j takes row j's sum over the lanes, shifts it into place, and
+// the warp adds the rows.  Lane 0 returns the total.
 template <bool SIGNED>
-__device__ __forceinline__ u192 gv_lane_total(const unsigned* col, int rows, int row0) {
+__device__ __forceinline__ u128 gv_lane_total(const unsigned* col, int rows, int p) {
   const int lane = threadIdx.x & 31;
-  u192 acc = {0ull, 0ull, 0ull};
-  for (int j = rows - 1; j >= row0; --j) {
+  long long mine = 0;
+  for (int j = 0; j < rows; ++j) {
     const unsigned v = col[j * 32 + lane];
-    u192 s;
-    if constexpr (SIGNED) {
-      const long long x = (long long)__reduce_add_sync(0xffffffffu, v & 0xFFFFu) +
-                          ((long long)__reduce_add_sync(0xffffffffu, (int)v >> 16) << 16);
-      const unsigned long long ext = (unsigned long long)(x >> 63);
-      s = {(unsigned long long)x, ext, ext};
-    } else {
-      s = {__reduce_add_sync(0xffffffffu, v), 0ull, 0ull};
-    }
-    acc = shl192(acc, GV_LIMB_BITS);
-    add192(acc, s);
+    long long s;
+    if constexpr (SIGNED)
+      s = (long long)__reduce_add_sync(0xffffffffu, v & 0xFFFFu) +
+          ((long long)__reduce_add_sync(0xffffffffu, (int)v >> 16) << 16);
+    else
+      s = (long long)__reduce_add_sync(0xffffffffu, v);
+    if (lane == j) mine = s;
   }
-  return acc;
-}
-// The total in a tile's fixed point: v 2^p as a 128-bit integer (bits below
-// its unit truncated).
-__device__ __forceinline__ u128 gv_tile_fixed(const u192& v, int p) {
-  const u192 r = p >= 0 ? shl192(v, p) : sar192(v, -p);
-  return u128{r.l0, r.l1};
+  const unsigned long long ext = (unsigned long long)(mine >> 63);
+  const int sh = GV_LIMB_BITS * lane + p;
+  u128 r = {0ull, 0ull};
+  if (lane < rows) {
+    if (sh >= 64)
+      r.hi = sh < 128 ? (unsigned long long)mine << (sh - 64) : 0ull;
+    else if (sh > 0)
+      r = u128{(unsigned long long)mine << sh, (unsigned long long)(mine >> (64 - sh))};
+    else
+      r = u128{(unsigned long long)(mine >> (sh > -64 ? -sh : 63)), ext};
+  }
+#pragma unroll
+  for (int m = 8; m > 0; m >>= 1) {
+    const u128 o = {shfl_xor_u64(r.lo, m), shfl_xor_u64(r.hi, m)};
+    r = add128(r, o);
+  }
+  return r;
 }
 
 // A bin's partial: 96 bits and an exponent code F + GV_BINE_OFF with the value
@@ -280,15 +283,21 @@ __device__ __forceinline__ GvPartial gv_partial_norm(unsigned long long lo, unsi
   return GvPartial{lo, (unsigned)hi, code};
 }
 __device__ __forceinline__ GvPartial gv_bin_partial(const unsigned* row, int L, int base) {
+  // a square of at least 2^46 (FP64: 2^62) has its top digit above two others:
+  // the top limb t is at least 2
   int t = L - 1;
-  unsigned a = row[t];
-  while (a == 0u && t > 0) a = row[--t];
+  unsigned a = row[t], b = row[t - 1], c = row[t - 2], d = row[t - 3];
+  while (a == 0u && t > 2) {
+    --t;
+    a = b;
+    b = c;
+    c = d;
+    d = t > 2 ? row[t - 3] : 0u;
+  }
   if (a == 0u) return GvPartial{0ull, 0u, 0};
-  const unsigned b = t > 0 ? row[t - 1] : 0u, c = t > 1 ? row[t - 2] : 0u,
-                 d = t > 2 ? row[t - 3] : 0u;
-  const u128 x = add128(add128(u128{(unsigned long long)d + ((unsigned long long)c << 22), 0ull},
-                               u128{(unsigned long long)b << 44, b >> 20}),
-                        u128{0ull, (unsigned long long)a << 2});
+  const u128 x = add128(u128{(unsigned long long)d + ((unsigned long long)c << 22),
+                             (unsigned long long)a << 2},
+                        u128{(unsigned long long)b << 44, b >> 20});
   // unit 2^(22 i - 2 GV_SQ_OFF) = 2^(2 F - 56) for the lowest digit i = base + t - 3
   return gv_partial_norm(x.lo, x.hi, 11 * (base + t - 3) - GV_SQ_OFF + GV_BIN_QBITS / 2 +
                                          GV_BINE_OFF);
