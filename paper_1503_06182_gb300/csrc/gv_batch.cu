@@ -465,7 +465,7 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
     if (cudaMemcpy(x.grid + GvGridLayout{x.d, nbins}.off_e64(), e.data(), e.size() * 8,
                    cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(x.par, x.params, sizeof x.params, cudaMemcpyHostToDevice) != cudaSuccess ||
-        gv::launch_grid_pack(x.d, nbins, x.grid, B->stream) != cudaSuccess ||
+        gv::launch_grid_pack(x.d, nbins, x.grid, nullptr, 0ull, B->stream) != cudaSuccess ||
         gv::launch_consts(x.ig, x.par, x.kconst, B->stream) != cudaSuccess ||
         gv::launch_reset(x.st, B->stream) != cudaSuccess)
       st = VEGAS_ECUDA;

@@ -108,6 +108,7 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 constexpr int kHostRecMax = 64;  // iterations whose records fit the mapped result block
 constexpr size_t kHostRecOff = 256;  // byte offset of the records in it
+constexpr size_t kHostGridOff = kHostRecOff + kHostRecMax * 2 * sizeof(double);  // of the edges
 static_assert(sizeof(GvState) <= kHostRecOff, "state fits before the records");
 
 // Autotuner cache: best events-per-thread per (integrand, precision, mode,
@@ -163,10 +164,12 @@ struct vegas_ctx {
   // ncall (plus_C); plus_valid: it exists on the device
   int strat = 0, beta_j = 3;
   void* plus_mem = nullptr;
+  size_t plus_bytes = 0;
   long long plus_nh = 0, plus_C = 0;
   int plus_s = 0, plus_tiles = 0;
   bool plus_valid = false;
-  long long plus_tab_C = 0;  // the C of the ab table on the device (0: none)
+  long long plus_tab_C = 0;  // the C of the tables on the device (0: none)
+  GvPlusFill plus_fill_host;  // what plus_fill holds
   GvPlusArgs pa;  // device arrays of the allocation (pointers only)
   GvPlusFill* plus_fill = nullptr;  // the stratified fill's data (device)
   // VEGAS+: the hypercube statistics, allocation and layout of an iteration
@@ -190,6 +193,13 @@ struct vegas_ctx {
   // fetching them is a synchronisation, not two copies
   void* hres = nullptr;
   void* hres_dev = nullptr;
+  // the grid's edges as the host knows them, in the same block: written by
+  // the host with a grid, and by the refinement of a stage's last iteration
+  double* hgrid = nullptr;
+  // the iteration counter: stages advance it by their iterations
+  unsigned long long it = 0;
+  bool in_flight = false;  // a stage was enqueued and not waited for yet
+  std::vector<double> upload;  // staging of a grid on its way to the device
   bool last_zero_copy = false;
   // derived constants currently on the device
   int consts_ig = -1;
@@ -359,14 +369,13 @@ GvPlusArgs plus_args(const vegas_ctx* c, const Plan& p, int k) {
 }
 
 // Device memory of a VEGAS+ allocation of nh hypercubes and n_tiles tiles
-// (zeroed; the allocation itself is made by the caller).
+// (zeroed; the allocation itself is made by the caller).  The block is kept
+// and laid out anew while it is large enough -- a warm-up stage of fewer calls
+// and its production stage share it -- so the pointers of a shape are a
+// function of the block, nh and n_tiles, which captured stages rely on.
 int ensure_plus(vegas_ctx* c, long long nh, int n_tiles) {
-  if (c->plus_mem && c->plus_nh == nh && c->plus_tiles >= n_tiles) return VEGAS_OK;
-  if (c->stream) cudaStreamSynchronize(c->stream);
-  if (c->plus_mem) cudaFree(c->plus_mem);
-  c->plus_mem = nullptr;
+  if (c->plus_mem && c->plus_nh == nh && c->plus_tiles == n_tiles) return VEGAS_OK;
   c->plus_valid = false;
-  clear_graphs(c);
   const long long nb = (nh + 255) / 256;
   size_t off = 0;
   const size_t o_off = off;
@@ -398,10 +407,19 @@ int ensure_plus(vegas_ctx* c, long long nh, int n_tiles) {
   off = align256(off + sizeof(GvPlusFill));
   const size_t o_tab = off;
   off = align256(off + (size_t)GV_PLUS_NTAB * 8 * 3);
-  if (cudaMalloc(&c->plus_mem, off) != cudaSuccess) {
-    cudaGetLastError();
+  if (off > c->plus_bytes) {
+    cudaStreamSynchronize(c->stream);
+    if (c->plus_mem) cudaFree(c->plus_mem);
     c->plus_mem = nullptr;
-    return VEGAS_ENOMEM;
+    c->plus_bytes = 0;
+    c->plus_nh = 0;
+    clear_graphs(c);
+    if (cudaMalloc(&c->plus_mem, off) != cudaSuccess) {
+      cudaGetLastError();
+      c->plus_mem = nullptr;
+      return VEGAS_ENOMEM;
+    }
+    c->plus_bytes = off;
   }
   char* b = (char*)c->plus_mem;
   GvPlusArgs& a = c->pa;
@@ -429,13 +447,9 @@ int ensure_plus(vegas_ctx* c, long long nh, int n_tiles) {
   a.inv = (const double*)(b + o_tab);
   a.abtab = (const double2*)(b + o_tab + (size_t)GV_PLUS_NTAB * 8);
   GV_TRY(cudaMemsetAsync(c->plus_mem, 0, off, c->stream));
-  std::vector<double> inv(GV_PLUS_NTAB, 0.0);
-  for (int n = 1; n < GV_PLUS_NTAB; ++n) inv[n] = 1.0 / (double)n;
-  // a pageable copy is staged before cudaMemcpyAsync returns
-  GV_TRY(cudaMemcpyAsync((void*)a.inv, inv.data(), inv.size() * 8, cudaMemcpyHostToDevice,
-                         c->stream));
   c->plus_nh = nh;
   c->plus_tab_C = 0;
+  c->plus_fill_host.nh = 0;  // plus_fill was zeroed
   c->plus_tiles = n_tiles;
   return VEGAS_OK;
 }
@@ -474,6 +488,7 @@ GvReduceArgs reduce_args(const vegas_ctx* c, const Plan& p, int k) {
     r.host_st = (GvState*)c->hres_dev;
     r.host_rec = (double*)((char*)c->hres_dev + kHostRecOff);
   }
+  if (c->hres_dev && !c->tuning) r.host_grid = (double*)((char*)c->hres_dev + kHostGridOff);
   if (p.plus) r.tiles_used = c->pa.tiles_used;
   r.k = k;
   r.last = k == p.itmx - 1;
@@ -736,19 +751,12 @@ int make_plan(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* param
   return VEGAS_OK;
 }
 
-// VEGAS+: the table of (C/(nh n), sqrt(1/(nh n))) for n < GV_PLUS_NTAB, in
-// the same FP64 operations as for any other n.
-int upload_abtab(vegas_ctx* c, long long C, long long nh) {
+// VEGAS+: the per-count tables for C calls and the layout's hypercubes.
+int ensure_tables(vegas_ctx* c, long long C) {
   if (c->plus_tab_C == C) return VEGAS_OK;
-  std::vector<double> t(2 * (size_t)GV_PLUS_NTAB, 0.0);
-  for (int n = 1; n < GV_PLUS_NTAB; ++n) {
-    const double nhd = (double)nh * (double)n;
-    t[2 * (size_t)n] = (double)C / nhd;
-    t[2 * (size_t)n + 1] = std::sqrt(1.0 / nhd);
-  }
-  // a pageable copy is staged before cudaMemcpyAsync returns
-  GV_TRY(cudaMemcpyAsync((void*)c->pa.abtab, t.data(), t.size() * 8, cudaMemcpyHostToDevice,
-                         c->stream));
+  GvPlusArgs a = c->pa;
+  a.ncall = C;
+  GV_TRY(gv::launch_plus_tables(a, c->stream));
   c->plus_tab_C = C;
   return VEGAS_OK;
 }
@@ -757,11 +765,12 @@ int upload_abtab(vegas_ctx* c, long long C, long long nh) {
 int ensure_allocation(vegas_ctx* c, const Plan& p) {
   int st = ensure_plus(c, p.nh, p.n_tiles);
   if (st) return st;
-  st = upload_abtab(c, p.ncall, p.nh);
+  st = ensure_tables(c, p.ncall);
   if (st) return st;
   c->plus_s = p.s;
   // the fill's view of the allocation (the workspace may have moved)
   GvPlusFill f;
+  memset(&f, 0, sizeof f);
   f.s = p.s;
   f.inv_s = 1.0f / (float)p.s;
   f.nh = p.nh;
@@ -779,8 +788,11 @@ int ensure_allocation(vegas_ctx* c, const Plan& p) {
   f.tpart = c->pa.tpart;
   f.inv = c->pa.inv;
   f.beta_j = c->beta_j;
-  // a pageable copy is staged before cudaMemcpyAsync returns
-  GV_TRY(cudaMemcpyAsync(c->plus_fill, &f, sizeof f, cudaMemcpyHostToDevice, c->stream));
+  if (c->plus_fill_host.nh == 0 || memcmp(&f, &c->plus_fill_host, sizeof f) != 0) {
+    // a pageable copy is staged before cudaMemcpyAsync returns
+    GV_TRY(cudaMemcpyAsync(c->plus_fill, &f, sizeof f, cudaMemcpyHostToDevice, c->stream));
+    memcpy(&c->plus_fill_host, &f, sizeof f);
+  }
   if (c->plus_valid && c->plus_C == p.ncall) return VEGAS_OK;
   GvPlusArgs a = plus_args(c, p, -1);
   a.uniform = 1;
@@ -909,6 +921,7 @@ int enqueue_stage(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* p
     if (st) return st;
   }
   c->hist_valid = p.nhist > 0;
+  c->in_flight = true;
   c->last_itmx = itmx;
   c->last_mode = mode;
   c->last_ept = p.ept;
@@ -935,6 +948,7 @@ int enqueue_stage(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* p
     st = enqueue_body(c, p, evp, false);
     if (st) return st;
     if (evp) c->pending_events = *evp;
+    c->it += (unsigned long long)itmx;
     c->pending = true;
     return VEGAS_OK;
   }
@@ -971,6 +985,7 @@ int enqueue_stage(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* p
   }
   GV_TRY(cudaGraphLaunch(ge->exec, c->stream));
   c->pending_events = ge->events;
+  c->it += (unsigned long long)itmx;
   c->pending = true;
   return VEGAS_OK;
 }
@@ -984,6 +999,7 @@ int fetch_stage(vegas_ctx* c, GvState* hs, std::vector<double>* per_iter) {
     // the finalising thread wrote the state and the records into the mapped
     // block; they are visible once the stream is done
     GV_TRY(cudaStreamSynchronize(c->stream));
+    c->in_flight = false;
     const volatile GvState* hv = (const volatile GvState*)c->hres;
     memset(hs, 0, sizeof *hs);
     hs->it = hv->it;
@@ -1007,6 +1023,7 @@ int fetch_stage(vegas_ctx* c, GvState* hs, std::vector<double>* per_iter) {
     GV_TRY(cudaMemcpyAsync(pin_rec, c->last_per_iter, nrec * sizeof(double),
                            cudaMemcpyDeviceToHost, c->stream));
     GV_TRY(cudaStreamSynchronize(c->stream));
+    c->in_flight = false;
     memcpy(hs, pin, sizeof(GvState));
     if (per_iter) per_iter->assign(pin_rec, pin_rec + nrec);
   }
@@ -1039,11 +1056,25 @@ int valid_grid(const double* e, int d, int N) {
   return 1;
 }
 
-int upload_grid(vegas_ctx* c, const double* edges) {
+// Wait for what is enqueued, if anything.
+int settle(vegas_ctx* c) {
+  if (c->in_flight) GV_TRY(cudaStreamSynchronize(c->stream));
+  c->in_flight = false;
+  return VEGAS_OK;
+}
+
+// Enqueue a grid (and, with set_it, the iteration counter c->it).  The caller
+// has waited for earlier stages, which write the host's copy of the grid.
+int upload_grid(vegas_ctx* c, const double* edges, bool set_it) {
   const size_t n = (size_t)c->ndim * (c->nbins + 1);
-  GV_TRY(cudaMemcpyAsync(c->grid + GvGridLayout{c->ndim, c->nbins}.off_e64(), edges, n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  GV_TRY(gv::launch_grid_pack(c->ndim, c->nbins, c->grid, c->stream));
-  GV_TRY(cudaStreamSynchronize(c->stream));
+  // from pageable memory of the context's own: staged before the call
+  // returns, whatever memory the caller's edges are in
+  c->upload.assign(edges, edges + n);
+  GV_TRY(cudaMemcpyAsync(c->grid + GvGridLayout{c->ndim, c->nbins}.off_e64(), c->upload.data(),
+                         n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+  GV_TRY(gv::launch_grid_pack(c->ndim, c->nbins, c->grid, set_it ? c->st : nullptr, c->it,
+                              c->stream));
+  if (c->hgrid) memcpy(c->hgrid, edges, n * sizeof(double));
   return VEGAS_OK;
 }
 
@@ -1098,13 +1129,15 @@ int vegas_init(int ndim, int nbins, uint64_t seed, vegas_ctx** out) {
   }
   c->own_stream = true;
   // the mapped result block (without it, results are copied)
-  if (cudaHostAlloc(&c->hres, kHostRecOff + kHostRecMax * 2 * sizeof(double),
+  if (cudaHostAlloc(&c->hres, kHostGridOff + (size_t)ndim * (nbins + 1) * sizeof(double),
                     cudaHostAllocMapped) == cudaSuccess) {
     if (cudaHostGetDevicePointer(&c->hres_dev, c->hres, 0) != cudaSuccess) {
       cudaGetLastError();
       cudaFreeHost(c->hres);
       c->hres = nullptr;
       c->hres_dev = nullptr;
+    } else {
+      c->hgrid = (double*)((char*)c->hres + kHostGridOff);
     }
   } else {
     cudaGetLastError();
@@ -1151,7 +1184,8 @@ int vegas_init(int ndim, int nbins, uint64_t seed, vegas_ctx** out) {
     std::vector<double> e((size_t)ndim * (nbins + 1));
     for (int a = 0; a < ndim; ++a)
       for (int i = 0; i <= nbins; ++i) e[(size_t)a * (nbins + 1) + i] = (double)i / nbins;
-    st = upload_grid(c, e.data());
+    st = upload_grid(c, e.data(), false);
+    if (!st && cudaStreamSynchronize(c->stream) != cudaSuccess) st = VEGAS_ECUDA;
   }
   if (st) {
     vegas_free(c);
@@ -1281,7 +1315,7 @@ int vegas_strat_set(vegas_ctx* c, int64_t ncall, const int32_t* counts) {
   const int n_tiles = (int)((ncall + 2 * nh + GV_TILE - 1) / GV_TILE);
   int st = ensure_plus(c, nh, n_tiles);
   if (st) return st;
-  st = upload_abtab(c, ncall, nh);
+  st = ensure_tables(c, ncall);
   if (st) return st;
   // the counts, their sums per CTA of 256 hypercubes and per group of 32
   // CTAs, and the total; then the layout
@@ -1411,6 +1445,10 @@ int vegas_grid_get(const vegas_ctx* c, double* edges) {
   if (!c || !edges) return VEGAS_EINVAL;
   const size_t n = (size_t)c->ndim * (c->nbins + 1);
   GV_TRY(cudaStreamSynchronize(c->stream));
+  if (c->hgrid) {
+    memcpy(edges, c->hgrid, n * sizeof(double));
+    return VEGAS_OK;
+  }
   GV_TRY(cudaMemcpy(edges, c->grid + GvGridLayout{c->ndim, c->nbins}.off_e64(), n * sizeof(double),
                     cudaMemcpyDeviceToHost));
   return VEGAS_OK;
@@ -1419,8 +1457,8 @@ int vegas_grid_get(const vegas_ctx* c, double* edges) {
 int vegas_grid_set(vegas_ctx* c, const double* edges) {
   if (!c || !edges) return VEGAS_EINVAL;
   if (!valid_grid(edges, c->ndim, c->nbins)) return VEGAS_EGRID;
-  GV_TRY(cudaStreamSynchronize(c->stream));
-  return upload_grid(c, edges);
+  const int st = settle(c);
+  return st ? st : upload_grid(c, edges, false);
 }
 
 int vegas_state_size(const vegas_ctx* c, size_t* bytes) {
@@ -1439,10 +1477,7 @@ int vegas_state_get(const vegas_ctx* c, void* buf, size_t bytes) {
   h.ndim = c->ndim;
   h.nbins = c->nbins;
   h.seed = c->seed;
-  GvState hs;
-  GV_TRY(cudaStreamSynchronize(c->stream));
-  GV_TRY(cudaMemcpy(&hs, c->st, sizeof hs, cudaMemcpyDeviceToHost));
-  h.it = hs.it;
+  h.it = c->it;
   h.batch = c->batch;
   h.fp32 = c->fp32;
   h.adapt = c->adapt;
@@ -1463,21 +1498,18 @@ int vegas_state_set(vegas_ctx* c, const void* buf, size_t bytes) {
   std::vector<double> e((size_t)c->ndim * (c->nbins + 1));
   memcpy(e.data(), (const char*)buf + sizeof h, e.size() * sizeof(double));
   if (!valid_grid(e.data(), c->ndim, c->nbins)) return VEGAS_EGRID;
-  GV_TRY(cudaStreamSynchronize(c->stream));
+  const int st = settle(c);
+  if (st) return st;
   c->seed = h.seed;
   c->batch = h.batch;
   c->fp32 = h.fp32;
   c->adapt = h.adapt;
   c->nonfinite_policy = h.nonfinite_policy;
   c->alpha = h.alpha;
-  GvState hs;
-  GV_TRY(cudaMemcpy(&hs, c->st, sizeof hs, cudaMemcpyDeviceToHost));
-  hs.it = h.it;
-  hs.it0 = h.it;
-  GV_TRY(cudaMemcpy(c->st, &hs, sizeof hs, cudaMemcpyHostToDevice));
-  clear_graphs(c);
+  // (captured stages stay: they are looked up by everything set here)
+  c->it = h.it;
   c->plus_valid = false;  // a VEGAS+ allocation is not part of a checkpoint
-  return upload_grid(c, e.data());
+  return upload_grid(c, e.data(), true);
 }
 
 int vegas_eval_events(vegas_ctx* c, int id, const double* params, int np, uint32_t iteration,

@@ -232,6 +232,7 @@ struct GvReduceArgs {
   // stages): the iteration records, and the state after the last iteration
   GvState* host_st = nullptr;
   double* host_rec = nullptr;
+  double* host_grid = nullptr;   // and the grid's edges [ndim][nbins + 1] after the last iteration
   int refine_follows;            // 1: each axis is refined by the CTA that completes it
   long long ncall;
   double inv_c, inv_cm1, inv_m1; // 1/C, 1/(C-1), 1/(k) for chi2/dof at the last iteration
@@ -463,6 +464,8 @@ namespace gv {
 cudaError_t launch_plus_finish(const GvPlusArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_plus_alloc(const GvPlusArgs& a, cudaStream_t s, bool pdl);
 cudaError_t launch_plus_layout(const GvPlusArgs& a, cudaStream_t s, bool pdl);
+// The tables of 1/n and of (C/(nh n), sqrt(1/(nh n))) for n < GV_PLUS_NTAB.
+cudaError_t launch_plus_tables(const GvPlusArgs& a, cudaStream_t s);
 cudaError_t launch_fill_plus(int ig, int form, const GvFillArgs& a, int n_tiles, size_t smem,
                              cudaStream_t s, bool pdl);
 cudaError_t launch_fill_adjoint(int form, int ept, const GvFillArgs& a, int n_tiles,
@@ -479,7 +482,10 @@ cudaError_t launch_reduce_batch(const GvReduceArgs* args, const int4* tasks, int
                                 int last, double inv_m1, size_t smem, cudaStream_t s);
 cudaError_t launch_consts(int integrand, const double* params, double* kconst, cudaStream_t s);
 cudaError_t launch_reset(GvState* st, cudaStream_t s);
-cudaError_t launch_grid_pack(int d, int N, double* grid, cudaStream_t s);
+// The tables of a grid whose edges are in place; with st, its counters are set
+// to it as well.
+cudaError_t launch_grid_pack(int d, int N, double* grid, GvState* st, unsigned long long it,
+                             cudaStream_t s);
 cudaError_t launch_rng_words(unsigned long long seed, uint32_t it, uint32_t batch,
                              unsigned long long ev0, long long n, int d, uint32_t* out,
                              cudaStream_t s);

@@ -306,7 +306,28 @@ __global__ void __launch_bounds__(kT, kMinBlocks) gv_plus_layout_kernel(const Gv
   if (h < a.nh) plus_layout_one(a, h, m, o);
 }
 
+// The tables of the per-count factors, in the same correctly rounded FP64
+// operations as for a count beyond them.
+__global__ void gv_plus_tables_kernel(const GvPlusArgs a) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= GV_PLUS_NTAB) return;
+  double inv = 0.0;
+  double2 f = make_double2(0.0, 0.0);
+  if (n > 0) {
+    const double nhd = (double)a.nh * (double)n;
+    inv = 1.0 / (double)n;
+    f = make_double2((double)a.ncall / nhd, sqrt(1.0 / nhd));
+  }
+  const_cast<double*>(a.inv)[n] = inv;
+  const_cast<double2*>(a.abtab)[n] = f;
+}
+
 namespace gv {
+
+cudaError_t launch_plus_tables(const GvPlusArgs& a, cudaStream_t s) {
+  gv_plus_tables_kernel<<<(GV_PLUS_NTAB + 255) / 256, 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_plus_finish(const GvPlusArgs& a, cudaStream_t s, bool pdl) {
   return gv_launch_prio(gv_plus_finish_kernel, dim3(kFC), dim3(kTF), 0, s, pdl, a.prio, a);

@@ -198,8 +198,9 @@ __device__ void finalize_iteration(const GvReduceArgs& a, int tid, int nthr, int
 // ---------------------------------------------------------------------------
 // Write the edges e_src (N+1 values) of axis ax into the grid pack with the
 // axis' derived tables.
+// (and the edges to mapped host memory, if given).
 __device__ __forceinline__ void pack_axis_tables(double* grid, const double* e_src, int ax, int d, int N, int tid,
-                                 int nthr) {
+                                 int nthr, double* host = nullptr) {
   const GvGridLayout L{d, N};
   double* e64 = grid + L.off_e64() + (size_t)ax * (N + 1);
   double* wd64 = grid + L.off_wd64() + (size_t)ax * N;
@@ -208,6 +209,7 @@ __device__ __forceinline__ void pack_axis_tables(double* grid, const double* e_s
   for (int i = tid; i <= N; i += nthr) {
     const double e = e_src[i];
     e64[i] = e;
+    if (host) host[(size_t)ax * (N + 1) + i] = e;
     if (i < N) {
       const double w = e_src[i + 1] - e;
       const double j = (double)N * w;
@@ -408,7 +410,7 @@ __device__ __forceinline__ void refine_axis(const GvReduceArgs& a, int ax, doubl
     for (int j = tid; j <= N; j += nthr) ne[j] = e[j];
   }
   gv_bar(bar, nthr);
-  pack_axis_tables(a.grid, ne, ax, a.ndim, N, tid, nthr);
+  pack_axis_tables(a.grid, ne, ax, a.ndim, N, tid, nthr, a.last ? a.host_grid : nullptr);
 }
 
 // Axes that one block of 32 slots can touch, and the dynamic shared memory
@@ -967,12 +969,15 @@ __global__ void gv_reset_kernel(GvState* st) {
   if (threadIdx.x == 0) st->nonfinite_iter = 0ull;
 }
 
-__global__ void gv_grid_pack_kernel(double* grid, int d, int N) {
-  // in place: each axis reads its own edges before writing them back unchanged
-  for (int ax = 0; ax < d; ++ax) {
-    pack_axis_tables(grid, grid + GvGridLayout{d, N}.off_e64() + (size_t)ax * (N + 1), ax, d, N,
-                     threadIdx.x, blockDim.x);
-    __syncthreads();
+// One CTA per axis, in place (the edges are written back unchanged).
+__global__ void gv_grid_pack_kernel(double* grid, int d, int N, GvState* st,
+                                    unsigned long long it) {
+  const int ax = blockIdx.x;
+  pack_axis_tables(grid, grid + GvGridLayout{d, N}.off_e64() + (size_t)ax * (N + 1), ax, d, N,
+                   threadIdx.x, blockDim.x);
+  if (st && ax == 0 && threadIdx.x == 0) {
+    st->it = it;
+    st->it0 = it;
   }
 }
 
@@ -1059,8 +1064,9 @@ cudaError_t launch_reset(GvState* st, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_grid_pack(int d, int N, double* grid, cudaStream_t s) {
-  gv_grid_pack_kernel<<<1, 256, 0, s>>>(grid, d, N);
+cudaError_t launch_grid_pack(int d, int N, double* grid, GvState* st, unsigned long long it,
+                             cudaStream_t s) {
+  gv_grid_pack_kernel<<<d, 128, 0, s>>>(grid, d, N, st, it);
   return cudaGetLastError();
 }
 
