@@ -98,8 +98,13 @@ __global__ void __launch_bounds__(GV_TILE / EPT, AdjBlocks<Real, EPT>::value)
       uint32_t r[MAXD];
       gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)(tile0 + slot), d, r);
       typename GvForm<Real>::Coord x[MAXD];
-      int bin[MAXD];
-      const GvJac<Real> J = gv_map_event<Real, MAXD>(r, d, N, s_jac, s_ew, x, bin);
+      GvJac<Real> J;
+#pragma unroll
+      for (int ax = 0; ax < MAXD; ++ax) {
+        int bin;
+        if (ax < d)
+          x[ax] = gv_map_axis<Real>(r[ax], N, s_jac + ax * N, s_ew + ax * N, ax == 0, J, bin);
+      }
       Real gr[1 + GV_NGRAD];
       if constexpr (GvForm<Real>::ID == GV_FORM_X64)
         gr[0] = gv_drell_yan_x<true>(x, K.k, gr + 1);

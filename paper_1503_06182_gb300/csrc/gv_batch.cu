@@ -3,7 +3,7 @@
 // The paper contrasts one run whose events all feed one grid with many
 // independent runs (Section 2.1); here many *different* integrations (uneven
 // dimension, call count and integrand) share the GPU.  Each iteration is
-//   one persistent fill launch per dimension class (at most 4, 8, 16 axes)
+//   one persistent fill launch per dimension class (at most 4, up to 16 axes)
 //   over a work list of (integration, tile) items,
 //   one reduce launch whose CTAs serve all integrations (task table) and
 //   refine each integration's axes as they complete,
@@ -101,7 +101,7 @@ struct vegas_batch {
   GvReduceArgs* d_red = nullptr;
   int4* d_red_tasks = nullptr;
   int n_red_tasks = 0;
-  // one work list per dimension class (members of at most 4, 8, 16 axes) and
+  // one work list per dimension class (members of at most 4, up to 16 axes) and
   // integrand
   struct FillClass {
     int maxd = 0, ig = 0, form = 0, n = 0, ctas = 0;
@@ -134,31 +134,31 @@ struct vegas_batch {
 namespace {
 
 // Work lists: dimension class, integrand and, in FP64, the arithmetic.
-constexpr int kMaxLists = 18;
+constexpr int kMaxLists = 12;
 
 // Dimension class of a member (the same classes as the single-context fill).
-int dim_class(int ig, int d) { return (d <= 4 && ig != VEGAS_EE3J) ? 4 : d <= 8 ? 8 : 16; }
+int dim_class(int ig, int d) { return (d <= 4 && ig != VEGAS_EE3J) ? 4 : 16; }
 
 // The list's fill launch (its counter reset first) and its occupancy.
 cudaError_t fill_class(vegas_batch* B, const vegas_batch::FillClass& c, int ept, int ctas,
                        cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(c.d_counter, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
-  static decltype(&gv::fill_batch_f4) const fs[3][3] = {
-      {gv::fill_batch_d4, gv::fill_batch_d8, gv::fill_batch_d16},
-      {gv::fill_batch_f4, gv::fill_batch_f8, gv::fill_batch_f16},
-      {gv::fill_batch_x4, gv::fill_batch_x8, gv::fill_batch_x16}};
-  auto f = fs[c.form][c.maxd == 4 ? 0 : (c.maxd == 8 ? 1 : 2)];
+  static decltype(&gv::fill_batch_f4) const fs[3][2] = {
+      {gv::fill_batch_d4, gv::fill_batch_d16},
+      {gv::fill_batch_f4, gv::fill_batch_f16},
+      {gv::fill_batch_x4, gv::fill_batch_x16}};
+  auto f = fs[c.form][c.maxd == 4 ? 0 : 1];
   return f(c.ig, ept, ctas, c.smem, s, B->d_fill, c.d_order, c.d_start, c.n, c.total,
            c.d_counter);
 }
 
 int class_occupancy(vegas_batch* B, const vegas_batch::FillClass& c, int ept) {
-  static decltype(&gv::fill_batch_occ_f4) const fs[3][3] = {
-      {gv::fill_batch_occ_d4, gv::fill_batch_occ_d8, gv::fill_batch_occ_d16},
-      {gv::fill_batch_occ_f4, gv::fill_batch_occ_f8, gv::fill_batch_occ_f16},
-      {gv::fill_batch_occ_x4, gv::fill_batch_occ_x8, gv::fill_batch_occ_x16}};
-  auto f = fs[c.form][c.maxd == 4 ? 0 : (c.maxd == 8 ? 1 : 2)];
+  static decltype(&gv::fill_batch_occ_f4) const fs[3][2] = {
+      {gv::fill_batch_occ_d4, gv::fill_batch_occ_d16},
+      {gv::fill_batch_occ_f4, gv::fill_batch_occ_f16},
+      {gv::fill_batch_occ_x4, gv::fill_batch_occ_x16}};
+  auto f = fs[c.form][c.maxd == 4 ? 0 : 1];
   return std::max(1, f(c.ig, ept, c.smem));
 }
 
@@ -478,10 +478,10 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
     int pos = 0, slot = 0;
     for (int cl = 0; cl < kMaxLists; ++cl) {
       {
-        const int maxd = cl % 3 == 0 ? 4 : (cl % 3 == 1 ? 8 : 16);
-        const int ig = cl / 3 % 3 == 0 ? VEGAS_GAUSS : (cl / 3 % 3 == 1 ? VEGAS_DY : VEGAS_EE3J);
-        const int form = precision ? GV_FORM_F32 : (cl < 9 ? GV_FORM_X64 : GV_FORM_F64);
-        if (precision && cl >= 9) continue;
+        const int maxd = cl % 2 == 0 ? 4 : 16;
+        const int ig = cl / 2 % 3 == 0 ? VEGAS_GAUSS : (cl / 2 % 3 == 1 ? VEGAS_DY : VEGAS_EE3J);
+        const int form = precision ? GV_FORM_F32 : (cl < 6 ? GV_FORM_X64 : GV_FORM_F64);
+        if (precision && cl >= 6) continue;
         std::vector<int> mem;
         for (int b = 0; b < n; ++b)
           if (B->m[b].ig == ig && B->m[b].form == form &&
@@ -507,9 +507,7 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
           acc += B->m[b].n_tiles;
           start.push_back(acc);
           c.smem = std::max<size_t>(c.smem,
-                            GvFillSmem(B->m[b].d, nbins, form, true, maxd > 4, 0, false,
-                                       false, true)
-                                .total);
+                            GvFillSmem(B->m[b].d, nbins, form, true, maxd > 4).total);
         }
         c.total = acc;
         B->cls.push_back(c);

@@ -81,59 +81,99 @@ __device__ __forceinline__ const GvX* gv_x_consts(const double* kconst) {
   return reinterpret_cast<const GvX*>(kconst + GV_NCONST);
 }
 
-template <int IG, typename Real, int MAXD>
-__device__ __forceinline__ Real gv_eval(const typename GvForm<Real>::Coord (&x)[MAXD], int d,
-                                        const GvConst<Real, GvTraits<IG>::NK>& K) {
-  if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
-    if constexpr (IG == GV_GAUSS)
-      return gv_gauss_x<MAXD>(x, d, K.k);
-    else if constexpr (IG == GV_DY)
-      return gv_drell_yan_x<false>(x, K.k, nullptr);
-    else if constexpr (IG == GV_DYNLO)
-      return gv_dy_nlo_x<MAXD>(x, d, K.k);
-    else
-      return gv_ee3j_x(x, K.k);
-  } else if constexpr (IG == GV_GAUSS) {
-    return gv_gauss<Real, MAXD>(x, d, K[GK_INV2S2], K[GK_SHIFT]);
-  } else if constexpr (IG == GV_DY) {
-    return gv_drell_yan<Real, false>(x, K, nullptr);
-  } else if constexpr (IG == GV_DYNLO) {
-    return gv_dy_nlo<Real, MAXD>(x, d, K);
-  } else {
-    return gv_ee3j<Real>(x, K);
-  }
-}
+// An integrand taken axis by axis: the variables that its formula needs at the
+// end stay (x), the others are consumed as they come, so that an event of many
+// axes holds few registers.  first(k, ..): axis k < 4, more(a, ..): axis
+// a >= 4, in order; then value and observable.  The observable (the
+// differential distributions of Section 3.2): Gauss x_0; Drell-Yan (both
+// forms) the dilepton mass m_ll = sqrt(tau s) in GeV, with tau as the
+// integrand forms it; 3-jet the thrust max(x1, x2, x3), x3 = 2 - x1 - x2.
+template <int IG, typename Real>
+struct GvStream {
+  using Coord = typename GvForm<Real>::Coord;
+  using W = typename GvForm<Real>::W;
+  using Const = GvConst<Real, GvTraits<IG>::NK>;
+  static constexpr bool X64 = GvForm<Real>::ID == GV_FORM_X64;
+  Coord x[IG == GV_EE3J ? 5 : 4];
+  Real f = Real();        // Gauss: the sum of squares; NLO-shaped: the factors' product
+  [[maybe_unused]] GvSumX q;  // Gauss, 64-bit significands: the sum of squares
 
-// The histogram observable of an event (the differential distributions of
-// Section 3.2): Gauss x_0; Drell-Yan (both forms) the dilepton mass
-// m_ll = sqrt(tau s) in GeV, with tau as the integrand forms it; 3-jet the
-// thrust max(x1, x2, x3), x3 = 2 - x1 - x2.
-template <int IG, typename Real, int MAXD>
-__device__ __forceinline__ typename GvForm<Real>::W gv_observable(
-    const typename GvForm<Real>::Coord (&x)[MAXD], const GvConst<Real, GvTraits<IG>::NK>& K) {
-  using Mt = GvMath<typename GvForm<Real>::W>;
-  if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
-    if constexpr (IG == GV_GAUSS) {
-      return x_to_double(x_from_q64(x[0]));
-    } else if constexpr (IG == GV_DY || IG == GV_DYNLO) {  // sqrt(s) 2^(log2(tau) / 2)
-      const unsigned long long lt = K[XK_B2].m - xi_mulhi(K[XK_A2].m, x[0]);
-      return x_to_double(x_mul(K[XK_SQRTS], x_exp2(lt, K[XK_B2].e - 1, true)));
-    } else {  // (x3 = 2 - x1 - x2 where it is below 1; elsewhere the weight is 0)
-      const unsigned long long x3 = 0ull - (x[0] + x[1]);
-      const unsigned long long t = x[0] > x[1] ? x[0] : x[1];
-      return x_to_double(x_from_q64(t > x3 ? t : x3));
-    }
-  } else if constexpr (IG == GV_GAUSS) {
-    return x[0];
-  } else if constexpr (IG == GV_DY || IG == GV_DYNLO) {
-    const Real tau = Mt::exp(Mt::fma(x[0], K[DK_L], K[DK_LOGTAULO]));
-    return Mt::sqrt(tau * K[DK_S]);
-  } else {
-    const Real x1 = x[0], x2 = x[1], x3 = (Real)2 - x1 - x2;
-    const Real t = x1 > x2 ? x1 : x2;
-    return t > x3 ? t : x3;
+  __device__ __forceinline__ void first(int k, const Coord& v, const Const& K) {
+    x[k] = v;
+    if constexpr (IG == GV_GAUSS) square(v);
   }
-}
+  __device__ __forceinline__ void more(int a, const Coord& v, const Const& K) {
+    if constexpr (IG == GV_GAUSS) {
+      square(v);
+    } else if constexpr (IG == GV_EE3J) {
+      if (a == 4) x[4] = v;
+    } else if constexpr (IG == GV_DYNLO) {
+      Real t;
+      if constexpr (X64)
+        t = gv_nlo_factor_x(v, K.k);
+      else
+        t = gv_nlo_factor<Real>(v, K);
+      if constexpr (X64)
+        f = a == 4 ? t : x_mul(f, t);
+      else
+        f = a == 4 ? t : f * t;
+    }
+  }
+  __device__ __forceinline__ void square(const Coord& v) {
+    if constexpr (X64) {
+      q.add(v);
+    } else {
+      const Real dx = v - (Real)0.5;
+      f = GvMath<Real>::fma(dx, dx, f);
+    }
+  }
+  __device__ __forceinline__ Real value(int d, const Const& K) const {
+    if constexpr (X64) {
+      if constexpr (IG == GV_GAUSS) return gv_gauss_x(q, K.k);
+      if constexpr (IG == GV_DY) return gv_drell_yan_x<false>(x, K.k, nullptr);
+      if constexpr (IG == GV_EE3J) return gv_ee3j_x(x, K.k);
+      if constexpr (IG == GV_DYNLO) {
+        const GvX g = gv_drell_yan_x<false>(x, K.k, nullptr);
+        return d > 4 ? x_mul(g, f) : g;
+      }
+    } else {
+      if constexpr (IG == GV_GAUSS)
+        return GvMath<Real>::exp(-f * K[GK_INV2S2]) - K[GK_SHIFT];
+      if constexpr (IG == GV_DY) return gv_drell_yan<Real, false>(x, K, nullptr);
+      if constexpr (IG == GV_EE3J) return gv_ee3j<Real>(x, K);
+      if constexpr (IG == GV_DYNLO) {
+        const Real g = gv_drell_yan<Real, false>(x, K, nullptr);
+        return d > 4 ? g * f : g;
+      }
+    }
+  }
+  __device__ __forceinline__ W observable(const Const& K) const {
+    if constexpr (X64) {
+      if constexpr (IG == GV_GAUSS) {
+        return x_to_double(x_from_q64(x[0]));
+      } else if constexpr (IG == GV_DY || IG == GV_DYNLO) {  // sqrt(s) 2^(log2(tau) / 2)
+        const unsigned long long lt = K[XK_B2].m - xi_mulhi(K[XK_A2].m, x[0]);
+        return x_to_double(x_mul(K[XK_SQRTS], x_exp2(lt, K[XK_B2].e - 1, true)));
+      } else {  // (x3 = 2 - x1 - x2 where it is below 1; elsewhere the weight is 0)
+        const unsigned long long x3 = 0ull - (x[0] + x[1]);
+        const unsigned long long t = x[0] > x[1] ? x[0] : x[1];
+        return x_to_double(x_from_q64(t > x3 ? t : x3));
+      }
+    } else {
+      using Mt = GvMath<Real>;
+      if constexpr (IG == GV_GAUSS) {
+        return x[0];
+      } else if constexpr (IG == GV_DY || IG == GV_DYNLO) {
+        const Real tau = Mt::exp(Mt::fma(x[0], K[DK_L], K[DK_LOGTAULO]));
+        return Mt::sqrt(tau * K[DK_S]);
+      } else {
+        const Real x1 = x[0], x2 = x[1], x3 = (Real)2 - x1 - x2;
+        const Real t = x1 > x2 ? x1 : x2;
+        return t > x3 ? t : x3;
+      }
+    }
+  }
+};
 
 // Histogram bin of v among nh bins over [lo, lo + nh / invw): 0 below (and
 // for a value that is not a number), nh + 1 above.
@@ -261,13 +301,13 @@ struct GvPair<GvX> {
 //   ew   [d*N]    GvBin32 (e, w, jm, je) in FP32, GvBin64 (e, w) on the FP64
 //                         pipe, GvBinX with 64-bit significands
 //   jac  [d*N]    f64     Jacobian factor N*(e_{i+1}-e_i) (FP64 pipe only)
-// After the first pass the forward fill's limbs lie over what follows evs (a
-// persistent kernel keeps the grid, so there they follow it):
+// After the first pass the forward fill's limbs lie over what follows evs:
 //   hist [d*N][L] u32     the bins' limbs
 //   hh   [nhist][L] u32, hw [nhist][LW] i32  the histogram's limbs of w^2 and w
 //   lq   [L][32] u32, lw [rows][32] i32   the lanes' columns of w^2 and of w
 // and beside both:
-//   bins [d][T]   u16     the events' bins (d > 4 classes only)
+//   bins [d][T]   u8      the events' bins (more than 4 axes), their high bytes
+//                         in as many again where N > 256
 //   po   [GV_PLUS_WIN] i32 hypercube offsets relative to the tile (VEGAS+)
 //   ps   [GV_PLUS_WIN + GV_TILE/GV_PLUS_SEG] double2  the tile's segments
 //                         (VEGAS+): each window hypercube's first, then each
@@ -295,7 +335,7 @@ __host__ __device__ inline bool gv_fill_hoistable(bool forward, bool plus, int d
 
 // Words of one event between the passes (GvEvent's layout).
 __host__ __device__ constexpr int gv_event_words32(bool f64, bool reg_bins, bool plus) {
-  return f64 ? (plus ? 4 : 2) + 2 : (plus ? 4 : 3);
+  return f64 ? (plus ? 4 : 2) + (reg_bins ? 2 : 1) : (plus ? 4 : (reg_bins ? 3 : 2));
 }
 
 struct GvFillSmem {
@@ -303,7 +343,7 @@ struct GvFillSmem {
   int L;
   __host__ __device__ GvFillSmem(int d, int N, int form, bool forward, bool bins_smem,
                                  int nhist = 0, bool plus = false, bool words = false,
-                                 bool keep_grid = false, int T = GV_TILE) {
+                                 int T = GV_TILE) {
     const unsigned dN = (unsigned)(d * N);
     const bool f64 = form != GV_FORM_F32;
     L = gv_limbs(d * N);
@@ -313,7 +353,7 @@ struct GvFillSmem {
     ew = wds > evs ? wds : evs;
     jac = ew + dN * (form == GV_FORM_X64 ? 32 : 16);
     const unsigned first = gv_align16(jac + (form == GV_FORM_F64 ? dN * 8 : 0));
-    limbs = keep_grid ? first : evs;
+    limbs = evs;
     hist = limbs;
     hh = hist + (forward ? dN * L * 4 : 0);
     hw = hh + (forward ? nhist * L * 4 : 0);
@@ -321,7 +361,7 @@ struct GvFillSmem {
     lw = lq + (forward ? L * 32 * 4 : 0);
     const unsigned second = gv_align16(lw + (forward ? gv_lane_rows(f64) * 32 * 4 : 0));
     bins = first > second ? first : second;
-    po = gv_align16(bins + ((forward && bins_smem) ? d * T * 2 : 0));
+    po = gv_align16(bins + ((forward && bins_smem) ? d * T * (N > 256 ? 2 : 1) : 0));
     ps = gv_align16(po + (plus ? GV_PLUS_WIN * 4 : 0));
     total = gv_align16(ps + (plus ? GV_PLUS_SEGS * 16 : 0));
   }
@@ -483,46 +523,38 @@ __device__ __forceinline__ void gv_stage_grid(const double* grid, int d, int N, 
   }
 }
 
-// Map one event's words through the grid: x, bins and the Jacobian.
-// FP64: x = e_i + f*(e_{i+1}-e_i) with f = (lo + 1/2) 2^-32, rounded as
+// One axis of an event: its word through the axis' row of the grid (s_ew, and
+// s_jac on the FP64 pipe): the variable, its bin, and the axis' factor into
+// the Jacobian J (which starts from the first factor).
+// FP64 pipe: x = e_i + f*(e_{i+1}-e_i) with f = (lo + 1/2) 2^-32, rounded as
 // written, J the FP64 product of the factors N (e_{i+1}-e_i); FP32: x with
-// FP32 edges and one fma, J as FP32 mantissa product and exponent sum.  The
-// product starts from the first factor (J = 1 * f0 * f1 ... exactly).
-// 64-bit significands: x = e + w (2 lo + 1) 2^-33 in fractions, J the product
-// of the normalised factors.
-template <typename Real, int MAXD>
-__device__ __forceinline__ GvJac<Real> gv_map_event(const uint32_t (&r)[MAXD], int d, int N,
-                                                    const double* s_jac,
-                                                    const typename GvPair<Real>::T* s_ew,
-                                                    typename GvForm<Real>::Coord (&x)[MAXD],
-                                                    int (&bin)[MAXD]) {
-  GvJac<Real> J;
-#pragma unroll
-  for (int a = 0; a < MAXD; ++a) {
-    if (a < d) {
-      const unsigned long long v = (unsigned long long)r[a] * (unsigned)N;
-      const int i = (int)(v >> 32);
-      const uint32_t lo = (uint32_t)v;
-      const auto ew = s_ew[a * N + i];
-      if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
-        x[a] = ew.e + xi_mul64x32(ew.w, lo) + (ew.w >> 33);
-        const GvX j = {ew.jm, (int)ew.je, 0u};
-        J.v = (a == 0) ? j : x_mul(J.v, j);
-      } else if constexpr (sizeof(Real) == 4) {
-        const float f = fmaf(__uint2float_rn(lo), 0x1p-32f, 0x1p-33f);
-        x[a] = fmaf(f, ew.w, ew.e);
-        J.m = (a == 0) ? ew.jm : __fmul_rn(J.m, ew.jm);
-        J.e = (a == 0) ? ew.je : J.e + ew.je;
-      } else {
-        const double f = ((double)lo + 0.5) * 0x1p-32;
-        x[a] = __dadd_rn(ew.e, __dmul_rn(f, ew.w));
-        const double jf = s_jac[a * N + i];
-        J.v = (a == 0) ? jf : __dmul_rn(J.v, jf);
-      }
-      bin[a] = i;
-    }
+// FP32 edges and one fma, J as FP32 mantissa product and exponent sum; 64-bit
+// significands: x = e + w (2 lo + 1) 2^-33 in fractions, J the product of the
+// normalised factors.
+template <typename Real>
+__device__ __forceinline__ typename GvForm<Real>::Coord gv_map_axis(
+    uint32_t r, int N, const double* s_jac, const typename GvPair<Real>::T* s_ew, bool first,
+    GvJac<Real>& J, int& bin) {
+  const unsigned long long v = (unsigned long long)r * (unsigned)N;
+  const int i = (int)(v >> 32);
+  const uint32_t lo = (uint32_t)v;
+  const auto ew = s_ew[i];
+  bin = i;
+  if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
+    const GvX j = {ew.jm, (int)ew.je, 0u};
+    J.v = first ? j : x_mul(J.v, j);
+    return ew.e + xi_mul64x32(ew.w, lo) + (ew.w >> 33);
+  } else if constexpr (sizeof(Real) == 4) {
+    const float f = fmaf(__uint2float_rn(lo), 0x1p-32f, 0x1p-33f);
+    J.m = first ? ew.jm : __fmul_rn(J.m, ew.jm);
+    J.e = first ? ew.je : J.e + ew.je;
+    return fmaf(f, ew.w, ew.e);
+  } else {
+    const double f = ((double)lo + 0.5) * 0x1p-32;
+    const double jf = s_jac[i];
+    J.v = first ? jf : __dmul_rn(J.v, jf);
+    return __dadd_rn(ew.e, __dmul_rn(f, ew.w));
   }
-  return J;
 }
 
 // |x| bits of a double, and its finiteness, on the integer pipes.
@@ -574,68 +606,68 @@ __device__ __forceinline__ GvSig<double> gv_sig(double x) {
 // at evs[j T + s]): FP32 form, 0: sign and significand of w (0: no weight),
 // 1: e2 + GV_SQ_OFF (12 bits) | bin 0 | bin 1 (10 bits each), 2: bin 2 | bin 3
 // | the histogram's bin; with VEGAS+, 2: bin 2 | bin 3 | e2 of q, 3: q's sign
-// and significand.  FP64 form: the double w (two words), then bins 0, 1, 2
-// and bin 3 | the histogram's bin; with VEGAS+ the double q at the end.  More
-// than 4 axes: the bins in s_bin.
-template <typename Real, int MAXD, bool PLUS, int T>
+// and significand.  FP64 form: the double w (two words), then bins 0, 1 and
+// bins 2, 3 | the histogram's bin; with VEGAS+ the double q at the end.  More
+// than 4 axes: the bins elsewhere, the histogram's bin in word 1 (FP64: 2).
+template <typename Real, bool REG, bool PLUS, int T>
 struct GvEvent {
-  static constexpr bool REG = MAXD <= 4;
-  unsigned* e;  // evs + slot
-  __device__ __forceinline__ static unsigned pack(const int (&bin)[MAXD], int d, int i, int j) {
-    unsigned r = 0u;
-    if (REG && i < MAXD && i < d) r = (unsigned)bin[i < MAXD ? i : 0];
-    if (REG && j < MAXD && j < d) r |= (unsigned)bin[j < MAXD ? j : 0] << 10;
-    return r;
-  }
-  __device__ __forceinline__ void put(const GvSig<float>& w, const GvSig<float>& q,
-                                      const int (&bin)[MAXD], int d, int hbin) const {
+  static constexpr bool F64 = sizeof(Real) == 8;
+  static constexpr int Q = F64 ? (REG ? 4 : 3) : 3;  // VEGAS+: first word of q's value
+  unsigned* e;                                       // evs + slot
+  // bins: 0, 1 and 2, 3 as pairs of 10 bits (at most 4 axes; else zero)
+  __device__ __forceinline__ void put(const GvSig<float>& w, const GvSig<float>& q, uint2 bins,
+                                      int hbin) const {
     e[0] = w.m | (w.neg ? 0x80000000u : 0u);
-    e[T] = ((unsigned)(w.e2 + GV_SQ_OFF) << 20) | pack(bin, d, 0, 1);
+    e[T] = ((unsigned)(w.e2 + GV_SQ_OFF) << 20) | (REG ? bins.x : (unsigned)hbin);
     if constexpr (PLUS) {
-      e[2 * T] = ((unsigned)(q.e2 + GV_SQ_OFF) << 20) | pack(bin, d, 2, 3);
-      e[3 * T] = q.m | (q.neg ? 0x80000000u : 0u);
-    } else {
-      e[2 * T] = ((unsigned)hbin << 20) | pack(bin, d, 2, 3);
+      e[2 * T] = ((unsigned)(q.e2 + GV_SQ_OFF) << 20) | bins.y;
+      e[Q * T] = q.m | (q.neg ? 0x80000000u : 0u);
+    } else if constexpr (REG) {
+      e[2 * T] = ((unsigned)hbin << 20) | bins.y;
     }
   }
-  __device__ __forceinline__ void put(double w, double q, const int (&bin)[MAXD], int d,
-                                      int hbin) const {
+  __device__ __forceinline__ void put(double w, double q, uint2 bins, int hbin) const {
     const unsigned long long b = (unsigned long long)__double_as_longlong(w);
     e[0] = (unsigned)b;
     e[T] = (unsigned)(b >> 32);
-    e[2 * T] = pack(bin, d, 0, 1);
-    e[3 * T] = ((unsigned)hbin << 20) | pack(bin, d, 2, 3);
+    if constexpr (REG) {
+      e[2 * T] = bins.x;
+      e[3 * T] = ((unsigned)hbin << 20) | bins.y;
+    } else {
+      e[2 * T] = (unsigned)hbin << 20;
+    }
     if constexpr (PLUS) {
       const unsigned long long c = (unsigned long long)__double_as_longlong(q);
-      e[4 * T] = (unsigned)c;
-      e[5 * T] = (unsigned)(c >> 32);
+      e[Q * T] = (unsigned)c;
+      e[(Q + 1) * T] = (unsigned)(c >> 32);
     }
   }
   __device__ __forceinline__ void none() const {
     e[0] = 0u;
-    if constexpr (sizeof(Real) == 8) e[T] = 0u;
-    if constexpr (PLUS) e[3 * T] = 0u;
-    if constexpr (PLUS && sizeof(Real) == 8) e[4 * T] = e[5 * T] = 0u;
+    if constexpr (F64) e[T] = 0u;
+    if constexpr (PLUS) e[Q * T] = 0u;
+    if constexpr (PLUS && F64) e[(Q + 1) * T] = 0u;
   }
   // the weight (VEGAS+: which = 1, the bins' quantity); m = 0: none
   template <int WHICH>
   __device__ __forceinline__ GvSig<Real> get() const {
-    if constexpr (sizeof(Real) == 4) {
-      const unsigned sm = e[WHICH ? 3 * T : 0];
+    if constexpr (!F64) {
+      const unsigned sm = e[WHICH ? Q * T : 0];
       const unsigned x = e[WHICH ? 2 * T : T];
       return GvSig<float>{sm & 0xFFFFFFu, (int)(x >> 20) - GV_SQ_OFF, (sm >> 31) != 0u};
     } else {
       const unsigned long long b =
-          ((unsigned long long)e[WHICH ? 5 * T : T] << 32) | e[WHICH ? 4 * T : 0];
+          ((unsigned long long)e[WHICH ? (Q + 1) * T : T] << 32) | e[WHICH ? Q * T : 0];
       return gv_sig(__longlong_as_double((long long)b));
     }
   }
   // bins 0, 1 (lo) and 2, 3 (hi), 10 bits each, for at most 4 axes
   __device__ __forceinline__ uint2 bins() const {
-    return sizeof(Real) == 4 ? make_uint2(e[T], e[2 * T]) : make_uint2(e[2 * T], e[3 * T]);
+    return F64 ? make_uint2(e[2 * T], e[3 * T]) : make_uint2(e[T], e[2 * T]);
   }
   __device__ __forceinline__ int hbin() const {
-    return (int)(e[sizeof(Real) == 4 ? 2 * T : 3 * T] >> 20);
+    if constexpr (F64) return (int)(e[(REG ? 3 : 2) * T] >> 20);
+    return REG ? (int)(e[2 * T] >> 20) : (int)(e[T] & 0xFFFFFu);
   }
 };
 
@@ -668,7 +700,8 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
   using W = typename GvForm<Real>::W;
   constexpr bool F64 = sizeof(W) == 8;
   using Pair = typename GvPair<Real>::T;
-  using Event = GvEvent<W, MAXD, PLUS, T>;
+  constexpr bool REG = MAXD <= 4;  // bins held in the event's words
+  using Event = GvEvent<W, REG, PLUS, T>;
   __shared__ int s_max[2][NW];
   const int d = a.ndim, N = a.nbins, dN = d * N, L = lay.L;
   const int hb = HIST ? a.nhist : 0;
@@ -679,7 +712,8 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
   const long long h0 = PLUS ? pf->tile_h0[tile] : 0;
   const double* s_jac = reinterpret_cast<const double*>(smem + lay.jac);
   const Pair* s_ew = reinterpret_cast<const Pair*>(smem + lay.ew);
-  unsigned short* s_bin = reinterpret_cast<unsigned short*>(smem + lay.bins);
+  unsigned char* s_bin = smem + lay.bins;                      // [d][T]
+  unsigned char* s_binh = N > 256 ? s_bin + d * T : nullptr;  // their high bytes
   unsigned* evs = reinterpret_cast<unsigned*>(smem + lay.wd);
   const int tid = threadIdx.x;
   const long long tile0 = tile * a.tile_events;
@@ -708,7 +742,7 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
     [[maybe_unused]] int jcur = -1;  // the open segment's window index
     [[maybe_unused]] double sg1 = 0.0, sg2 = 0.0;
     constexpr bool KEEP_DIGITS = MAXD <= 4;  // registers to spare only for few axes
-    [[maybe_unused]] unsigned cdig[MAXD];
+    [[maybe_unused]] unsigned cdig[PLUS ? MAXD : 1];
 #pragma unroll 1
     for (int k = 0; k < nk; ++k) {
       const int local = PLUS ? tid * EPT + k : k * B + tid;
@@ -718,15 +752,42 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
         event.none();
         continue;
       }
-      uint32_t r[MAXD];
-      if (words) {  // generated before the wait, by this thread
+      GvStream<IG, Real> S;
+      GvJac<Real> J;
+      uint2 bins = make_uint2(0u, 0u);
+      const auto put_bin = [&](int ax, int bin) {
+        if constexpr (!REG) {
+          s_bin[ax * T + slot] = (unsigned char)bin;
+          if (s_binh) s_binh[ax * T + slot] = (unsigned char)(bin >> 8);
+        }
+      };
+      const auto axes4 = [&](const uint32_t* r) {  // axes 0..3
 #pragma unroll
-        for (int j = 0; j < MAXD; ++j)
-          if (j < d) r[j] = evs[j * T + slot];
-      } else {
-        gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)(tile0 + local), d, r);
-      }
+        for (int k = 0; k < 4; ++k) {
+          if (k < d) {
+            int bin;
+            S.first(k, gv_map_axis<Real>(r[k], N, s_jac + k * N, s_ew + k * N, k == 0, J, bin), K);
+            if constexpr (REG)
+              (k < 2 ? bins.x : bins.y) |= (unsigned)bin << (10 * (k & 1));
+            else
+              put_bin(k, bin);
+          }
+        }
+      };
+      const auto axis = [&](int ax, uint32_t r) {  // an axis past those
+        int bin;
+        S.more(ax, gv_map_axis<Real>(r, N, s_jac + ax * N, s_ew + ax * N, false, J, bin), K);
+        put_bin(ax, bin);
+      };
       if constexpr (PLUS) {
+        uint32_t r[MAXD];
+        if (words) {  // generated before the wait, by this thread
+#pragma unroll
+          for (int j = 0; j < MAXD; ++j)
+            if (j < d) r[j] = evs[j * T + slot];
+        } else {
+          gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)(tile0 + local), d, r);
+        }
         while (jc + 1 < GV_PLUS_WIN && s_off[jc + 1] <= local) ++jc;
         if (jc != jcur) {  // a new hypercube: close the previous segment
           if (jcur >= 0)
@@ -740,22 +801,48 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
         if (!KEEP_DIGITS)
           gv_plus_digits<MAXD>((unsigned)(h0 + jc), d, (unsigned)pf->s, pf->inv_s, cdig);
         gv_plus_strat<MAXD>(cdig, d, (unsigned)pf->s, pf->magic, r);
-      }
-      typename GvForm<Real>::Coord x[MAXD];
-      int bin[MAXD];
-      const GvJac<Real> J = gv_map_event<Real, MAXD>(r, d, N, s_jac, s_ew, x, bin);
-      if constexpr (!Event::REG) {
+        axes4(r);
 #pragma unroll
-        for (int ax = 0; ax < MAXD; ++ax)
-          if (ax < d) s_bin[ax * T + slot] = (unsigned short)bin[ax];
+        for (int ax = 4; ax < MAXD; ++ax)
+          if (ax < d) axis(ax, r[ax]);
+      } else {
+        // one Philox block (4 axes) at a time
+        const unsigned long long ev = (unsigned long long)(tile0 + local);
+        const auto block = [&](int j, uint32_t (&r)[4]) {
+          if (words) {  // generated before the wait, by this thread
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (4 * j + k < d) r[k] = evs[(4 * j + k) * T + slot];
+          } else {
+            const uint4 o = gv_philox(make_uint4((uint32_t)ev, (uint32_t)(ev >> 32), it,
+                                                 (a.batch << 8) | (uint32_t)j),
+                                      (uint32_t)a.seed, (uint32_t)(a.seed >> 32));
+            r[0] = o.x;
+            r[1] = o.y;
+            r[2] = o.z;
+            r[3] = o.w;
+          }
+        };
+        uint32_t r[4];
+        block(0, r);
+        axes4(r);
+        if constexpr (!REG) {
+#pragma unroll 1
+          for (int j = 1; 4 * j < d; ++j) {
+            block(j, r);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (4 * j + k < d) axis(4 * j + k, r[k]);
+          }
+        }
       }
-      const Real g = gv_eval<IG, Real, MAXD>(x, d, K);
+      const Real g = S.value(d, K);
       int hbin = 0;
       if constexpr (HIST) {
         if constexpr (F64)
-          hbin = gv_hist_bin<W>(gv_observable<IG, Real, MAXD>(x, K), a.h_lo, a.h_invw, hb - 2);
+          hbin = gv_hist_bin<W>(S.observable(K), a.h_lo, a.h_invw, hb - 2);
         else
-          hbin = gv_hist_bin<W>(gv_observable<IG, Real, MAXD>(x, K), a.h_lo_f, a.h_invw_f, hb - 2);
+          hbin = gv_hist_bin<W>(S.observable(K), a.h_lo_f, a.h_invw_f, hb - 2);
       }
       if constexpr (!F64) {
         const unsigned u = __float_as_uint(__fmul_rn(J.m, g));
@@ -788,7 +875,7 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
         if (fin && (kw > 0 || kq > 0)) {
           if (kw <= 0) sw = GvSig<float>{0u, 0, false};
           if (PLUS && kq <= 0) sq = GvSig<float>{0u, 0, false};
-          event.put(sw, sq, bin, d, hbin);
+          event.put(sw, sq, bins, hbin);
         } else {
           event.none();
         }
@@ -811,7 +898,7 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
           fin = gv_finite_bits(gv_abs_bits(wv)) && gv_finite_bits(gv_abs_bits(qk));
         }
         if (fin) {
-          event.put(wv, qk, bin, d, hbin);
+          event.put(wv, qk, bins, hbin);
           if (gv_abs_bits(wv) != 0ull) mw = max(mw, gv_scale_exp(gv_abs_bits(wv)) - 53);
           if constexpr (PLUS)
             if (gv_abs_bits(qk) != 0ull) mq = max(mq, gv_scale_exp(gv_abs_bits(qk)) - 53);
@@ -879,15 +966,20 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
       const Event event{evs + slot};
       const auto add_bins = [&](const unsigned (&l)[4], int pos) {
         unsigned row = a_hist + 4u * (unsigned)pos;
-        const uint2 b = Event::REG ? event.bins() : make_uint2(0u, 0u);
+        if constexpr (REG) {
+          const uint2 b = event.bins();
 #pragma unroll
-        for (int ax = 0; ax < MAXD; ++ax) {
-          if (ax < d) {
-            unsigned bin;
-            if constexpr (Event::REG)
-              bin = ((ax < 2 ? b.x : b.y) >> (10 * (ax & 1))) & 0x3FFu;
-            else
-              bin = s_bin[ax * T + slot];
+          for (int ax = 0; ax < 4; ++ax) {
+            if (ax < d) {
+              gv_bin_add_square<W>(l, row + (((ax < 2 ? b.x : b.y) >> (10 * (ax & 1))) & 0x3FFu) * L4);
+              row += axis4;
+            }
+          }
+        } else {
+#pragma unroll 4
+          for (int ax = 0; ax < d; ++ax) {
+            unsigned bin = s_bin[ax * T + slot];
+            if (s_binh) bin |= (unsigned)s_binh[ax * T + slot] << 8;
             gv_bin_add_square<W>(l, row + bin * L4);
             row += axis4;
           }
@@ -972,7 +1064,7 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
 // The Philox words of a tile's events at counter `it` into shared memory
 // (word a of slot s at s_words[a T + s]); each thread makes the words of the
 // events it will evaluate, so no barrier is needed before use.
-template <int MAXD, int T, int B, bool PLUS>
+template <int T, int B, bool PLUS>
 __device__ __forceinline__ void gv_tile_words(const GvFillArgs& a, uint32_t it, long long tile,
                                               unsigned* s_words) {
   const int d = a.ndim;
@@ -982,30 +1074,32 @@ __device__ __forceinline__ void gv_tile_words(const GvFillArgs& a, uint32_t it, 
   for (int k = 0; k < nk; ++k) {
     const int local = PLUS ? (int)threadIdx.x * (T / B) + k : k * B + (int)threadIdx.x;
     const int slot = k * B + (int)threadIdx.x;
-    uint32_t r[MAXD];
-    gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)(t0 + local), d, r);
-#pragma unroll
-    for (int j = 0; j < MAXD; ++j)
-      if (j < d) s_words[j * T + slot] = r[j];
+    const unsigned long long ev = (unsigned long long)(t0 + local);
+#pragma unroll 1
+    for (int j = 0; 4 * j < d; ++j) {
+      const uint4 o = gv_philox(
+          make_uint4((uint32_t)ev, (uint32_t)(ev >> 32), it, (a.batch << 8) | (uint32_t)j),
+          (uint32_t)a.seed, (uint32_t)(a.seed >> 32));
+      unsigned* w = s_words + 4 * j * T + slot;
+      w[0] = o.x;
+      w[T] = o.y;
+      w[2 * T] = o.z;
+      w[3 * T] = o.w;
+    }
   }
 }
 
 // Minimum resident CTAs per SM in the fill's launch bound (0: none), i.e. its
-// register budget.  FP32 fills of at most 8 axes: 64 registers at any width
-// (the stratified fill of at most 4 axes included; the stratified fill of up
-// to 8 axes, which keeps its range's segment sums, takes 80 with three
-// 256-thread CTAs: at 64 it spilled ~250 bytes).  FP32 fills of up to 16 axes without
-// VEGAS+, 4 events per thread: three 256-thread CTAs, 80 registers (111 for
-// the 13-axis NLO-shaped weight unbounded).  FP64 fills: none (they would
-// spill).
+// register budget: 64 registers for FP32 fills at any width, 80 for the
+// stratified ones of 5 to 8 axes and none above (they would spill); FP64
+// fills: none.
 template <typename Real, int EPT, int MAXD, bool PLUS>
 struct GvFillBlocks {
   static constexpr int B = GV_TILE / EPT;
   static constexpr int value = GvForm<Real>::ID != GV_FORM_F32 ? 0
+                               : (PLUS && MAXD == 16)  ? 0
                                : (PLUS && MAXD == 8)   ? 3
-                               : MAXD <= 8             ? 65536 / (64 * B)
-                               : (!PLUS && EPT == 4)   ? 3
-                                                       : 0;
+                                                       : 65536 / (64 * B);
 };
 
 template <int IG, typename Real, int EPT, int MAXD, bool HIST = false, bool PLUS = false>
@@ -1014,7 +1108,7 @@ __global__ void __launch_bounds__(GV_TILE / EPT, (GvFillBlocks<Real, EPT, MAXD, 
   constexpr int B = GV_TILE / EPT, T = GV_TILE;
   extern __shared__ __align__(16) unsigned char smem[];
   const int d = a.ndim, N = a.nbins;
-  const bool hoist = MAXD <= 8 && a.hoist;  // set by the host (gv_fill_hoistable)
+  const bool hoist = a.hoist;  // set by the host (gv_fill_hoistable)
   const GvFillSmem lay(d, N, GvForm<Real>::ID, true, MAXD > 4, HIST ? a.nhist : 0, PLUS, hoist);
   // the tile's words at the counter this iteration should have (the stage's
   // first counter, which no running kernel writes, plus the iteration index),
@@ -1023,7 +1117,7 @@ __global__ void __launch_bounds__(GV_TILE / EPT, (GvFillBlocks<Real, EPT, MAXD, 
   uint32_t itg = 0u;
   if (hoist) {
     itg = (uint32_t)(a.st->it0 + (unsigned long long)a.kst);
-    gv_tile_words<MAXD, T, B, PLUS>(a, itg, blockIdx.x, s_words);
+    gv_tile_words<T, B, PLUS>(a, itg, blockIdx.x, s_words);
   }
   gv_wait_prior_grid();  // grid, constants and iteration counter come from earlier kernels
   if constexpr (PLUS) {
@@ -1054,7 +1148,7 @@ __global__ void __launch_bounds__(GV_TILE / EPT, (GvFillBlocks<Real, EPT, MAXD, 
     }
   }
   const uint32_t it = (uint32_t)a.st->it;
-  if (hoist && it != itg) gv_tile_words<MAXD, T, B, PLUS>(a, it, blockIdx.x, s_words);  // (not expected)
+  if (hoist && it != itg) gv_tile_words<T, B, PLUS>(a, it, blockIdx.x, s_words);  // (not expected)
   __syncthreads();
   gv_fill_tile<IG, Real, EPT, MAXD, HIST, PLUS>(a, blockIdx.x, smem, lay, it,
                                                 hoist);
@@ -1081,33 +1175,28 @@ __global__ void gv_eval_events_kernel(const GvFillArgs a, uint32_t it, const lon
     K.load(a.kconst);
   uint32_t r[MAXD];
   gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)events[j], d, r);
-  typename GvForm<Real>::Coord x[MAXD];
+  GvStream<IG, Real> S;
   GvJac<Real> J;
 #pragma unroll
   for (int ax = 0; ax < MAXD; ++ax) {
     if (ax < d) {
-      const unsigned long long v = (unsigned long long)r[ax] * (unsigned)N;
-      const int i = (int)(v >> 32);
-      const uint32_t lo = (uint32_t)v;
-      const int k = ax * N + i;
-      if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
-        const GvBinX b = gv_bin_x(e64[ax * (N + 1) + i], wd64[k], N);
-        x[ax] = b.e + xi_mul64x32(b.w, lo) + (b.w >> 33);
-        const GvX f = {b.jm, (int)b.je, 0u};
-        J.v = (ax == 0) ? f : x_mul(J.v, f);
-      } else if constexpr (sizeof(Real) == 4) {
-        const float f = fmaf(__uint2float_rn(lo), 0x1p-32f, 0x1p-33f);
-        x[ax] = fmaf(f, b32[k].w, b32[k].e);
-        J.m = (ax == 0) ? b32[k].jm : __fmul_rn(J.m, b32[k].jm);
-        J.e = (ax == 0) ? b32[k].je : J.e + b32[k].je;
-      } else {
-        const double f = ((double)lo + 0.5) * 0x1p-32;
-        x[ax] = __dadd_rn(e64[ax * (N + 1) + i], __dmul_rn(f, wd64[k]));
-        J.v = (ax == 0) ? jac[k] : __dmul_rn(J.v, jac[k]);
-      }
-      bins[j * d + ax] = i;
+      // the bin's record, as gv_stage_grid stages it, on its own
+      const int i = (int)(((unsigned long long)r[ax] * (unsigned)N) >> 32), k = ax * N + i;
+      typename GvPair<Real>::T rec;
+      if constexpr (GvForm<Real>::ID == GV_FORM_X64)
+        rec = gv_bin_x(e64[ax * (N + 1) + i], wd64[k], N);
+      else if constexpr (sizeof(Real) == 4)
+        rec = b32[k];
+      else
+        rec = GvBin64{e64[ax * (N + 1) + i], wd64[k]};
+      int bin;
+      const auto x = gv_map_axis<Real>(r[ax], N, jac + ax * N, &rec - i, ax == 0, J, bin);
+      if (ax < 4)
+        S.first(ax < 4 ? ax : 0, x, K);
+      else
+        S.more(ax, x, K);
+      bins[j * d + ax] = bin;
     }
   }
-  const Real g = gv_eval<IG, Real, MAXD>(x, d, K);
-  w[j] = gv_weight(J, g);
+  w[j] = gv_weight(J, S.value(d, K));
 }

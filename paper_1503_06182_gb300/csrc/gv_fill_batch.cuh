@@ -1,7 +1,7 @@
 // gv_fill_batch.cuh -- the persistent fill kernel of the batched form and its
 // launch helpers, instantiated per precision and dimension class in
-// gv_batch_{f,d,x}{4,8,16}.cu (so that they compile in parallel).  Each class
-// (at most 4, 8 or 16 axes) and integrand runs its own work list with code
+// gv_batch_{f,d,x}{4,16}.cu (so that they compile in parallel).  Each class
+// (at most 4, or up to 16 axes) and integrand runs its own work list with code
 // unrolled for it: one kernel holding the three integrands needed the
 // registers of two (219 instead of 96-126 at 16 axes, one CTA per SM
 // instead of two).
@@ -23,7 +23,6 @@ __global__ void __launch_bounds__(GV_TILE / EPT,
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long s_item;
   __shared__ int s_pos;
-  int cur = -1;
   for (;;) {
     if (threadIdx.x == 0) {
       const long long item = (long long)atomicAdd(counter, 1ull);
@@ -49,13 +48,12 @@ __global__ void __launch_bounds__(GV_TILE / EPT,
     const int b = order[pos];
     const long long tile = item - item_start[pos];
     const GvFillArgs a = args[b];
-    const GvFillSmem lay(a.ndim, a.nbins, GvForm<Real>::ID, true, MAXD > 4, 0, false, false, true);
-    if (b != cur) {
-      gv_stage_grid<Real>(a.grid, a.ndim, a.nbins, reinterpret_cast<double*>(smem + lay.jac),
-                          reinterpret_cast<typename GvPair<Real>::T*>(smem + lay.ew),
-                          threadIdx.x, B);
-      cur = b;
-    }
+    const GvFillSmem lay(a.ndim, a.nbins, GvForm<Real>::ID, true, MAXD > 4);
+    // staged for every tile: the limbs of the tile before lie over it (kept
+    // beside them, the grid cost a resident CTA)
+    gv_stage_grid<Real>(a.grid, a.ndim, a.nbins, reinterpret_cast<double*>(smem + lay.jac),
+                        reinterpret_cast<typename GvPair<Real>::T*>(smem + lay.ew), threadIdx.x,
+                        B);
     const uint32_t it = (uint32_t)a.st->it;
     __syncthreads();
     gv_fill_tile<IG, Real, EPT, MAXD>(a, tile, smem, lay, it);
@@ -154,11 +152,8 @@ inline int gv_fill_batch_occ_ig(int ept, size_t smem) {
   }                                                                                           \
   }
 GV_DECLARE_FILL_BATCH(f4)
-GV_DECLARE_FILL_BATCH(f8)
 GV_DECLARE_FILL_BATCH(f16)
 GV_DECLARE_FILL_BATCH(d4)
-GV_DECLARE_FILL_BATCH(d8)
 GV_DECLARE_FILL_BATCH(d16)
 GV_DECLARE_FILL_BATCH(x4)
-GV_DECLARE_FILL_BATCH(x8)
 GV_DECLARE_FILL_BATCH(x16)

@@ -39,7 +39,6 @@ static cudaError_t gv_launch_fill_maxd(int ept, const GvFillArgs& a, int n_tiles
                                        cudaStream_t s, bool pdl) {
   if (a.ndim <= 4 && IG != GV_EE3J)
     return gv_launch_fill_ept<IG, Real, 4>(ept, a, n_tiles, smem, s, pdl);
-  if (a.ndim <= 8) return gv_launch_fill_ept<IG, Real, 8>(ept, a, n_tiles, smem, s, pdl);
   if (a.ndim <= 16) return gv_launch_fill_ept<IG, Real, 16>(ept, a, n_tiles, smem, s, pdl);
   return cudaErrorInvalidValue;
 }
@@ -51,7 +50,6 @@ static cudaError_t gv_launch_fill_hist_t(const GvFillArgs& a, int n_tiles, size_
                                          cudaStream_t s, bool pdl) {
   if (a.ndim <= 4 && IG != GV_EE3J)
     return gv_launch_fill_t<IG, Real, 4, 4, true>(a, n_tiles, smem, s, pdl);
-  if (a.ndim <= 8) return gv_launch_fill_t<IG, Real, 4, 8, true>(a, n_tiles, smem, s, pdl);
   if (a.ndim <= 16) return gv_launch_fill_t<IG, Real, 4, 16, true>(a, n_tiles, smem, s, pdl);
   return cudaErrorInvalidValue;
 }

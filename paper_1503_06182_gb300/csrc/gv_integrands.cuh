@@ -116,22 +116,9 @@ struct GvConst {
   __device__ __forceinline__ Real operator[](int i) const { return v[i]; }
 };
 
-// ---------------------------------------------------------------------------
-// Gaussian product minus a constant: g = exp(-sum_a (x_a - 1/2)^2 / (2 sigma^2))
-// - shift (shift = 0 unless given: negative weights, as NLO subtractions give).
-// ---------------------------------------------------------------------------
-template <typename Real, int MAXD>
-__device__ __forceinline__ Real gv_gauss(const Real (&x)[MAXD], int d, Real inv2s2, Real shift) {
-  Real acc = (Real)0;
-#pragma unroll
-  for (int a = 0; a < MAXD; ++a) {
-    if (a < d) {
-      const Real dx = x[a] - (Real)0.5;
-      acc = GvMath<Real>::fma(dx, dx, acc);
-    }
-  }
-  return GvMath<Real>::exp(-acc * inv2s2) - shift;
-}
+// The Gaussian product minus a constant, g = exp(-sum_a (x_a - 1/2)^2 / (2
+// sigma^2)) - shift (shift = 0 unless given: negative weights, as NLO
+// subtractions give), is summed axis by axis (GvStream).
 
 // ---------------------------------------------------------------------------
 // LO pp -> gamma*/Z -> mu- mu+ (four variables: tau, rapidity, cos theta, phi).
@@ -238,21 +225,12 @@ __device__ __forceinline__ Real gv_drell_yan(const Real* x, const GvConst<Real, 
 // further axis, exp(beta cos(2 pi x_k)) / I0(beta) (each factor integrates to
 // 1 over [0,1]).  More axes, more work per event, the same integral.
 // ---------------------------------------------------------------------------
-template <typename Real, int MAXD>
-__device__ __forceinline__ Real gv_dy_nlo(const Real (&x)[MAXD], int d,
-                                          const GvConst<Real, NK_NK>& K) {
+template <typename Real>
+__device__ __forceinline__ Real gv_nlo_factor(Real x, const GvConst<Real, NK_NK>& K) {
   using Mt = GvMath<Real>;
-  Real g = gv_drell_yan<Real, false>(x, K, nullptr);
-  Real f = (Real)1;
-#pragma unroll
-  for (int a = 4; a < MAXD; ++a) {
-    if (a < d) {
-      Real sn, cs;
-      Mt::sincospi((Real)2 * x[a], &sn, &cs);
-      f = f * (Mt::exp(K[NK_BETA] * cs) * K[NK_INVI0]);
-    }
-  }
-  return g * f;
+  Real sn, cs;
+  Mt::sincospi((Real)2 * x, &sn, &cs);
+  return Mt::exp(K[NK_BETA] * cs) * K[NK_INVI0];
 }
 
 // ---------------------------------------------------------------------------

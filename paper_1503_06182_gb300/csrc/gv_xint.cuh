@@ -42,36 +42,38 @@
 // Gaussian product minus a constant.  The squares are summed exactly (128
 // bits and a carry word).
 // ---------------------------------------------------------------------------
-template <int MAXD>
-GV_X_FN GvX gv_gauss_x(const unsigned long long (&x)[MAXD], int d, const GvX* K) {
+struct GvSumX {
   unsigned long long lo = 0ull, mid = 0ull;
   unsigned top = 0u;
-#ifdef __CUDA_ARCH__
-#pragma unroll
-#endif
-  for (int a = 0; a < MAXD; ++a) {
-    if (a < d) {
-      const unsigned long long h = 1ull << 63, dx = x[a] >= h ? x[a] - h : h - x[a];
-      const unsigned long long pl = dx * dx, ph = xi_mulhi(dx, dx);
-      lo += pl;
-      const unsigned long long c = lo < pl ? 1ull : 0ull;
-      mid += ph + c;  // ph < 2^63: no carry within
-      top += mid < ph + c ? 1u : 0u;
-    }
+  GV_X_FN void add(unsigned long long x) {
+    const unsigned long long h = 1ull << 63, dx = x >= h ? x - h : h - x;
+    const unsigned long long pl = dx * dx, ph = xi_mulhi(dx, dx);
+    lo += pl;
+    const unsigned long long c = ph + (lo < pl ? 1ull : 0ull);  // ph < 2^63: no carry within
+    mid += c;
+    top += mid < c ? 1u : 0u;
   }
+};
+GV_X_FN GvX gv_gauss_x(const GvSumX& s, const GvX* K) {
   GvX q;
-  if (top) {
-    const int k = 64 - xi_clz((unsigned long long)top);
-    q = GvX{((unsigned long long)top << (64 - k)) | (mid >> k), -64 + k, 0u};
-  } else if (mid) {
-    const int lz = xi_clz(mid);
-    q = GvX{lz ? (mid << lz) | (lo >> (64 - lz)) : mid, -64 - lz, 0u};
+  if (s.top) {
+    const int k = 64 - xi_clz((unsigned long long)s.top);
+    q = GvX{((unsigned long long)s.top << (64 - k)) | (s.mid >> k), -64 + k, 0u};
+  } else if (s.mid) {
+    const int lz = xi_clz(s.mid);
+    q = GvX{lz ? (s.mid << lz) | (s.lo >> (64 - lz)) : s.mid, -64 - lz, 0u};
   } else {
-    q = x_norm(lo, -128);
+    q = x_norm(s.lo, -128);
   }
   const GvX t = x_mul(q, K[XK_INV2S2]);
   const GvX g = x_exp2(t.m, t.e, true);
   return K[XK_MSHIFT].m ? x_add(g, K[XK_MSHIFT]) : g;
+}
+template <int MAXD>
+GV_X_FN GvX gv_gauss_x(const unsigned long long (&x)[MAXD], int d, const GvX* K) {
+  GvSumX s;
+  for (int a = 0; a < d; ++a) s.add(x[a]);
+  return gv_gauss_x(s, K);
 }
 
 // 1 - q for a fraction q
@@ -153,18 +155,13 @@ GV_X_FN GvX gv_drell_yan_x(const unsigned long long* x, const GvX* K, GvX* grad)
 // ---------------------------------------------------------------------------
 // NLO-shaped stand-in: Drell-Yan times exp(beta cos 2 pi x_k) / I0(beta).
 // ---------------------------------------------------------------------------
+GV_X_FN GvX gv_nlo_factor_x(unsigned long long x, const GvX* K) {
+  return x_mul(x_exp2(x_mul(K[XK_BETA2], x_from_q62(x_cos_turn(x)))), K[XK_INVI0]);
+}
 template <int MAXD>
 GV_X_FN GvX gv_dy_nlo_x(const unsigned long long (&x)[MAXD], int d, const GvX* K) {
   GvX g = gv_drell_yan_x<false>(x, K, nullptr);
-#ifdef __CUDA_ARCH__
-#pragma unroll 1
-#endif
-  for (int a = 4; a < MAXD; ++a) {
-    if (a < d) {
-      const GvX f = x_exp2(x_mul(K[XK_BETA2], x_from_q62(x_cos_turn(x[a]))));
-      g = x_mul(g, x_mul(f, K[XK_INVI0]));
-    }
-  }
+  for (int a = 4; a < d; ++a) g = x_mul(g, gv_nlo_factor_x(x[a], K));
   return g;
 }
 
