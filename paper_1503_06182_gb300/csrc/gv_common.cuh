@@ -26,7 +26,7 @@
 // in the FP64 form) to a row of 22-bit limbs at absolute positions
 // (gv_limbs.cuh) and publishes a bin's sum as at least 66 bits with its own
 // exponent code; the iteration's sum aligns the tiles' to the bin's largest
-// code with 32 more bits.  Both truncations depend on the data alone, so the
+// code with 20 more bits.  Both truncations depend on the data alone, so the
 // bin sums stay launch-shape independent.
 #pragma once
 #include <cstdint>
@@ -45,7 +45,7 @@
 #define GV_MAXPARAMS 16
 #define GV_BINE_OFF 1200      // stored bin exponent F + GV_BINE_OFF (0: no nonzero weight)
 #define GV_BIN_QBITS 56       // bits of one w^2 below its bin's scale in a tile
-#define GV_BIN_XBITS 32       // extra low bits of the iteration's bin sums
+#define GV_BIN_XBITS 20       // extra low bits of the iteration's bin sums
 #define GV_BIN_FB (GV_BIN_QBITS + GV_BIN_XBITS)  // bin sums in units of 2^(2F - GV_BIN_FB)
 #define GV_HIST_MAX 1000      // histogram bins of the observable (plus underflow and overflow)
 
