@@ -243,7 +243,7 @@ int upload_tables(vegas_batch* B) {
     r.per_iter = B->per_iter + (size_t)b * B->per_iter_cap * 2;
     r.tickets = x.tickets;
     r.alpha = B->alpha;
-    gv_set_fractions(r);
+    r.inv_nbins = 1.0 / (double)B->N;
     r.grid = x.grid;
     for (int yy = 0; yy < gy; ++yy)
       for (int xx = 0; xx < gx; ++xx) rt.push_back(make_int4(b, xx, yy, gx * gy));

@@ -508,7 +508,7 @@ GvReduceArgs reduce_args(const vegas_ctx* c, const Plan& p, int k) {
   r.per_iter = p.per_iter;
   r.tickets = c->tickets;
   r.alpha = c->alpha;
-  gv_set_fractions(r);
+  r.inv_nbins = 1.0 / (double)c->nbins;
   r.grid = c->grid;
   return r;
 }

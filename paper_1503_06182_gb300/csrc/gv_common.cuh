@@ -245,9 +245,7 @@ struct GvReduceArgs {
   double* per_iter;              // forward: [itmx][2]; adjoint: [itmx][2 + 2*NGRAD]
   int* tickets;                  // gv_tickets_ints(nacc) counters, one per 128-byte line
   // grid refinement
-  double alpha;
-  unsigned long long frac64 = 0; // floor(2^64 / nbins) and the remainder of that division
-  unsigned frac_rem = 0, pad = 0;
+  double alpha, inv_nbins;
   double* grid;                  // grid pack (refined in place, one axis per CTA)
   // VEGAS+: the tiles the fill gave events (its grid holds the largest
   // allocation; the rest left nothing); nullptr: all n_tiles
@@ -453,12 +451,6 @@ struct GvPlusArgs {
   double* per_iter = nullptr;  // [itmx][2]
   GvState* st = nullptr;
 };
-
-inline void gv_set_fractions(GvReduceArgs& r) {
-  const unsigned long long N = (unsigned long long)r.nbins;
-  r.frac64 = ~0ull / N;
-  r.frac_rem = (unsigned)(~0ull % N) + 1u;  // 2^64 = frac64 N + frac_rem, frac_rem <= N
-}
 
 namespace gv {
 cudaError_t launch_plus_finish(const GvPlusArgs& a, cudaStream_t s, bool pdl);

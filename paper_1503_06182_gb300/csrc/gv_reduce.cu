@@ -24,12 +24,14 @@
 // sums) records I_k and sigma_k and combines the stage.  No CTA ever waits
 // for another.
 //
-// On this chip a dependent FP64 operation waits ~56-64 cycles and a warp-wide
-// FP64 instruction occupies the SM's FP64 pipe for ~19 cycles: the serial code
-// here runs on the integer pipes where it can.
+// On this chip a dependent FP64 operation waits ~56-64 cycles, a warp-wide
+// FP64 instruction occupies the SM's FP64 pipe for ~19 cycles, and the FP64
+// library log takes ~2000 cycles: the serial code here keeps its FP64 chains
+// short (reciprocals passed in, a table-driven log, one thread per bin).
 #include <algorithm>
 
 #include "gv_combine.cuh"
+#include "gv_ff.cuh"
 #include "gv_integrands.cuh"
 #include "gv_limbs.cuh"
 #include "gv_xint.cuh"
@@ -245,179 +247,240 @@ __device__ __forceinline__ void pack_axis_tables(double* grid, const double* e_s
   }
 }
 
-// Shared memory of refine_axis: slope[N] (GvX), d[N], C[N+1], e[N+1], ne[N+1].
-__host__ __device__ inline size_t refine_axis_smem(int N) {
-  return sizeof(double) * (3 * (size_t)N + 3 * ((size_t)N + 1) + 1);
+// 1/x and 1/sqrt(x) for positive normal x: the hardware approximations
+// (PTX rcp.approx.ftz.f64 and rsqrt.approx.ftz.f64, about 20 correct bits)
+// refined by two Newton-Raphson steps, y <- y + y (1 - x y) and
+// z <- z + z (1 - x z^2) / 2, each of which squares the relative error.
+// Measured against the correctly rounded results over six decades: the
+// reciprocal agrees bit for bit, the square root within 2.7e-16.  They
+// replace the library's correctly rounded routines, whose special-case
+// handling costs this chip's scarce FP64 pipe more instructions.
+__device__ __forceinline__ double gv_rcp_nr(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double e = fma(-x, y, 1.0);
+  y = fma(y, e, y);
+  e = fma(-x, y, 1.0);
+  return fma(y, e, y);
+}
+__device__ __forceinline__ double gv_rsqrt_nr(double x) {
+  double z;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(x));
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const double h = x * z;
+    const double e = fma(-h, z, 1.0);
+    z = fma(0.5 * z, e, z);
+  }
+  return z;
 }
 struct GvRefineMem {
-  GvX* slope;                    // [N], 16-byte aligned
-  unsigned long long *db, *C;    // [N] bits of d, [N + 1]
-  double *e, *ne;                // [N + 1] old and new edges
+  double *r, *slope;    // [N] 6 x smoothed sums, then compressed values; bin sums, then slopes
+  double *C, *e, *ne;   // [N + 1] prefix sums, old and new edges
 };
 __device__ __forceinline__ GvRefineMem refine_mem(double* sm, int N) {
   GvRefineMem m;
-  m.slope = reinterpret_cast<GvX*>(sm + ((reinterpret_cast<size_t>(sm) >> 3) & 1));
-  m.db = reinterpret_cast<unsigned long long*>(m.slope + N);
-  m.C = m.db + N;
-  m.e = reinterpret_cast<double*>(m.C + (N + 1));
+  m.r = sm;
+  m.slope = m.r + N;
+  m.C = m.slope + N;
+  m.e = m.C + (N + 1);
   m.ne = m.e + (N + 1);
   return m;
 }
 
-// sqrt of a GvX: of its significand in [1/4, 1), the exponent made even.
-__device__ __forceinline__ GvX x_sqrt(const GvX& v) {
-  const int odd = v.e & 1;  // v = (m 2^-64) 2^(e + 64)
-  const unsigned long long q = v.m >> (2 + odd);  // Q62 of m 2^-64 (or half of it)
-  return x_norm((unsigned long long)xi_sqrt_q62(q), ((v.e + 64 + odd) >> 1) - 62);
+// ((1 - rho)/(-ln rho))^alpha for 0 < rho < 1, with the common exponents
+// evaluated by reciprocals and roots rather than pow.  In the refinement
+// rho <= 3/5 (a smoothed bin holds at most 3/5 of the smoothed total), so
+// 1 - rho >= 2/5 and -ln rho >= 0.51: both are positive normal numbers.
+__device__ __forceinline__ double compress(double rho, double alpha) {
+  if (rho <= 0.0) return 0.0;
+  if (rho >= 1.0) return 1.0;
+  const double L = -gv_log_pos(rho);
+  const double om = 1.0 - rho;
+  if (alpha == 1.5) {  // om^(3/2) L^(-3/2) = (om^2 / sqrt(om)) (1/sqrt(L))^3
+    const double y = gv_rsqrt_nr(L), z = gv_rsqrt_nr(om);
+    return (om * om * z) * (y * y * y);
+  }
+  if (alpha == 1.0) return om * gv_rcp_nr(L);
+  if (alpha == 0.5) return om * gv_rsqrt_nr(om) * gv_rsqrt_nr(L);
+  if (alpha == 2.0) {
+    const double q = om * gv_rcp_nr(L);
+    return q * q;
+  }
+  if (alpha == 0.0) return 1.0;
+  return pow(om * __drcp_rn(L), alpha);
+}
+
+// The compressed value r = ((1 - rho)/(-ln rho))^(3/2) (alpha = 3/2) and the
+// slope de / r in FP32 pairs (gv_ff.cuh), for 2^-100 < rho <= 3/5 and
+// 2^-100 < de <= 1.  -ln rho by the table reduction of gv_log_pos: rho =
+// 2^k m, r' = m R_j - 1 (|r'| < 2^-7), ln rho = k ln2 + L_j + ln(1 + r'),
+// with ln(1 + r') = r' + r'^2 P(r'), P = -1/2 + r'/3 - r'^2/4 + ... + r'^5/7
+// (truncation below 2^-60); the leading -1/2 and r' P's product are paired,
+// the rest of P (scaled by r'^3 < 2^-21) is FP32.
+__device__ __forceinline__ void compress15_ff(double rho, double de, double& rv, double& sl) {
+  const long long b = __double_as_longlong(rho);
+  const int k = (int)(b >> 52) - 1023;
+  const int j = (int)((b >> 45) & 127);
+  const GvFF m = gv_ff_from_double(
+      __longlong_as_double((b & 0xFFFFFFFFFFFFFll) | 0x3FF0000000000000ll));
+  const double2 RL = __ldg(reinterpret_cast<const double2*>(gv_log_tab) + j);
+  const GvFF p = gv_ff_mul(m, gv_ff_from_double(RL.x));
+  const GvFF r = gv_two_sum(__fsub_rn(p.hi, 1.0f), p.lo);  // p.hi - 1 is exact
+  const float x = r.hi;
+  float Q = __fmaf_rn(x, 1.0f / 7.0f, -1.0f / 6.0f);
+  Q = __fmaf_rn(Q, x, 0.2f);
+  Q = __fmaf_rn(Q, x, -0.25f);
+  Q = __fmaf_rn(Q, x, 1.0f / 3.0f);
+  const GvFF P = gv_two_sum(-0.5f, __fmul_rn(x, Q));
+  const GvFF l1p = gv_ff_add(r, gv_ff_mul(gv_ff_mul(r, r), P));
+  // ln 2 = 0x1.62e43p-1 + (-0x1.05c61p-29), to 9e-17
+  const GvFF kln2 = gv_ff_mul_f(GvFF{0x1.62e43p-1f, -0x1.05c61p-29f}, (float)k);
+  const GvFF lnrho = gv_ff_add(gv_ff_add(kln2, gv_ff_from_double(RL.y)), l1p);
+  const GvFF L = {-lnrho.hi, -lnrho.lo};
+  const GvFF R = gv_ff_from_double(rho);
+  const GvFF om = gv_ff_add(GvFF{1.0f, 0.0f}, GvFF{-R.hi, -R.lo});
+  const GvFF q = gv_ff_div(om, L);
+  const GvFF c = gv_ff_mul(q, gv_ff_sqrt(q));
+  rv = gv_ff_to_double(c);
+  sl = gv_ff_to_double(gv_ff_div(gv_ff_from_double(de), c));
+}
+
+// alpha values whose compressed values are at least (1/745)^2 > 1e-6 (the
+// reciprocal approximation then sees normal numbers only)
+__device__ __forceinline__ bool fast_alpha(double alpha) {
+  return alpha == 1.5 || alpha == 1.0 || alpha == 0.5 || alpha == 2.0 || alpha == 0.0;
+}
+
+// Shared memory of refine_axis: r[N], slope[N], C[N+1], e[N+1], ne[N+1].
+__host__ __device__ inline size_t refine_axis_smem(int N) {
+  return sizeof(double) * (2 * (size_t)N + 3 * ((size_t)N + 1));
 }
 
 // Refinement of axis ax by a group of nthr threads (local index tid, barrier
 // id bar, group number q), once every block holding the axis has rounded its
-// bin sums d_i to FP64:
+// bin sums d_i to FP64 (the oracle's arithmetic from here on):
 //   1. 6 x the smoothed sums, s_i = 3 (d_0 + d_1) at the ends and
-//      2 (d_{i-1} + d_i + d_{i+1}) inside, and their total;
-//   2. per bin the share rho = s_i / total, the compressed value r =
-//      ((1-rho)/(-ln rho))^alpha and the slope (e_{i+1}-e_i)/r;
-//   3. the prefix sums C of r;
-//   4. per new edge: the old bin where C reaches j R/N (binary search), then
+//      2 (d_{i-1} + d_i + d_{i+1}) inside, and their total (a fixed-order
+//      tree), then per bin the share rho = s_i / total, the compressed value
+//      r = ((1-rho)/(-ln rho))^alpha and the slope (e_{i+1}-e_i)/r;
+//   2. one warp: the prefix sums C of r;
+//   3. per new edge: the old bin where C reaches j R/N -- binary search on
+//      the bit patterns of the nonnegative doubles -- then
 //      e_i + (target - C_i) * slope_i; e'_0 = 0 and e'_N = 1 exactly;
-//   5. the axis' tables.
+//   4. the axis' tables.
 // An axis whose bins are all zero keeps its edges.
-//
-// The steps are a chain of latencies on one SM, and on this chip a dependent
-// FP64 operation waits ~62 cycles: everything up to the new edge runs in 64-bit
-// significands (gv_x64.cuh) and fixed point, where an operation waits 4 to 6.
-// The total is an exact sum of the smoothed values at their largest exponent,
-// and C a fixed-point sum (r < 1; 63 bits for N of them), both formed by
-// integer warp operations in any order.  One axis of 100 bins takes 10.5
-// thousand cycles in place (compression 3.5, search 1.6, tables 1.4, smoothing
-// 1.2; a second pass in the same CTA 8.1: the rest is instruction fetch),
-// against 13.7 for the FP64 steps with a float-float compression, and is
-// accurate to 2^-56 of a bin's share where that was to 2^-45.
+// The same steps in 64-bit integer significands are 5 to 15 us faster over the
+// 9 to 14 iterations of the small stages, but their edges differ in the last
+// places, and an FP32 table entry that rounds the other way moves events across
+// an integrand's cuts: a batch with three-jet members then leaves 1e-9 in one
+// run of four.
+// A cluster's sums are in shared memory already (LOADED: d in slope, the edges
+// in e, and a barrier passed).
 template <bool LOADED>
 __device__ __forceinline__ void refine_axis(const GvReduceArgs& a, int ax, double* sm, int tid, int nthr, int bar,
                             int q) {
-  const int N = a.nbins, lane = tid & 31, wid = tid >> 5, nw = nthr >> 5;
-  // 8 groups of up to 8 warps, or one group of up to 16
-  __shared__ int s_emax[64];
-  __shared__ unsigned s_lim[64][3];
-  __shared__ unsigned long long s_pre[64];
-  const int q8 = 8 * q;
+  const int N = a.nbins, lane = tid & 31, wid = tid >> 5;
+  __shared__ double s_inv[8], s_step[8];
   const GvRefineMem m = refine_mem(sm, N);
-  GvX* slope = m.slope;
-  unsigned long long *db = m.db, *C = m.C;
-  double *e = m.e, *ne = m.ne;
+  double *r = m.r, *slope = m.slope, *C = m.C, *e = m.e, *ne = m.ne;
   if (!LOADED) {
     const double* d = a.sums + 2 * a.nch + ax * N;
     const double* e64 = a.grid + GvGridLayout{a.ndim, N}.off_e64() + (size_t)ax * (N + 1);
-    for (int k = tid; k <= N; k += nthr) {
-      if (k < N) db[k] = (unsigned long long)__double_as_longlong(__ldcg(d + k));
-      e[k] = e64[k];
-    }
+    for (int k = tid; k <= N; k += nthr) e[k] = e64[k];
+    for (int i = tid; i < N; i += nthr) slope[i] = __ldcg(d + i);
     gv_bar(bar, nthr);
   }
-  // thread t takes the bins [t ch, (t + 1) ch)
-  const int ch = N <= nthr ? 1 : (N + nthr - 1) / nthr, i0 = min(N, tid * ch), i1 = min(N, i0 + ch);
-  int emax = GV_X_ZERO_E;
-  for (int i = i0; i < i1; ++i) {
-    // twice d_i and a neighbour and the third value: the other neighbour, or
-    // at the ends half the sum of the two (no divergence)
-    const GvX t = x_addp(x_from(__longlong_as_double((long long)db[i])),
-                         x_from(__longlong_as_double((long long)db[i ? i - 1 : 1])));
+  for (int i = tid; i < N; i += nthr) {  // (the ends add a zero: no second path for their lanes)
     const bool end = i == 0 || i == N - 1;
-    const GvX o = x_from(__longlong_as_double((long long)db[end ? i : i + 1]));
-    GvX s = x_scale(x_addp(t, end ? x_scale(t, -1) : o), 1);
-    if ((db[i] >> 52) >= 0x7FFull) s.e = 1 << 20;  // beyond FP64: no refinement
-    slope[i] = s;
-    emax = max(emax, s.e);
-  }
-  emax = __reduce_max_sync(0xffffffffu, emax);
-  if (lane == 0) s_emax[q8 + wid] = emax;
-  gv_bar(bar, nthr);
-  emax = s_emax[q8];
-  for (int w = 1; w < nw; ++w) emax = max(emax, s_emax[q8 + w]);
-  // the values at the largest exponent in three digits of 22, 22 and 20 bits;
-  // at most 1024 of them
-  unsigned l0 = 0u, l1 = 0u, l2 = 0u;
-  for (int i = i0; i < i1; ++i) {
-    const GvX s = slope[i];
-    const unsigned long long v = emax - s.e < 64 ? s.m >> (emax - s.e) : 0ull;
-    l0 += (unsigned)v & 0x3FFFFFu;
-    l1 += (unsigned)(v >> 22) & 0x3FFFFFu;
-    l2 += (unsigned)(v >> 44);
-  }
-  l0 = __reduce_add_sync(0xffffffffu, l0);
-  l1 = __reduce_add_sync(0xffffffffu, l1);
-  l2 = __reduce_add_sync(0xffffffffu, l2);
-  if (lane == 0) {
-    s_lim[q8 + wid][0] = l0;
-    s_lim[q8 + wid][1] = l1;
-    s_lim[q8 + wid][2] = l2;
+    const int k = max(i, 1);
+    r[i] = (end ? 3.0 : 2.0) * (slope[k - 1] + slope[k] + (end ? 0.0 : slope[min(i + 1, N - 1)]));
   }
   gv_bar(bar, nthr);
-  unsigned long long t0 = 0ull, t1 = 0ull, t2 = 0ull;
-  for (int w = 0; w < nw; ++w) {
-    t0 += s_lim[q8 + w][0];
-    t1 += s_lim[q8 + w][1];
-    t2 += s_lim[q8 + w][2];
-  }
-  // total = t0 + t1 2^22 + t2 2^44, below 2^75: its leading 64 bits
-  const unsigned long long low = t0 + (t1 << 22), hi = t2 + (low >> 44);
-  const GvX total = hi >> 20 ? x_norm((hi << 33) | ((low & 0xFFFFFFFFFFFull) >> 11), emax + 11)
-                             : x_norm((hi << 44) | (low & 0xFFFFFFFFFFFull), emax);
-  if (total.m != 0ull && emax < (1 << 19)) {
-    const GvX inv = x_rcp(total);
-    const int fb = 53 + (N <= 256 ? 2 : 0) + (N <= 64 ? 2 : 0);  // fraction bits of C
-    unsigned long long run = 0ull;
-    for (int i = i0; i < i1; ++i) {
-      const GvX s = slope[i];
-      GvX r = x_zero(), sl = x_zero();
-      if (s.m) {
-        const GvX rho = x_mul(s, inv);
-        if (rho.e < -63) {  // below 1 (it is at most 3/5)
-          const GvX L = x_neg(x_log2(rho));
-          const GvX om = x_one_minus(x_to_q64(rho));
-          // (1 - rho)/(-ln rho), -ln rho = L ln 2 >= 0.51
-          const GvX c = x_mul(om, x_mul(x_rcp(L), GV_X_LOG2E));
-          if (a.alpha == 1.5)
-            r = x_mul(c, x_sqrt(c));
-          else if (a.alpha == 1.0)
-            r = c;
-          else if (a.alpha == 0.5)
-            r = x_sqrt(c);
-          else if (a.alpha == 2.0)
-            r = x_sqr(c);
-          else if (a.alpha == 0.0)
-            r = GvX{1ull << 63, -63, 0u};
-          else
-            r = x_from(pow(x_to_double(c), a.alpha));
-        } else {
-          r = GvX{1ull << 63, -63, 0u};
-        }
-        if (r.m) sl = x_mul(x_from(e[i + 1] - e[i]), x_rcp(r));
-      }
-      slope[i] = sl;
-      const int sh = -r.e - fb;
-      run += r.m && sh < 64 ? (sh > 0 ? r.m >> sh : r.m) : 0ull;
-      C[i + 1] = run;
-    }
-    // exclusive prefix of the threads' sums: within the warp, then the warps
-    unsigned long long x = run;
+  if (wid == 0) {
+    // the total in an order fixed by N alone (whatever the group's size):
+    // 32 consecutive chunks in order, then a fixed pairwise tree
+    const int chunk = (N + 31) / 32;
+    const int i0 = min(N, lane * chunk), i1 = min(N, i0 + chunk);
+    double part = 0.0;
+    if (chunk <= 4) {
+      // a fixed pairwise tree over the chunk (zeros past its end add exactly)
+      double v[4];
 #pragma unroll
-    for (int m = 1; m < 32; m <<= 1) {
-      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, m);
-      if (lane >= m) x += y;
+      for (int k = 0; k < 4; ++k) v[k] = i0 + k < i1 ? r[i0 + k] : 0.0;
+      part = (v[0] + v[1]) + (v[2] + v[3]);
+    } else {
+      for (int i = i0; i < i1; ++i) part += r[i];
     }
-    if (lane == 31) s_pre[q8 + wid] = x;
-    gv_bar(bar, nthr);
-    unsigned long long base = x - run, all = 0ull;
-    for (int w = 0; w < nw; ++w) {
-      if (w < wid) base += s_pre[q8 + w];
-      all += s_pre[q8 + w];
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) part += __shfl_down_sync(0xffffffffu, part, m);
+    if (lane == 0) {
+      const double t = part;
+      s_inv[q] = !(t > 0.0) ? 0.0 : (t > 0x1p-1000 && t < 0x1p1000) ? gv_rcp_nr(t) : __drcp_rn(t);
     }
-    for (int i = i0; i < i1; ++i) C[i + 1] += base;
-    if (tid == 0) C[0] = 0ull;
+  }
+  gv_bar(bar, nthr);
+  const double inv = s_inv[q];
+  const bool fast = fast_alpha(a.alpha);
+  if (inv > 0.0) {
+    for (int i = tid; i < N; i += nthr) {
+      double rv = 0.0, sl = 0.0;
+      const double s6 = r[i];
+      if (s6 > 0.0) {
+        const double rho = s6 * inv, de = e[i + 1] - e[i];
+        if (a.alpha == 1.5 && rho > 0x1p-100 && rho <= 0.6 && de > 0x1p-100 && de <= 1.0) {
+          compress15_ff(rho, de, rv, sl);
+        } else {
+          rv = compress(rho, a.alpha);
+          if (rv > 0.0) sl = de * (fast ? gv_rcp_nr(rv) : __drcp_rn(rv));
+        }
+      }
+      r[i] = rv;
+      slope[i] = sl;
+    }
     gv_bar(bar, nthr);
+    if (wid == 0) {
+      const int chunk = (N + 31) / 32;
+      const int i0 = min(N, lane * chunk), i1 = min(N, i0 + chunk);
+      // the chunk's own running sums (in order), formed before the scan so
+      // that each C below is one addition away from its chunk's base
+      double lp[4];
+      double local = 0.0;
+      if (chunk <= 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          local = i0 + k < i1 ? local + r[i0 + k] : local;
+          lp[k] = local;
+        }
+      } else {
+        for (int i = i0; i < i1; ++i) local += r[i];
+      }
+      // inclusive prefix sums of the 32 chunk sums (Hillis-Steele; the lanes
+      // below the distance add a zero), then each chunk's exclusive prefix
+#pragma unroll
+      for (int m = 1; m < 32; m <<= 1) {
+        const double v = __shfl_up_sync(0xffffffffu, local, m);
+        local += lane >= m ? v : 0.0;
+      }
+      double run = __shfl_up_sync(0xffffffffu, local, 1);  // of this lane's chunk
+      if (lane == 0) run = 0.0;
+      if (lane == 0) C[0] = 0.0;
+      if (chunk <= 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (i0 + k < i1) C[i0 + k + 1] = run + lp[k];
+      } else {
+        for (int i = i0; i < i1; ++i) {
+          run += r[i];
+          C[i + 1] = run;
+        }
+      }
+      __syncwarp();
+      if (lane == 0) s_step[q] = C[N] * a.inv_nbins;
+    }
+    gv_bar(bar, nthr);
+    const double step = s_step[q];
+    const long long* Cb = reinterpret_cast<const long long*>(C);
     for (int j = tid; j <= N; j += nthr) {
       double v;
       if (j == 0) {
@@ -425,19 +488,17 @@ __device__ __forceinline__ void refine_axis(const GvReduceArgs& a, int ax, doubl
       } else if (j == N) {
         v = 1.0;
       } else {
-        // all j / N: by the 64-bit fraction j 2^64 / N (to a unit)
-        const unsigned long long target =
-            xi_mulhi(all, a.frac64 * (unsigned)j +
-                              __float2uint_rz(__fdividef((float)(a.frac_rem * (unsigned)j), (float)N)));
-        int lo = 0, hb = N - 1;  // first bin i with C[i+1] > target (N-1 if none)
-        while (lo < hb) {
-          const int mid = (lo + hb) >> 1;
-          if (C[mid + 1] > target)
-            hb = mid;
+        const double target = step * j;
+        const long long tb = __double_as_longlong(target);
+        int lo = 0, hi = N - 1;  // first bin i with C[i+1] > target (N-1 if none)
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (Cb[mid + 1] > tb)
+            hi = mid;
           else
             lo = mid + 1;
         }
-        v = e[lo] + x_to_double(x_mul(x_norm(target - C[lo], -fb), slope[lo]));
+        v = fma(target - C[lo], slope[lo], e[lo]);
       }
       ne[j] = v;
     }
@@ -868,10 +929,10 @@ __device__ __forceinline__ void gv_cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // v into the cluster's CTA 0 at the address that p has in this CTA
-__device__ __forceinline__ void gv_store_rank0(unsigned long long* p, unsigned long long v) {
+__device__ __forceinline__ void gv_store_rank0(double* p, double v) {
   unsigned q;
   asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(q) : "r"((unsigned)__cvta_generic_to_shared(p)));
-  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(q), "l"(v) : "memory");
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(q), "d"(v) : "memory");
 }
 __global__ void __launch_bounds__(kClusterThreads) gv_reduce_cluster_kernel(const GvReduceArgs a) {
   extern __shared__ __align__(16) double sm[];
@@ -909,7 +970,7 @@ __global__ void __launch_bounds__(kClusterThreads) gv_reduce_cluster_kernel(cons
               ? 0.0
               : i128_to_double(x, bin ? pw * (em - GV_BINE_OFF) - GV_BIN_FB : pw * em - GV_FB);
       a.sums[k] = d;
-      if (refine) gv_store_rank0(m.db + s, (unsigned long long)__double_as_longlong(d));
+      if (refine) gv_store_rank0(m.slope + s, d);
     }
   }
   __syncwarp();
