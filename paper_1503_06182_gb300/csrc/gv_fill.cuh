@@ -71,7 +71,8 @@ struct GvTraits<GV_DYNLO> {
 };
 static_assert(XK_N <= GV_NCONST_X, "room for the GvX constants");
 
-// The GvX constants stay in (shared) memory: too many for registers.
+// The GvX constants stay in (shared) memory: too many for registers.  1 / I0
+// of the NLO-shaped integrand is there to the power of its further axes.
 template <int NC>
 struct GvConst<GvX, NC> {
   const GvX* k;
@@ -79,6 +80,11 @@ struct GvConst<GvX, NC> {
 };
 __device__ __forceinline__ const GvX* gv_x_consts(const double* kconst) {
   return reinterpret_cast<const GvX*>(kconst + GV_NCONST);
+}
+template <int IG>
+__device__ __forceinline__ GvX gv_x_const(const double* kconst, int i, int d) {
+  const GvX c = gv_x_consts(kconst)[i];
+  return IG == GV_DYNLO && i == XK_INVI0 ? gv_nlo_norm_x(c, d - 4) : c;
 }
 
 // An integrand taken axis by axis: the variables that its formula needs at the
@@ -96,7 +102,8 @@ struct GvStream {
   static constexpr bool X64 = GvForm<Real>::ID == GV_FORM_X64;
   Coord x[IG == GV_EE3J ? 5 : 4];
   Real f = Real();        // Gauss: the sum of squares; NLO-shaped: the factors' product
-  [[maybe_unused]] GvSumX q;  // Gauss, 64-bit significands: the sum of squares
+  // 64-bit significands: Gauss: the sum of squares; NLO-shaped: of the cosines
+  [[maybe_unused]] std::conditional_t<IG == GV_DYNLO, GvSumCos, GvSumX> q;
 
   __device__ __forceinline__ void first(int k, const Coord& v, const Const& K) {
     x[k] = v;
@@ -108,15 +115,12 @@ struct GvStream {
     } else if constexpr (IG == GV_EE3J) {
       if (a == 4) x[4] = v;
     } else if constexpr (IG == GV_DYNLO) {
-      Real t;
-      if constexpr (X64)
-        t = gv_nlo_factor_x(v, K.k);
-      else
-        t = gv_nlo_factor<Real>(v, K);
-      if constexpr (X64)
-        f = a == 4 ? t : x_mul(f, t);
-      else
+      if constexpr (X64) {
+        q.add(v);
+      } else {
+        const Real t = gv_nlo_factor<Real>(v, K);
         f = a == 4 ? t : f * t;
+      }
     }
   }
   __device__ __forceinline__ void square(const Coord& v) {
@@ -134,7 +138,7 @@ struct GvStream {
       if constexpr (IG == GV_EE3J) return gv_ee3j_x(x, K.k);
       if constexpr (IG == GV_DYNLO) {
         const GvX g = gv_drell_yan_x<false>(x, K.k, nullptr);
-        return d > 4 ? x_mul(g, f) : g;
+        return d > 4 ? gv_nlo_x(g, q, K[XK_INVI0], K.k) : g;
       }
     } else {
       if constexpr (IG == GV_GAUSS)
@@ -727,7 +731,7 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
     if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
       constexpr int NX = GvTraits<IG>::NX;
       __shared__ GvX s_k[NX];
-      if (tid < NX) s_k[tid] = gv_x_consts(a.kconst)[tid];
+      if (tid < NX) s_k[tid] = gv_x_const<IG>(a.kconst, tid, d);
       __syncthreads();
       K.k = s_k;
     } else {
@@ -761,16 +765,39 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
           if (s_binh) s_binh[ax * T + slot] = (unsigned char)(bin >> 8);
         }
       };
-      const auto axes4 = [&](const uint32_t* r) {  // axes 0..3
+      // four coordinates before the first is used or its bin stored: their loads
+      // and products overlap (ten iterations of 1e6 Drell-Yan events 429 -> 417
+      // us in FP32, 1249 -> 1207 in FP64; the Gaussian and three jets, whose
+      // axes do less, gain nothing)
+      const auto map4 = [&](int ax, const uint32_t* r, auto use) {
+        typename GvForm<Real>::Coord v[4];
+        int bin[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (k < d) {
-            int bin;
-            S.first(k, gv_map_axis<Real>(r[k], N, s_jac + k * N, s_ew + k * N, k == 0, J, bin), K);
-            if constexpr (REG)
-              (k < 2 ? bins.x : bins.y) |= (unsigned)bin << (10 * (k & 1));
-            else
-              put_bin(k, bin);
+        for (int k = 0; k < 4; ++k)
+          v[k] = gv_map_axis<Real>(r[k], N, s_jac + (ax + k) * N, s_ew + (ax + k) * N,
+                                   ax + k == 0, J, bin[k]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) use(k, v[k], bin[k]);
+      };
+      const auto first = [&](int k, const auto& v, int bin) {
+        S.first(k, v, K);
+        if constexpr (REG)
+          (k < 2 ? bins.x : bins.y) |= (unsigned)bin << (10 * (k & 1));
+        else
+          put_bin(k, bin);
+      };
+      const auto axes4 = [&](const uint32_t* r) {  // axes 0..3
+        if constexpr (IG == GV_DY || IG == GV_DYNLO) {
+          map4(0, r, first);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (IG != GV_GAUSS || k < d) {  // (the others have four or more)
+              int bin;
+              const auto v =
+                  gv_map_axis<Real>(r[k], N, s_jac + k * N, s_ew + k * N, k == 0, J, bin);
+              first(k, v, bin);
+            }
           }
         }
       };
@@ -830,9 +857,16 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
 #pragma unroll 1
           for (int j = 1; 4 * j < d; ++j) {
             block(j, r);
+            if ((IG == GV_DY || IG == GV_DYNLO) && 4 * j + 4 <= d) {
+              map4(4 * j, r, [&](int k, const auto& v, int bin) {
+                S.more(4 * j + k, v, K);
+                put_bin(4 * j + k, bin);
+              });
+            } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-              if (4 * j + k < d) axis(4 * j + k, r[k]);
+              for (int k = 0; k < 4; ++k)
+                if (4 * j + k < d) axis(4 * j + k, r[k]);
+            }
           }
         }
       }
@@ -1161,18 +1195,23 @@ __global__ void gv_eval_events_kernel(const GvFillArgs a, uint32_t it, const lon
                                       long long n, double* w, int* bins) {
   constexpr int MAXD = GV_MAXD;
   const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
   const int d = a.ndim, N = a.nbins;
+  GvConst<Real, GvTraits<IG>::NK> K;
+  if constexpr (GvForm<Real>::ID == GV_FORM_X64) {
+    __shared__ GvX s_k[GvTraits<IG>::NX];
+    if (threadIdx.x < GvTraits<IG>::NX)
+      s_k[threadIdx.x] = gv_x_const<IG>(a.kconst, (int)threadIdx.x, d);
+    __syncthreads();
+    K.k = s_k;
+  } else {
+    K.load(a.kconst);
+  }
+  if (j >= n) return;
   const GvGridLayout L{d, N};
   const double* e64 = a.grid + L.off_e64();
   const double* wd64 = a.grid + L.off_wd64();
   const double* jac = a.grid + L.off_jac();
   const GvBin32* b32 = reinterpret_cast<const GvBin32*>(a.grid + L.off_bin32());
-  GvConst<Real, GvTraits<IG>::NK> K;
-  if constexpr (GvForm<Real>::ID == GV_FORM_X64)
-    K.k = gv_x_consts(a.kconst);
-  else
-    K.load(a.kconst);
   uint32_t r[MAXD];
   gv_event_words<MAXD>(a.seed, it, a.batch, (unsigned long long)events[j], d, r);
   GvStream<IG, Real> S;

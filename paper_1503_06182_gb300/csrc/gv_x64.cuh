@@ -466,7 +466,21 @@ GV_X_FN GvTurn xi_turn(unsigned long long p) {
 }
 GV_X_FN long long x_cos_turn(unsigned long long p) {
   const GvTurn t = xi_turn(p);
-  const long long v = (t.quadrant & 1u) ? xi_sin_quarter(t.u, t.z) : xi_cos_quarter(t.z);
+  // both polynomials have one shape: the coefficients are selected, so that
+  // the lanes of a warp do not take two paths
+  const bool odd = (t.quadrant & 1u) != 0u;
+  const unsigned z32 = (unsigned)(t.z >> 32);
+  unsigned q = (odd ? 0x5beb7u : 0x48319u) - xi_mulhi32(z32, odd ? 0xd57u : 0x950u);
+  q = (odd ? 0x1e8f435u : 0x1b6e24fu) - xi_mulhi32(z32, q);
+  q = (odd ? 0x78c1d3f8u : 0x7e74e28eu) - xi_mulhi32(z32, q);
+  unsigned long long p4 = (odd ? 0x0002a0f0690fdcf0ull : 0x000069b47ca8812aull) -
+                          xi_mulhi(t.z, (unsigned long long)q << (odd ? 13 : 10));
+  p4 = (odd ? 0x004cb4b3398af616ull : 0x000f0fa83448dd5dull) - xi_mulhi(t.z, p4);
+  p4 = (odd ? 0x0519af19dd6ab874ull : 0x0155d3c7e3cbff9full) - xi_mulhi(t.z, p4);
+  p4 = (odd ? 0x295779cc4b7ca57dull : 0x103c1f081b5ac3b3ull) - xi_mulhi(t.z, p4);
+  p4 = (odd ? 0x6487ed5110b4611aull : 0x4ef4f326f9177969ull) - xi_mulhi(t.z, p4);
+  p4 = xi_mulhi(odd ? t.u : t.z, p4);
+  const long long v = (long long)(odd ? p4 : 0x4000000000000000ull - p4);
   // quadrant 0: cos, 1: -sin d, 2: -cos, 3: sin d
   const bool neg = t.quadrant == 0u   ? false
                    : t.quadrant == 1u ? !t.neg

@@ -153,16 +153,45 @@ GV_X_FN GvX gv_drell_yan_x(const unsigned long long* x, const GvX* K, GvX* grad)
 }
 
 // ---------------------------------------------------------------------------
-// NLO-shaped stand-in: Drell-Yan times exp(beta cos 2 pi x_k) / I0(beta).
+// NLO-shaped stand-in: Drell-Yan times exp(beta cos 2 pi x_k) / I0(beta) for
+// each further axis.  The cosines are summed exactly (Q62, as 16 hi + lo), so
+// that an event takes one exponential instead of one per axis.
 // ---------------------------------------------------------------------------
-GV_X_FN GvX gv_nlo_factor_x(unsigned long long x, const GvX* K) {
-  return x_mul(x_exp2(x_mul(K[XK_BETA2], x_from_q62(x_cos_turn(x)))), K[XK_INVI0]);
+struct GvSumCos {
+  long long hi = 0;
+  unsigned lo = 0u;
+  GV_X_FN void add(unsigned long long x) {
+    const long long v = x_cos_turn(x);
+    hi += v >> 4;
+    lo += (unsigned)v & 15u;
+  }
+  GV_X_FN GvX value() const {  // |sum| <= 12: below 2^62 in hi
+    long long h = hi + (long long)(lo >> 4);
+    unsigned l = lo & 15u;
+    const unsigned s = h < 0 ? 1u : 0u;
+    if (s) {
+      h = -h - (l ? 1 : 0);
+      l = (16u - l) & 15u;
+    }
+    const unsigned long long m = (unsigned long long)h;
+    return m >> 60 ? x_norm((m << 2) | (l >> 2), -60, s) : x_norm((m << 4) | l, -62, s);
+  }
+};
+// 1 / I0(beta)^n
+GV_X_FN GvX gv_nlo_norm_x(const GvX& inv, int n) {
+  GvX r = {1ull << 63, -63, 0u};
+  for (int k = 0; k < n; ++k) r = x_mul(r, inv);
+  return r;
+}
+GV_X_FN GvX gv_nlo_x(const GvX& dy, const GvSumCos& c, const GvX& norm, const GvX* K) {
+  return x_mul(x_mul(dy, norm), x_exp2(x_mul(K[XK_BETA2], c.value())));
 }
 template <int MAXD>
 GV_X_FN GvX gv_dy_nlo_x(const unsigned long long (&x)[MAXD], int d, const GvX* K) {
-  GvX g = gv_drell_yan_x<false>(x, K, nullptr);
-  for (int a = 4; a < d; ++a) g = x_mul(g, gv_nlo_factor_x(x[a], K));
-  return g;
+  const GvX g = gv_drell_yan_x<false>(x, K, nullptr);
+  GvSumCos c;
+  for (int a = 4; a < d; ++a) c.add(x[a]);
+  return gv_nlo_x(g, c, gv_nlo_norm_x(K[XK_INVI0], d - 4), K);
 }
 
 // ---------------------------------------------------------------------------
@@ -179,8 +208,9 @@ GV_X_FN GvX gv_ee3j_x(const unsigned long long* x, const GvX* K) {
   // cos of the angle between 1 and 2: 1 - 2 (1 - x3) / (x1 x2)
   const GvX q = x_mul(x_from_q64(s), x_rcp(x_norm(xi_mulhi(x1, x2), -64)));
   const int sh = -63 - q.e;  // 2 q in Q62
-  const long long q2 = sh <= 0 ? 2 * one : (sh < 64 ? (long long)(q.m >> sh) : 0ll);
-  const long long c12 = one - (q2 > 2 * one - 1 ? 2 * one - 1 : q2);
+  const unsigned long long q2 = sh <= 0 ? ~0ull : (sh < 64 ? q.m >> sh : 0ull);
+  const unsigned long long two = ~0ull >> 1;  // 2 less a unit
+  const long long c12 = one - (long long)(q2 > two ? two : q2);
   const long long v12 = one - xi_mulq62(c12, c12);
   const long long s12 = xi_sqrt_q62(v12 > 0 ? (unsigned long long)v12 : 0ull);
   // event plane: p1 along z, p2 in the x-z plane, p3 balances
