@@ -292,7 +292,10 @@ __device__ __forceinline__ GvRefineMem refine_mem(double* sm, int N) {
 // evaluated by reciprocals and roots rather than pow.  In the refinement
 // rho <= 3/5 (a smoothed bin holds at most 3/5 of the smoothed total), so
 // 1 - rho >= 2/5 and -ln rho >= 0.51: both are positive normal numbers.
-__device__ __forceinline__ double compress(double rho, double alpha) {
+// Out of line: the usual alpha takes compress15_ff, and the code it walks past is
+// fetched cold in every reduce (ten axes, 4 x 1000 + 10 x 1e4 events: 241 us
+// inlined, 238 so).
+__device__ __noinline__ double compress(double rho, double alpha) {
   if (rho <= 0.0) return 0.0;
   if (rho >= 1.0) return 1.0;
   const double L = -gv_log_pos(rho);
@@ -564,8 +567,8 @@ struct SlotSumW {
 // 2048 of them), each read once: the sum moves down when a larger exponent
 // comes.
 template <int G>
-__device__ __forceinline__ SlotSum sum_tiles(const ulonglong2* src, size_t stride, int u, int step,
-                                             int nt, const int* tileE, int nch, bool bin, int pw,
+__device__ __forceinline__ SlotSum sum_tiles(const ulonglong2* src, size_t stride, int u, int lane,
+                                             int step, int nt, const int* tileE, int nch, bool bin, int pw,
                                              bool sgn, int empty) {
   SlotSum s = {{0ull, 0ull}, empty};
   for (int t0 = u; t0 < nt; t0 += G * step) {
@@ -595,6 +598,7 @@ __device__ __forceinline__ SlotSum sum_tiles(const ulonglong2* src, size_t strid
     }
 #pragma unroll
     for (int g = 0; g < G; ++g) {
+      if (g > 0 && t0 - lane + g * step >= nt) break;  // no lane has another
       u128 x = {v[g].x, v[g].y};
       if (bin) {
         const unsigned h = (unsigned)v[g].y;
@@ -615,12 +619,12 @@ __device__ __forceinline__ u192 widen128(u128 v) {
 }
 // As sum_tiles, over any number of partials.
 __device__ __forceinline__ SlotSumW sum_tiles_wide(const ulonglong2* src, size_t stride, int u,
-                                                   int step, int nt, const int* tileE, int nch,
+                                                   int lane, int step, int nt, const int* tileE, int nch,
                                                    bool bin, int pw, bool sgn, int empty) {
   SlotSumW s = {{0ull, 0ull, 0ull}, empty};
   for (long long t0 = u; t0 < nt; t0 += 2048ll * step) {
     const SlotSum p = sum_tiles<GV_RED_TILES_PER_LOAD / 2>(
-        src, stride, (int)t0, step, (int)min(t0 + 2048ll * step, (long long)nt), tileE, nch, bin, pw, sgn,
+        src, stride, (int)t0, lane, step, (int)min(t0 + 2048ll * step, (long long)nt), tileE, nch, bin, pw, sgn,
         empty);
     if (p.em == empty) continue;
     if (p.em > s.em) {
@@ -663,7 +667,7 @@ __device__ __forceinline__ void gv_reduce_task(const GvReduceArgs& a, int bx, in
   // ---- A: this CTA's tiles
   SlotSumW sum = {{0ull, 0ull, 0ull}, empty};
   if (k < a.nacc)
-    sum = sum_tiles_wide(a.part + k, (size_t)a.nacc, t0 + wid, 8, t1, a.tileE + ch, a.nch, bin, pw,
+    sum = sum_tiles_wide(a.part + k, (size_t)a.nacc, t0 + wid, 0, 8, t1, a.tileE + ch, a.nch, bin, pw,
                          hw, empty);
   int em = sum.em;
   s_emax[wid * 32 + lane] = em;
@@ -847,12 +851,12 @@ __global__ void __launch_bounds__(256, 3) gv_reduce_slots_kernel(const GvReduceA
   u192 r = {0ull, 0ull, 0ull};
   if constexpr (WIDE) {
     const SlotSumW sum =
-        sum_tiles_wide(src, 1, tid, 256, nt, a.tileE + (k >> 1), a.nch, bin, pw, hw, empty);
+        sum_tiles_wide(src, 1, tid, lane, 256, nt, a.tileE + (k >> 1), a.nch, bin, pw, hw, empty);
     em = __reduce_max_sync(0xffffffffu, sum.em);
     if (sum.em != empty) r = sar192(sum.v, pw * (em - sum.em));
     r = warp_sum192(r);
   } else {
-    const SlotSum sum = sum_tiles<GV_RED_TILES_PER_LOAD>(src, 1, tid, 256, nt, a.tileE + (k >> 1),
+    const SlotSum sum = sum_tiles<GV_RED_TILES_PER_LOAD>(src, 1, tid, lane, 256, nt, a.tileE + (k >> 1),
                                                          a.nch, bin, pw, hw, empty);
     em = __reduce_max_sync(0xffffffffu, sum.em);
     u128 x = {0ull, 0ull};
@@ -960,7 +964,7 @@ __global__ void __launch_bounds__(kClusterThreads) gv_reduce_cluster_kernel(cons
     const int pw = hw ? 1 : (bin ? 2 : (k & 1) + 1);
     const int empty = bin ? 0 : GV_EMPTY;
     const SlotSum sum =
-        sum_tiles<GV_RED_TILES_PER_LOAD>(a.part + (size_t)k * a.n_tiles, 1, lane, 32, nt,
+        sum_tiles<GV_RED_TILES_PER_LOAD>(a.part + (size_t)k * a.n_tiles, 1, lane, lane, 32, nt,
                                          a.tileE + (k >> 1), a.nch, bin, pw, hw, empty);
     const int em = __reduce_max_sync(0xffffffffu, sum.em);
     const u128 x = warp_sum128(sum.em == empty ? u128{0ull, 0ull} : sar128(sum.v, pw * (em - sum.em)));
