@@ -548,8 +548,13 @@ int enqueue_body(vegas_ctx* c, const Plan& p, std::vector<cudaEvent_t>* ev, bool
 // host).  In a stage, the fills of iterations k > 0 make their Philox words
 // while the previous refinement runs, and a shape whose CTAs are all
 // resident at once does that for every tile: single fill launches, timed
-// alone, miss it.  4 is kept unless another candidate is more than 0.5%
-// faster.
+// alone, miss it.  The candidates are 1, 2 and 4: a stage whose tiles are one
+// round of the SMs wants more threads in each (ten iterations of 1e5 calls with
+// 1 and 4: FP32 NLO on 13 axes 178 and 224 us, FP64 Drell-Yan 240 and 268), a
+// larger one fewer (1e6 FP32 Drell-Yan calls 493 and 322 us).  8 leaves 640
+// threads on an SM and is behind in every one of them (325 us there, and 463
+// against 421 after an L2 flush, which the trials do not show; 1e5 FP64
+// Drell-Yan 344).  4 is kept unless another is more than 0.5% faster.
 constexpr int kTuneRep = 5;
 int autotune_chained(vegas_ctx* c, Plan& p, const std::string& key) {
   const size_t gbytes = grid_doubles(c->ndim, c->nbins) * sizeof(double);
@@ -572,8 +577,7 @@ int autotune_chained(vegas_ctx* c, Plan& p, const std::string& key) {
   int st = VEGAS_OK;
   float best = 1e30f, t4 = 1e30f;
   int best_ept = 4;
-  for (const int ept : {1, 2, 4, 8}) {
-    if (c->ndim > 8 && ept == 8) continue;
+  for (const int ept : {1, 2, 4}) {
     // a shape the device cannot launch (registers, shared memory) is skipped
     if (launch_fill_plan(c, t, ept) != cudaSuccess) {
       cudaGetLastError();

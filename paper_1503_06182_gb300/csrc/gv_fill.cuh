@@ -365,14 +365,14 @@ struct GvFillSmem {
   // a copy's rows, and words to 8 past a multiple of 32: the same row stands in
   // other banks in each copy
   __host__ __device__ unsigned copy_bytes(int nhist, bool f64) const {
-    const unsigned w = (unsigned)(nhist * (L + gv_hist_w_limbs(f64)));
+    const unsigned w = (unsigned)(nhist * (L + gv_hist_w_limbs(f64, L)));
     return 4u * (w + (40u - w % 32u) % 32u);
   }
   __host__ __device__ void place(int d, int N, int form, bool forward, bool bins_smem, int nhist,
                                  bool plus, bool words, int T) {
     const unsigned dN = (unsigned)(d * N);
     const bool f64 = form != GV_FORM_F32;
-    L = gv_limbs(d * N);
+    L = gv_limbs(d * N, nhist == 0 && !plus);
     const unsigned evs = forward ? gv_event_words32(f64, !bins_smem, plus) * T * 4 : 0;
     const unsigned wds = words ? (d + 3) / 4 * 4 * T * 4 : 0;
     wd = 0;
@@ -386,7 +386,7 @@ struct GvFillSmem {
     hs = forward && nhist > 0 ? copy_bytes(nhist, f64) : 0;
     lq = hh + hc * hs;
     lw = lq + (forward ? L * 32 * 4 : 0);
-    const unsigned second = gv_align16(lw + (forward ? gv_lane_rows(f64) * 32 * 4 : 0));
+    const unsigned second = gv_align16(lw + (forward ? gv_lane_rows(f64, L) * 32 * 4 : 0));
     bins = first > second ? first : second;
     po = gv_align16(bins + ((forward && bins_smem) ? d * T * (N > 256 ? 2 : 1) : 0));
     ps = gv_align16(po + (plus ? GV_PLUS_WIN * 4 : 0));
@@ -394,7 +394,7 @@ struct GvFillSmem {
   }
   // bytes of the limbs, from `limbs`
   __host__ __device__ unsigned limb_bytes(bool f64) const {
-    return lw + gv_lane_rows(f64) * 32 * 4 - limbs;
+    return lw + gv_lane_rows(f64, L) * 32 * 4 - limbs;
   }
 };
 
@@ -978,7 +978,7 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
   [[maybe_unused]] int* hw = reinterpret_cast<int*>(smem + lay.hw);            // [hb][HW]
   unsigned* lq = reinterpret_cast<unsigned*>(smem + lay.lq);
   int* lw = reinterpret_cast<int*>(smem + lay.lw);
-  constexpr int HW = gv_hist_w_limbs(F64);
+  [[maybe_unused]] const int HW = gv_hist_w_limbs(F64, L);
   const int lane = tid & 31, wid = tid >> 5;
   const unsigned a_hist = gv_shared_address(hist), a_lq = gv_shared_address(lq + lane),
                  a_lw = gv_shared_address(lw + lane);
@@ -1091,12 +1091,15 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
     if (have_w && wid == 0)
       sum = add128(sum, gv_lane_total<false>(lq, L, 22 * vw.base - 2 * GV_SQ_OFF - 2 * E + GV_FB));
     else if (have_w && wid == 1)
-      sum = add128(sum, gv_lane_total<true>(reinterpret_cast<const unsigned*>(lw), gv_lane_rows(F64),
+      sum = add128(sum, gv_lane_total<true>(reinterpret_cast<const unsigned*>(lw), gv_lane_rows(F64, L),
                                             22 * vw.wbase - GV_SQ_OFF - E + GV_FB));
     ulonglong2* o = out + (size_t)(2 + tid) * ks;
     for (int k = tid; k < dN; k += B, o += (size_t)B * ks) {
       GvPartial v = gv_bin_partial(hist + k * L, L, vq.base);
-      if (!first) v = gv_partial_add(v, gv_load_partial(o));
+      if (!first) {  // few bins have weights below the first window
+        if (v.code == 0) continue;
+        v = gv_partial_add(v, gv_load_partial(o));
+      }
       gv_store_partial(o, v);
     }
     if constexpr (HIST) {
@@ -1104,7 +1107,10 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
       for (int k = tid; k < hb; k += B) {
         ulonglong2* o = out + (2 + dN + k) * ks;
         GvPartial v = gv_bin_partial(hh + k * L, L, vw.base);
-        if (!first) v = gv_partial_add(v, gv_load_partial(o));
+        if (!first) {
+          if (v.code == 0) continue;  // (nor has the bin a sum of w)
+          v = gv_partial_add(v, gv_load_partial(o));
+        }
         gv_store_partial(o, v);
         o = out + (2 + dN + hb + k) * ks;
         v = gv_hist_partial(hw + k * HW, HW, vw.hbase);

@@ -31,14 +31,29 @@
 #define GV_SQ_OFF 1144  // 11 x 104: keeps every limb index positive (h >= -1126)
 #define GV_W21_OFF 1155 // 21 x 55: the histogram's 21-bit digits of w
 
-// Limbs per bin: 9 up to 1024 bins in all; above, fewer, so that the largest
-// shapes still fit shared memory.  Odd, so that consecutive bins start in
-// different banks.
-__host__ __device__ inline int gv_limbs(int dN) { return dN <= 1024 ? 9 : (dN <= 2048 ? 7 : 5); }
+// Limbs per bin: 9 up to 1024 bins in all (weights down to 2^-55 of the tile's
+// largest in one pass); above, fewer, so that the largest shapes still fit
+// shared memory.  Odd, so that consecutive bins start in different banks.  Plain
+// fills of up to 512 bins have 13 (2^-99): on a grid adapted over 40 iterations
+// nearly every tile has an event below 2^-55, and a second pass; ten iterations
+// of 1e6 Drell-Yan events then take 382 us with 9 and 330 with 13, on a fresh
+// grid 314 and 326, and three jets of 1e7 events 2.71 and 2.74 ms.  With a
+// histogram (535 and 562 us) or strata (1033 and 1131) the room is better spent
+// on a fourth CTA per SM.
+__host__ __device__ inline int gv_limbs(int dN, bool plain) {
+  return plain && dN <= 512 ? 13 : (dN <= 1024 ? 9 : (dN <= 2048 ? 7 : 5));
+}
 // Rows of the per-lane columns of w (22-bit digits) and limbs per histogram
-// bin of w (21-bit digits), for the window of 9 limbs.
-__host__ __device__ constexpr int gv_lane_rows(bool f64) { return f64 ? 7 : 5; }
-__host__ __device__ constexpr int gv_hist_w_limbs(bool f64) { return f64 ? 9 : 7; }
+// bin of w (21-bit digits).  The largest weight stands at most 11 (L - 4) + 31
+// bits above the lowest 22-bit digit (+ 30 above a 21-bit one): digit 3 (4) for
+// L <= 9, digit 5 (6) for L = 13; its 24 or 53 bits reach 1 (2) or 3 digits
+// further.
+__host__ __device__ constexpr int gv_lane_rows(bool f64, int L = 9) {
+  return (f64 ? 7 : 5) + (L > 9 ? 2 : 0);
+}
+__host__ __device__ constexpr int gv_hist_w_limbs(bool f64, int L) {
+  return (f64 ? 9 : 7) + (L > 9 ? 2 : 0);
+}
 
 struct u192 {
   unsigned long long l0, l1, l2;
@@ -236,7 +251,9 @@ template <bool SIGNED>
 __device__ __forceinline__ u128 gv_lane_total(const unsigned* col, int rows, int p) {
   const int lane = threadIdx.x & 31;
   long long mine = 0;
-  for (int j = 0; j < rows; ++j) {
+  // a row of unsigned digits adds up to less than 2^32: those below 2^-32 of a
+  // unit are nothing
+  for (int j = SIGNED ? 0 : max(0, (-32 - p) / GV_LIMB_BITS); j < rows; ++j) {
     const unsigned v = col[j * 32 + lane];
     long long s;
     if constexpr (SIGNED)
