@@ -56,7 +56,7 @@ FLOPS_ADJOINT_FP32 = 110 + 72 + 5
 # operations): 83 + 3 x 21 + 25 + 15 + 3 x 15 + grid map 4 x 5 = 251.
 FP64_OPS_PER_EVENT_DY = 83 + 3 * 21 + 25 + 15 + 3 * 15 + 4 * 5
 SM_COUNT, FP32_LANES_PER_SM, SM_MAX_MHZ = 152, 128, 2070.0
-# Per events-per-thread shape of the FP32 Drell-Yan fill (1e6 calls, 977
+# Per events-per-thread shape of the FP32 Drell-Yan fill (1e6 calls, 1042
 # tiles), from one-kernel ncu captures (profiles/fill_drell_yan_fp32_ept*_1e6.md):
 # the DRAM bytes (read + write) of one launch, and its warp instructions
 # (smsp__inst_executed.sum).  The fill is issue-bound, so its instruction rate
@@ -64,12 +64,12 @@ SM_COUNT, FP32_LANES_PER_SM, SM_MAX_MHZ = 152, 128, 2070.0
 # binding roofline.  Valid while the fill's sources are the ones captured
 # (their SHA-256 below) and only for the shape the timed run used; otherwise
 # both are reported as unknown (null).
-FILL_CAPTURES = {4: {"traffic_bytes": 83_456, "warp_instructions": 21_418_973},
-                 8: {"traffic_bytes": 121_600, "warp_instructions": 19_412_189}}
+FILL_CAPTURES = {4: {"traffic_bytes": 36_096, "warp_instructions": 15_493_135},
+                 8: {"traffic_bytes": 36_096, "warp_instructions": 14_138_535}}
 SMSP_PER_SM = 4
 FILL_SOURCES = ("gv_fill.cuh", "gv_fill_inst.cuh", "gv_fill_dy_f32.cu", "gv_integrands.cuh",
-                "gv_common.cuh")
-FILL_SOURCES_SHA256 = "b6e6780f442ab04756baca4c51db64638d12551e4734af9a48e958c1e9bed140"
+                "gv_limbs.cuh", "gv_common.cuh")
+FILL_SOURCES_SHA256 = "d1c8431f6e49a6f234cd53b38c3a2df0f4c5a0eb77f2523a36dd5dc579e8ce36"
 # HBM copy bandwidth measured by the driver on the GB300s (used when
 # MEASURED_PEAKS.json is absent: the profiling recipe's fallback)
 HBM_FALLBACK_GBS = 6800.0

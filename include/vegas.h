@@ -72,8 +72,8 @@ extern "C" {
                                  exact integer sums in both forms */
 #define VEGAS_OPT_ADAPT 2     /* 1 = refine the grid after every iteration (default), 0 = frozen */
 #define VEGAS_OPT_EPT 3       /* events per thread of the fill kernel: 0 = autotuned (trial
-                                 launches per shape; 4 unless another candidate is more than 2%
-                                 faster), or 1, 2, 4, 8 (8 only for ndim <= 8: VEGAS_EINVAL
+                                 launches per shape of 1, 2 and 4; 4 unless another is
+                                 measurably faster), or 1, 2, 4, 8 (8 only for ndim <= 8: VEGAS_EINVAL
                                  above).  Results do not depend on it. */
 #define VEGAS_OPT_NONFINITE 4 /* 0 = return VEGAS_ENONFINITE if any weight is not finite (default),
                                  1 = set such weights to 0 and count them silently */
@@ -310,7 +310,7 @@ int vegas_get_ept(const vegas_ctx* ctx, int* ept);
 
 /* ---- batched integrations (many independent VEGAS runs per launch) ----
  * n integrations of uneven dimension, call count and integrand run as one
- * persistent fill launch per iteration, dimension class (at most 4, 8, 16
+ * persistent fill launch per iteration, dimension class (at most 4, up to 16
  * axes) and integrand over a work list of (integration, tile) items taken
  * largest-first from a device counter, then one reduce and
  * one refine launch serving every integration; the itmx iterations are

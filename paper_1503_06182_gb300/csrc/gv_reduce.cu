@@ -2,16 +2,16 @@
 // optimisation (Section 2.1: the grid optimisation is serial so that it can
 // use the results of all events).
 //
-// gv_reduce_kernel sums the tile partials exactly.  Its grid is (slot blocks
-// of 32) x (tile ranges): each CTA owns 32 slots and a range of tiles; its 8
-// warps stride over the tiles, align every partial to the largest exponent
-// the slot has in the range (channel sums: the tiles' scales; bin sums: the
-// bins' own exponent codes, gv_limbs.cuh)
-// and add in 192-bit integers; the warps' sums are combined in shared memory
-// and published with that exponent.  No sum is formed with atomics.  Integer
-// addition is associative, and the alignment depends only on the data and on
-// the reduce grid, a function of the tile count alone: the totals do not
-// depend on the fill's launch shape or on timing.
+// Forward stages and small adjoint ones: gv_reduce_cluster_kernel and
+// gv_reduce_slots_kernel (below).  gv_reduce_kernel and the batched form: the
+// grid is (slot blocks of 32) x (tile ranges): each CTA owns 32 slots and a
+// range of tiles; its 8 warps stride over the tiles and add the partials at the
+// largest exponent the slot has so far (channel sums: the tiles' scales; bin
+// sums: the bins' own exponent codes, gv_limbs.cuh), in 128-bit integers; the
+// warps' sums are combined in shared memory in 192 bits and published with
+// their exponent.  No sum is formed with atomics.  The order depends on the
+// reduce grid alone, a function of the tile count: the totals do not depend on
+// the fill's launch shape or on timing.
 //
 // Tickets instead of waiting: each CTA publishes its sums and counts itself
 // on its block of 32 slots; the CTA that completes a block combines the

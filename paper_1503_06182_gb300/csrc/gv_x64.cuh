@@ -8,8 +8,9 @@
 // quantity is bounded: 11 bits more than FP64 keeps, in less time.  A weight
 // is rounded once, to FP64, at the end.  One fill of 1e6 Drell-Yan events on 4
 // axes: 350 us on the FP64 pipe (a warp instruction per ~19 cycles per SM, the
-// pipe full), 99 us here (2160 instructions per event, 61% of issue slots);
-// 1e5 events of the NLO-shaped weight on 13 axes: 230 and 50 us.  Weights at
+// pipe full), 95 us here (about 2100 instructions per event);
+// 1e5 events of the NLO-shaped weight on 13 axes: 230 us there, 50 with an
+// exponential per axis and fewer with one per event.  Weights at
 // random points: 2^-54.2 rms from 200-bit values, of which the final rounding
 // alone makes 2^-54.8.
 //
