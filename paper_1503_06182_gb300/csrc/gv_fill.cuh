@@ -515,8 +515,9 @@ __device__ __forceinline__ void gv_plus_strat(const unsigned (&c)[MAXD], int d, 
   }
 }
 
-// A bin's record from its edge and width (e in [0, 1), 0 < w < 1, exact to
-// 2^-64); N w is exact: 53 + 10 bits.
+// A bin's record from its edge and width (e in [0, 1), 0 < w <= 1, exact to
+// 2^-64; a width is 1 where the other bins of the axis are below 2^-53); N w is
+// exact: 53 + 10 bits.
 __device__ __forceinline__ GvBinX gv_bin_x(double e, double w, int N) {
   const GvX E = x_from(e), W = x_from(w);
   const GvX j = x_norm((W.m >> 11) * (unsigned long long)N, W.e + 11);

@@ -281,10 +281,12 @@ GV_X_FN double x_to_double(const GvX& v) {
   const unsigned long long rest = v.m & ((1ull << (sh - 1)) - 1ull);
   return xi_double(sign | (q + ((half && (rest || (q & 1ull))) ? 1ull : 0ull)));
 }
-// a fraction in [0, 1) as GvX; a GvX in [0, 1) as a fraction (truncated)
+// a fraction in [0, 1) as GvX; a GvX in [0, 1] as a fraction (truncated; 1, which
+// a grid's width or an exponential can round to, is the largest fraction)
 GV_X_FN GvX x_from_q64(unsigned long long q) { return x_norm(q, -64); }
 GV_X_FN unsigned long long x_to_q64(const GvX& v) {
   const int sh = -64 - v.e;
+  if (sh < 0) return ~0ull;
   return sh < 64 ? v.m >> sh : 0ull;
 }
 
