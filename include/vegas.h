@@ -116,7 +116,8 @@ int vegas_set_option(vegas_ctx* ctx, int key, double value);
 int vegas_set_stream(vegas_ctx* ctx, void* stream);
 
 /* Device workspace for the per-tile partials and per-iteration records of a
- * call with (ncall, itmx): bytes needed. */
+ * call with (ncall, itmx), and of every call with at most that many of each:
+ * bytes needed. */
 int vegas_workspace_size(const vegas_ctx* ctx, int64_t ncall, int itmx, size_t* bytes);
 
 /* Hand the context a caller-owned DEVICE buffer of `bytes` bytes (256-byte

@@ -227,14 +227,13 @@ void clear_graphs(vegas_ctx* c) {
 
 size_t grid_doubles(int d, int N) { return GvGridLayout{d, N}.doubles(); }
 
-// events: the fill's capacity (ncall, or ncall + 2 nh with VEGAS+); plus_f:
-// room for the per-event J g of VEGAS+
 // chained iterations per autotuning trial (iteration records are sized for them)
 constexpr int kTuneIter = 8;
 
-size_t workspace_bytes(int d, int N, int64_t ncall, int itmx, int mode, int nhist, int T,
-                       bool plus_f = false) {
-  const int64_t n_tiles = (ncall + T - 1) / T;
+// A function that grows with n_tiles and itmx.  plus_f: room for the segments
+// of VEGAS+, whose fill has a capacity of plus_events (ncall + 2 nh).
+size_t workspace_bytes(int d, int N, int64_t n_tiles, int itmx, int mode, int nhist,
+                       bool plus_f = false, int64_t plus_events = 0) {
   const int nch = mode ? GV_MAXCH : 1;
   const int nacc = mode ? 2 * GV_MAXCH : 2 + d * N + 2 * nhist;
   int tpc = 0, gx = 0, gy = 0;
@@ -244,7 +243,9 @@ size_t workspace_bytes(int d, int N, int64_t ncall, int itmx, int mode, int nhis
   b += align256((size_t)std::max(itmx, kTuneIter) * (2 + 2 * GV_NGRAD) * 8);
   b += align256((size_t)gy * gx * 32 * sizeof(GvSlot));
   // VEGAS+: segment sums (16 B) per range and per hypercube (nh <= ncall / 4)
-  if (plus_f) b += align256((size_t)(ncall / GV_PLUS_SEG + 1) * 16) + align256((size_t)(ncall / 4 + 1) * 16);
+  if (plus_f)
+    b += align256((size_t)(plus_events / GV_PLUS_SEG + 1) * 16) +
+         align256((size_t)(plus_events / 4 + 1) * 16);
   return b;
 }
 
@@ -734,7 +735,8 @@ int make_plan(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* param
   int gx = 0, gy = 0;
   gv::reduce_grid(p.n_tiles, p.nacc, &p.tiles_per_cta, &gx, &gy);
   p.reduce_ctas = gx * gy;
-  const size_t need = workspace_bytes(c->ndim, c->nbins, cap, itmx, mode, p.nhist, p.tile_events, p.plus != 0);
+  const size_t need =
+      workspace_bytes(c->ndim, c->nbins, p.n_tiles, itmx, mode, p.nhist, p.plus != 0, cap);
   int st = ensure_workspace(c, need);
   if (st) return st;
   char* w = (char*)c->ws;
@@ -1288,10 +1290,11 @@ int vegas_set_stream(vegas_ctx* c, void* stream) {
 int vegas_workspace_size(const vegas_ctx* c, int64_t ncall, int itmx, size_t* bytes) {
   if (!c || !bytes || ncall < 2 || itmx < 1) return VEGAS_EINVAL;
   const int nhist = c->hist_nh > 0 ? c->hist_nh + 2 : 0;
-  // FP64's tiles are no larger than FP32's: room for either
-  const int T = std::min(gv_tile_events(ncall, GV_FORM_F32), gv_tile_events(ncall, GV_FORM_X64));
-  *bytes = std::max(workspace_bytes(c->ndim, c->nbins, ncall, itmx, 0, nhist, T),
-                    workspace_bytes(c->ndim, c->nbins, ncall, itmx, 1, 0, T));
+  // room for either precision, and for every stage of fewer calls
+  const int64_t tiles =
+      std::max(gv_most_tiles(ncall, GV_FORM_F32), gv_most_tiles(ncall, GV_FORM_X64));
+  *bytes = std::max(workspace_bytes(c->ndim, c->nbins, tiles, itmx, 0, nhist),
+                    workspace_bytes(c->ndim, c->nbins, tiles, itmx, 1, 0));
   return VEGAS_OK;
 }
 

@@ -31,8 +31,8 @@
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
+#include "gv_tiles.cuh"
 
-#define GV_TILE 1024          // most events of a tile (see gv_tile_events)
 #define GV_FB 96              // fixed-point bits below a tile's scale
 #define GV_MAXD 16            // maximum number of axes
 #define GV_NGRAD 5            // Drell-Yan gradient components
@@ -50,37 +50,6 @@
 #define GV_HIST_MAX 1000      // histogram bins of the observable (plus underflow and overflow)
 
 enum { GV_GAUSS = 0, GV_DY = 1, GV_EE3J = 2, GV_DYNLO = 3 };
-
-// Arithmetic of an event: the FP64 pipe, FP32, or 64-bit significands on the
-// integer pipes (gv_x64.cuh).
-enum { GV_FORM_F64 = 0, GV_FORM_F32 = 1, GV_FORM_X64 = 2 };
-
-// Events per tile of a stage of ncall events (plain forward stages, single or
-// batched): 128 to GV_TILE, a function of the call count and the arithmetic
-// alone, so that results do not depend on the launch shape.  One tile is one
-// CTA: the size minimises the rounds of tiles over the 152 SMs times a tile's
-// time, its events plus a fixed part (staging, zeroing, epilogue) worth t0
-// events.  A smaller size has to save 4% of that: its tiles cost a batch, whose
-// members share the SMs, more partials (64 members of 1e4 to 1e7 calls 20.5 ms
-// with powers of two, 20.8 so; 20.9 if any saving counts).  Ten iterations with
-// 128 and with 1024 events a tile: 1e4 calls of the FP64 NLO-shaped weight on
-// 13 axes 297 and 619 us, of FP64 Drell-Yan 199 and 287, of FP32 Drell-Yan 159
-// and 162.  Against the powers of two: an FP64 fit step of 1e5 calls (149 tiles
-// of 672 instead of 98 of 1024) 585 and 495 us, the Gaussian on four axes 209
-// and 197, ten iterations of 1e6 FP32 NLO events (1042 of 960) 750 and 727.
-inline int gv_tile_events(long long ncall, int form) {
-  const long long t0 = form == GV_FORM_F32 ? 256 : 96;
-  long long best = 0;
-  int T = GV_TILE;
-  for (int t = GV_TILE; t >= 128; t -= 32) {
-    const long long tiles = (ncall + t - 1) / t, cost = (tiles + 151) / 152 * (t + t0);
-    if (best == 0 || 100 * cost < 96 * best) {
-      best = cost;
-      T = t;
-    }
-  }
-  return T;
-}
 
 // Whether the FP64 form runs on 64-bit significands: parameters of ordinary
 // size (every derived constant finite, momentum fractions above 2^-60, y_cut
