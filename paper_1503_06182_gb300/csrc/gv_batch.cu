@@ -73,7 +73,7 @@ struct Member {
   GvState* st;
   double* par;
   double* kconst;
-  GvSlot* cpart;
+  unsigned long long* cpart;
   double* sums;
   ulonglong2* part;
   int* tileE;
@@ -419,7 +419,7 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
     q[3] = off;
     off = a256(off + GV_NCONST_ALL * 8);
     q[4] = off;  // cpart
-    off = a256(off + (size_t)x.gy * x.gx * 32 * sizeof(GvSlot));
+    off = a256(off + (size_t)x.gy * x.gx * 32 * GV_SLOT_BYTES);
     q[5] = off;
     off = a256(off + (size_t)x.nacc * 8);
     q[7] = off;
@@ -448,7 +448,7 @@ int vegas_batch_create(int n, const int* ndim, const int64_t* ncall, const int* 
     x.st = (GvState*)(base + q[1]);
     x.par = (double*)(base + q[2]);
     x.kconst = (double*)(base + q[3]);
-    x.cpart = (GvSlot*)(base + q[4]);
+    x.cpart = (unsigned long long*)(base + q[4]);
     x.sums = (double*)(base + q[5]);
     x.part = (ulonglong2*)(base + q[7]);
     x.tileE = (int*)(base + q[8]);

@@ -241,7 +241,7 @@ size_t workspace_bytes(int d, int N, int64_t n_tiles, int itmx, int mode, int nh
   size_t b = align256((size_t)n_tiles * nacc * 16);
   b += align256((size_t)n_tiles * nch * 4);
   b += align256((size_t)std::max(itmx, kTuneIter) * (2 + 2 * GV_NGRAD) * 8);
-  b += align256((size_t)gy * gx * 32 * sizeof(GvSlot));
+  b += align256((size_t)gy * gx * 32 * GV_SLOT_BYTES);
   // VEGAS+: segment sums (16 B) per range and per hypercube (nh <= ncall / 4)
   if (plus_f)
     b += align256((size_t)(plus_events / GV_PLUS_SEG + 1) * 16) +
@@ -318,7 +318,7 @@ struct Plan {
   ulonglong2* part;
   int* tileE;
   double* per_iter;
-  GvSlot* cpart;
+  unsigned long long* cpart;
 };
 
 GvFillArgs fill_args(const vegas_ctx* c, const Plan& p, int k = 0) {
@@ -746,9 +746,9 @@ int make_plan(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* param
   w += align256((size_t)p.n_tiles * p.nch * 4);
   p.per_iter = (double*)w;
   w += align256((size_t)std::max(itmx, kTuneIter) * (2 + 2 * GV_NGRAD) * 8);
-  p.cpart = (GvSlot*)w;
+  p.cpart = (unsigned long long*)w;
   if (p.plus) {
-    w += align256((size_t)gy * gx * 32 * sizeof(GvSlot));
+    w += align256((size_t)gy * gx * 32 * GV_SLOT_BYTES);
     p.seg_r = (double2*)w;
     w += align256((size_t)(cap / GV_PLUS_SEG + 1) * 16);
     p.seg_h = (double2*)w;

@@ -25,8 +25,8 @@
 // precision.  A tile adds each w^2 (exact in the FP32 form, to 2^-62 of itself
 // in the FP64 form) to a row of 22-bit limbs at absolute positions
 // (gv_limbs.cuh) and publishes a bin's sum as at least 66 bits with its own
-// exponent code; the iteration's sum aligns the tiles' to the bin's largest
-// code with 20 more bits.  Both truncations depend on the data alone, so the
+// exponent code; the iteration's sum keeps at least 32 bits below the largest of
+// them (gv_slotsum.cuh).  Both truncations depend on the data alone, so the
 // bin sums stay launch-shape independent.
 #pragma once
 #include <cstdint>
@@ -45,8 +45,6 @@
 #define GV_MAXPARAMS 16
 #define GV_BINE_OFF 1200      // stored bin exponent F + GV_BINE_OFF (0: no nonzero weight)
 #define GV_BIN_QBITS 56       // bits of one w^2 below its bin's scale in a tile
-#define GV_BIN_XBITS 20       // extra low bits of the iteration's bin sums
-#define GV_BIN_FB (GV_BIN_QBITS + GV_BIN_XBITS)  // bin sums in units of 2^(2F - GV_BIN_FB)
 #define GV_HIST_MAX 1000      // histogram bins of the observable (plus underflow and overflow)
 
 enum { GV_GAUSS = 0, GV_DY = 1, GV_EE3J = 2, GV_DYNLO = 3 };
@@ -170,14 +168,9 @@ struct GvFillArgs {
   const struct GvPlusFill* plus = nullptr;
 };
 
-// One slot's sum as a 192-bit two's complement integer with its exponent:
-// channel slot 2c (sum v) / 2c+1 (sum v^2): value = v 2^(pw e - GV_FB),
-// pw = 1 / 2, e a tile scale (GV_EMPTY: nothing nonzero); bin slot: value =
-// v 2^(2 (e - GV_BINE_OFF) - GV_BIN_FB), e a stored bin exponent (0: empty).
-struct __align__(16) GvSlot {
-  unsigned long long l0, l1, l2;
-  int e, pad;
-};
+// What a tile range of the two-level reduce publishes of one slot: the counters
+// of gv_slotsum.cuh and their window.
+#define GV_SLOT_BYTES (7 * 8)
 
 // Tickets of the reduce kernel, each on its own 128-byte line: one per slot
 // block of 32 slots, one per axis (and one spare line).
@@ -213,7 +206,7 @@ struct GvReduceArgs {
   const ulonglong2* part;
   const int* tileE;
   GvState* st;
-  GvSlot* cpart;                 // [tile ranges][32 * slot blocks] one CTA's sums
+  unsigned long long* cpart;                 // [tile ranges][7][32 * slot blocks] one CTA's sums
   double* sums;                  // [nacc] FP64 sums of the last iteration
   double* per_iter;              // forward: [itmx][2]; adjoint: [itmx][2 + 2*NGRAD]
   int* tickets;                  // gv_tickets_ints(nacc) counters, one per 128-byte line

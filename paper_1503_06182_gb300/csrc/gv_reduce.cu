@@ -5,13 +5,12 @@
 // Forward stages and small adjoint ones: gv_reduce_cluster_kernel and
 // gv_reduce_slots_kernel (below).  gv_reduce_kernel and the batched form: the
 // grid is (slot blocks of 32) x (tile ranges): each CTA owns 32 slots and a
-// range of tiles; its 8 warps stride over the tiles and add the partials at the
-// largest exponent the slot has so far (channel sums: the tiles' scales; bin
-// sums: the bins' own exponent codes, gv_limbs.cuh), in 128-bit integers; the
-// warps' sums are combined in shared memory in 192 bits and published with
-// their exponent.  No sum is formed with atomics.  The order depends on the
-// reduce grid alone, a function of the tile count: the totals do not depend on
-// the fill's launch shape or on timing.
+// range of tiles; its 8 warps stride over the tiles, the warps' sums are combined
+// in shared memory and published.  All of them form a slot's sum by the rule of
+// gv_slotsum.cuh (channel sums: at the tiles' scales; bin sums: at the bins' own
+// exponent codes, gv_limbs.cuh).  No sum is formed with atomics, and none depends
+// on the order of its tiles: the totals are the same in every kernel, launch shape
+// and batch.
 //
 // Tickets instead of waiting: each CTA publishes its sums and counts itself
 // on its block of 32 slots; the CTA that completes a block combines the
@@ -34,31 +33,12 @@
 #include "gv_ff.cuh"
 #include "gv_integrands.cuh"
 #include "gv_limbs.cuh"
+#include "gv_slotsum.cuh"
 #include "gv_xint.cuh"
 
-// Slots (GvSlot: 192 bits and an exponent) are written by one thread and read
-// by CTAs that took a ticket after the writer's fence: L2 loads.
-__device__ __forceinline__ u192 slot_value(const GvSlot& s) { return {s.l0, s.l1, s.l2}; }
-__device__ __forceinline__ GvSlot load_slot(const GvSlot* p) {
-  const ulonglong2 a = __ldcg(reinterpret_cast<const ulonglong2*>(p));
-  const ulonglong2 b = __ldcg(reinterpret_cast<const ulonglong2*>(p) + 1);
-  GvSlot s;
-  s.l0 = a.x;
-  s.l1 = a.y;
-  s.l2 = b.x;
-  s.e = (int)(unsigned)(b.y & 0xFFFFFFFFull);
-  s.pad = 0;
-  return s;
-}
-__device__ __forceinline__ void store_slot(GvSlot* p, const u192& v, int e) {
-  reinterpret_cast<ulonglong2*>(p)[0] = make_ulonglong2(v.l0, v.l1);
-  reinterpret_cast<ulonglong2*>(p)[1] = make_ulonglong2(v.l2, (unsigned long long)(unsigned)e);
-}
-
-// value * 2^q rounded to nearest-even, assembled with integer operations only
-// (the integer is two's complement; results stay in the normal range for
-// every sum this library forms): from its magnitude's leading 64 bits (bit 63
-// set, worth 2^(e - 63)) and whether anything lies below them.
+// A value rounded to nearest-even, assembled with integer operations only, from
+// its magnitude's leading 64 bits (bit 63 set, worth 2^(e - 63)) and whether
+// anything lies below them.
 __device__ __forceinline__ double assemble_double(unsigned long long window, bool sticky, int e,
                                                   bool neg) {
   // round the 64-bit window to 53 bits (nearest, ties to even)
@@ -88,58 +68,11 @@ __device__ __forceinline__ double assemble_double(unsigned long long window, boo
   }
   return neg ? -r : r;
 }
-__device__ __forceinline__ double i128_to_double(u128 v, int q) {
-  const bool neg = (long long)v.hi < 0;
-  if (neg) {
-    v.lo = 0ull - v.lo;
-    v.hi = ~v.hi + (v.lo == 0ull ? 1ull : 0ull);
-  }
-  if (v.hi == 0ull) {
-    if (v.lo == 0ull) return 0.0;
-    const int lz = __clzll((long long)v.lo);
-    return assemble_double(v.lo << lz, false, 63 - lz + q, neg);
-  }
-  const int lz = __clzll((long long)v.hi);
-  const unsigned long long window = lz ? (v.hi << lz) | (v.lo >> (64 - lz)) : v.hi;
-  return assemble_double(window, (v.lo << lz) != 0ull, 127 - lz + q, neg);
-}
-__device__ double u192_to_double(u192 v, int q) {
-  const bool neg = (long long)v.l2 < 0;
-  if (neg) {
-    v.l0 = ~v.l0;
-    v.l1 = ~v.l1;
-    v.l2 = ~v.l2;
-    v.l0 += 1ull;
-    const unsigned long long c0 = v.l0 == 0ull ? 1ull : 0ull;
-    v.l1 += c0;
-    v.l2 += (c0 && v.l1 == 0ull) ? 1ull : 0ull;
-  }
-  int top;
-  if (v.l2)
-    top = 191 - __clzll((long long)v.l2);
-  else if (v.l1)
-    top = 127 - __clzll((long long)v.l1);
-  else if (v.l0)
-    top = 63 - __clzll((long long)v.l0);
-  else
-    return 0.0;
-  // 64-bit window with the leading one at bit 63, plus a sticky bit
+__device__ __forceinline__ double acc_to_double(const GvAcc& a) {
   unsigned long long window;
-  bool sticky = false;
-  if (top >= 63) {
-    const int sh = top - 63;
-    window = sar192(v, sh).l0;
-    if (sh >= 128) {
-      sticky = v.l0 != 0ull || v.l1 != 0ull || (sh > 128 && (v.l2 << (192 - sh)) != 0ull);
-    } else if (sh >= 64) {
-      sticky = v.l0 != 0ull || (sh > 64 && (v.l1 << (128 - sh)) != 0ull);
-    } else if (sh > 0) {
-      sticky = (v.l0 << (64 - sh)) != 0ull;
-    }
-  } else {
-    window = v.l0 << (63 - top);
-  }
-  return assemble_double(window, sticky, top + q, neg);
+  bool sticky, neg;
+  int e;
+  return acc_window(a, &window, &sticky, &e, &neg) ? assemble_double(window, sticky, e, neg) : 0.0;
 }
 
 // Barrier of a group of nthr threads (a multiple of 32); id 0 is the whole CTA.
@@ -521,136 +454,196 @@ __host__ __device__ inline int gv_axes_per_block(int N) {
 
 #define GV_RED_TILES_PER_LOAD 8
 
-// Arithmetic shift right of a 128-bit value by s >= 0, in words: two selects
-// and a funnel shift each.
-__device__ __forceinline__ u128 sar128(u128 v, int s) {
-  s = min(s, 127);
-  unsigned w0 = (unsigned)v.lo, w1 = (unsigned)(v.lo >> 32);
-  unsigned w2 = (unsigned)v.hi, w3 = (unsigned)(v.hi >> 32);
-  const unsigned ext = (unsigned)((int)w3 >> 31);
-  if (s & 64) {
-    w0 = w2;
-    w1 = w3;
-    w2 = ext;
-    w3 = ext;
+// Tile partials.  Channel slots: 128-bit two's complement at
+// 2^(pw e - GV_FB), e the tile's scale; bin slots (axis bins and histogram bins):
+// a 96-bit value, unsigned for sums of w^2 (pw = 2) or two's complement for the
+// histogram's sums of w (pw = 1, sgn), at
+// 2^(pw (e - GV_BINE_OFF) - GV_BIN_QBITS), e its exponent code.
+//
+// Bit position and top word of a partial v of tile t; one slot's partials.
+struct SlotPartials {
+  const ulonglong2* src;
+  size_t stride;
+  const int* tileE;
+  int nch, pw;
+  bool bin, sgn;
+  __device__ __forceinline__ ulonglong2 load(int t) const { return __ldcg(src + t * stride); }
+  __device__ __forceinline__ int position(const ulonglong2& v, int t) const {
+    if (bin) {
+      const int e = (int)(v.y >> 32);
+      return e == 0 ? 0 : pw * (e - GV_BINE_OFF) - GV_BIN_QBITS + GV_POS_OFF;
+    }
+    const int e = __ldcg(tileE + (size_t)t * nch);
+    return e == GV_EMPTY ? 0 : pw * e - GV_FB + GV_POS_OFF;
   }
-  if (s & 32) {
-    w0 = w1;
-    w1 = w2;
-    w2 = w3;
-    w3 = ext;
+  __device__ __forceinline__ unsigned word3(const ulonglong2& v) const {
+    return bin ? (sgn ? (unsigned)((int)v.y >> 31) : 0u) : (unsigned)(v.y >> 32);
   }
-  w0 = __funnelshift_r(w0, w1, s);
-  w1 = __funnelshift_r(w1, w2, s);
-  w2 = __funnelshift_r(w2, w3, s);
-  w3 = __funnelshift_r(w3, ext, s);
-  return u128{w0 | ((unsigned long long)w1 << 32), w2 | ((unsigned long long)w3 << 32)};
+};
+// The partials t0 + g step below nt, g < G, and their positions (0: none): every
+// load before the first use, and no branch among them (a load under a condition
+// that also uses it waits for it: 8 round trips through L2 instead of one).
+// Returns the highest position.
+template <int G>
+__device__ __forceinline__ int load_tiles(const SlotPartials& s, int t0, int step, int nt,
+                                          ulonglong2 (&v)[G], int (&pos)[G]) {
+  int top = 0;
+#pragma unroll
+  for (int g = 0; g < G; ++g) v[g] = s.load(min(t0 + g * step, nt - 1));
+  if (s.bin) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) pos[g] = s.position(v[g], 0);
+  } else {
+#pragma unroll
+    for (int g = 0; g < G; ++g) pos[g] = s.position(v[g], min(t0 + g * step, nt - 1));
+  }
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    if (t0 + g * step >= nt) pos[g] = 0;
+    top = max(top, pos[g]);
+  }
+  return top;
 }
 
-// Tile partials.  Channel slots: 128-bit two's complement at
-// 2^(pw e - GV_FB); bin slots (axis bins and histogram bins): a 96-bit value,
-// unsigned for sums of w^2 (pw = 2) or two's complement for the histogram's
-// sums of w (pw = 1, sgn), at 2^(pw (e - GV_BINE_OFF) - GV_BIN_QBITS), with
-// GV_BIN_XBITS more low bits in the sums.
-// A slot's running sum over them, at the largest exponent seen so far.  128-bit for up to 2048 partials (a bin's of 96 bits, 20 more low bits,
-// 11 bits of headroom; a channel's of 107); a longer run is summed in 192 bits
-// over segments of 2048.
-struct SlotSum {
-  u128 v;
-  int em;
-};
-struct SlotSumW {
-  u192 v;
-  int em;
-};
-// The sum of the partials src[t stride], t = u, u + step, .. below nt (at most
-// 2048 of them), each read once: the sum moves down when a larger exponent
-// comes.
+// The sum of the partials t = u, u + step, .. below nt, each read once: the window
+// moves up when a higher one comes.  (`lane`: of threads with consecutive u, 0
+// otherwise.)
 template <int G>
-__device__ __forceinline__ SlotSum sum_tiles(const ulonglong2* src, size_t stride, int u, int lane,
-                                             int step, int nt, const int* tileE, int nch, bool bin, int pw,
-                                             bool sgn, int empty) {
-  SlotSum s = {{0ull, 0ull}, empty};
+__device__ __forceinline__ GvAcc sum_tiles(const SlotPartials& p, int u, int lane, int step,
+                                           int nt) {
+  GvAcc s = acc_zero();
   for (int t0 = u; t0 < nt; t0 += G * step) {
-    // every load before the first use, and no branch among them (a load under
-    // a condition that also uses it waits for it: 8 round trips through L2
-    // instead of one)
     ulonglong2 v[G];
-    int et[G], cm = empty;
-#pragma unroll
-    for (int g = 0; g < G; ++g) v[g] = __ldcg(src + (size_t)min(t0 + g * step, nt - 1) * stride);
-    if (bin) {
-#pragma unroll
-      for (int g = 0; g < G; ++g) et[g] = (int)(v[g].y >> 32);
-    } else {
-#pragma unroll
-      for (int g = 0; g < G; ++g)
-        et[g] = __ldcg(tileE + (size_t)min(t0 + g * step, nt - 1) * nch);
-    }
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      if (t0 + g * step >= nt) et[g] = empty;
-      cm = max(cm, et[g]);
-    }
-    if (cm > s.em) {
-      if (s.em != empty) s.v = sar128(s.v, pw * (cm - s.em));
-      s.em = cm;
-    }
+    int pos[G];
+    const int top = load_tiles(p, t0, step, nt, v, pos);
+    if ((top >> 5) > s.g) acc_raise(s, top >> 5);
+    unsigned far = 0u;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       if (g > 0 && t0 - lane + g * step >= nt) break;  // no lane has another
-      u128 x = {v[g].x, v[g].y};
-      if (bin) {
-        const unsigned h = (unsigned)v[g].y;
-        x.hi = ((sgn ? (unsigned long long)(long long)(int)h : h) << GV_BIN_XBITS) |
-               (x.lo >> (64 - GV_BIN_XBITS));
-        x.lo <<= GV_BIN_XBITS;
-      }
-      const bool none = et[g] == empty;
-      x.lo = none ? 0ull : x.lo;
-      x.hi = none ? 0ull : x.hi;
-      s.v = add128(s.v, sar128(x, none ? 0 : pw * (s.em - et[g])));
+      const int o = s.g - (pos[g] >> 5);
+      const bool near = pos[g] != 0 && o <= 1;
+      if (pos[g] != 0 && o > 1) far |= 1u << g;
+      acc_add_near(s, near ? (unsigned)v[g].x : 0u, near ? (unsigned)(v[g].x >> 32) : 0u,
+                   near ? (unsigned)v[g].y : 0u, near ? p.word3(v[g]) : 0u, pos[g], o);
+    }
+    // read again: few, and their code stays out of the loop above
+    while (far) {
+      const int t = t0 + (__ffs((int)far) - 1) * step;
+      far &= far - 1u;
+      const ulonglong2 x = p.load(t);
+      const int q = p.position(x, t);
+      acc_add_far(s, (unsigned)x.x, (unsigned)(x.x >> 32), (unsigned)x.y, p.word3(x), q,
+                  s.g - (q >> 5));
     }
   }
   return s;
 }
-__device__ __forceinline__ u192 widen128(u128 v) {
-  return u192{v.lo, v.hi, (unsigned long long)((long long)v.hi >> 63)};
-}
-// As sum_tiles, over any number of partials.
-__device__ __forceinline__ SlotSumW sum_tiles_wide(const ulonglong2* src, size_t stride, int u,
-                                                   int lane, int step, int nt, const int* tileE, int nch,
-                                                   bool bin, int pw, bool sgn, int empty) {
-  SlotSumW s = {{0ull, 0ull, 0ull}, empty};
-  for (long long t0 = u; t0 < nt; t0 += 2048ll * step) {
-    const SlotSum p = sum_tiles<GV_RED_TILES_PER_LOAD / 2>(
-        src, stride, (int)t0, lane, step, (int)min(t0 + 2048ll * step, (long long)nt), tileE, nch, bin, pw, sgn,
-        empty);
-    if (p.em == empty) continue;
-    if (p.em > s.em) {
-      if (s.em != empty) s.v = sar192(s.v, pw * (p.em - s.em));
-      s.em = p.em;
-    }
-    add192(s.v, sar192(widen128(p.v), pw * (s.em - p.em)));
+
+// The sum over a warp of at most 32 G partials, one slot: the highest position
+// first.  In every lane.
+template <int G>
+__device__ __forceinline__ double warp_sum_tiles(const SlotPartials& p, int nt) {
+  constexpr unsigned all = 0xffffffffu, M = (1u << 26) - 1u;
+  const int lane = threadIdx.x & 31;
+  ulonglong2 v[G];
+  int pos[G];
+  const int g0 = __reduce_max_sync(all, load_tiles(p, lane, 32, nt, v, pos)) >> 5;
+  if (g0 == 0) return 0.0;
+  GvAccFixed a = {{0u, 0u, 0u, 0u, 0u, 0u}};
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    if (32 * g >= nt) break;
+    const bool any = pos[g] != 0;
+    acc_add_fixed(a, any ? (unsigned)v[g].x : 0u, any ? (unsigned)(v[g].x >> 32) : 0u,
+                  any ? (unsigned)v[g].y : 0u, any ? p.word3(v[g]) : 0u, any ? pos[g] : 32 * g0, g0);
   }
-  return s;
+  // in eight parts of 26 bits: of the even and the odd ones no two overlap
+  unsigned s[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int j = 26 * i / 32, r = 26 * i % 32;
+    s[i] = __reduce_add_sync(
+        all, i == 7 ? a.w[5] >> r : __funnelshift_r(a.w[j], a.w[min(j + 1, 5)], r) & M);
+  }
+  unsigned long long q[4], h[3];
+  q[0] = s[0] | ((unsigned long long)s[2] << 52);
+  q[1] = ((unsigned long long)s[2] >> 12) | ((unsigned long long)s[4] << 40);
+  q[2] = ((unsigned long long)s[4] >> 24) | ((unsigned long long)s[6] << 28);
+  h[0] = ((unsigned long long)s[1] << 26);
+  h[1] = ((unsigned long long)s[3] << 14);
+  h[2] = ((unsigned long long)s[5] << 2) | ((unsigned long long)s[7] << 54);
+  asm("add.cc.u64 %0, %0, %3;\n\t"
+      "addc.cc.u64 %1, %1, %4;\n\t"
+      "addc.u64 %2, %2, %5;"
+      : "+l"(q[0]), "+l"(q[1]), "+l"(q[2])
+      : "l"(h[0]), "l"(h[1]), "l"(h[2]));
+  q[3] = (unsigned long long)((long long)q[2] >> 63);
+  unsigned long long window;
+  bool sticky, neg;
+  int e;
+  return acc_leading(q, g0, &window, &sticky, &e, &neg) ? assemble_double(window, sticky, e, neg)
+                                                        : 0.0;
+}
+
+// The sum over a warp's lanes, in every lane: counters in a low part
+// of 27 bits and the rest, which fits 32 bits for 2^21 partials a lane; more
+// (`many`) take three parts.
+__device__ __forceinline__ GvAcc warp_sum_acc(GvAcc a, bool many) {
+  constexpr unsigned M = (1u << 27) - 1u, all = 0xffffffffu;
+  const int g = __reduce_max_sync(all, a.g);
+  if (a.g < g) acc_raise(a, g);
+#pragma unroll
+  for (int j = 0; j < GV_SLOT_WORDS; ++j) {
+    const long long v = (long long)a.w[j];
+    unsigned long long t = __reduce_add_sync(all, (unsigned)v & M);
+    if (!many)
+      t += (unsigned long long)(long long)__reduce_add_sync(all, (int)(v >> 27)) << 27;
+    else
+      t += ((unsigned long long)__reduce_add_sync(all, (unsigned)(v >> 27) & M) << 27) +
+           ((unsigned long long)__reduce_add_sync(all, (unsigned)(v >> 54)) << 54);
+    a.w[j] = t;
+  }
+  return a;
 }
 
 // One reduce CTA (256 threads) of one integration: slot block bx (32 slots,
 // one per lane), tile range by, of nblk CTAs in total for that integration.
-//   A. every CTA: the largest exponent of each slot over its tiles, then the
-//      tiles' partials aligned to it and summed -- the CTA's sums, published
-//      with that exponent (no atomics);
+//   A. every CTA: each slot's sum over its tiles (no atomics), published;
 //   B. the CTA that completes a slot block (ticket): the block's sums over all
-//      tile ranges at their largest exponent, each rounded once to FP64;
+//      tile ranges, each rounded once to FP64;
 //   C. the CTA whose block completes an axis (second ticket) refines the
 //      axis; the CTA that completes block 0 (the channel sums) finalises the
 //      iteration.
-// Integer sums of values aligned by rules that depend only on the data:
-// nothing here depends on the launch shape or on timing.
+// The sums depend on the data alone (gv_slotsum.cuh), not on the launch shape or
+// on timing.
+static_assert(GV_SLOT_BYTES == 8 * (GV_SLOT_WORDS + 1), "a published sum");
+struct GvTaskMem {
+  unsigned long long w[GV_SLOT_WORDS][8][32];  // the warps' sums: counters ..
+  int g[8][32];                                // .. and windows
+  int flags[4], won[GV_MAXD];
+};
+// The sum over the CTA's warps of their lanes' sums: warp j < GV_SLOT_WORDS
+// returns counter j, and every warp the window.
+__device__ __forceinline__ unsigned long long task_combine(GvTaskMem& m, const GvAcc& a, int* g) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int j = 0; j < GV_SLOT_WORDS; ++j) m.w[j][wid][lane] = a.w[j];
+  m.g[wid][lane] = a.g;
+  __syncthreads();
+  int top = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) top = max(top, m.g[w][lane]);
+  *g = top;
+  unsigned long long t = 0ull;
+  if (wid < GV_SLOT_WORDS) {
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += acc_word(&m.w[0][w][lane], 8 * 32, m.g[w][lane], top, wid);
+  }
+  return t;
+}
 __device__ __forceinline__ void gv_reduce_task(const GvReduceArgs& a, int bx, int by, int nblk,
-                               u192 (*s_part)[32], int* s_emax, int* s_flags, int* s_won,
-                               double* sm) {
+                                               GvTaskMem& mem, double* sm) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int k = bx * 32 + lane;
   const int gx = (a.nacc + 31) / 32, gy = nblk / gx;
@@ -660,86 +653,60 @@ __device__ __forceinline__ void gv_reduce_task(const GvReduceArgs& a, int bx, in
   // the histogram's sums of w: the last nhist slots
   const bool hw = bin && a.nhist > 0 && k >= a.nacc - a.nhist;
   const int pw = hw ? 1 : (bin ? 2 : (k & 1) + 1);
-  const int empty = bin ? 0 : GV_EMPTY;
-  const int ch = k >> 1;
+  const size_t row = 32 * (size_t)gx;  // of the published sums: [range][counters, window][row]
   gv_wait_prior_grid();
 
   // ---- A: this CTA's tiles
-  SlotSumW sum = {{0ull, 0ull, 0ull}, empty};
+  GvAcc sum = acc_zero();
   if (k < a.nacc)
-    sum = sum_tiles_wide(a.part + k, (size_t)a.nacc, t0 + wid, 0, 8, t1, a.tileE + ch, a.nch, bin, pw,
-                         hw, empty);
-  int em = sum.em;
-  s_emax[wid * 32 + lane] = em;
-  __syncthreads();
-#pragma unroll
-  for (int w = 0; w < 8; ++w) em = max(em, s_emax[w * 32 + lane]);
-  u192 r = sum.em == empty ? sum.v : sar192(sum.v, pw * (em - sum.em));
-  s_part[wid][lane] = r;
-  __syncthreads();
-  if (wid == 0) {
-    u192 t = s_part[0][lane];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) add192(t, s_part[w][lane]);
-    if (k < a.nacc) store_slot(a.cpart + (size_t)by * (32 * gx) + k, t, em);
+    sum = sum_tiles<GV_RED_TILES_PER_LOAD / 2>(
+        SlotPartials{a.part + k, (size_t)a.nacc, a.tileE + (k >> 1), a.nch, pw, bin, hw}, t0 + wid,
+        0, 8, t1);
+  int g;
+  unsigned long long t = task_combine(mem, sum, &g);
+  if (wid <= GV_SLOT_WORDS) {
+    a.cpart[(size_t)(by * (GV_SLOT_WORDS + 1) + wid) * row + k] =
+        wid < GV_SLOT_WORDS ? t : (unsigned long long)g;
     __threadfence();
   }
   __syncthreads();
   if (threadIdx.x == 0)
-    s_flags[0] = atomicAdd(a.tickets + gv_ticket_group(bx), 1) == gy - 1 ? 1 : 0;
+    mem.flags[0] = atomicAdd(a.tickets + gv_ticket_group(bx), 1) == gy - 1 ? 1 : 0;
   __syncthreads();
-  if (!s_flags[0]) return;
+  if (!mem.flags[0]) return;
 
   // ---- B: this CTA completes slot block bx
   __threadfence();  // the other CTAs' sums, published before their tickets
   gv_allow_next_grid();  // what is left is short: the next fill's CTAs may come in
   if (threadIdx.x == 0) a.tickets[gv_ticket_group(bx)] = 0;
-  constexpr int YC = 2;  // tile ranges per warp held in registers (gy <= 16)
-  GvSlot cs[YC];
-  const bool held = gy <= 8 * YC;
-  em = empty;
+  sum = acc_zero();
+#pragma unroll 1
+  for (int y = wid; y < gy; y += 8) {
+    const unsigned long long* c = a.cpart + (size_t)y * (GV_SLOT_WORDS + 1) * row + k;
+    GvAcc r;
 #pragma unroll
-  for (int q = 0; q < YC; ++q) {
-    const int y = wid + 8 * q;
-    cs[q].e = empty;
-    if (held && k < a.nacc && y < gy) cs[q] = load_slot(a.cpart + (size_t)y * (32 * gx) + k);
-    em = max(em, cs[q].e);
+    for (int j = 0; j < GV_SLOT_WORDS; ++j) r.w[j] = __ldcg(c + j * row);
+    r.g = (int)__ldcg(c + GV_SLOT_WORDS * row);
+    const int top = max(r.g, sum.g);
+    acc_raise(r, top);
+    acc_raise(sum, top);
+#pragma unroll
+    for (int j = 0; j < GV_SLOT_WORDS; ++j) sum.w[j] += r.w[j];
   }
-  if (!held && k < a.nacc)
-    for (int y = wid; y < gy; y += 8)
-      em = max(em, __ldcg(&a.cpart[(size_t)y * (32 * gx) + k].e));
-  s_emax[wid * 32 + lane] = em;
-  __syncthreads();
-#pragma unroll
-  for (int w = 0; w < 8; ++w) em = max(em, s_emax[w * 32 + lane]);
-  r = {0ull, 0ull, 0ull};
-  if (k < a.nacc && em != empty) {
-    if (held) {
-#pragma unroll
-      for (int q = 0; q < YC; ++q)
-        if (cs[q].e != empty) add192(r, sar192(slot_value(cs[q]), pw * (em - cs[q].e)));
-    } else {
-      for (int y = wid; y < gy; y += 8) {
-        const GvSlot c = load_slot(a.cpart + (size_t)y * (32 * gx) + k);
-        if (c.e != empty) add192(r, sar192(slot_value(c), pw * (em - c.e)));
-      }
-    }
-  }
-  s_part[wid][lane] = r;
+  t = task_combine(mem, sum, &g);
+  __syncthreads();  // (a counter may be read at another's place)
+  if (wid < GV_SLOT_WORDS) mem.w[wid][0][lane] = t;
   __syncthreads();
   const int N = a.nbins;
   // the axis bins of this block (the histogram slots after them have no axis)
   const int j_first = max(0, bx * 32 - 2 * a.nch);
   const int j_last = min(min(a.nacc - 1, bx * 32 + 31) - 2 * a.nch, a.ndim * N - 1);
   if (wid == 0) {
-    u192 t = s_part[0][lane];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) add192(t, s_part[w][lane]);
     // the slot's sum over all events, rounded once to FP64
-    if (k < a.nacc)
-      a.sums[k] = em == empty ? 0.0
-                              : u192_to_double(t, bin ? pw * (em - GV_BINE_OFF) - GV_BIN_FB
-                                                      : pw * em - GV_FB);
+#pragma unroll
+    for (int j = 0; j < GV_SLOT_WORDS; ++j) sum.w[j] = mem.w[j][0][lane];
+    sum.g = g;
+    if (k < a.nacc) a.sums[k] = acc_to_double(sum);
     __threadfence();
     // second tickets, one lane per axis the block touches: the block whose
     // count completes an axis refines it
@@ -757,12 +724,12 @@ __device__ __forceinline__ void gv_reduce_task(const GvReduceArgs& a, int bx, in
       }
     }
     const unsigned mask = __ballot_sync(0xffffffffu, won);
-    if (won) s_won[__popc(mask & ((1u << lane) - 1u))] = ax0 + lane;
-    if (lane == 0) s_flags[1] = __popc(mask);
+    if (won) mem.won[__popc(mask & ((1u << lane) - 1u))] = ax0 + lane;
+    if (lane == 0) mem.flags[1] = __popc(mask);
   }
   __syncthreads();
   // block 0 holds the channel sums: it finalises the iteration
-  const int n_won = s_flags[1], fin = bx == 0;
+  const int n_won = mem.flags[1], fin = bx == 0;
   if (n_won == 0 && !fin) return;
 
   // ---- C
@@ -779,7 +746,7 @@ __device__ __forceinline__ void gv_reduce_task(const GvReduceArgs& a, int bx, in
     if (q < ng) {
       const int per = (int)(refine_axis_smem(a.nbins) / sizeof(double));
       for (int it = q; it < n_won; it += ng)
-        refine_axis<false>(a, s_won[it], sm + (size_t)q * per, threadIdx.x - 32 * wpg * q, 32 * wpg,
+        refine_axis<false>(a, mem.won[it], sm + (size_t)q * per, threadIdx.x - 32 * wpg * q, 32 * wpg,
                     2 + q, q);
     }
   }
@@ -787,18 +754,14 @@ __device__ __forceinline__ void gv_reduce_task(const GvReduceArgs& a, int bx, in
 
 __global__ void __launch_bounds__(256) gv_reduce_kernel(const GvReduceArgs a) {
   extern __shared__ __align__(16) double sm[];
-  __shared__ u192 s_part[8][32];
-  __shared__ int s_emax[256], s_flags[4], s_won[GV_MAXD];
-  gv_reduce_task(a, blockIdx.x, blockIdx.y, gridDim.x * gridDim.y, s_part, s_emax, s_flags,
-                 s_won, sm);
+  __shared__ GvTaskMem mem;
+  gv_reduce_task(a, blockIdx.x, blockIdx.y, gridDim.x * gridDim.y, mem, sm);
 }
 
 // ---------------------------------------------------------------------------
 // Single-level reduce of an iteration with slot-major partials (slot k of tile
-// t at part[k n_tiles + t]): a CTA owns one slot and reads it over every tile,
-// aligned to the largest exponent and added in 128-bit integers (192-bit for
-// more than 2048 tiles), rounded once to FP64.  The order is fixed by the
-// number of tiles.  Compared with the two-level reduce there is no published
+// t at part[k n_tiles + t]): a CTA owns one slot and reads it over every tile;
+// the sum is rounded once to FP64.  Compared with the two-level reduce there is no published
 // per-range sum and no ticket between the levels: one L2 round trip for the
 // partials, then one fence and one ticket per slot.
 // Tickets: the CTA that completes the channel slots finalises the iteration,
@@ -806,36 +769,15 @@ __global__ void __launch_bounds__(256) gv_reduce_kernel(const GvReduceArgs a) {
 // another.  Bound by latency up to some thousand tiles, then by the partials'
 // traffic: ten iterations of 1e7 three-jet events (502 slots of 9766 tiles,
 // 78 MB) 2.88 ms when the loads waited for one another and the exponents were
-// read first, 2.77 ms now.
+// read first, 2.77 with each thread's sum in one 128-bit integer at its largest
+// exponent so far, 2.79 with sums that no order can change (1e6 Drell-Yan events
+// 417 and 421 us).
 // ---------------------------------------------------------------------------
-// Sum over a warp of 128-bit values (mod 2^128), in five digits of 26 bits.
-__device__ __forceinline__ u128 warp_sum128(u128 v) {
-  constexpr unsigned M = (1u << 26) - 1u;
-  const unsigned all = 0xffffffffu;
-  const unsigned d0 = __reduce_add_sync(all, (unsigned)v.lo & M);
-  const unsigned d1 = __reduce_add_sync(all, (unsigned)(v.lo >> 26) & M);
-  const unsigned d2 = __reduce_add_sync(all, (unsigned)((v.lo >> 52) | (v.hi << 12)) & M);
-  const unsigned d3 = __reduce_add_sync(all, (unsigned)(v.hi >> 14) & M);
-  const unsigned d4 = __reduce_add_sync(all, (unsigned)(v.hi >> 40));
-  const u128 a = {(unsigned long long)d0 + ((unsigned long long)d1 << 26),
-                  ((unsigned long long)d3 << 14) + ((unsigned long long)d4 << 40)};
-  return add128(a, u128{(unsigned long long)d2 << 52, d2 >> 12});
-}
-__device__ __forceinline__ u192 warp_sum192(u192 v) {
-#pragma unroll
-  for (int m = 16; m > 0; m >>= 1) {
-    const u192 o = {shfl_xor_u64(v.l0, m), shfl_xor_u64(v.l1, m), shfl_xor_u64(v.l2, m)};
-    add192(v, o);
-  }
-  return v;
-}
-
 // Three CTAs per SM: 80 registers hold eight partials in flight.
-template <bool WIDE>
 __global__ void __launch_bounds__(256, 3) gv_reduce_slots_kernel(const GvReduceArgs a) {
   extern __shared__ __align__(16) double sm[];
-  __shared__ int s_emax[8];
-  __shared__ u192 s_sum[8];
+  __shared__ unsigned long long s_w[8][GV_SLOT_WORDS];
+  __shared__ int s_g[8];
   __shared__ int s_won, s_fin;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int k = blockIdx.x;
@@ -843,46 +785,34 @@ __global__ void __launch_bounds__(256, 3) gv_reduce_slots_kernel(const GvReduceA
   // the histogram's sums of w: the last nhist slots
   const bool hw = bin && a.nhist > 0 && k >= a.nacc - a.nhist;
   const int pw = hw ? 1 : (bin ? 2 : (k & 1) + 1);
-  const int empty = bin ? 0 : GV_EMPTY;
-  const ulonglong2* src = a.part + (size_t)k * a.n_tiles;
+  const SlotPartials part = {a.part + (size_t)k * a.n_tiles, 1, a.tileE + (k >> 1), a.nch, pw, bin,
+                             hw};
   gv_wait_prior_grid();
   const int nt = a.tiles_used ? min(a.n_tiles, __ldcg(a.tiles_used)) : a.n_tiles;
-  int em;
-  u192 r = {0ull, 0ull, 0ull};
-  if constexpr (WIDE) {
-    const SlotSumW sum =
-        sum_tiles_wide(src, 1, tid, lane, 256, nt, a.tileE + (k >> 1), a.nch, bin, pw, hw, empty);
-    em = __reduce_max_sync(0xffffffffu, sum.em);
-    if (sum.em != empty) r = sar192(sum.v, pw * (em - sum.em));
-    r = warp_sum192(r);
-  } else {
-    const SlotSum sum = sum_tiles<GV_RED_TILES_PER_LOAD>(src, 1, tid, lane, 256, nt, a.tileE + (k >> 1),
-                                                         a.nch, bin, pw, hw, empty);
-    em = __reduce_max_sync(0xffffffffu, sum.em);
-    u128 x = {0ull, 0ull};
-    if (sum.em != empty) x = sar128(sum.v, pw * (em - sum.em));
-    r = widen128(warp_sum128(x));
-  }
-  // the warps' sums at their own largest exponents
+  GvAcc sum = warp_sum_acc(sum_tiles<GV_RED_TILES_PER_LOAD>(part, tid, lane, 256, nt),
+                           nt > (1 << 28));
   if (lane == 0) {
-    s_emax[wid] = em;
-    s_sum[wid] = r;
+#pragma unroll
+    for (int j = 0; j < GV_SLOT_WORDS; ++j) s_w[wid][j] = sum.w[j];
+    s_g[wid] = sum.g;
   }
   __syncthreads();
+  if (wid == 0) {  // lane j adds the warps' counters j
+    int g = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) g = max(g, s_g[w]);
+    unsigned long long t = 0ull;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += acc_word(s_w[w], 1, s_g[w], g, lane);
+#pragma unroll
+    for (int j = 0; j < GV_SLOT_WORDS; ++j) sum.w[j] = __shfl_sync(0xffffffffu, t, j);
+    sum.g = g;
+  }
   if (tid == 0) {
     s_won = -1;
     s_fin = 0;
-#pragma unroll
-    for (int w = 1; w < 8; ++w) em = max(em, s_emax[w]);
-    r = {0ull, 0ull, 0ull};
-#pragma unroll
-    for (int w = 0; w < 8; ++w)
-      if (s_emax[w] != empty) add192(r, sar192(s_sum[w], pw * (em - s_emax[w])));
     // the slot's sum over all events, rounded once to FP64
-    const int q = bin ? pw * (em - GV_BINE_OFF) - GV_BIN_FB : pw * em - GV_FB;
-    a.sums[k] = em == empty ? 0.0
-                : WIDE      ? u192_to_double(r, q)
-                            : i128_to_double(u128{r.l0, r.l1}, q);
+    a.sums[k] = acc_to_double(sum);
     __threadfence();
     if (k < 2 * a.nch) {
       int* tk = a.tickets + gv_ticket_done(a.nacc);
@@ -962,17 +892,9 @@ __global__ void __launch_bounds__(kClusterThreads) gv_reduce_cluster_kernel(cons
     const int k = k0 + s;
     const bool bin = !channels, hw = bin && !axis && k >= a.nacc - a.nhist;
     const int pw = hw ? 1 : (bin ? 2 : (k & 1) + 1);
-    const int empty = bin ? 0 : GV_EMPTY;
-    const SlotSum sum =
-        sum_tiles<GV_RED_TILES_PER_LOAD>(a.part + (size_t)k * a.n_tiles, 1, lane, lane, 32, nt,
-                                         a.tileE + (k >> 1), a.nch, bin, pw, hw, empty);
-    const int em = __reduce_max_sync(0xffffffffu, sum.em);
-    const u128 x = warp_sum128(sum.em == empty ? u128{0ull, 0ull} : sar128(sum.v, pw * (em - sum.em)));
+    const double d = warp_sum_tiles<GV_RED_TILES_PER_LOAD>(
+        SlotPartials{a.part + (size_t)k * a.n_tiles, 1, a.tileE + (k >> 1), a.nch, pw, bin, hw}, nt);
     if (lane == 0) {
-      const double d =
-          em == empty
-              ? 0.0
-              : i128_to_double(x, bin ? pw * (em - GV_BINE_OFF) - GV_BIN_FB : pw * em - GV_FB);
       a.sums[k] = d;
       if (refine) gv_store_rank0(m.slope + s, d);
     }
@@ -997,8 +919,7 @@ __global__ void __launch_bounds__(256, 4) gv_reduce_batch_kernel(const GvReduceA
                                                               const int4* tasks, int k, int last,
                                                               double inv_m1) {
   extern __shared__ __align__(16) double sm[];
-  __shared__ u192 s_part[8][32];
-  __shared__ int s_emax[256], s_flags[4], s_won[GV_MAXD];
+  __shared__ GvTaskMem mem;
   // the integration's arguments in shared memory, read where used (a copy in
   // registers held ~40 of them for the whole task)
   __shared__ GvReduceArgs s_a;
@@ -1014,7 +935,7 @@ __global__ void __launch_bounds__(256, 4) gv_reduce_batch_kernel(const GvReduceA
     s_a.inv_m1 = inv_m1;
   }
   __syncthreads();
-  gv_reduce_task(s_a, t.y, t.z, t.w, s_part, s_emax, s_flags, s_won, sm);
+  gv_reduce_task(s_a, t.y, t.z, t.w, mem, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -1236,14 +1157,12 @@ cudaError_t launch_reduce(const GvReduceArgs& a, size_t smem, cudaStream_t s, bo
 // every SM for their partials: ten iterations of 1e6 events (977 tiles, four
 // axes of 100 bins) 409 us with a CTA per slot and 434 with clusters; 98 tiles
 // 209 and 203.
-constexpr int kClusterTiles = 256;
+constexpr int kClusterTiles = 32 * GV_RED_TILES_PER_LOAD;
 cudaError_t launch_reduce_slots(const GvReduceArgs& a, size_t smem, cudaStream_t s, bool pdl) {
   if (a.n_tiles > kClusterTiles) {
-    const bool wide = a.n_tiles > 2048;
-    auto* kernel = wide ? gv_reduce_slots_kernel<true> : gv_reduce_slots_kernel<false>;
-    const cudaError_t e = allow_smem((const void*)kernel, smem);
+    const cudaError_t e = allow_smem((const void*)gv_reduce_slots_kernel, smem);
     if (e != cudaSuccess) return e;
-    return gv_launch(kernel, dim3(a.nacc), dim3(256), smem, s, pdl, a);
+    return gv_launch(gv_reduce_slots_kernel, dim3(a.nacc), dim3(256), smem, s, pdl, a);
   }
   const cudaError_t e = allow_smem((const void*)gv_reduce_cluster_kernel, smem);
   if (e != cudaSuccess) return e;
