@@ -25,9 +25,10 @@
 // precision.  A tile adds each w^2 (exact in the FP32 form, to 2^-62 of itself
 // in the FP64 form) to a row of 22-bit limbs at absolute positions
 // (gv_limbs.cuh) and publishes a bin's sum as at least 66 bits with its own
-// exponent code; the iteration's sum keeps at least 32 bits below the largest of
-// them (gv_slotsum.cuh).  Both truncations depend on the data alone, so the
-// bin sums stay launch-shape independent.
+// position; the iteration's sum keeps at least 32 bits below the largest of
+// them (gv_slotsum.cuh).  What either drops depends on the data alone, so the
+// bin sums stay launch-shape independent; a tile's part is within 2^-66 of the
+// bin's largest w^2 per event.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -43,8 +44,6 @@
 #define GV_NCONST_X 24        // and the 64-bit-significand constants (GvX) after all of them
 #define GV_NCONST_ALL (GV_NCONST + 2 * GV_NCONST_X)  // doubles in all
 #define GV_MAXPARAMS 16
-#define GV_BINE_OFF 1200      // stored bin exponent F + GV_BINE_OFF (0: no nonzero weight)
-#define GV_BIN_QBITS 56       // bits of one w^2 below its bin's scale in a tile
 #define GV_HIST_MAX 1000      // histogram bins of the observable (plus underflow and overflow)
 
 enum { GV_GAUSS = 0, GV_DY = 1, GV_EE3J = 2, GV_DYNLO = 3 };

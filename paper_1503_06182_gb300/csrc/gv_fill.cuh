@@ -699,12 +699,13 @@ struct GvEvent {
   }
 };
 
+// In memory: 48 bits of the upper word (two's complement), the position above.
 __device__ __forceinline__ void gv_store_partial(ulonglong2* p, const GvPartial& v) {
-  *p = make_ulonglong2(v.lo, (unsigned long long)v.hi | ((unsigned long long)(unsigned)v.code << 32));
+  *p = make_ulonglong2(v.lo, (v.hi & 0xFFFFFFFFFFFFull) | ((unsigned long long)(unsigned)v.pos << 48));
 }
 __device__ __forceinline__ GvPartial gv_load_partial(const ulonglong2* p) {
   const ulonglong2 v = *p;
-  return GvPartial{v.x, (unsigned)v.y, (int)(v.y >> 32)};
+  return GvPartial{v.x, (unsigned long long)((long long)(v.y << 16) >> 16), (int)(v.y >> 48)};
 }
 
 // ---------------------------------------------------------------------------
@@ -991,7 +992,10 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
   const size_t ks = a.slot_major ? (size_t)a.n_tiles : (size_t)1;
   ulonglong2* out = a.part + (a.slot_major ? (size_t)tile : (size_t)tile * a.nacc);
   int E = GV_EMPTY;         // the tile's scale: |w| < 2^E
-  u128 sum = {0ull, 0ull};  // warp 0: of w^2, warp 1: of w, at the tile's scale
+  // the tile's sums (gv_lane_sum) of w^2 and of w, by the last two warps: the first
+  // ones have more bins below (wsum 0 and 1; the others 2 and more)
+  const int wsum = NW - 1 - wid;
+  u192 sum = {0ull, 0ull, 0ull};
   // weights at limb indices of at least up_w have been added (VEGAS+: q, up_q)
   int up_w = 0x40000000;
   [[maybe_unused]] int up_q = 0x40000000;
@@ -1089,17 +1093,18 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
         for (int k = tid; k < hb * (L + HW); k += B)
           hh[k] += hh[k + hsw] + hh[k + 2 * hsw] + hh[k + 3 * hsw];
     }
-    if (have_w && wid == 0)
-      sum = add128(sum, gv_lane_total<false>(lq, L, 22 * vw.base - 2 * GV_SQ_OFF - 2 * E + GV_FB));
-    else if (have_w && wid == 1)
-      sum = add128(sum, gv_lane_total<true>(reinterpret_cast<const unsigned*>(lw), gv_lane_rows(F64, L),
-                                            22 * vw.wbase - GV_SQ_OFF - E + GV_FB));
+    if (have_w && wsum == 0)
+      add192(sum, gv_lane_sum<false>(lq, L, vw.base - gv_square_cut(E)));
+    else if (have_w && wsum == 1)
+      add192(sum, gv_lane_sum<true>(reinterpret_cast<const unsigned*>(lw), gv_lane_rows(F64, L),
+                                    vw.wbase - gv_w_cut(E)));
     ulonglong2* o = out + (size_t)(2 + tid) * ks;
     for (int k = tid; k < dN; k += B, o += (size_t)B * ks) {
       GvPartial v = gv_bin_partial(hist + k * L, L, vq.base);
       if (!first) {  // few bins have weights below the first window
-        if (v.code == 0) continue;
-        v = gv_partial_add(v, gv_load_partial(o));
+        if (v.pos == 0) continue;
+        const GvPartial x = gv_load_partial(o);
+        if (x.pos) v = gv_bin_partial_more(x, hist + k * L, L, vq.base);
       }
       gv_store_partial(o, v);
     }
@@ -1109,8 +1114,9 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
         ulonglong2* o = out + (2 + dN + k) * ks;
         GvPartial v = gv_bin_partial(hh + k * L, L, vw.base);
         if (!first) {
-          if (v.code == 0) continue;  // (nor has the bin a sum of w)
-          v = gv_partial_add(v, gv_load_partial(o));
+          if (v.pos == 0) continue;  // (nor has the bin a sum of w)
+          const GvPartial x = gv_load_partial(o);
+          if (x.pos) v = gv_bin_partial_more(x, hh + k * L, L, vw.base);
         }
         gv_store_partial(o, v);
         o = out + (2 + dN + hb + k) * ks;
@@ -1124,7 +1130,12 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
     up_w = vw.base;
     if constexpr (PLUS) up_q = vq.base;
   }
-  if (lane == 0 && wid < 2) out[wid == 0 ? ks : (size_t)0] = make_ulonglong2(sum.lo, sum.hi);
+  if (lane == 0 && wsum < 2) {  // at the tile's scale, bits below a unit dropped once
+    if (E != GV_EMPTY)
+      sum = sar192(sum, wsum == 0 ? 2 * E - GV_FB + 2 * GV_SQ_OFF - 22 * gv_square_cut(E)
+                                 : E - GV_FB + GV_SQ_OFF - 22 * gv_w_cut(E));
+    out[wsum == 0 ? ks : (size_t)0] = make_ulonglong2(sum.l0, sum.l1);
+  }
   if (tid == 0) a.tileE[tile] = E;
   if constexpr (PLUS) {
     // the hypercubes this tile holds whole (the barriers above ordered the

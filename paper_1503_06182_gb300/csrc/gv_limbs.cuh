@@ -24,6 +24,7 @@
 // 3-jet (5 axes, 1e7 events) 336 and 234 us.
 #pragma once
 #include "gv_common.cuh"
+#include "gv_slotsum.cuh"
 
 #define GV_LIMB_BITS 22
 #define GV_LIMB_MASK 0x3FFFFFu
@@ -281,23 +282,54 @@ __device__ __forceinline__ u128 gv_lane_total(const unsigned* col, int rows, int
   return r;
 }
 
-// A bin's partial: 96 bits and an exponent code F + GV_BINE_OFF with the value
-// in units of 2^(2 F - GV_BIN_QBITS).  From the row's top nonzero limb and the
-// three below it (zeros below the row), so the value is at least 2^66.
-struct GvPartial {
-  unsigned long long lo;
-  unsigned hi;
-  int code;  // 0: empty
-};
-__device__ __forceinline__ GvPartial gv_partial_norm(unsigned long long lo, unsigned long long hi,
-                                                     int code) {
-  if (hi >> 32) {  // 97 or 98 bits: drop one digit
-    lo = (lo >> GV_LIMB_BITS) | (hi << (64 - GV_LIMB_BITS));
-    hi >>= GV_LIMB_BITS;
-    code += GV_LIMB_BITS / 2;
+// The same for the forward fill, whose passes may cut the events into windows of
+// either row length: the rows from absolute digit index `cut` on (row 0 is index
+// j0 + cut), exactly, in units of that digit; lower ones drop.  Every lane below
+// 16 returns the total.
+template <bool SIGNED>
+__device__ __forceinline__ u192 gv_lane_sum(const unsigned* col, int rows, int j0) {
+  const int lane = threadIdx.x & 31;
+  long long mine = 0;
+#pragma unroll 4
+  for (int j = max(0, -j0); j < rows; ++j) {
+    const unsigned v = col[j * 32 + lane];
+    long long s;
+    if constexpr (SIGNED)
+      s = (long long)__reduce_add_sync(0xffffffffu, v & 0xFFFFu) +
+          ((long long)__reduce_add_sync(0xffffffffu, (int)v >> 16) << 16);
+    else
+      s = (long long)__reduce_add_sync(0xffffffffu, v);
+    if (lane == j) mine = s;
   }
-  return GvPartial{lo, (unsigned)hi, code};
+  const unsigned long long ext = (unsigned long long)(mine >> 63);
+  const int sh = GV_LIMB_BITS * (j0 + lane), q = sh >> 6, r = sh & 63;
+  const unsigned long long lo = (unsigned long long)mine << r;
+  const unsigned long long hi = r ? (unsigned long long)(mine >> (64 - r)) : ext;
+  u192 v = {0ull, 0ull, 0ull};
+  if (mine != 0)
+    v = q == 0 ? u192{lo, hi, ext} : (q == 1 ? u192{0ull, lo, hi} : u192{0ull, 0ull, q == 2 ? lo : 0ull});
+#pragma unroll
+  for (int m = 8; m > 0; m >>= 1) {
+    const u192 o = {shfl_xor_u64(v.l0, m), shfl_xor_u64(v.l1, m), shfl_xor_u64(v.l2, m)};
+    add192(v, o);
+  }
+  return v;
 }
+// Where those totals are cut for a tile of scale E: 22 to 43 bits below a unit of
+// 2^(2 E - GV_FB) (squares) or 2^(E - GV_FB).
+__device__ __forceinline__ int gv_square_cut(int E) { return (2 * E - GV_FB + 2 * GV_SQ_OFF) / 22 - 1; }
+__device__ __forceinline__ int gv_w_cut(int E) { return (E - GV_FB + GV_SQ_OFF + 2200) / 22 - 101; }
+
+// A bin's partial: a 112-bit integer at a bit position (gv_slotsum.cuh).  Of a
+// bin's sums of w^2 it holds the limb of the largest digit index at which any of
+// the tile's events has a nonzero digit in the bin, and the three below it, each
+// summed over all events: at least 66 bits, at most 99.  What the limbs further
+// down would carry into these is dropped, up to one unit per event.  So the
+// partial is a function of the bin's events, whatever windows of limbs took them.
+struct GvPartial {
+  unsigned long long lo, hi;
+  int pos;  // 0: empty
+};
 __device__ __forceinline__ GvPartial gv_bin_partial(const unsigned* row, int L, int base) {
   // a square of at least 2^46 (FP64: 2^62) has its top digit above two others:
   // the top limb t is at least 2
@@ -310,35 +342,34 @@ __device__ __forceinline__ GvPartial gv_bin_partial(const unsigned* row, int L, 
     c = d;
     d = t > 2 ? row[t - 3] : 0u;
   }
-  if (a == 0u) return GvPartial{0ull, 0u, 0};
+  if (a == 0u) return GvPartial{0ull, 0ull, 0};
   const u128 x = add128(u128{(unsigned long long)d + ((unsigned long long)c << 22),
                              (unsigned long long)a << 2},
                         u128{(unsigned long long)b << 44, b >> 20});
-  // unit 2^(22 i - 2 GV_SQ_OFF) = 2^(2 F - 56) for the lowest digit i = base + t - 3
-  return gv_partial_norm(x.lo, x.hi, 11 * (base + t - 3) - GV_SQ_OFF + GV_BIN_QBITS / 2 +
-                                         GV_BINE_OFF);
+  return GvPartial{x.lo, x.hi, 22 * (base + t - 3) - 2 * GV_SQ_OFF + GV_POS_OFF};
 }
-// The sum of two partials of a bin (a later pass over lower weights): the
-// smaller unit aligned to the larger one, bits below it dropped.
-__device__ __forceinline__ GvPartial gv_partial_add(GvPartial x, GvPartial y) {
-  if (x.code == 0) return y;
-  if (y.code == 0) return x;
-  if (x.code < y.code) {
-    const GvPartial t = x;
-    x = y;
-    y = t;
+// x of the windows so far, and the limbs of a lower one that x's digits reach.
+// (The lower window's events have no digit above x's: theirs end at two limbs
+// above its first window, where the smallest top digit of that stands.)
+__device__ __forceinline__ GvPartial gv_bin_partial_more(GvPartial x, const unsigned* row, int L,
+                                                         int base) {
+  const int j = (x.pos - GV_POS_OFF + 2 * GV_SQ_OFF) / 22 - base;  // x's lowest digit; j >= 0
+  u128 r = {x.lo, x.hi};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const unsigned long long v = j + i < L ? row[j + i] : 0u;
+    const int sh = 22 * i;  // at most 66
+    r = add128(r, sh < 64 ? u128{v << sh, sh ? v >> (64 - sh) : 0ull} : u128{0ull, v << (sh - 64)});
   }
-  const u192 s = sar192(u192{y.lo, y.hi, 0ull}, 2 * (x.code - y.code));
-  const u128 r = add128(u128{x.lo, x.hi}, u128{s.l0, s.l1});
-  return gv_partial_norm(r.lo, r.hi, x.code);
+  return GvPartial{r.lo, r.hi, x.pos};
 }
-// A histogram bin's partial of w: 96-bit two's complement in units of
-// 2^(F - GV_BIN_QBITS), from its row of signed 21-bit digits.
+// A histogram bin's partial of w: two's complement, from its row of signed 21-bit
+// digits.
 __device__ __forceinline__ GvPartial gv_hist_partial(const int* row, int rows, int hbase) {
   int t = rows - 1;
   int a = row[t];
   while (a == 0 && t > 0) a = row[--t];
-  if (a == 0) return GvPartial{0ull, 0u, 0};
+  if (a == 0) return GvPartial{0ull, 0ull, 0};
   u192 v = {(unsigned long long)(long long)a, (unsigned long long)((long long)a >> 63), 0ull};
 #pragma unroll
   for (int i = 1; i <= 3; ++i) {
@@ -347,28 +378,19 @@ __device__ __forceinline__ GvPartial gv_hist_partial(const int* row, int rows, i
     const unsigned long long ext = (unsigned long long)(q >> 63);
     add192(v, u192{(unsigned long long)q, ext, ext});
   }
-  return GvPartial{v.l0, (unsigned)v.l1,
-                   21 * (hbase + t - 3) - GV_W21_OFF + GV_BIN_QBITS + GV_BINE_OFF};
+  return GvPartial{v.l0, v.l1, 21 * (hbase + t - 3) - GV_W21_OFF + GV_POS_OFF};
 }
+// The sum of two (a later pass over lower weights): the lower one aligned to the
+// higher one's unit, bits below it dropped.  (|value| < 2^95: no overflow.)
 __device__ __forceinline__ GvPartial gv_hist_partial_add(GvPartial x, GvPartial y) {
-  if (x.code == 0) return y;
-  if (y.code == 0) return x;
-  if (x.code < y.code) {
+  if (x.pos == 0) return y;
+  if (y.pos == 0) return x;
+  if (x.pos < y.pos) {
     const GvPartial t = x;
     x = y;
     y = t;
   }
-  const unsigned long long xh = (unsigned long long)(long long)(int)x.hi;
-  const unsigned long long yh = (unsigned long long)(long long)(int)y.hi;
-  const unsigned long long ye = (unsigned long long)((long long)yh >> 63);
-  const u192 s = sar192(u192{y.lo, yh, ye}, x.code - y.code);
-  u192 r = {x.lo, xh, (unsigned long long)((long long)xh >> 63)};
-  add192(r, s);
-  // |x|, |y| < 2^95: halve if the sum leaves 95 bits (it stays two's complement)
-  const long long top = (long long)r.l1;
-  if (top != (long long)(int)top) {
-    r = sar192(r, 1);
-    x.code += 1;
-  }
-  return GvPartial{r.l0, (unsigned)r.l1, x.code};
+  const u192 s = sar192(u192{y.lo, y.hi, (unsigned long long)((long long)y.hi >> 63)}, x.pos - y.pos);
+  const u128 r = add128(u128{x.lo, x.hi}, u128{s.l0, s.l1});
+  return GvPartial{r.lo, r.hi, x.pos};
 }

@@ -8,8 +8,8 @@
 // range of tiles; its 8 warps stride over the tiles, the warps' sums are combined
 // in shared memory and published.  All of them form a slot's sum by the rule of
 // gv_slotsum.cuh (channel sums: at the tiles' scales; bin sums: at the bins' own
-// exponent codes, gv_limbs.cuh).  No sum is formed with atomics, and none depends
-// on the order of its tiles: the totals are the same in every kernel, launch shape
+// positions, gv_limbs.cuh).  No sum is formed with atomics, and none depends on
+// the order of its tiles: the totals are the same in every kernel, launch shape
 // and batch.
 //
 // Tickets instead of waiting: each CTA publishes its sums and counts itself
@@ -454,30 +454,32 @@ __host__ __device__ inline int gv_axes_per_block(int N) {
 
 #define GV_RED_TILES_PER_LOAD 8
 
-// Tile partials.  Channel slots: 128-bit two's complement at
-// 2^(pw e - GV_FB), e the tile's scale; bin slots (axis bins and histogram bins):
-// a 96-bit value, unsigned for sums of w^2 (pw = 2) or two's complement for the
-// histogram's sums of w (pw = 1, sgn), at
-// 2^(pw (e - GV_BINE_OFF) - GV_BIN_QBITS), e its exponent code.
-//
-// Bit position and top word of a partial v of tile t; one slot's partials.
+// One slot's tile partials.  Channel slots: 128-bit two's complement at
+// 2^(pw e - GV_FB), e the tile's scale, pw = 1 (sums of v) or 2 (of v^2); bin slots
+// (axis bins and histogram bins): 112 bits and their position (GvPartial).
 struct SlotPartials {
   const ulonglong2* src;
   size_t stride;
   const int* tileE;
   int nch, pw;
-  bool bin, sgn;
+  bool bin;
+  __device__ __forceinline__ SlotPartials(const GvReduceArgs& a, int k, size_t first, size_t stride_)
+      : src(a.part + first),
+        stride(stride_),
+        tileE(a.tileE + (k >> 1)),
+        nch(a.nch),
+        pw((k & 1) + 1),
+        bin(a.has_bins && k >= 2 * a.nch) {}
   __device__ __forceinline__ ulonglong2 load(int t) const { return __ldcg(src + t * stride); }
+  // bit position of a partial v of tile t (0: none), and its top word
   __device__ __forceinline__ int position(const ulonglong2& v, int t) const {
-    if (bin) {
-      const int e = (int)(v.y >> 32);
-      return e == 0 ? 0 : pw * (e - GV_BINE_OFF) - GV_BIN_QBITS + GV_POS_OFF;
-    }
+    if (bin) return (int)(v.y >> 48);
     const int e = __ldcg(tileE + (size_t)t * nch);
     return e == GV_EMPTY ? 0 : pw * e - GV_FB + GV_POS_OFF;
   }
   __device__ __forceinline__ unsigned word3(const ulonglong2& v) const {
-    return bin ? (sgn ? (unsigned)((int)v.y >> 31) : 0u) : (unsigned)(v.y >> 32);
+    const unsigned h = (unsigned)(v.y >> 32);
+    return bin ? (unsigned)(int)(short)h : h;
   }
 };
 // The partials t0 + g step below nt, g < G, and their positions (0: none): every
@@ -649,19 +651,13 @@ __device__ __forceinline__ void gv_reduce_task(const GvReduceArgs& a, int bx, in
   const int gx = (a.nacc + 31) / 32, gy = nblk / gx;
   const int t0 = by * a.tiles_per_cta;
   const int t1 = min(a.n_tiles, t0 + a.tiles_per_cta);
-  const bool bin = a.has_bins && k >= 2 * a.nch;
-  // the histogram's sums of w: the last nhist slots
-  const bool hw = bin && a.nhist > 0 && k >= a.nacc - a.nhist;
-  const int pw = hw ? 1 : (bin ? 2 : (k & 1) + 1);
   const size_t row = 32 * (size_t)gx;  // of the published sums: [range][counters, window][row]
   gv_wait_prior_grid();
 
   // ---- A: this CTA's tiles
   GvAcc sum = acc_zero();
   if (k < a.nacc)
-    sum = sum_tiles<GV_RED_TILES_PER_LOAD / 2>(
-        SlotPartials{a.part + k, (size_t)a.nacc, a.tileE + (k >> 1), a.nch, pw, bin, hw}, t0 + wid,
-        0, 8, t1);
+    sum = sum_tiles<GV_RED_TILES_PER_LOAD / 2>(SlotPartials(a, k, k, a.nacc), t0 + wid, 0, 8, t1);
   int g;
   unsigned long long t = task_combine(mem, sum, &g);
   if (wid <= GV_SLOT_WORDS) {
@@ -781,12 +777,7 @@ __global__ void __launch_bounds__(256, 3) gv_reduce_slots_kernel(const GvReduceA
   __shared__ int s_won, s_fin;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int k = blockIdx.x;
-  const bool bin = a.has_bins && k >= 2 * a.nch;
-  // the histogram's sums of w: the last nhist slots
-  const bool hw = bin && a.nhist > 0 && k >= a.nacc - a.nhist;
-  const int pw = hw ? 1 : (bin ? 2 : (k & 1) + 1);
-  const SlotPartials part = {a.part + (size_t)k * a.n_tiles, 1, a.tileE + (k >> 1), a.nch, pw, bin,
-                             hw};
+  const SlotPartials part(a, k, (size_t)k * a.n_tiles, 1);
   gv_wait_prior_grid();
   const int nt = a.tiles_used ? min(a.n_tiles, __ldcg(a.tiles_used)) : a.n_tiles;
   GvAcc sum = warp_sum_acc(sum_tiles<GV_RED_TILES_PER_LOAD>(part, tid, lane, 256, nt),
@@ -890,10 +881,8 @@ __global__ void __launch_bounds__(kClusterThreads) gv_reduce_cluster_kernel(cons
   }
   for (int s = wid * kClusterCtas + rank; s < n; s += kClusterSlots) {
     const int k = k0 + s;
-    const bool bin = !channels, hw = bin && !axis && k >= a.nacc - a.nhist;
-    const int pw = hw ? 1 : (bin ? 2 : (k & 1) + 1);
     const double d = warp_sum_tiles<GV_RED_TILES_PER_LOAD>(
-        SlotPartials{a.part + (size_t)k * a.n_tiles, 1, a.tileE + (k >> 1), a.nch, pw, bin, hw}, nt);
+        SlotPartials(a, k, (size_t)k * a.n_tiles, 1), nt);
     if (lane == 0) {
       a.sums[k] = d;
       if (refine) gv_store_rank0(m.slope + s, d);
