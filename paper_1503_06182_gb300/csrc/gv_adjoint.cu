@@ -30,7 +30,8 @@ template <typename Real>
 struct AdjSmem {
   static constexpr bool F64 = GvForm<Real>::ID != GV_FORM_F32;
   static constexpr int WORDS = F64 ? 2 * kNch : kNch + 1;  // per event
-  static constexpr int ROWS = kL + gv_lane_rows(F64);      // per channel: of v^2, then of v
+  static constexpr int SQ = kL + (F64 ? GvSig<double>::LOW : 0);
+  static constexpr int ROWS = SQ + gv_lane_rows(F64);      // per channel: of v^2, then of v
   static constexpr size_t lanes = (size_t)WORDS * GV_TILE * 4;
   static constexpr size_t grid = lanes + (size_t)kNch * ROWS * 32 * 4;
 };
@@ -219,9 +220,10 @@ __global__ void __launch_bounds__(GV_TILE / EPT, AdjBlocks<Real, EPT>::value)
           const int pos = limb - win.x;
           if (pos >= 0) {
             unsigned l[4];
-            gv_square_digits(s, h + GV_SQ_OFF - 11 * limb, l);
-            gv_lane_add_square<W>(l, a_cols + (c * Lay::ROWS + pos) * 128);
-            gv_lane_add_w(s, a_cols + (c * Lay::ROWS + kL) * 128, win.y);
+            const int rem = h + GV_SQ_OFF - 11 * limb;
+            gv_square_digits(s, rem, l);
+            gv_lane_add_square(s, rem, l, a_cols + (c * Lay::ROWS + pos) * 128);
+            gv_lane_add_w(s, a_cols + (c * Lay::ROWS + Lay::SQ) * 128, win.y);
           } else {
             mE[c] = max(mE[c], s.e2);
           }
@@ -238,8 +240,9 @@ __global__ void __launch_bounds__(GV_TILE / EPT, AdjBlocks<Real, EPT>::value)
       if (!win.w) continue;
       const unsigned* col = cols + c * Lay::ROWS * 32;
       const u128 t =
-          (j & 1) ? gv_lane_total<false>(col, kL, 22 * win.x - 2 * GV_SQ_OFF - 2 * E + GV_FB)
-                  : gv_lane_total<true>(col + kL * 32, gv_lane_rows(F64),
+          (j & 1) ? gv_lane_total<false>(col, Lay::SQ, 22 * (win.x - GvSig<W>::LOW) -
+                                                           2 * GV_SQ_OFF - 2 * E + GV_FB)
+                  : gv_lane_total<true>(col + Lay::SQ * 32, gv_lane_rows(F64),
                                         22 * win.y - GV_SQ_OFF - E + GV_FB);
       if (lane == 0) s_sum[j] = add128(s_sum[j], t);
     }

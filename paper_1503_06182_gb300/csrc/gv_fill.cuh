@@ -311,7 +311,7 @@ struct GvPair<GvX> {
 //        hc copies (events of a warp share few bins of an observable with a
 //        peak: 8 passes per atomic for Drell-Yan masses, 4 with lane l adding
 //        to copy l % 4; ten iterations of 1e6 events with 60 bins 553 -> 537 us)
-//   lq   [L][32] u32, lw [rows][32] i32   the lanes' columns of w^2 and of w
+//   lq   [L (FP64: + 2)][32] u32, lw [rows][32] i32   the lanes' columns of w^2 and w
 // and beside both:
 //   bins [d][T]   u8      the events' bins (more than 4 axes), their high bytes
 //                         in as many again where N > 256
@@ -385,7 +385,7 @@ struct GvFillSmem {
     hw = hh + (forward ? nhist * L * 4 : 0);
     hs = forward && nhist > 0 ? copy_bytes(nhist, f64) : 0;
     lq = hh + hc * hs;
-    lw = lq + (forward ? L * 32 * 4 : 0);
+    lw = lq + (forward ? (L + (f64 ? GvSig<double>::LOW : 0)) * 32 * 4 : 0);
     const unsigned second = gv_align16(lw + (forward ? gv_lane_rows(f64, L) * 32 * 4 : 0));
     bins = first > second ? first : second;
     po = gv_align16(bins + ((forward && bins_smem) ? d * T * (N > 256 ? 2 : 1) : 0));
@@ -1056,8 +1056,9 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
         if (s.m != 0 && limb < up_w) {
           if (pos >= 0) {
             unsigned l[4];
-            gv_square_digits(s, h + GV_SQ_OFF - 11 * limb, l);
-            gv_lane_add_square<W>(l, a_lq + pos * 128);
+            const int rem = h + GV_SQ_OFF - 11 * limb;
+            gv_square_digits(s, rem, l);
+            gv_lane_add_square(s, rem, l, a_lq + pos * 128);
             gv_lane_add_w(s, a_lw, vw.wbase);
             if constexpr (!PLUS) add_bins(l, pos);
             if constexpr (HIST) {
@@ -1094,7 +1095,8 @@ __device__ __forceinline__ void gv_fill_tile(const GvFillArgs& a, long long tile
           hh[k] += hh[k + hsw] + hh[k + 2 * hsw] + hh[k + 3 * hsw];
     }
     if (have_w && wsum == 0)
-      add192(sum, gv_lane_sum<false>(lq, L, vw.base - gv_square_cut(E)));
+      add192(sum, gv_lane_sum<false>(lq, L + GvSig<W>::LOW,
+                                     vw.base - GvSig<W>::LOW - gv_square_cut(E)));
     else if (have_w && wsum == 1)
       add192(sum, gv_lane_sum<true>(reinterpret_cast<const unsigned*>(lw), gv_lane_rows(F64, L),
                                     vw.wbase - gv_w_cut(E)));

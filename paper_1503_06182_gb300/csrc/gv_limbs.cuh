@@ -129,6 +129,7 @@ struct GvSig;
 template <>
 struct GvSig<float> {
   static constexpr int H = 0;  // the square's digits are those of m^2 2^(2 (e2 + H))
+  static constexpr int LOW = 0;  // digits of the square below those
   static constexpr int BITS = 24;
   unsigned m;
   int e2;
@@ -136,7 +137,8 @@ struct GvSig<float> {
 };
 template <>
 struct GvSig<double> {
-  static constexpr int H = 21;  // of floor(m^2 2^-42), 64 bits
+  static constexpr int H = 21;   // of floor(m^2 2^-42), 64 bits
+  static constexpr int LOW = 2;  // the other 42 bits
   static constexpr int BITS = 53;
   unsigned long long m;
   int e2;
@@ -153,7 +155,7 @@ __device__ __forceinline__ void gv_square_digits(const GvSig<float>& w, int rem,
   l[2] = (__funnelshift_r(lo, hi, 24u) >> (20u - s)) & GV_LIMB_MASK;
   l[3] = rem == 10 ? hi >> 14 : 0u;
 }
-// FP64: the high 64 bits of the 106-bit square (truncated below 2^-62 of it).
+// FP64: the high 64 bits of the 106-bit square.
 __device__ __forceinline__ void gv_square_digits(const GvSig<double>& w, int rem,
                                                  unsigned (&l)[4]) {
   const unsigned long long P = __umul64hi(w.m << 11, w.m << 11);
@@ -162,6 +164,15 @@ __device__ __forceinline__ void gv_square_digits(const GvSig<double>& w, int rem
   l[1] = __funnelshift_r((unsigned)P, (unsigned)(P >> 32), 22u - s) & GV_LIMB_MASK;
   l[2] = (unsigned)(P >> (44u - s)) & GV_LIMB_MASK;
   l[3] = (unsigned)(P >> 46) >> (20u - s);
+}
+// The low 42 bits: the two digits below l[0] and the bits of l[0] below s (zero
+// there).  The tile's own sums take them, the bins do not (a bin drops digits of
+// that size anyway).
+__device__ __forceinline__ void gv_square_low(const GvSig<double>& w, int rem, unsigned (&l)[3]) {
+  const unsigned long long q = (w.m * w.m & 0x3FFFFFFFFFFull) << (2u * (unsigned)rem + 2u);
+  l[0] = (unsigned)q & GV_LIMB_MASK;
+  l[1] = (unsigned)(q >> 22) & GV_LIMB_MASK;
+  l[2] = (unsigned)(q >> 44);
 }
 
 // The window of one pass: the squares' limb indices [base, base + L - 4] (their
@@ -205,15 +216,24 @@ __device__ __forceinline__ void gv_lane_add_w(const GvSig<double>& w, unsigned l
   gv_red<256>(p, gv_signed_digit((unsigned)(w.m >> (44u - sh)) & GV_LIMB_MASK, s));
   gv_red<384>(p, gv_signed_digit((unsigned)(w.m >> 45) >> (21u - sh), s));
 }
-template <typename Real>
-__device__ __forceinline__ void gv_lane_add_square(const unsigned (&l)[4], unsigned p) {
+// (p: the row of the lowest digit, LOW rows below l[0]'s)
+__device__ __forceinline__ void gv_lane_add_square(const GvSig<float>& w, int rem,
+                                                   const unsigned (&l)[4], unsigned p) {
   gv_red<0>(p, l[0]);
   gv_red<128>(p, l[1]);
   gv_red<256>(p, l[2]);
-  if constexpr (sizeof(Real) == 8)
-    gv_red<384>(p, l[3]);
-  else
-    gv_red_nonzero<384>(p, l[3]);
+  gv_red_nonzero<384>(p, l[3]);
+}
+__device__ __forceinline__ void gv_lane_add_square(const GvSig<double>& w, int rem,
+                                                   const unsigned (&l)[4], unsigned p) {
+  unsigned low[3];
+  gv_square_low(w, rem, low);
+  gv_red<0>(p, low[0]);
+  gv_red<128>(p, low[1]);
+  gv_red<256>(p, l[0] | low[2]);
+  gv_red<384>(p, l[1]);
+  gv_red<512>(p, l[2]);
+  gv_red<640>(p, l[3]);
 }
 // The square's digits into a bin's row at address p.
 template <typename Real>
@@ -253,6 +273,7 @@ __device__ __forceinline__ u128 gv_lane_total(const unsigned* col, int rows, int
   long long mine = 0;
   // a row of unsigned digits adds up to less than 2^32: those below 2^-32 of a
   // unit are nothing
+#pragma unroll 4
   for (int j = SIGNED ? 0 : max(0, (-32 - p) / GV_LIMB_BITS); j < rows; ++j) {
     const unsigned v = col[j * 32 + lane];
     long long s;
