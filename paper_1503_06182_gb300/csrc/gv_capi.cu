@@ -108,7 +108,8 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 constexpr int kHostRecMax = 64;  // iterations whose records fit the mapped result block
 constexpr size_t kHostRecOff = 256;  // byte offset of the records in it
-constexpr size_t kHostGridOff = kHostRecOff + kHostRecMax * 2 * sizeof(double);  // of the edges
+constexpr size_t kHostItOff = kHostRecOff + kHostRecMax * 2 * sizeof(double);  // of the counter
+constexpr size_t kHostGridOff = kHostItOff + 64;                               // of the edges
 static_assert(sizeof(GvState) <= kHostRecOff, "state fits before the records");
 
 // Autotuner cache: best events-per-thread per (integrand, precision, mode,
@@ -193,13 +194,17 @@ struct vegas_ctx {
   // fetching them is a synchronisation, not two copies
   void* hres = nullptr;
   void* hres_dev = nullptr;
-  // the grid's edges as the host knows them, in the same block: written by
-  // the host with a grid, and by the refinement of a stage's last iteration
+  // the grid's edges and the iteration counter in the same block: written by
+  // the host with a grid or a state, and by the device in a stage's last
+  // iteration (whoever launched it: a caller may have captured it).  stale: the
+  // launches of a stage failed part way, so the device alone knows them
   double* hgrid = nullptr;
-  // the iteration counter: stages advance it by their iterations
-  unsigned long long it = 0;
-  bool in_flight = false;  // a stage was enqueued and not waited for yet
-  std::vector<double> upload;  // staging of a grid on its way to the device
+  volatile unsigned long long* hit = nullptr;
+  bool stale = false;
+  std::vector<double> upload;  // a grid on its way to the device
+  // something was enqueued and not waited for yet; captured: a caller captured a
+  // stage and may replay it at any time
+  bool in_flight = false, captured = false;
   bool last_zero_copy = false;
   // derived constants currently on the device
   int consts_ig = -1;
@@ -489,7 +494,10 @@ GvReduceArgs reduce_args(const vegas_ctx* c, const Plan& p, int k) {
     r.host_st = (GvState*)c->hres_dev;
     r.host_rec = (double*)((char*)c->hres_dev + kHostRecOff);
   }
-  if (c->hres_dev && !c->tuning) r.host_grid = (double*)((char*)c->hres_dev + kHostGridOff);
+  if (c->hres_dev && !c->tuning) {
+    r.host_grid = (double*)((char*)c->hres_dev + kHostGridOff);
+    r.host_it = (unsigned long long*)((char*)c->hres_dev + kHostItOff);
+  }
   if (p.plus) r.tiles_used = c->pa.tiles_used;
   r.k = k;
   r.last = k == p.itmx - 1;
@@ -951,10 +959,17 @@ int enqueue_stage(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* p
       }
       evp = &ge->events;
     }
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess)
+      cudaGetLastError();  // (the legacy stream while another one captures)
+    else if (cs != cudaStreamCaptureStatusNone)
+      c->captured = true;
     st = enqueue_body(c, p, evp, false);
-    if (st) return st;
+    if (st) {
+      c->stale = true;
+      return st;
+    }
     if (evp) c->pending_events = *evp;
-    c->it += (unsigned long long)itmx;
     c->pending = true;
     return VEGAS_OK;
   }
@@ -991,7 +1006,6 @@ int enqueue_stage(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* p
   }
   GV_TRY(cudaGraphLaunch(ge->exec, c->stream));
   c->pending_events = ge->events;
-  c->it += (unsigned long long)itmx;
   c->pending = true;
   return VEGAS_OK;
 }
@@ -1062,25 +1076,39 @@ int valid_grid(const double* e, int d, int N) {
   return 1;
 }
 
-// Wait for what is enqueued, if anything.
-int settle(vegas_ctx* c) {
-  if (c->in_flight) GV_TRY(cudaStreamSynchronize(c->stream));
-  c->in_flight = false;
+// The iteration counter, the context's work done.
+int read_counter(const vegas_ctx* c, unsigned long long* it) {
+  if (c->hit && !c->stale) {
+    *it = *c->hit;
+    return VEGAS_OK;
+  }
+  GvState hs;
+  GV_TRY(cudaMemcpy(&hs, c->st, sizeof hs, cudaMemcpyDeviceToHost));
+  *it = hs.it;
   return VEGAS_OK;
 }
 
-// Enqueue a grid (and, with set_it, the iteration counter c->it).  The caller
-// has waited for earlier stages, which write the host's copy of the grid.
-int upload_grid(vegas_ctx* c, const double* edges, bool set_it) {
+// Enqueue a grid and, unless it is null, the iteration counter.  Waits for earlier
+// work first, if there is any: it may write the host's copy of the grid, or still
+// read `upload`.  (Waiting for an idle stream costs 2 to 3 us.)
+int upload_grid(vegas_ctx* c, const double* edges, const unsigned long long* it) {
   const size_t n = (size_t)c->ndim * (c->nbins + 1);
-  // from pageable memory of the context's own: staged before the call
-  // returns, whatever memory the caller's edges are in
+  if (c->in_flight || c->captured) GV_TRY(cudaStreamSynchronize(c->stream));
+  c->in_flight = true;
+  if (c->hgrid) {
+    unsigned long long now = 0;
+    const int st = it ? VEGAS_OK : read_counter(c, &now);
+    if (st) return st;
+    memcpy(c->hgrid, edges, n * sizeof(double));
+    *c->hit = it ? *it : now;
+    c->stale = false;
+  }
+  // from memory of the context's own, whatever memory the caller's edges are in
   c->upload.assign(edges, edges + n);
   GV_TRY(cudaMemcpyAsync(c->grid + GvGridLayout{c->ndim, c->nbins}.off_e64(), c->upload.data(),
                          n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  GV_TRY(gv::launch_grid_pack(c->ndim, c->nbins, c->grid, set_it ? c->st : nullptr, c->it,
+  GV_TRY(gv::launch_grid_pack(c->ndim, c->nbins, c->grid, it ? c->st : nullptr, it ? *it : 0ull,
                               c->stream));
-  if (c->hgrid) memcpy(c->hgrid, edges, n * sizeof(double));
   return VEGAS_OK;
 }
 
@@ -1144,6 +1172,8 @@ int vegas_init(int ndim, int nbins, uint64_t seed, vegas_ctx** out) {
       c->hres_dev = nullptr;
     } else {
       c->hgrid = (double*)((char*)c->hres + kHostGridOff);
+      c->hit = (volatile unsigned long long*)((char*)c->hres + kHostItOff);
+      *c->hit = 0ull;
     }
   } else {
     cudaGetLastError();
@@ -1190,7 +1220,7 @@ int vegas_init(int ndim, int nbins, uint64_t seed, vegas_ctx** out) {
     std::vector<double> e((size_t)ndim * (nbins + 1));
     for (int a = 0; a < ndim; ++a)
       for (int i = 0; i <= nbins; ++i) e[(size_t)a * (nbins + 1) + i] = (double)i / nbins;
-    st = upload_grid(c, e.data(), false);
+    st = upload_grid(c, e.data(), nullptr);
     if (!st && cudaStreamSynchronize(c->stream) != cudaSuccess) st = VEGAS_ECUDA;
   }
   if (st) {
@@ -1279,7 +1309,7 @@ int vegas_set_option(vegas_ctx* c, int key, double v) {
 
 int vegas_set_stream(vegas_ctx* c, void* stream) {
   if (!c) return VEGAS_EINVAL;
-  if (c->stream) cudaStreamSynchronize(c->stream);
+  cudaStreamSynchronize(c->stream);  // (the legacy stream's work too: a grid may be on its way)
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   c->own_stream = false;
   c->stream = (cudaStream_t)stream;
@@ -1452,7 +1482,7 @@ int vegas_grid_get(const vegas_ctx* c, double* edges) {
   if (!c || !edges) return VEGAS_EINVAL;
   const size_t n = (size_t)c->ndim * (c->nbins + 1);
   GV_TRY(cudaStreamSynchronize(c->stream));
-  if (c->hgrid) {
+  if (c->hgrid && !c->stale) {
     memcpy(edges, c->hgrid, n * sizeof(double));
     return VEGAS_OK;
   }
@@ -1464,8 +1494,7 @@ int vegas_grid_get(const vegas_ctx* c, double* edges) {
 int vegas_grid_set(vegas_ctx* c, const double* edges) {
   if (!c || !edges) return VEGAS_EINVAL;
   if (!valid_grid(edges, c->ndim, c->nbins)) return VEGAS_EGRID;
-  const int st = settle(c);
-  return st ? st : upload_grid(c, edges, false);
+  return upload_grid(c, edges, nullptr);
 }
 
 int vegas_state_size(const vegas_ctx* c, size_t* bytes) {
@@ -1484,14 +1513,19 @@ int vegas_state_get(const vegas_ctx* c, void* buf, size_t bytes) {
   h.ndim = c->ndim;
   h.nbins = c->nbins;
   h.seed = c->seed;
-  h.it = c->it;
+  int st = vegas_grid_get(c, (double*)((char*)buf + sizeof h));  // (waits)
+  if (st) return st;
+  unsigned long long it = 0;
+  st = read_counter(c, &it);
+  if (st) return st;
+  h.it = it;
   h.batch = c->batch;
   h.fp32 = c->fp32;
   h.adapt = c->adapt;
   h.nonfinite_policy = c->nonfinite_policy;
   h.alpha = c->alpha;
   memcpy(buf, &h, sizeof h);
-  return vegas_grid_get(c, (double*)((char*)buf + sizeof h));
+  return VEGAS_OK;
 }
 
 int vegas_state_set(vegas_ctx* c, const void* buf, size_t bytes) {
@@ -1505,8 +1539,6 @@ int vegas_state_set(vegas_ctx* c, const void* buf, size_t bytes) {
   std::vector<double> e((size_t)c->ndim * (c->nbins + 1));
   memcpy(e.data(), (const char*)buf + sizeof h, e.size() * sizeof(double));
   if (!valid_grid(e.data(), c->ndim, c->nbins)) return VEGAS_EGRID;
-  const int st = settle(c);
-  if (st) return st;
   c->seed = h.seed;
   c->batch = h.batch;
   c->fp32 = h.fp32;
@@ -1514,9 +1546,9 @@ int vegas_state_set(vegas_ctx* c, const void* buf, size_t bytes) {
   c->nonfinite_policy = h.nonfinite_policy;
   c->alpha = h.alpha;
   // (captured stages stay: they are looked up by everything set here)
-  c->it = h.it;
   c->plus_valid = false;  // a VEGAS+ allocation is not part of a checkpoint
-  return upload_grid(c, e.data(), true);
+  const unsigned long long it = h.it;
+  return upload_grid(c, e.data(), &it);
 }
 
 int vegas_eval_events(vegas_ctx* c, int id, const double* params, int np, uint32_t iteration,

@@ -198,6 +198,7 @@ struct GvReduceArgs {
   GvState* host_st = nullptr;
   double* host_rec = nullptr;
   double* host_grid = nullptr;   // and the grid's edges [ndim][nbins + 1] after the last iteration
+  unsigned long long* host_it = nullptr;  // and the counter
   int refine_follows;            // 1: each axis is refined by the CTA that completes it
   long long ncall;
   double inv_c, inv_cm1, inv_m1; // 1/C, 1/(C-1), 1/(k) for chi2/dof at the last iteration
