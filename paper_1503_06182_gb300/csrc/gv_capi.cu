@@ -546,8 +546,6 @@ cudaError_t launch_fill_plan(const vegas_ctx* c, const Plan& p, int ept, bool pd
   return launch_fill_any(p.ig, p.form, ept, a, p.n_tiles, p.smem, c->stream, pdl);
 }
 
-// Pick events per thread by timing one fill launch per candidate.  Runs
-// between two setup kernels, so the trial launches leave no trace.
 int enqueue_body(vegas_ctx* c, const Plan& p, std::vector<cudaEvent_t>* ev, bool capture);
 
 // Events per thread for a plain forward stage, by timing what a stage runs:
@@ -627,8 +625,11 @@ int autotune_chained(vegas_ctx* c, Plan& p, const std::string& key) {
   return VEGAS_OK;
 }
 
+// Events per thread of a stage: a gradient stage's by timing one fill launch per
+// candidate, between two setup kernels, so that the trial launches leave no trace.
 int autotune(vegas_ctx* c, Plan& p) {
-  const std::string key = tune_key(c->device, p.ig, p.form, p.mode, c->ndim, c->nbins, p.tile_events, p.n_tiles);
+  const std::string key =
+      tune_key(c->device, p.ig, p.form, p.mode, c->ndim, c->nbins, p.tile_events, p.n_tiles);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(key);
@@ -637,22 +638,17 @@ int autotune(vegas_ctx* c, Plan& p) {
       return VEGAS_OK;
     }
   }
-  if (p.mode == 0 && !p.plus && !p.nhist) return autotune_chained(c, p, key);
-  const int cands_fwd[] = {1, 2, 4, 8};
-  const int cands_adj[] = {1, 2, 4};
-  const int* cands = p.mode ? cands_adj : cands_fwd;
-  const int nc = p.mode ? 3 : 4;
+  // (forward stages with a histogram or strata have one shape)
+  if (p.mode == 0) return autotune_chained(c, p, key);
   cudaEvent_t e0, e1;
   GV_TRY(cudaEventCreate(&e0));
   GV_TRY(cudaEventCreate(&e1));
-  // the fastest candidate, but 4 events per thread (the best for every forward
-  // fill measured) unless another is more than 2% faster: a few trial launches
-  // are noisy enough to flip a 10% difference now and then
+  // the fastest candidate, but 4 events per thread unless another is more than 2%
+  // faster: a few trial launches are noisy enough to flip a 10% difference now and
+  // then
   float best = 1e30f, t4 = 1e30f;
   int best_ept = 4;
-  for (int i = 0; i < nc; ++i) {
-    const int ept = cands[i];
-    if (c->ndim > 8 && ept == 8) continue;
+  for (const int ept : {1, 2, 4}) {
     cudaError_t err = launch_fill_plan(c, p, ept);  // warm-up
     if (err != cudaSuccess) {
       cudaGetLastError();
@@ -734,7 +730,7 @@ int make_plan(vegas_ctx* c, int64_t ncall, int itmx, int ig, const double* param
                            p.plus != 0, false);
     const GvFillSmem words(c->ndim, c->nbins, p.form, mode == 0, c->ndim > 4, p.nhist,
                            p.plus != 0, true);
-    p.hoist = gv_fill_hoistable(mode == 0, p.plus != 0, c->ndim) &&
+    p.hoist = gv_fill_hoistable(mode == 0, c->ndim) &&
                       words.total <= GV_WORDS_SMEM_MAX
                   ? 1
                   : 0;

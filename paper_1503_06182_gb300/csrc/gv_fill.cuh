@@ -329,8 +329,7 @@ __host__ __device__ inline unsigned gv_align16(unsigned b) { return (b + 15u) & 
 // would take the layout past GV_WORDS_SMEM_MAX (the host sets
 // GvFillArgs::hoist accordingly).
 #define GV_WORDS_SMEM_MAX (200 * 1024)
-__host__ __device__ inline bool gv_fill_hoistable(bool forward, bool plus, int d) {
-  (void)plus;  // the stratified fill stratifies the hoisted words after its wait
+__host__ __device__ inline bool gv_fill_hoistable(bool forward, int d) {
   return forward && d <= 8;
 }
 

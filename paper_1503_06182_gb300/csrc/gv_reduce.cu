@@ -80,13 +80,11 @@ __device__ __forceinline__ void gv_bar(int id, int nthr) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthr) : "memory");
 }
 
-// The iteration's finalisation, by the threads [0, nthr) of a group (local
-// thread index tid, barrier id bar): the iteration record, the stage's
-// combination and the per-iteration state.
-__device__ void finalize_iteration(const GvReduceArgs& a, int tid, int nthr, int bar) {
+// The iteration's finalisation, by one warp of a group (tid: the thread's index in
+// the group): the iteration record, the stage's combination and the per-iteration
+// state.
+__device__ void finalize_iteration(const GvReduceArgs& a, int tid) {
   const int lane = tid & 31, wid = tid >> 5;
-  (void)nthr;
-  (void)bar;
   GvState* st = a.st;
   // the sums, each rounded once to FP64 by the CTA that completed its block
   if (wid == 0) {
@@ -732,12 +730,10 @@ __device__ __forceinline__ void gv_reduce_task(const GvReduceArgs& a, int bx, in
   // ---- C
   if (n_won) __threadfence();  // the other blocks' sums, published before their tickets
   // the won axes and the finalisation side by side on groups of warps: the
-  // finalisation takes warp 7 (all warps if no axis was won), the axes the
-  // other warps, min(n_won, 7) groups, each with its own barrier and shared
-  // memory
-  if (fin && (n_won == 0 || wid == 7)) {
-    const int nw = n_won == 0 ? 8 : 1, w0 = 8 - nw;
-    finalize_iteration(a, threadIdx.x - 32 * w0, 32 * nw, 1);
+  // finalisation takes warp 7, the axes the other warps, min(n_won, 7) groups,
+  // each with its own barrier and shared memory
+  if (fin && wid == 7) {
+    finalize_iteration(a, threadIdx.x - 32 * 7);
   } else if (n_won > 0) {
     const int ng = min(n_won, 7), wpg = (fin ? 7 : 8) / ng, q = wid / wpg;
     if (q < ng) {
@@ -827,7 +823,7 @@ __global__ void __launch_bounds__(256, 3) gv_reduce_slots_kernel(const GvReduceA
   __threadfence();  // the other slots' sums, published before their tickets
   gv_allow_next_grid();  // what is left is short: the next fill's CTAs may come in
   if (fin)
-    finalize_iteration(a, tid, 256, 1);
+    finalize_iteration(a, tid);
   else
     refine_axis<false>(a, won, sm, tid, 256, 2, 0);
 }
@@ -896,15 +892,15 @@ __global__ void __launch_bounds__(kClusterThreads) gv_reduce_cluster_kernel(cons
   if (rank != 0) return;
   const int nthr = min(kClusterThreads, (N + 31) & ~31);
   if (channels) {
-    if (wid == 0) finalize_iteration(a, lane, 32, 1);
+    if (wid == 0) finalize_iteration(a, lane);
   } else if (refine && tid < nthr) {
     refine_axis<true>(a, c, sm, tid, nthr, 2, 0);
   }
 }
 
 // Batched: one launch reduces many integrations; task i names the
-// integration and the block coordinates of CTA i.  Four CTAs per SM, as
-// above (72 registers otherwise).
+// integration and the block coordinates of CTA i.  Four CTAs per SM (64
+// registers).
 __global__ void __launch_bounds__(256, 4) gv_reduce_batch_kernel(const GvReduceArgs* args,
                                                               const int4* tasks, int k, int last,
                                                               double inv_m1) {

@@ -21,8 +21,8 @@ enum { GV_FORM_F64 = 0, GV_FORM_F32 = 1, GV_FORM_X64 = 2 };
 // with powers of two, 20.8 so; 20.9 if any saving counts).  Ten iterations with
 // 128 and with 1024 events a tile: 1e4 calls of the FP64 NLO-shaped weight on
 // 13 axes 297 and 619 us, of FP64 Drell-Yan 199 and 287, of FP32 Drell-Yan 159
-// and 162.  Against the powers of two: an FP64 fit step of 1e5 calls (149 tiles
-// of 672 instead of 98 of 1024) 585 and 495 us, the Gaussian on four axes 209
+// and 162.  Against the powers of two: an FP64 fit step of 1e5 calls (143 tiles
+// of 704 instead of 98 of 1024) 585 and 495 us, the Gaussian on four axes 209
 // and 197, ten iterations of 1e6 FP32 NLO events (1042 of 960) 750 and 727.
 inline int gv_tile_events(long long ncall, int form) {
   const long long t0 = form == GV_FORM_F32 ? 256 : 96;
