@@ -1125,8 +1125,10 @@ void reduce_grid(int n_tiles, int nacc, int* tiles_per_cta, int* gx, int* gy) {
   *gy = (n_tiles + tpc - 1) / tpc;
 }
 
+// Above 48 KB, static shared memory (up to 13.7 KB: the two-level reduce's sums)
+// included, a kernel has to opt in.
 static cudaError_t allow_smem(const void* k, size_t smem) {
-  if (smem <= 48 * 1024) return cudaSuccess;
+  if (smem + sizeof(GvTaskMem) + 1024 <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
