@@ -64,12 +64,12 @@ SM_COUNT, FP32_LANES_PER_SM, SM_MAX_MHZ = 152, 128, 2070.0
 # binding roofline.  Valid while the fill's sources are the ones captured
 # (their SHA-256 below) and only for the shape the timed run used; otherwise
 # both are reported as unknown (null).
-FILL_CAPTURES = {4: {"traffic_bytes": 36_096, "warp_instructions": 15_493_135},
-                 8: {"traffic_bytes": 36_096, "warp_instructions": 14_138_535}}
+FILL_CAPTURES = {4: {"traffic_bytes": 41_984, "warp_instructions": 15_803_631},
+                 8: {"traffic_bytes": 41_984, "warp_instructions": 14_419_855}}
 SMSP_PER_SM = 4
 FILL_SOURCES = ("gv_fill.cuh", "gv_fill_inst.cuh", "gv_fill_dy_f32.cu", "gv_integrands.cuh",
-                "gv_limbs.cuh", "gv_common.cuh")
-FILL_SOURCES_SHA256 = "d1c8431f6e49a6f234cd53b38c3a2df0f4c5a0eb77f2523a36dd5dc579e8ce36"
+                "gv_limbs.cuh", "gv_slotsum.cuh", "gv_tiles.cuh", "gv_common.cuh")
+FILL_SOURCES_SHA256 = "a3adece0f371600b1ced12c9811cda3194627379e14ccc91ca8e8f4d6f2c1e80"
 # HBM copy bandwidth measured by the driver on the GB300s (used when
 # MEASURED_PEAKS.json is absent: the profiling recipe's fallback)
 HBM_FALLBACK_GBS = 6800.0
@@ -400,7 +400,11 @@ def run_gpu(args):
                                 "peak_source": hbm_src, "frac": red_gbs / hbm}},
         "peaks_measured": peaks,
         "fp64_path": {"value": value64, "unit": UNIT,
-                      "roofline": {"bound": "fp64", "kernel": "gv_fill_kernel<drell_yan, double>",
+                      "roofline": {"bound": "alu (integer multiplies)",
+                                   "kernel": "gv_fill_kernel<drell_yan, GvX>",
+                                   "note": "the FP64 operations' count against the FP64 pipe's "
+                                           "rate; they run on 64-bit significands in the "
+                                           "integer pipes, so the fraction may pass 1",
                                    "kernel_avg_ms": fill64, "fp64_ops_per_event":
                                        FP64_OPS_PER_EVENT_DY, "achieved": ach64,
                                    "peak": peaks["dfma_tflops"], "unit": "TFLOP/s",

@@ -13,9 +13,9 @@
 // the weights, 48 KB); the second pass adds each value's and its square's
 // digits to per-lane columns of limbs (gv_limbs.cuh): about 45 instructions a
 // channel, where 128-bit shifts and adds in registers and a reduce-scatter of
-// twelve 128-bit sums per warp took twice that.  1e7 FP32 events on 4 axes: 370
-// before, 283 us now (1136 and 918 instructions per event, 83% of issue slots,
-// 1.7 warps waiting to issue); 1e5 FP64 events 75 and 38 us.
+// twelve 128-bit sums per warp took twice that.  1e8 FP32 events on 4 axes: 3.60
+// ms before, 2.74 now (1136 and 925 instructions per event, 84% of issue slots);
+// 1e5 FP64 events 75 and 38 us.
 #include "gv_fill_inst.cuh"
 
 namespace {

@@ -11,12 +11,12 @@
 //            finish converts the sums to FP64 and records the iteration.
 //
 // Exact accumulation.  Every tile takes its scale from its largest |v| (an
-// order-free max): E_t with max|v| < 2^E_t.  Each v is rounded once to an
-// integer multiple of 2^(E_t - GV_FB) (v^2 to 2^(2 E_t - GV_FB)); from then on
-// only integer additions happen, which are associative.  The result is
-// therefore bit-identical for any block size, events per thread, tile-to-CTA
-// schedule and batching -- the paper's "independent of the number of
-// threads" (Section 2.2) made exact -- and it is more accurate than the
+// order-free max): E_t with max|v| < 2^E_t.  It adds v and v^2 in integer digits,
+// exactly, and cuts the sums once to integer multiples of 2^(E_t - GV_FB) and
+// 2^(2 E_t - GV_FB); from then on only integer additions happen, which are
+// associative.  The result is therefore bit-identical for any block size, events
+// per thread, tile-to-CTA schedule and batching -- the paper's "independent of the
+// number of threads" (Section 2.2) made exact -- and it is more accurate than the
 // Kahan sums the paper uses for the same purpose.
 //
 // Bin sums carry their own scale.  The grid refinement compresses every

@@ -19,9 +19,9 @@
 // sums took 128-bit shifts, adds and shuffles in every thread; they now go to
 // per-lane columns of limbs with the same digits.  Bound by instruction issue
 // before and after.  One FP32 fill of 1e6 events alone, before and now:
-// Drell-Yan (4 axes) 28.7 and 22.3 us, 685 and 495 instructions per event;
-// NLO-shaped (13 axes) 97 and 50 us; with a 60-bin histogram 34.5 and 28.1 us;
-// 3-jet (5 axes, 1e7 events) 336 and 234 us.
+// Drell-Yan (4 axes) 28.7 and 22.0 us, 685 and 506 instructions per event;
+// NLO-shaped (13 axes) 97 and 50 us; with a 60-bin histogram 34.5 and 26.4 us;
+// 3-jet (5 axes, 1e7 events) 336 and 237 us.
 #pragma once
 #include "gv_common.cuh"
 #include "gv_slotsum.cuh"
