@@ -1305,7 +1305,8 @@ int vegas_set_option(vegas_ctx* c, int key, double v) {
 
 int vegas_set_stream(vegas_ctx* c, void* stream) {
   if (!c) return VEGAS_EINVAL;
-  cudaStreamSynchronize(c->stream);  // (the legacy stream's work too: a grid may be on its way)
+  // (of the legacy stream's work too, if there is any: a grid may be on its way)
+  if (c->stream || c->in_flight) cudaStreamSynchronize(c->stream);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   c->own_stream = false;
   c->stream = (cudaStream_t)stream;

@@ -484,19 +484,20 @@ struct SlotPartials {
 // The partials t0 + g step below nt, g < G, and their positions (0: none): every
 // load before the first use, and no branch among them (a load under a condition
 // that also uses it waits for it: 8 round trips through L2 instead of one).
-// Returns the highest position.
+// Returns the highest position.  (nt = 0 reads the first tile and takes nothing.)
 template <int G>
 __device__ __forceinline__ int load_tiles(const SlotPartials& s, int t0, int step, int nt,
                                           ulonglong2 (&v)[G], int (&pos)[G]) {
+  const int end = max(nt, 1) - 1;
   int top = 0;
 #pragma unroll
-  for (int g = 0; g < G; ++g) v[g] = s.load(min(t0 + g * step, nt - 1));
+  for (int g = 0; g < G; ++g) v[g] = s.load(min(t0 + g * step, end));
   if (s.bin) {
 #pragma unroll
     for (int g = 0; g < G; ++g) pos[g] = s.position(v[g], 0);
   } else {
 #pragma unroll
-    for (int g = 0; g < G; ++g) pos[g] = s.position(v[g], min(t0 + g * step, nt - 1));
+    for (int g = 0; g < G; ++g) pos[g] = s.position(v[g], min(t0 + g * step, end));
   }
 #pragma unroll
   for (int g = 0; g < G; ++g) {
